@@ -5,59 +5,92 @@
 // is the paper's decoding mask (figure "TiDAR Attention Masks"; Section 3.1): drafted
 // tokens causal, every mask block bidirectional inside itself and blind to the other
 // blocks.  The mask is never materialised: a query tile derives, from its rows' metadata,
-// which 64-key tiles it needs (cached pages up to the largest nvis, and only the local
+// which 64-key pages it needs (cached pages up to the largest nvis, and only the local
 // rows of the blocks it contains), skips all others, and applies the per-row bound only
-// on tiles that straddle it.
+// on pages that straddle it.
 //
-// Tiling: the G = Hq/Hkv query heads that share a KV head are packed into one 128-row
-// MMA tile (floor(128/G) slots x G heads), so K/V are read once per KV head.  Per key
-// tile: S = Q K^T (M 128, N 64, K hd) into TMEM (double buffered); the softmax warps read S
-// (one thread per row), keep a reference max and the running sum, and write P (bf16, two keys per
-// 32-bit column) back into the first half of the S buffer it came from; O += P V (M 128, N hd,
-// K 64, P as the tensor-memory operand, V as the MN-major shared-memory operand) accumulates in
-// TMEM over all key tiles.  P never touches shared memory: with P staged there the kernel moved
-// 128 KB through shared memory per key tile (Q 32 and K 16 read by Q K^T, P 16 written and read,
-// V 16, and the 32 KB the TMA writes), 1000 cycles at 128 B per cycle against 512 cycles of MMAs.
-// The reference max is only raised when a tile exceeds it by more than 2^8 (P stays <= 256,
+// Tiling: the G = Hq/Hkv query heads that share a KV head are packed into 128-row MMA tiles
+// (floor(128/G) slots x G heads), so K/V are read once per KV head.  A CTA runs two streams, A and B, of
+// (128-row query tile) x (64-key page) steps.  Per step j of stream T: S = Q_T K^T (M 128, N 64, K hd) into
+// TMEM (double buffered); the stream's four softmax warps read S (one thread per row), keep a reference max
+// and the running sum, and write P (bf16, two keys per 32-bit column) back over the first half of the
+// S buffer it came from; O_T += P V (M 128, N hd, K 64, P as the tensor-memory operand, V as the MN-major
+// shared-memory operand) accumulates in TMEM over all steps.  The streams take turns on the tensor pipe, and
+// each has the scores of its next step waiting when it finishes one, so neither the pipe nor the softmax warps wait
+// for the other's latency.
+// What bounds it: shared memory.  A step's operands are 64 KB read (Q 32, K 16, V 16) and up to 32 KB written by
+// the loads, 500 - 750 cycles at 128 B per cycle against 512 cycles of MMAs (a product with N = 64 takes 48 cycles, not
+// 32, for the 6 KB it reads); a step takes 0.53 - 0.56 us, 0.93 - 0.98 kcycles, on an SM.  Whole calls, 32/8
+// heads of 128, 272 rows, 1 k / 4 k / 16 k / 32 k cached positions: 22.6 / 33 / 85 / 156 us; the kernel before this one
+// (two CTAs per SM, one tile and one stream each, the same split for every sequence) took 26.4 / 40 / 97 / 197 us.
+//   PAIR of tiles: A and B are two query tiles, each K/V page serves both: half the loads, and 80
+//     instead of 96 KB through shared memory per step.
+//   SINGLE tile: A and B are the same query tile and take the pages in turn; their two results are merged through
+//     shared memory at the end.  Twice the parallelism for the same rows and half the partial results.
+//
+// One thread issues all MMAs, and a commit covers everything issued before it: the barrier that announces
+// the scores of step j + 2 (their products are issued right behind P V of step j, and the barrier is committed
+// to even when there are no such scores) also says that P V of step j has read its P and updated O.
+// The reference max is only raised when a step exceeds it by more than 2^8 (P stays <= 256,
 // exact enough in bf16/fp32); raising it rescales the rows of O in TMEM, which happens in the
-// first tiles only.  Barriers that either side can run ahead on exist once per S buffer (a
-// parity wait cannot tell two completions from none).  The CTA needs
-// <= 113 KB of shared memory, 256 TMEM columns and < 170 registers per thread, so two CTAs
-// share an SM and fill each other's dependency stalls.  The key range of a query tile can be
-// split over several CTAs; partial (max, sum, O) results are merged by attn_combine_kernel.
+// first steps only.
+//
+// As in the projections, the thread that issues MMAs never tests an mbarrier (the test would wait for the MMAs
+// queued before it and the pipe would run dry): a watcher warp does, and releases it through
+// hardware barriers.
+//
+// Work distribution.  Which CTA does what is planned on the device, once per pass (plan_block):
+// every layer of a pass has the same rows, hence the same query tiles and key ranges.  The plan decides whether
+// tiles are paired, cuts key ranges into items of about equal time, whatever the sequences' lengths
+// are, and lists long items first (a causal first pass would otherwise end on its longest rows).
+// Partial (max, sum, O) results of a tile with several items are merged by attn_combine_kernel.
 #pragma once
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 
 namespace attn_tc {
 
-constexpr int KT = 64;               // keys per tile (= page size)
-constexpr int K_STAGES = 3, V_STAGES = 2;   // K runs a tile further ahead: Q K^T of tile i + 1 is issued before P V of tile i
-constexpr int THREADS = 192;         // warp 0: TMA, warp 1: MMA, warps 2..5: softmax
-constexpr int MAX_SPLITS = 8;
+constexpr int PAGE = 64;             // keys per step (= page size)
+constexpr int STAGES = 5;            // K pages and V pages in flight, each
+constexpr int THREADS = 384;         // warp 0: K loads, 1: MMA, 2: watcher, 3: Q and V loads; warps 4..7 / 8..11: softmax of stream A / B
+constexpr int MAX_SPLITS = 32;       // items per tile
+constexpr int SLOTS_PER_SM = 2;      // partial results that fit the scratch = grid of a pass whose key ranges may be split
 constexpr float RAISE_THRESHOLD = 8.f;   // log2 units
 
-struct Args {
+// Pages [p_begin, p_end) of the query tile that covers slots [row0, min(row0 + spt, row_end)) of sequence slot `seq`
+// and, if pair, of the tile behind it.  Its keys in pages: n_cache_pages cached ones, then step-local rows from loc_lo on.
+struct __align__(16) Item { int32_t row0, row_end, seq, p_begin, p_end, n_cache_pages, loc_lo, pair, split, pad[3]; };
+// A query tile: its items are item0 .. item0 + n_items - 1 (n_items = 0: no rows); in a pair, sub says which half it is.
+struct __align__(16) Tile { int32_t row0, row_end, item0, n_items, sub, pad[3]; };
+
+// Units (up to two query tiles of one sequence) of a pass and where the plan goes.
+struct PlanArgs {
   int R;                    // rows (slots) of the pass
   int rows_per_group;       // slots per sequence group (k(k+1) for a step; R for a first pass)
-  int tiles_per_group;      // ceil(rows_per_group / spt)
-  int n_groups;
-  // Groups of different sizes (a step whose sequences use different block lengths): query tile t
-  // covers rows [tile_row0[t], tile_row0[t] + spt) of the group that ends at tile_rend[t]; null =
-  // equal groups, derived from rows_per_group.  n_tiles = number of query tiles in either case.
-  const int32_t *tile_row0, *tile_rend; int n_tiles;
+  int units_per_group;      // ceil(rows_per_group / (2 spt))
+  // Groups of different sizes (a step whose sequences use different block lengths): unit u
+  // covers rows [unit_row0[u], unit_row0[u] + 2 spt) of the group that ends at unit_rend[u]; null =
+  // equal groups, derived from rows_per_group.  n_units = number of units in either case.
+  const int32_t *unit_row0, *unit_rend; int n_units;
+  int spt;                  // slots per query tile = 128 / G
+  int Hkv;
+  int n_sms, max_items;     // items a pass may have; n_units = every unit is one item
+  Item *items; Tile *tiles; // out: [max_items] (unused ones are zero), [2 n_units] (only where items may be split)
+};
+
+struct Args {
   int spt;                  // slots per query tile = 128 / G
   int G, Hq, Hkv;
-  int splits;
-  const int32_t *seq, *nvis, *loc0, *nloc;   // per row
+  const Item *items; const Tile *tiles;
+  const int32_t *nvis, *loc0, *nloc;         // per row
   const int32_t *page_table; int pages_per_seq;
   int page_base_k, page_base_v;              // offsets in the page dimension of the K / V tensor maps
   float scale_log2;                          // log2(e) / sqrt(hd)
   bf16 *O;                                   // [R][Hq*hd]
-  float *part_O;                             // [splits][R][Hq][hd]  (splits > 1)
-  float *part_ml;                            // [splits][R][Hq][2]
+  float *part_O;                             // [CTA][tile of the pair][hd / 4][128 rows][4]: a warp's stores are contiguous
+  float2 *part_ml;                           // [CTA][tile of the pair][128 rows] (reference max, sum)
   int *status;
-  unsigned long long *tile_count;            // diagnostics: += key tiles this CTA visits (null = off)
+  unsigned long long *tile_count;            // diagnostics: += steps this CTA computes (null = off)
 };
 
 // Shared memory of one CTA; everything is dynamic so that the 1024-byte alignment the
@@ -65,59 +98,211 @@ struct Args {
 template <int HD>
 struct Smem {
   static constexpr int NH = HD / 64;                 // 64-element halves of a head
-  static constexpr int Q_BYTES = 128 * HD * 2;
-  static constexpr int KV_BYTES = KT * HD * 2;
+  static constexpr int Q_BYTES = 128 * HD * 2;       // one query tile
+  static constexpr int KV_BYTES = PAGE * HD * 2;
   static constexpr int Q_OFF = 0;
-  static constexpr int K_OFF = Q_OFF + Q_BYTES;
-  static constexpr int V_OFF = K_OFF + K_STAGES * KV_BYTES;
-  static constexpr int BAR_OFF = V_OFF + V_STAGES * KV_BYTES;    // mbarriers and a few words
-  static constexpr int TOTAL = BAR_OFF + 256;
-  static constexpr int TMEM_COLS = 256;              // 2 x 64 (S) + HD (O) <= 256
+  static constexpr int K_OFF = Q_OFF + 2 * Q_BYTES;
+  static constexpr int V_OFF = K_OFF + STAGES * KV_BYTES;
+  static constexpr int BAR_OFF = V_OFF + STAGES * KV_BYTES;      // mbarriers and a few words
+  static constexpr int TOTAL = BAR_OFF + 512;
+  static constexpr int XCHG_OFF = K_OFF;             // single tile: the streams' results, [stream][hd / 8][128 rows][4] floats; (max, sum) behind them
+  static constexpr int XCHG_ML_OFF = XCHG_OFF + 128 * HD * 4;
+  static constexpr int TMEM_COLS = 512;              // 2 streams x (2 x 64 (S) + HD (O)), rounded up to a power of two
 };
+static_assert(Smem<128>::XCHG_ML_OFF + 2 * 128 * 8 <= Smem<128>::BAR_OFF && Smem<64>::XCHG_ML_OFF + 2 * 128 * 8 <= Smem<64>::BAR_OFF, "exchange area fits the K/V rings");
 
 struct Ctl {                                         // lives at Smem::BAR_OFF
-  uint64_t q_full, k_full[K_STAGES], k_empty[K_STAGES], v_full[V_STAGES], v_empty[V_STAGES], s_full[2], s_empty[2], p_full[2];
+  uint64_t q_full, k_full[STAGES], k_empty[STAGES], v_full[STAGES], v_empty[STAGES], s_full[2][2], p_full[2][2];
   uint32_t tmem_base;
-  int abort_flag, max_nvis, loc_lo, loc_hi;
+  int abort_flag;
 };
-static_assert(sizeof(Ctl) <= 256, "control block must fit its slot");
+static_assert(sizeof(Ctl) <= 512, "control block must fit its slot");
+
+// Plans a pass's attention (see the head of this file); run by one whole block, a multiple of 128 threads.
+//
+// The entities of a plan are the units (tiles paired) or the tiles (not paired).  Every entity's key range is cut
+// into the fewest items of at most `limit` us.  Pairing and limit minimise an estimate of
+// the kernel's time: a CTA costs OVERHEAD us (first loads, first scores, result) and per page PAIR_PAGE or
+// SINGLE_PAGE us; a partial result costs its store (PAIR_STORE, SINGLE_STORE) and the merge kernel; CTAs beyond one per
+// SM run in later waves, of which on average half a CTA's time is lost at the end.
+// Everything is kept in shared memory until the plan is made: a trip to global memory and back costs as much as all
+// of the arithmetic.
+// (Measured inside the kernel, head_dim 128, all SMs busy: 1.05 us per page of a pair, 0.56 of a single tile.)
+constexpr float OVERHEAD = 5.f, PAIR_PAGE = 1.05f, SINGLE_PAGE = 0.56f, PAIR_STORE = 2.5f, SINGLE_STORE = 1.5f, MERGE = 3.f;
+constexpr int PLAN_UNITS = 256;                        // up to this many units are planned; beyond, every unit is one item
+constexpr int CAND = 32;                               // limits tried per pairing: longest / (1 + i / 2)
+
+// What a row sees: cached positions [0, nvis), local rows [loc0, loc0 + nloc).
+struct RowKeys { int nvis, loc0, nloc, seq; };
+
+template <typename ROW>
+__device__ inline void plan_block(const PlanArgs &p, ROW row_keys) {
+  struct Keys { short n_cache, n_pages; int loc_lo; };
+  __shared__ Keys keys[3][PLAN_UNITS];                 // tile 0, tile 1, the unit
+  __shared__ int unit_row0[PLAN_UNITS], unit_rend[PLAN_UNITS], unit_seq[PLAN_UNITS];
+  __shared__ float ent_us[3 * PLAN_UNITS];             // units, then tiles
+  __shared__ short ent_n[2 * PLAN_UNITS], order_s[2 * PLAN_UNITS], place_s[2 * PLAN_UNITS];
+  __shared__ int longest_us[2];                        // longest unit / tile, as float bits
+  __shared__ unsigned long long best;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+  const bool planned = p.n_units <= PLAN_UNITS, splits = p.max_items > p.n_units;
+  if (threadIdx.x == 0) best = ~0ull;
+  if (threadIdx.x < 2) longest_us[threadIdx.x] = 0;
+  __syncthreads();
+  for (int u = warp; u < p.n_units; u += n_warps) {
+    int row0, row_end;
+    if (p.unit_row0) { row0 = p.unit_row0[u]; row_end = p.unit_rend[u]; }
+    else {
+      const int i = u % p.units_per_group, grp = u / p.units_per_group;
+      row0 = grp * p.rows_per_group + i * 2 * p.spt;
+      row_end = min((grp + 1) * p.rows_per_group, p.R);
+    }
+    int nvis[2] = {0, 0}, lo[2] = {0x7fffffff, 0x7fffffff}, hi[2] = {0, 0}, seq = 0;
+    for (int r = row0 + lane; r < min(row0 + 2 * p.spt, row_end); r += 32) {
+      const RowKeys k = row_keys(r);
+      const int t = r >= row0 + p.spt;
+      seq = k.seq;
+      if (t) { nvis[1] = max(nvis[1], k.nvis); if (k.nloc > 0) { lo[1] = min(lo[1], k.loc0); hi[1] = max(hi[1], k.loc0 + k.nloc); } }
+      else { nvis[0] = max(nvis[0], k.nvis); if (k.nloc > 0) { lo[0] = min(lo[0], k.loc0); hi[0] = max(hi[0], k.loc0 + k.nloc); } }
+    }
+    seq = __shfl_sync(0xffffffffu, seq, 0);            // (row0 itself is lane 0's)
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      nvis[t] = __reduce_max_sync(0xffffffffu, nvis[t]); lo[t] = __reduce_min_sync(0xffffffffu, lo[t]); hi[t] = __reduce_max_sync(0xffffffffu, hi[t]);
+    }
+    if (lane < 3) {                                    // lane 0 / 1: the tiles, lane 2: the unit
+      const int nv = lane == 0 ? nvis[0] : lane == 1 ? nvis[1] : max(nvis[0], nvis[1]);
+      const int l = lane == 0 ? lo[0] : lane == 1 ? lo[1] : min(lo[0], lo[1]), h = lane == 0 ? hi[0] : lane == 1 ? hi[1] : max(hi[0], hi[1]);
+      const bool two = row0 + p.spt < row_end;
+      const int n_cache = (nv + PAGE - 1) / PAGE, n_pages = n_cache + (h > l ? (h - l + PAGE - 1) / PAGE : 0);
+      if (planned) {
+        keys[lane][u] = Keys{(short)n_cache, (short)n_pages, l};
+        const float us = n_pages * (lane == 2 && two ? PAIR_PAGE : SINGLE_PAGE);
+        ent_us[lane == 2 ? u : p.n_units + 2 * u + lane] = us;
+        atomicMax(&longest_us[lane == 2 ? 0 : 1], __float_as_int(us));
+        if (lane == 0) { unit_row0[u] = row0; unit_rend[u] = row_end; unit_seq[u] = seq; }
+      } else if (lane == 2) {                          // every unit one item, listed back to front (a causal pass lists its rows in ascending length)
+        Item it{};
+        it.row0 = row0; it.row_end = row_end; it.seq = seq; it.p_end = n_pages; it.n_cache_pages = n_cache; it.loc_lo = l; it.pair = two;
+        p.items[p.n_units - 1 - u] = it;
+      }
+    }
+  }
+  if (!planned) return;
+  __syncthreads();
+  bool paired = true;
+  float limit = 1e30f;
+  auto limit_of = [&](int cnd) { return fmaxf(__int_as_float(longest_us[cnd / CAND]) / (1.f + 0.5f * (cnd % CAND)), 0.1f) * 1.0001f; };
+  // pieces of an entity of cost us under a limit, at most one per page
+  auto pieces = [&](float us, float lim, bool dbl) { return (int)fminf(ceilf(us / lim), us * (dbl ? 1.0001f / PAIR_PAGE : 1.0001f / SINGLE_PAGE)); };
+  if (splits) {
+    const int per = blockDim.x / (2 * CAND) >= 16 ? 16 : blockDim.x / (2 * CAND) >= 4 ? 4 : 2;       // threads per candidate
+    const int cnd = threadIdx.x / per, sub = threadIdx.x % per;
+    const bool live_cnd = cnd < 2 * CAND, pr = cnd < CAND;
+    const float lim = limit_of(live_cnd ? cnd : 0);
+    const int n_ent = live_cnd ? (pr ? p.n_units : 2 * p.n_units) : 0, e0 = pr ? 0 : p.n_units;
+    int items = 0, live = 0, most = 0; float us_sum = 0.f, us_max = 0.f;
+    for (int e = sub; e < n_ent; e += per) {
+      const float us = ent_us[e0 + e];
+      if (us <= 0.f) continue;
+      const bool dbl = pr && unit_row0[e] + p.spt < unit_rend[e];
+      const int k = pieces(us, lim, dbl);
+      const float store = k > 1 ? (dbl ? PAIR_STORE : SINGLE_STORE) : 0.f;
+      items += k; ++live; most = max(most, k);
+      us_sum += us + k * (OVERHEAD + store);
+      us_max = fmaxf(us_max, __fdividef(us, (float)k) + (k > 1 ? 0.5f * SINGLE_PAGE : 0.f) + store + OVERHEAD);
+    }
+    for (int o = per >> 1; o > 0; o >>= 1) {
+      items += __shfl_xor_sync(0xffffffffu, items, o); live += __shfl_xor_sync(0xffffffffu, live, o); most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+      us_sum += __shfl_xor_sync(0xffffffffu, us_sum, o); us_max = fmaxf(us_max, __shfl_xor_sync(0xffffffffu, us_max, o));
+    }
+    if (live_cnd && sub == 0 && items <= p.max_items && most <= MAX_SPLITS) {
+      float us = us_max;
+      if (items * p.Hkv > p.n_sms) us = fmaxf(us, p.Hkv * us_sum / p.n_sms + 0.5f * us_max);
+      if (items > live) us += MERGE + 0.3f * items / live;
+      atomicMin(&best, ((unsigned long long)__float_as_uint(us) << 32) | (unsigned)cnd);     // us > 0: its bits order like its value
+    }
+    __syncthreads();
+    if (best != ~0ull) { const int c = (int)(best & 0xffffffffu); paired = c < CAND; limit = limit_of(c); }
+  }
+  const int n_ent = paired ? p.n_units : 2 * p.n_units, e0 = paired ? 0 : p.n_units;
+  for (int e = threadIdx.x; e < n_ent; e += blockDim.x) {
+    const float us = ent_us[e0 + e];
+    const int k = us <= 0.f ? 0 : splits ? max(1, pieces(us, limit, paired && unit_row0[e] + p.spt < unit_rend[e])) : 1;
+    ent_n[e] = (short)k; ent_us[e0 + e] = k ? us / k : -1.f;
+  }
+  __syncthreads();
+  // longest items first: entity e goes to place `rank`
+  for (int e = threadIdx.x; e < n_ent; e += blockDim.x) {
+    const float us = ent_us[e0 + e];
+    int rank = 0;
+#pragma unroll 4
+    for (int f = 0; f < n_ent; ++f) { const float v = ent_us[e0 + f]; rank += v > us || (v == us && f < e); }
+    order_s[rank] = (short)e;
+  }
+  __syncthreads();
+  if (warp == 0) {                                     // places of the items: running sum over the order
+    int base = 0;
+    for (int r0 = 0; r0 < n_ent; r0 += 32) {
+      const int e = r0 + lane < n_ent ? order_s[r0 + lane] : -1;
+      const int n = e >= 0 ? ent_n[e] : 0;
+      int sum = n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) { const int v = __shfl_up_sync(0xffffffffu, sum, o); if (lane >= o) sum += v; }
+      if (e >= 0) place_s[e] = (short)(base + sum - n);
+      base += __shfl_sync(0xffffffffu, sum, 31);
+    }
+    for (int i = base + lane; i < p.max_items; i += 32) p.items[i] = Item{};       // unused places: no rows, no pages
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < 2 * p.n_units; t += blockDim.x) {                  // what the merge kernel needs
+    const int u = t >> 1, e = paired ? u : t;
+    Tile w{};
+    w.row0 = unit_row0[u] + (t & 1) * p.spt; w.row_end = unit_rend[u];
+    w.n_items = w.row0 < w.row_end ? ent_n[e] : 0; w.item0 = place_s[e]; w.sub = paired ? t & 1 : 0;
+    p.tiles[t] = w;
+  }
+  for (int e = warp; e < n_ent; e += n_warps) {
+    const int u = paired ? e : e >> 1, n = ent_n[e];
+    const Keys k = keys[paired ? 2 : e & 1][u];
+    for (int j = lane; j < n; j += 32) {
+      Item it{};
+      it.row0 = unit_row0[u] + (paired ? 0 : (e & 1) * p.spt); it.row_end = unit_rend[u]; it.seq = unit_seq[u];
+      it.n_cache_pages = k.n_cache; it.loc_lo = k.loc_lo;
+      it.p_begin = k.n_pages * j / n; it.p_end = k.n_pages * (j + 1) / n;
+      it.pair = paired && unit_row0[u] + p.spt < unit_rend[u]; it.split = n > 1;
+      p.items[place_s[e] + j] = it;
+    }
+  }
+}
 
 template <int HD>
-__global__ void __launch_bounds__(THREADS, 2)
+__global__ void __launch_bounds__(THREADS, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                const __grid_constant__ CUtensorMap tmKloc, const __grid_constant__ CUtensorMap tmVloc, const Args a, const TlSlot tl) {
   using L = Smem<HD>;
   constexpr int NH = L::NH;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   pdl_trigger();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = sm100::warp_index(), lane = threadIdx.x & 31;
   const uint32_t smem0 = sm100::smem_u32(smem_raw);
   if (smem0 & 1023u) {                               // cannot place swizzled tiles: report, touch nothing
     if (threadIdx.x == 0 && a.status) atomicExch(a.status, 3);
     return;
   }
   Ctl &ctl = *reinterpret_cast<Ctl *>(smem_raw + L::BAR_OFF);
+  const int rows_used = a.spt * a.G;                                   // MMA rows of a tile that carry data
 
-  // ---- which work item ----
-  int w = blockIdx.x;
-  const int sp = w % a.splits; w /= a.splits;
-  const int kvh = w % a.Hkv; w /= a.Hkv;
-  int row0, row_end;                                                   // first slot of the tile; slots of its group end at row_end
-  if (a.tile_row0) { row0 = a.tile_row0[w]; row_end = a.tile_rend[w]; }
-  else {
-    const int tile = w % a.tiles_per_group, grp = w / a.tiles_per_group;
-    row0 = grp * a.rows_per_group + tile * a.spt;
-    row_end = min((grp + 1) * a.rows_per_group, a.R);
-  }
-  const int rows_used = a.spt * a.G;                                   // MMA rows that carry data
-
+  if (warp == 2 && lane < 5) sm100::prefetch_tensormap(lane == 0 ? &tmQ : lane == 1 ? &tmK : lane == 2 ? &tmV : lane == 3 ? &tmKloc : &tmVloc);
   if (threadIdx.x == 0) {
-    ctl.abort_flag = 0; ctl.max_nvis = 0; ctl.loc_lo = 0x7fffffff; ctl.loc_hi = 0;
+    ctl.abort_flag = 0;
     sm100::mbar_init(sm100::smem_u32(&ctl.q_full), 1);
-    for (int s = 0; s < K_STAGES; ++s) { sm100::mbar_init(sm100::smem_u32(&ctl.k_full[s]), 1); sm100::mbar_init(sm100::smem_u32(&ctl.k_empty[s]), 1); }
-    for (int s = 0; s < V_STAGES; ++s) { sm100::mbar_init(sm100::smem_u32(&ctl.v_full[s]), 1); sm100::mbar_init(sm100::smem_u32(&ctl.v_empty[s]), 1); }
-    for (int b = 0; b < 2; ++b) { sm100::mbar_init(sm100::smem_u32(&ctl.s_full[b]), 1); sm100::mbar_init(sm100::smem_u32(&ctl.s_empty[b]), 1); }
-    for (int b = 0; b < 2; ++b) sm100::mbar_init(sm100::smem_u32(&ctl.p_full[b]), 4);
+    for (int s = 0; s < STAGES; ++s) {
+      sm100::mbar_init(sm100::smem_u32(&ctl.k_full[s]), 1); sm100::mbar_init(sm100::smem_u32(&ctl.k_empty[s]), 1);
+      sm100::mbar_init(sm100::smem_u32(&ctl.v_full[s]), 1); sm100::mbar_init(sm100::smem_u32(&ctl.v_empty[s]), 1);
+    }
+    for (int t = 0; t < 2; ++t)
+      for (int b = 0; b < 2; ++b) { sm100::mbar_init(sm100::smem_u32(&ctl.s_full[t][b]), 1); sm100::mbar_init(sm100::smem_u32(&ctl.p_full[t][b]), 4); }
     sm100::fence_mbar_init();
   }
   if (warp == 1) {
@@ -125,259 +310,321 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     sm100::tmem_alloc(sm100::smem_u32(&ctl.tmem_base), L::TMEM_COLS);
     sm100::tmem_relinquish();
   }
-  __syncthreads();
-  pdl_wait();                 // everything below reads what earlier kernels of the pass wrote
-  if (threadIdx.x == 0) tl_go(tl);
-
-  // ---- per-row metadata (softmax threads own one MMA row each) and the tile's key range ----
-  const int my_row = (warp & 3) * 32 + lane;             // MMA row = TMEM lane (softmax warps only)
-  int my_slot = -1, my_nvis = 0, my_loc0 = 0, my_nloc = 0, my_head = 0;
-  if (warp >= 2) {
-    const int sl = my_row / a.G;
-    const int pr = row0 + sl;
-    if (sl < a.spt && pr < row_end) {
-      my_slot = pr; my_head = kvh * a.G + my_row % a.G;
-      my_nvis = a.nvis[pr]; my_nloc = a.nloc[pr]; my_loc0 = a.loc0[pr];
-      atomicMax(&ctl.max_nvis, my_nvis);
-      if (my_nloc > 0) { atomicMin(&ctl.loc_lo, my_loc0); atomicMax(&ctl.loc_hi, my_loc0 + my_nloc); }
-    }
-  }
   sm100::tc_fence_before();
   __syncthreads();
   sm100::tc_fence_after();
   const uint32_t tmem = ctl.tmem_base;
-  const uint32_t tmem_S = tmem, tmem_O = tmem + 2 * KT;               // S: 2 x 64 columns, O: HD columns
-  const int max_nvis = ctl.max_nvis;
-  const int loc_lo = ctl.loc_lo, loc_hi = ctl.loc_hi;
-  const int n_cache_tiles = (max_nvis + KT - 1) / KT;
-  const int n_loc_tiles = loc_hi > loc_lo ? (loc_hi - loc_lo + KT - 1) / KT : 0;
-  const int nt_all = n_cache_tiles + n_loc_tiles;
-  const int t_begin = (int)((long long)nt_all * sp / a.splits), t_end = (int)((long long)nt_all * (sp + 1) / a.splits);
-  const int nt = t_end - t_begin;
-  const int seq = row0 < a.R ? a.seq[row0] : 0;
+  const uint32_t tmem_S = tmem, tmem_O = tmem + 4 * PAGE;             // per stream: 2 x 64 columns of S, HD columns of O
   volatile int *abortp = &ctl.abort_flag;
-  if (threadIdx.x == 0 && a.tile_count) atomicAdd(a.tile_count, (unsigned long long)nt);
+  pdl_wait();                 // everything below reads what earlier kernels of the pass wrote
+  if (threadIdx.x == 0) tl_go(tl);
 
-  if (warp == 0) {
-    // ===================== TMA producer =====================
-    if (lane == 0 && nt > 0) {
+  // ---- which work item (every thread reads it: no barrier before the first loads go out) ----
+  const int kvh = blockIdx.x % a.Hkv, item_no = blockIdx.x / a.Hkv;
+  const Item item = a.items[item_no];                                  // all zero where the grid is larger than the plan: nothing to do
+  const int row0 = item.row0, p_begin = item.p_begin, np = item.p_end - item.p_begin;
+  const bool pair = item.pair != 0;
+  const int ahead = pair ? 2 : 4;                                      // pages whose scores are computed ahead: two steps of every stream
+  if (threadIdx.x == 0 && a.tile_count && np > 0) atomicAdd(a.tile_count, (unsigned long long)np * (pair ? 2 : 1));
+
+  if (warp == 0 || warp == 3) {
+    // ===================== K producer / Q and V producer =====================
+    // Lane i holds the i-th entry of a group of 32 entries of the page table, so that a page's load does not wait for
+    // its entry.  One load per page (the halves of the head are a dimension of the tensor map), and K and V each have
+    // a warp of their own: issuing a page's four loads one after the other from one warp took 1700 cycles per
+    // page (of 64 keys), three times as long as the page's MMAs.
+    if (np > 0) {
+      const bool is_k = warp == 0;
       const uint64_t pol = sm100::policy_evict_last();
-      const uint32_t qb = sm100::smem_u32(&ctl.q_full);
-      sm100::mbar_expect_tx(qb, (uint32_t)(NH * rows_used * 128));
-      for (int h = 0; h < NH; ++h)
-        sm100::tma_load_3d(smem0 + L::Q_OFF + h * (128 * 128), &tmQ, qb, h * 64, kvh * a.G, row0, pol);
-      int ks = 0, vs = 0; uint32_t kph = 0, vph = 0;
-      auto load_tile = [&](int t, bool is_k) -> bool {
-        const bool is_cache = t < n_cache_tiles;
-        const int page = is_cache ? a.page_table[(size_t)seq * a.pages_per_seq + t] : 0;
-        const int lrow = loc_lo + (t - n_cache_tiles) * KT;
-        const int st = is_k ? ks : vs;
-        if (!sm100::mbar_wait(sm100::smem_u32(is_k ? &ctl.k_empty[st] : &ctl.v_empty[st]), (is_k ? kph : vph) ^ 1u, abortp)) return false;
-        const uint32_t fb = sm100::smem_u32(is_k ? &ctl.k_full[st] : &ctl.v_full[st]);
-        sm100::mbar_expect_tx(fb, (uint32_t)L::KV_BYTES);
-        for (int h = 0; h < NH; ++h) {
-          const uint32_t dst = smem0 + (is_k ? L::K_OFF : L::V_OFF) + st * L::KV_BYTES + h * (KT * 128);
-          if (is_cache) sm100::tma_load_4d(dst, is_k ? &tmK : &tmV, fb, h * 64, 0, kvh, (is_k ? a.page_base_k : a.page_base_v) + page, pol);
-          else sm100::tma_load_3d(dst, is_k ? &tmKloc : &tmVloc, fb, h * 64, kvh, lrow, pol);
+      if (!is_k && sm100::elect_one()) {
+        const uint32_t qb = sm100::smem_u32(&ctl.q_full);
+        sm100::mbar_expect_tx(qb, (uint32_t)(NH * rows_used * 128 * (pair ? 2 : 1)));
+        for (int t = 0; t < (pair ? 2 : 1); ++t)
+          for (int h = 0; h < NH; ++h)
+            sm100::tma_load_3d(smem0 + L::Q_OFF + t * L::Q_BYTES + h * (128 * 128), &tmQ, qb, h * 64, kvh * a.G, row0 + t * a.spt, pol);
+      }
+      const int32_t *table = a.page_table + (size_t)item.seq * a.pages_per_seq;
+      const int n_table = min(item.n_cache_pages, item.p_end) - p_begin;         // pages of this item that the table backs
+      int cur = lane < n_table ? table[p_begin + lane] : 0, next = 0;
+      const CUtensorMap *tm = is_k ? &tmK : &tmV, *tm_loc = is_k ? &tmKloc : &tmVloc;
+      const int base = is_k ? a.page_base_k : a.page_base_v;
+      const uint32_t full0 = sm100::smem_u32(is_k ? ctl.k_full : ctl.v_full), empty0 = sm100::smem_u32(is_k ? ctl.k_empty : ctl.v_empty);
+      const uint32_t dst0 = smem0 + (is_k ? L::K_OFF : L::V_OFF);
+      int s = 0; uint32_t ph = 1u;
+      for (int p = 0; p < np; ++p) {
+        if ((p & 31) == 0) {
+          if (p) cur = next;
+          next = p + 32 + lane < n_table ? table[p_begin + p + 32 + lane] : 0;
         }
-        if (is_k) { if (++ks == K_STAGES) { ks = 0; kph ^= 1u; } }
-        else { if (++vs == V_STAGES) { vs = 0; vph ^= 1u; } }
-        return true;
-      };
-      // K of tile t + 1 goes out before V of tile t, in the order the MMA warp consumes them
-      bool ok = load_tile(t_begin, true);
-      for (int t = t_begin; t < t_end && ok; ++t) {
-        if (t + 1 < t_end) ok = load_tile(t + 1, true);
-        if (ok) ok = load_tile(t, false);
+        const int page = __shfl_sync(0xffffffffu, cur, p & 31) + base;
+        if (!__all_sync(0xffffffffu, sm100::mbar_wait(empty0 + (uint32_t)s * 8u, ph, abortp))) break;
+        if (sm100::elect_one()) {
+          const uint32_t fb = full0 + (uint32_t)s * 8u, dst = dst0 + (uint32_t)s * L::KV_BYTES;
+          sm100::mbar_expect_tx(fb, (uint32_t)L::KV_BYTES);
+          if (p < n_table) sm100::tma_load_5d(dst, tm, fb, 0, 0, 0, kvh, page, pol);
+          else sm100::tma_load_4d(dst, tm_loc, fb, 0, item.loc_lo + (p_begin + p - item.n_cache_pages) * PAGE, 0, kvh, pol);
+        }
+        __syncwarp();
+        if (++s == STAGES) { s = 0; ph ^= 1u; }
       }
     }
   } else if (warp == 1) {
     // ===================== MMA issuer =====================
-    if (lane == 0 && nt > 0) {
-      const uint32_t idesc_qk = sm100::make_idesc_bf16(128, KT);
-      const uint32_t idesc_pv = sm100::make_idesc_bf16(128, HD) | (1u << 16);      // B (= V) is MN-major
-      bool ok = sm100::mbar_wait(sm100::smem_u32(&ctl.q_full), 0, abortp);
+    // Runs the same schedule as the watcher to the end whatever happens, one barrier operation each per event.
+    const uint32_t idesc_qk = sm100::make_idesc_bf16(128, PAGE);
+    const uint32_t idesc_pv = sm100::make_idesc_bf16(128, HD) | (1u << 16);      // B (= V) is MN-major
+    // descriptors are built once; the issue loop only adds 16-byte-unit offsets
+    const uint64_t q_desc = sm100::make_desc_sw128(smem0 + L::Q_OFF);
+    const uint64_t k_desc0 = sm100::make_desc_sw128(smem0 + L::K_OFF);
+    const uint64_t v_desc0 = sm100::make_desc_sw128_mn(smem0 + L::V_OFF, PAGE * 128);
+    constexpr uint64_t KV16 = L::KV_BYTES >> 4, Q16 = L::Q_BYTES >> 4;
+    // scores of page p (ring stage s) for stream t, into S buffer b
+    auto issue_qk = [&](int t, int b, int s) {
+      const uint64_t qd = q_desc + (pair && t ? Q16 : 0), kd = k_desc0 + (uint64_t)s * KV16;
+      const uint32_t d = tmem_S + (uint32_t)((t * 2 + b) * PAGE);
+#pragma unroll
+      for (int kk = 0; kk < HD / 16; ++kk)             // 64-element half kk / 4 of the head, 16 elements of it
+        sm100::mma_bf16_ss(d, qd + (kk / 4) * (128 * 128 / 16) + (kk % 4) * 2, kd + (kk / 4) * (PAGE * 128 / 16) + (kk % 4) * 2, idesc_qk, kk > 0 ? 1u : 0u);
+    };
+    for (int p = 0; p < min(ahead, np); ++p) {
+      sm100::named_bar_sync(9u + (uint32_t)p, 64);
       sm100::tc_fence_after();
-      int ks = 0; uint32_t kph = 0;          // K ring position of the next QK^T
-      int vs = 0; uint32_t vph = 0;          // V ring position of the next PV
-      // descriptors are built once; the issue loop only adds 16-byte-unit offsets
-      const uint64_t q_desc = sm100::make_desc_sw128(smem0 + L::Q_OFF);
-      const uint64_t k_desc0 = sm100::make_desc_sw128(smem0 + L::K_OFF);
-      const uint64_t v_desc0 = sm100::make_desc_sw128_mn(smem0 + L::V_OFF, KT * 128);
-      constexpr uint64_t KV16 = L::KV_BYTES >> 4;
-      auto issue_qk = [&](int i) -> bool {   // i: tile counter of this CTA
-        const int b = i & 1; const uint32_t bph = (uint32_t)(i >> 1) & 1u;
-        if (!sm100::mbar_wait(sm100::smem_u32(&ctl.k_full[ks]), kph, abortp)) return false;
-        if (!sm100::mbar_wait(sm100::smem_u32(&ctl.s_empty[b]), bph ^ 1u, abortp)) return false;
-        sm100::tc_fence_after();
-        const uint64_t kd = k_desc0 + (uint64_t)ks * KV16;
-        const uint32_t d = tmem_S + b * KT;
-#pragma unroll
-        for (int kk = 0; kk < HD / 16; ++kk) {
-          // 64-element half kk/4 of the head: Q halves are 128 rows x 128 B apart, K halves 64 rows x 128 B
-          sm100::mma_bf16_ss(d, q_desc + (kk / 4) * (128 * 128 / 16) + (kk % 4) * 2, kd + (kk / 4) * (KT * 128 / 16) + (kk % 4) * 2, idesc_qk,
-                             kk > 0 ? 1u : 0u);
+      if (sm100::elect_one()) {
+        for (int t = pair ? 0 : p & 1; t < (pair ? 2 : (p & 1) + 1); ++t) {
+          const int b = pair ? p : p >> 1;
+          issue_qk(t, b, p);
+          sm100::mma_commit(sm100::smem_u32(&ctl.s_full[t][b]));
         }
-        sm100::mma_commit(sm100::smem_u32(&ctl.k_empty[ks]));
-        sm100::mma_commit(sm100::smem_u32(&ctl.s_full[b]));
-        if (++ks == K_STAGES) { ks = 0; kph ^= 1u; }
-        return true;
-      };
-      if (ok) ok = issue_qk(0);
-      for (int i = 0; i < nt && ok; ++i) {
-        if (i + 1 < nt) { ok = issue_qk(i + 1); if (!ok) break; }
-        if (!sm100::mbar_wait(sm100::smem_u32(&ctl.v_full[vs]), vph, abortp)) { ok = false; break; }
-        // (one barrier per S buffer: the softmax warps may finish tile i + 1 before this thread has seen tile i,
-        // and a parity wait cannot tell two completions from none)
-        if (!sm100::mbar_wait(sm100::smem_u32(&ctl.p_full[i & 1]), (uint32_t)(i >> 1) & 1u, abortp)) { ok = false; break; }
-        sm100::tc_fence_after();
-        const uint64_t vd = v_desc0 + (uint64_t)vs * KV16;
-        const uint32_t p_tmem = tmem_S + (uint32_t)((i & 1) * KT);
-#pragma unroll
-        for (int kk = 0; kk < KT / 16; ++kk)       // 16 keys per instruction: 8 columns of P, 16 V rows (2048 B)
-          sm100::mma_bf16_ts(tmem_O, p_tmem + kk * 8, vd + kk * (16 * 128 / 16), idesc_pv, (i > 0 || kk > 0) ? 1u : 0u);
-        sm100::mma_commit(sm100::smem_u32(&ctl.v_empty[vs]));
-        // P consumed and O up to date through tile i: the S buffer P lived in is free for tile i + 2
-        sm100::mma_commit(sm100::smem_u32(&ctl.s_empty[i & 1]));
-        if (++vs == V_STAGES) { vs = 0; vph ^= 1u; }
+        sm100::mma_commit(sm100::smem_u32(&ctl.k_empty[p]));
       }
+      __syncwarp();
     }
-  } else {
+    int sv = 0, sk = ahead % STAGES;                   // ring stages of V(p) and K(p + ahead)
+    for (int p = 0; p < np; ++p) {
+      const int j = pair ? p : p >> 1, b = j & 1;
+      const uint64_t vd = v_desc0 + (uint64_t)sv * KV16;
+      for (int t = pair ? 0 : p & 1; t < (pair ? 2 : (p & 1) + 1); ++t) {
+        const bool last_stream = !pair || t == 1;
+        sm100::named_bar_sync(1u + (uint32_t)(t * 2 + b), 64);
+        sm100::tc_fence_after();
+        if (sm100::elect_one()) {
+          const uint32_t p_tmem = tmem_S + (uint32_t)((t * 2 + b) * PAGE), o_tmem = tmem_O + (uint32_t)(t * HD);
+#pragma unroll
+          for (int kk = 0; kk < PAGE / 16; ++kk)       // 16 keys per instruction: 8 columns of P, 16 V rows (2048 B)
+            sm100::mma_bf16_ts(o_tmem, p_tmem + kk * 8, vd + kk * (16 * 128 / 16), idesc_pv, (j > 0 || kk > 0) ? 1u : 0u);
+          if (last_stream) sm100::mma_commit(sm100::smem_u32(&ctl.v_empty[sv]));
+          if (p + ahead < np) {
+            issue_qk(t, b, sk);
+            if (last_stream) sm100::mma_commit(sm100::smem_u32(&ctl.k_empty[sk]));
+          }
+          sm100::mma_commit(sm100::smem_u32(&ctl.s_full[t][b]));       // step j + 2's scores, or only "P V of step j is done"
+        }
+        __syncwarp();
+      }
+      if (++sv == STAGES) sv = 0;
+      if (++sk == STAGES) sk = 0;
+    }
+  } else if (warp == 2) {
+    // ===================== watcher =====================
+    // Waits (bounded) for what each group of MMAs needs and arrives on the group's hardware barrier.  A barrier
+    // cannot be arrived on twice before the MMA warp has passed it: P of step j + 2 needs the scores whose products
+    // are issued behind step j's.  After a failed wait that argument no longer holds, so from then on the watcher
+    // meets the MMA warp at every barrier instead.
+    bool failed = false;
+    auto release = [&](uint32_t id, uint32_t bar0, uint32_t par0, uint32_t bar1, uint32_t par1, uint32_t bar2, uint32_t par2) {
+      if (!failed) {
+        bool ok = true;
+        if (lane == 0)
+          ok = (!bar1 || sm100::mbar_wait(bar1, par1, abortp)) && (!bar2 || sm100::mbar_wait(bar2, par2, abortp)) && sm100::mbar_wait(bar0, par0, abortp);
+        failed = !__shfl_sync(0xffffffffu, ok, 0);
+      }
+      if (!failed) sm100::named_bar_arrive(id, 64);
+      else sm100::named_bar_sync(id, 64);
+    };
+    for (int p = 0; p < min(ahead, np); ++p)
+      release(9u + (uint32_t)p, sm100::smem_u32(&ctl.k_full[p]), 0, p ? 0u : sm100::smem_u32(&ctl.q_full), 0, 0u, 0);
+    int sv = 0, sk = ahead % STAGES; uint32_t phv = 0, phk = (uint32_t)(ahead / STAGES) & 1u;
+    for (int p = 0; p < np; ++p) {
+      const int j = pair ? p : p >> 1, b = j & 1;
+      for (int t = pair ? 0 : p & 1; t < (pair ? 2 : (p & 1) + 1); ++t) {
+        const bool first_stream = !pair || t == 0;
+        release(1u + (uint32_t)(t * 2 + b), sm100::smem_u32(&ctl.p_full[t][b]), (uint32_t)(j >> 1) & 1u, first_stream ? sm100::smem_u32(&ctl.v_full[sv]) : 0u, phv,
+                first_stream && p + ahead < np ? sm100::smem_u32(&ctl.k_full[sk]) : 0u, phk);
+      }
+      if (++sv == STAGES) { sv = 0; phv ^= 1u; }
+      if (++sk == STAGES) { sk = 0; phk ^= 1u; }
+    }
+  } else if (warp >= 4) {
     // ===================== softmax =====================
+    const int t = (warp - 4) >> 2;                       // stream
+    const int tile = pair ? t : 0;
+    const int my_row = (warp & 3) * 32 + lane;           // this thread's MMA row = TMEM lane
+    const int nj = pair ? np : (np + 1 - t) >> 1;        // steps of this stream
+    // (a row without a slot sees everything, so that its warp does not mask page after page for it)
+    int my_slot = -1, my_nvis = 0x7fffffff, my_loc0 = item.loc_lo, my_nloc = 1 << 30;
+    {
+      const int pr = row0 + tile * a.spt + my_row / a.G;
+      if (my_row < rows_used && pr < item.row_end) { my_slot = pr; my_nvis = a.nvis[pr]; my_nloc = a.nloc[pr]; my_loc0 = a.loc0[pr]; }
+    }
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
+    const uint32_t s_addr0 = tmem_S + (uint32_t)(t * 2 * PAGE) + lane_addr, o_addr = tmem_O + (uint32_t)(t * HD) + lane_addr;
+    const uint32_t s_bar0 = sm100::smem_u32(&ctl.s_full[t][0]), p_bar0 = sm100::smem_u32(&ctl.p_full[t][0]);
+    // wait until the scores of step j are there (for j >= nj: until P V of step j - 2 is done).  A parity wait means what it says
+    // because the barrier's next completion needs a P that this warp has not yet written.  A wait that gives up must
+    // take the whole warp out: the TMEM accesses are warp-collective.
+    auto wait_s = [&](int j) { return __all_sync(0xffffffffu, sm100::mbar_wait(s_bar0 + (uint32_t)(j & 1) * 8u, (uint32_t)(j >> 1) & 1u, abortp)) != 0; };
     float m_ref = -INFINITY, l_run = 0.f;
     bool ok = true;
-    for (int i = 0; i < nt && ok; ++i) {
-      const int t = t_begin + i;
-      const int b = i & 1; const uint32_t bph = (uint32_t)(i >> 1) & 1u;
-      // a wait that gives up must take the whole warp out: the TMEM loads below are warp-collective
-      if (!__all_sync(0xffffffffu, sm100::mbar_wait(sm100::smem_u32(&ctl.s_full[b]), bph, abortp))) { ok = false; break; }
+    for (int j = 0; j < nj; ++j) {
+      if (!(ok = wait_s(j))) break;
       sm100::tc_fence_after();
-      uint32_t sv[64];
+      const uint32_t s_addr = s_addr0 + (uint32_t)((j & 1) * PAGE);
+      uint32_t sv[2][32];
+      sm100::tmem_ld32(s_addr, sv[0]);
+      sm100::tmem_ld32(s_addr + 32, sv[1]);
+      sm100::tmem_wait_ld();
+      // Visible keys of the page for my row: [lo, hi) in page-local indices.  Masking is skipped
+      // for pages that are visible in full (all cached pages but the last ones of a row).
       {
-        uint32_t v0[32], v1[32];
-        sm100::tmem_ld32(tmem_S + lane_addr + b * KT, v0);
-        sm100::tmem_ld32(tmem_S + lane_addr + b * KT + 32, v1);
-        sm100::tmem_wait_ld();
+        const int p = p_begin + (pair ? j : 2 * j + t);
+        int lo = 0, hi = 0;
+        if (p < item.n_cache_pages) hi = my_nvis - p * PAGE;
+        else if (my_nloc > 0) { lo = my_loc0 - (item.loc_lo + (p - item.n_cache_pages) * PAGE); hi = lo + my_nloc; }
+        if (lo > 0 || hi < PAGE) {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) { sv[j] = v0[j]; sv[32 + j] = v1[j]; }
-      }
-
-      // visible keys of this tile for my row: [lo, hi) in tile-local indices
-      int lo = 0, hi = 0;
-      if (my_slot >= 0) {
-        if (t < n_cache_tiles) { lo = 0; hi = min(KT, my_nvis - t * KT); }
-        else {
-          const int base = loc_lo + (t - n_cache_tiles) * KT;           // local row of key 0
-          lo = max(0, my_loc0 - base); hi = my_nloc > 0 ? min(KT, my_loc0 + my_nloc - base) : 0;
+          for (int c = 0; c < PAGE; ++c)
+            if (c < lo || c >= hi) sv[c / 32][c & 31] = 0xff800000u;               // -inf
         }
       }
-      // Softmax of the tile in base 2.  The scores stay raw in sv: the scale is applied inside
-      // one FMA per element (s * scale - m), masking is skipped for tiles that are visible in
-      // full (all cached keys but the last tile of a row), and the max and the sum run as
-      // four independent chains: this loop, not the MMAs, bounds the kernel.
-      if (lo > 0 || hi < KT) {
-#pragma unroll
-        for (int j = 0; j < 64; ++j)
-          if (j < lo || j >= hi) sv[j] = 0xff800000u;          // -inf
-      }
+      // Softmax in base 2.  The scores stay raw: the scale is applied inside one FMA per two elements (s * scale - m), and
+      // the max and the sum run as independent chains.
       float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-      for (int j = 0; j < 64; j += 4) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) mx4[u] = fmaxf(mx4[u], __uint_as_float(sv[j + u]));
-      }
-      const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * a.scale_log2;     // scale > 0; -inf stays -inf
-      // raise the reference only when this tile exceeds it by more than the threshold
+      for (int c = 0; c < 64; c += 2) mx4[(c >> 1) & 3] = sm100::max3(mx4[(c >> 1) & 3], __uint_as_float(sv[c / 32][c & 31]), __uint_as_float(sv[c / 32][(c & 31) + 1]));
+      const float mx = sm100::max3(mx4[0], mx4[1], fmaxf(mx4[2], mx4[3])) * a.scale_log2;      // scale > 0; -inf stays -inf
+      // raise the reference only when this step exceeds it by more than the threshold
       // (-inf + threshold = -inf, so the first visible key always sets it)
       const float m_new = (mx > m_ref + RAISE_THRESHOLD) ? mx : m_ref;
       const float alpha = (m_new == m_ref) ? 1.f : exp2f(m_ref - m_new);      // m_ref = -inf gives 0
       const float neg_m = (m_new == -INFINITY) ? 0.f : -m_new;
-      float sum4[4] = {0.f, 0.f, 0.f, 0.f};
-      uint32_t pk[32];
-#pragma unroll
-      for (int j = 0; j < 64; j += 4) {
-        float p[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          p[u] = sm100::ex2_approx(fmaf(__uint_as_float(sv[j + u]), a.scale_log2, neg_m));   // -inf -> 0
-          sum4[u] += p[u];
-        }
-        __nv_bfloat162 h01 = __floats2bfloat162_rn(p[0], p[1]), h23 = __floats2bfloat162_rn(p[2], p[3]);
-        pk[j >> 1] = *reinterpret_cast<uint32_t *>(&h01);
-        pk[(j >> 1) + 1] = *reinterpret_cast<uint32_t *>(&h23);
-      }
-      const float sum = (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
-      l_run = l_run * alpha + sum;
       m_ref = m_new;
-
-      if (i > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
-        // O is rescaled in place, so P V of tile i - 1 must be complete: completion (i - 1) / 2 of the
-        // barrier of its S buffer.  A parity wait means what it says only while the barrier is at most
-        // one completion away from the one waited for, which holds although most tiles never wait
-        // here: completion (i - 3) / 2 happened before the Q K^T of tile i - 1 was issued, and the
-        // next one needs the P of tile i + 1.
-        if (!__all_sync(0xffffffffu, sm100::mbar_wait(sm100::smem_u32(&ctl.s_empty[(i - 1) & 1]), (uint32_t)((i - 1) >> 1) & 1u, abortp))) { ok = false; break; }
+      if (j > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
+        // O is rescaled in place: P V of step j - 1 must be done; that of step j waits for P
+        if (!(ok = wait_s(j + 1))) break;
         sm100::tc_fence_after();
-#pragma unroll
-        for (int c = 0; c < HD / 32; ++c) {
-          uint32_t v[32];
-          sm100::tmem_ld32(tmem_O + lane_addr + c * 32, v);
+#pragma unroll 2
+        for (int c = 0; c < HD / 16; ++c) {
+          uint32_t v[16];
+          sm100::tmem_ld16(o_addr + c * 16, v);
           sm100::tmem_wait_ld();
 #pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) * alpha);
-          sm100::tmem_st32(tmem_O + lane_addr + c * 32, v);
+          for (int i = 0; i < 16; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
+          sm100::tmem_st16(o_addr + c * 16, v);
         }
-        sm100::tmem_wait_st();
-        sm100::tc_fence_before();
       }
-      // P -> the first 32 columns of this tile's S buffer (my row = my TMEM lane; the scores are in registers)
-      sm100::tmem_st32(tmem_S + lane_addr + b * KT, pk);
+      const sm100::f32x2 scale2 = sm100::pack2(a.scale_log2, a.scale_log2), neg_m2 = sm100::pack2(neg_m, neg_m);
+      sm100::f32x2 sum2[2] = {0ull, 0ull};           // (0, 0)
+      uint32_t pk[32];
+#pragma unroll
+      for (int c = 0; c < 64; c += 2) {
+        float x, y;
+        sm100::unpack2(sm100::fma2(sm100::pack2(__uint_as_float(sv[c / 32][c & 31]), __uint_as_float(sv[c / 32][(c & 31) + 1])), scale2, neg_m2), x, y);
+        x = sm100::ex2_approx(x); y = sm100::ex2_approx(y);           // -inf -> 0
+        sum2[(c >> 1) & 1] = sm100::add2(sum2[(c >> 1) & 1], sm100::pack2(x, y));
+        __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+        pk[c >> 1] = *reinterpret_cast<uint32_t *>(&h);
+      }
+      sm100::tmem_st32(s_addr, pk);
       sm100::tmem_wait_st();
       sm100::tc_fence_before();
       __syncwarp();
-      if (lane == 0) sm100::mbar_arrive(sm100::smem_u32(&ctl.p_full[b]));
+      if (lane == 0) sm100::mbar_arrive(p_bar0 + (uint32_t)(j & 1) * 8u);
+      float sa, sb;
+      sm100::unpack2(sm100::add2(sum2[0], sum2[1]), sa, sb);
+      l_run = l_run * alpha + (sa + sb);
     }
-    // ---- output: O is complete once the last PV has finished ----
-    // (the last two products, each on its own buffer's barrier; the bound on the distance holds as above)
-    if (ok && nt > 1) ok = sm100::mbar_wait(sm100::smem_u32(&ctl.s_empty[(nt - 2) & 1]), (uint32_t)((nt - 2) >> 1) & 1u, abortp);
-    if (ok && nt > 0) ok = sm100::mbar_wait(sm100::smem_u32(&ctl.s_empty[(nt - 1) & 1]), (uint32_t)((nt - 1) >> 1) & 1u, abortp);
-    ok = __all_sync(0xffffffffu, ok);
-    if (ok) {
-      sm100::tc_fence_after();
-      const float inv = (a.splits == 1) ? 1.f / l_run : 1.f;
-      bf16 *o = a.O + ((size_t)max(my_slot, 0) * a.Hq + my_head) * HD;
-      const size_t pidx = ((size_t)sp * a.R + max(my_slot, 0)) * a.Hq + my_head;
-      float *po = a.part_O + pidx * HD;
+    // ---- output: O is complete once the last P V has finished ----
+    if (ok && nj > 1) ok = wait_s(nj);                   // (P V of the last step but one; in order, so that the parity wait below is unambiguous)
+    if (ok && nj > 0) ok = wait_s(nj + 1);
+    sm100::tc_fence_after();
+    bf16 *o = a.O + ((size_t)max(my_slot, 0) * a.Hq + kvh * a.G + my_row % a.G) * HD;
+    const size_t part = (size_t)blockIdx.x * 2 + tile;
+    float *po = a.part_O + (part * (HD / 4) * 128 + my_row) * 4;
+    auto write32 = [&](const float (&v)[32], int col, float inv) {       // columns [col, col + 32) of this row
+      if (my_slot < 0) return;
+      if (!item.split) {
 #pragma unroll
-      for (int c = 0; c < HD / 32; ++c) {
-        uint32_t v[32];
-        if (nt > 0) { sm100::tmem_ld32(tmem_O + lane_addr + c * 32, v); sm100::tmem_wait_ld(); }
-        else {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) v[j] = 0u;
+        for (int i = 0; i < 32; i += 8) {
+          uint4 u;
+          __nv_bfloat162 h0 = __floats2bfloat162_rn(v[i] * inv, v[i + 1] * inv), h1 = __floats2bfloat162_rn(v[i + 2] * inv, v[i + 3] * inv),
+                         h2 = __floats2bfloat162_rn(v[i + 4] * inv, v[i + 5] * inv), h3 = __floats2bfloat162_rn(v[i + 6] * inv, v[i + 7] * inv);
+          u.x = *reinterpret_cast<uint32_t *>(&h0); u.y = *reinterpret_cast<uint32_t *>(&h1);
+          u.z = *reinterpret_cast<uint32_t *>(&h2); u.w = *reinterpret_cast<uint32_t *>(&h3);
+          *reinterpret_cast<uint4 *>(o + col + i) = u;
         }
-        if (my_slot >= 0) {
-          if (a.splits == 1) {
+      } else {
 #pragma unroll
-            for (int j = 0; j < 32; j += 8) {
-              uint4 u;
-              __nv_bfloat162 h0 = __floats2bfloat162_rn(__uint_as_float(v[j]) * inv, __uint_as_float(v[j + 1]) * inv),
-                             h1 = __floats2bfloat162_rn(__uint_as_float(v[j + 2]) * inv, __uint_as_float(v[j + 3]) * inv),
-                             h2 = __floats2bfloat162_rn(__uint_as_float(v[j + 4]) * inv, __uint_as_float(v[j + 5]) * inv),
-                             h3 = __floats2bfloat162_rn(__uint_as_float(v[j + 6]) * inv, __uint_as_float(v[j + 7]) * inv);
-              u.x = *reinterpret_cast<uint32_t *>(&h0); u.y = *reinterpret_cast<uint32_t *>(&h1);
-              u.z = *reinterpret_cast<uint32_t *>(&h2); u.w = *reinterpret_cast<uint32_t *>(&h3);
-              *reinterpret_cast<uint4 *>(o + c * 32 + j) = u;
-            }
-          } else {
+        for (int i = 0; i < 32; i += 4)
+          *reinterpret_cast<float4 *>(po + (size_t)((col + i) / 4) * (128 * 4)) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+      }
+    };
+    auto load32 = [&](int col, float (&v)[32]) {
+      uint32_t w[32];
+      sm100::tmem_ld32(o_addr + col, w);
+      sm100::tmem_wait_ld();
 #pragma unroll
-            for (int j = 0; j < 32; j += 4)
-              *reinterpret_cast<uint4 *>(po + c * 32 + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+      for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(w[i]);
+    };
+    if (pair) {
+      if (ok && nj > 0) {
+        const float inv = item.split ? 1.f : 1.f / l_run;
+#pragma unroll
+        for (int c = 0; c < HD; c += 32) { float v[32]; load32(c, v); write32(v, c, inv); }
+        if (my_slot >= 0 && item.split) a.part_ml[part * 128 + my_row] = make_float2(m_ref, l_run);
+      }
+    } else if (np > 0) {
+      // The streams' halves of the same rows: each hands the other's columns over and finishes its own.  All MMAs have
+      // read the K/V rings once every warp has got here (a failed stream only has to show up).
+      float4 *xo = reinterpret_cast<float4 *>(smem_raw + L::XCHG_OFF);   // [stream that reads][HD / 8][128]
+      float2 *xml = reinterpret_cast<float2 *>(smem_raw + L::XCHG_ML_OFF);
+      sm100::named_bar_sync(13, 256);
+      if (ok) {
+        xml[t * 128 + my_row] = make_float2(m_ref, l_run);
+#pragma unroll
+        for (int c = 0; c < HD / 2; c += 32) {
+          float v[32];
+          if (nj > 0) load32((1 - t) * (HD / 2) + c, v);
+          else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) v[i] = 0.f;
           }
+#pragma unroll
+          for (int i = 0; i < 32; i += 4) xo[((1 - t) * (HD / 8) + (c + i) / 4) * 128 + my_row] = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
         }
       }
-      if (my_slot >= 0 && a.splits > 1) { a.part_ml[pidx * 2] = m_ref; a.part_ml[pidx * 2 + 1] = l_run; }
+      sm100::named_bar_sync(13, 256);
+      if (ok) {
+        const float2 other = xml[(1 - t) * 128 + my_row];
+        const float M = fmaxf(m_ref, other.x);
+        const float wm = m_ref == -INFINITY ? 0.f : exp2f(m_ref - M), wo = other.x == -INFINITY ? 0.f : exp2f(other.x - M);
+        const float l = wm * l_run + wo * other.y, inv = item.split ? 1.f : 1.f / l;
+#pragma unroll
+        for (int c = 0; c < HD / 2; c += 32) {
+          float v[32];
+          if (nj > 0) load32(t * (HD / 2) + c, v);
+          else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) v[i] = 0.f;
+          }
+#pragma unroll
+          for (int i = 0; i < 32; i += 4) {
+            const float4 x = xo[(t * (HD / 8) + (c + i) / 4) * 128 + my_row];
+            v[i] = wm * v[i] + wo * x.x; v[i + 1] = wm * v[i + 1] + wo * x.y; v[i + 2] = wm * v[i + 2] + wo * x.z; v[i + 3] = wm * v[i + 3] + wo * x.w;
+          }
+          write32(v, t * (HD / 2) + c, inv);
+        }
+        if (t == 0 && my_slot >= 0 && item.split) a.part_ml[part * 128 + my_row] = make_float2(M, l);
+      }
     }
   }
 
@@ -397,35 +644,47 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   if (threadIdx.x == 0) tl_end(tl);
 }
 
-// Merge the per-split partial results: O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s.
-// HD / 4 threads per (row, head), four consecutive columns each: 16-byte loads, 8-byte stores.
+// Merge the partial results of the query tiles that were split: O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s.
+// HD / 16 blocks of 256 threads per (query tile, KV head); a thread takes 8 columns of one MMA row, neighbouring
+// threads neighbouring rows, which is how the partial results lie in memory.
 template <int HD>
-__global__ void attn_combine_kernel(const float *__restrict__ part_O, const float *__restrict__ part_ml, int splits, int R, int Hq,
-                               bf16 *__restrict__ O, TlSlot tl) {
+__global__ void __launch_bounds__(256)
+attn_combine_kernel(const Args a, TlSlot tl) {
   pdl_trigger();
   pdl_wait();
   if (threadIdx.x == 0) tl_go(tl);
-  constexpr int PER = HD / 4;
-  const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const size_t wid = gid / PER;
-  const int c4 = (int)(gid % PER);
-  if (wid >= (size_t)R * Hq) { if (threadIdx.x == 0) tl_end(tl); return; }
-  float M = -INFINITY;
-  for (int s = 0; s < splits; ++s) M = fmaxf(M, part_ml[((size_t)s * R * Hq + wid) * 2]);
-  float den = 0.f;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int s = 0; s < splits; ++s) {
-    const size_t idx = (size_t)s * R * Hq + wid;
-    const float m = part_ml[idx * 2], l = part_ml[idx * 2 + 1];
-    const float wgt = (m == -INFINITY) ? 0.f : exp2f(m - M);
-    den += wgt * l;
-    const float4 v = reinterpret_cast<const float4 *>(part_O + idx * HD)[c4];
-    acc.x = fmaf(wgt, v.x, acc.x); acc.y = fmaf(wgt, v.y, acc.y); acc.z = fmaf(wgt, v.z, acc.z); acc.w = fmaf(wgt, v.w, acc.w);
+  constexpr int BLOCKS = HD / 16;
+  const int w = blockIdx.x / BLOCKS, kvh = w % a.Hkv;
+  const int cg = (blockIdx.x % BLOCKS) * 2 + (threadIdx.x >> 7), m = threadIdx.x & 127;
+  const Tile t = a.tiles[w / a.Hkv];
+  const int slot = t.row0 + m / a.G;
+  if (t.n_items > 1 && m < a.spt * a.G && slot < t.row_end) {
+    const size_t part = ((size_t)t.item0 * a.Hkv + kvh) * 2 + t.sub;
+    const float2 *ml = a.part_ml + part * 128 + m;
+    const float4 *po = reinterpret_cast<const float4 *>(a.part_O) + part * (HD / 4) * 128 + (size_t)cg * 2 * 128 + m;
+    const size_t ml_step = (size_t)a.Hkv * 2 * 128, po_step = (size_t)a.Hkv * 2 * (HD / 4) * 128;
+    float M = -INFINITY;
+#pragma unroll 4
+    for (int s = 0; s < t.n_items; ++s) M = fmaxf(M, ml[s * ml_step].x);
+    float den = 0.f;
+    float acc[8] = {};
+#pragma unroll 4
+    for (int s = 0; s < t.n_items; ++s) {
+      const float2 v = ml[s * ml_step];
+      const float4 x = po[s * po_step], y = po[s * po_step + 128];
+      const float wgt = (v.x == -INFINITY) ? 0.f : exp2f(v.x - M);
+      den += wgt * v.y;
+      acc[0] = fmaf(wgt, x.x, acc[0]); acc[1] = fmaf(wgt, x.y, acc[1]); acc[2] = fmaf(wgt, x.z, acc[2]); acc[3] = fmaf(wgt, x.w, acc[3]);
+      acc[4] = fmaf(wgt, y.x, acc[4]); acc[5] = fmaf(wgt, y.y, acc[5]); acc[6] = fmaf(wgt, y.z, acc[6]); acc[7] = fmaf(wgt, y.w, acc[7]);
+    }
+    const float inv = 1.f / den;
+    __nv_bfloat162 h0 = __floats2bfloat162_rn(acc[0] * inv, acc[1] * inv), h1 = __floats2bfloat162_rn(acc[2] * inv, acc[3] * inv),
+                   h2 = __floats2bfloat162_rn(acc[4] * inv, acc[5] * inv), h3 = __floats2bfloat162_rn(acc[6] * inv, acc[7] * inv);
+    uint4 u;
+    u.x = *reinterpret_cast<uint32_t *>(&h0); u.y = *reinterpret_cast<uint32_t *>(&h1);
+    u.z = *reinterpret_cast<uint32_t *>(&h2); u.w = *reinterpret_cast<uint32_t *>(&h3);
+    *reinterpret_cast<uint4 *>(a.O + ((size_t)slot * a.Hq + kvh * a.G + m % a.G) * HD + cg * 8) = u;
   }
-  const float inv = 1.f / den;
-  __nv_bfloat162 h0 = __floats2bfloat162_rn(acc.x * inv, acc.y * inv), h1 = __floats2bfloat162_rn(acc.z * inv, acc.w * inv);
-  uint2 u; u.x = *reinterpret_cast<uint32_t *>(&h0); u.y = *reinterpret_cast<uint32_t *>(&h1);
-  reinterpret_cast<uint2 *>(O + wid * HD)[c4] = u;
   if (threadIdx.x == 0) tl_end(tl);
 }
 

@@ -3,6 +3,7 @@
 #pragma once
 #include "common.cuh"
 #include "sm100_ptx.cuh"
+#include "attn_tc.cuh"
 
 // Four consecutive split-K partial sums starting at p (fp32 or bf16 slabs).
 template <typename T> __device__ __forceinline__ float4 load4(const T *p);
@@ -105,38 +106,54 @@ __global__ void assemble_prefill_kernel(RowMeta m, int seq, int row0, int n_prom
   embed_row_to_f32(embed + (size_t)id * d, X + (size_t)r * d, d);
 }
 
-// Row metadata for the stand-alone attention entry point (same slot layout as a step).
+// What row r of the stand-alone attention entry points sees (same slot layout as a step).
 // seq_len comes from the caller: it is clamped to [0, n_max] (n_max = the positions the page
 // table can back minus the k causal slots), so that no row looks past the table.
-__global__ void attn_meta_kernel(RowMeta m, const int32_t *__restrict__ seq_len, int k, int R, int n_max) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= R) return;
+__device__ __forceinline__ attn_tc::RowKeys attn_row_keys(const int32_t *__restrict__ seq_len, int k, int n_max, int r) {
   const int T = k * (k + 1);
   const int s = r / T, slot = r % T;
   const int n = min(max(seq_len[s], 0), n_max);
-  m.seq[r] = s;
-  if (slot < k) {
-    m.pos[r] = n + slot; m.nvis[r] = n + slot + 1; m.loc0[r] = 0; m.nloc[r] = 0;
-  } else {
-    const int b = (slot - k) / k;
-    m.pos[r] = n + b + 1 + (slot - k) % k; m.nvis[r] = n + b + 1; m.loc0[r] = s * k * k + b * k; m.nloc[r] = k;
-  }
+  if (slot < k) return attn_tc::RowKeys{n + slot + 1, 0, 0, s};
+  const int b = (slot - k) / k;
+  return attn_tc::RowKeys{n + b + 1, s * k * k + b * k, k, s};
+}
+__global__ void attn_meta_kernel(RowMeta m, const int32_t *__restrict__ seq_len, int k, int R, int n_max) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= R) return;
+  const attn_tc::RowKeys w = attn_row_keys(seq_len, k, n_max, r);
+  m.seq[r] = w.seq; m.nvis[r] = w.nvis; m.loc0[r] = w.loc0; m.nloc[r] = w.nloc;
+}
+// The same for the tensor-core attention kernel, with its work plan (the first block).
+__global__ void __launch_bounds__(512) attn_meta_plan_kernel(RowMeta m, const int32_t *__restrict__ seq_len, int k, int R, int n_max, attn_tc::PlanArgs plan) {
+  pdl_trigger();
+  pdl_wait();
+  if (blockIdx.x == 0) { attn_tc::plan_block(plan, [&](int r) { return attn_row_keys(seq_len, k, n_max, r); }); return; }
+  const int r = (blockIdx.x - 1) * blockDim.x + threadIdx.x;
+  if (r >= R) return;
+  const attn_tc::RowKeys w = attn_row_keys(seq_len, k, n_max, r);
+  m.seq[r] = w.seq; m.nvis[r] = w.nvis; m.loc0[r] = w.loc0; m.nloc[r] = w.nloc;
 }
 
-// cos/sin of pos * theta^(-2i/hd), evaluated in double once per pass (shared by every
-// layer and head), stored as float.
-__global__ void rope_table_kernel(const int32_t *__restrict__ pos, int R, int half, double theta,
-                                  float *__restrict__ cs, float *__restrict__ sn, TlSlot tl) {
+// What every layer of a pass shares, computed once per pass from the row metadata: cos/sin of
+// pos * theta^(-2i/hd) (evaluated in double, stored as float), one thread per (row, i), and, when
+// plan.tiles is set, the attention work plan (the first block).
+__global__ void __launch_bounds__(256) pass_setup_kernel(RowMeta m, int R, int half, double theta,
+                                  float *__restrict__ cs, float *__restrict__ sn, attn_tc::PlanArgs plan, TlSlot tl) {
   pdl_trigger();
   pdl_wait();
   if (threadIdx.x == 0) tl_go(tl);
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= R * half) { if (threadIdx.x == 0) tl_end(tl); return; }
-  const int r = t / half, i = t % half;
-  const double inv = pow(theta, -(double)i / (double)half);
-  double s, c;
-  sincos((double)pos[r] * inv, &s, &c);
-  cs[t] = (float)c; sn[t] = (float)s;
+  const int first = plan.tiles ? 1 : 0;
+  if (first && blockIdx.x == 0) attn_tc::plan_block(plan, [&](int r) { return attn_tc::RowKeys{m.nvis[r], m.loc0[r], m.nloc[r], m.seq[r]}; });
+  else {
+    const int t = (blockIdx.x - first) * blockDim.x + threadIdx.x;
+    if (t < R * half) {
+      const int r = t / half, i = t % half;
+      const double inv = pow(theta, -(double)i / (double)half);
+      double s, c;
+      sincos((double)m.pos[r] * inv, &s, &c);
+      cs[t] = (float)c; sn[t] = (float)s;
+    }
+  }
   if (threadIdx.x == 0) tl_end(tl);
 }
 

@@ -18,6 +18,8 @@
 
 namespace {
 
+constexpr int MAX_SMS = 160;      // scratch is sized for this many (a B200 has 148)
+
 std::string g_init_error;
 
 struct SeqState {
@@ -51,11 +53,11 @@ struct tidar_ctx {
   RowMeta meta{};
   int32_t *d_blk_len = nullptr;    // [max_batch]: drafts a sequence's block holds (the block length of its last pass)
   // a step whose sequences use different block lengths: per listed sequence its k, first row, first local row;
-  // per query tile of the attention kernel its first row and the end of its sequence's rows
-  int32_t *d_step_k = nullptr, *d_step_off = nullptr, *d_step_loc = nullptr, *d_tile_row0 = nullptr, *d_tile_rend = nullptr;
+  // per attention unit (two query tiles) its first row and the end of its sequence's rows
+  int32_t *d_step_k = nullptr, *d_step_off = nullptr, *d_step_loc = nullptr, *d_unit_row0 = nullptr, *d_unit_rend = nullptr;
   int32_t *h_lay = nullptr;        // pinned staging for those five arrays
   size_t lay_ints = 0;
-  int mixed_tiles = 0;             // query tiles of the current mixed step
+  int mixed_units = 0;             // attention units of the current mixed step
   float *d_run_max = nullptr, *d_run_sum = nullptr, *d_tgt_logit = nullptr, *d_logprob = nullptr;   // likelihood scoring, per row
   int32_t *d_target = nullptr;
   std::vector<CUtensorMap> tm_lm_chunks;   // the LM head in vocabulary chunks of lm_chunk rows (scoring)
@@ -88,10 +90,11 @@ struct tidar_ctx {
   struct AMap { const void *p; int rows, cols, box; CUtensorMap tm; };
   std::vector<AMap> amaps;
   CUtensorMap tm_q, tm_kv, tm_kloc, tm_vloc;
-  float *attn_part_O = nullptr, *attn_part_ml = nullptr;
+  float *attn_part_O = nullptr; float2 *attn_part_ml = nullptr;
+  attn_tc::Item *plan_items = nullptr; attn_tc::Tile *plan_tiles = nullptr;       // attention work plan of the current pass
   int n_sms = 0;
-  // the launches of one decode step as an executable graph, valid for one (k, n_seqs, attention split)
-  struct StepGraph { int k = 0, n_seqs = 0, splits = 0, mixed_R = 0, tiles = 0, mixed_K = 0; bool ar = false, timeline = false; cudaGraphExec_t exec = nullptr; int64_t launches = 0; } sg;
+  // the launches of one decode step as an executable graph, valid for one (k, n_seqs)
+  struct StepGraph { int k = 0, n_seqs = 0, mixed_R = 0, tiles = 0, mixed_K = 0; bool ar = false, timeline = false; cudaGraphExec_t exec = nullptr; int64_t launches = 0; } sg;
   bool graphs_ok = true;
   bool slab_bf16 = false;          // split-K partial sums of the step in bf16 instead of fp32 (config debug bit 2)
   int32_t *d_status = nullptr, *cand_idx = nullptr;
@@ -184,7 +187,7 @@ void layout(tidar_ctx &x, void *arena, size_t *bytes) {
   x.lay_ints = 3 * (size_t)(c.max_batch + 1) + 2 * (size_t)(x.R_head + c.max_batch);
   x.d_step_k = cv.take<int32_t>(x.lay_ints);
   x.d_step_off = x.d_step_k + (c.max_batch + 1); x.d_step_loc = x.d_step_off + (c.max_batch + 1);
-  x.d_tile_row0 = x.d_step_loc + (c.max_batch + 1); x.d_tile_rend = x.d_tile_row0 + (x.R_head + c.max_batch);
+  x.d_unit_row0 = x.d_step_loc + (c.max_batch + 1); x.d_unit_rend = x.d_unit_row0 + (x.R_head + c.max_batch);
   x.d_run_max = cv.take<float>(R); x.d_run_sum = cv.take<float>(R); x.d_tgt_logit = cv.take<float>(R); x.d_logprob = cv.take<float>(R);
   x.d_target = cv.take<int32_t>(R);
   x.d_block = cv.take<int32_t>((size_t)c.max_batch * c.k_max);
@@ -197,8 +200,11 @@ void layout(tidar_ctx &x, void *arena, size_t *bytes) {
   x.d_status = cv.take<int32_t>(64);
   x.d_tl = cv.take<unsigned long long>(2 * tidar_ctx::TL_MAX + 8);   // timeline slots, then diagnostic counters
   if (c.impl == 0) {
-    x.attn_part_O = cv.take<float>((size_t)attn_tc::MAX_SPLITS * R * c.n_q_heads * c.head_dim);
-    x.attn_part_ml = cv.take<float>((size_t)attn_tc::MAX_SPLITS * R * c.n_q_heads * 2);
+    const size_t slots = (size_t)attn_tc::SLOTS_PER_SM * MAX_SMS;
+    x.attn_part_O = cv.take<float>(slots * 2 * 128 * c.head_dim);
+    x.attn_part_ml = cv.take<float2>(slots * 2 * 128);
+    x.plan_tiles = cv.take<attn_tc::Tile>(2 * R);     // a unit of two query tiles holds at least one row
+    x.plan_items = cv.take<attn_tc::Item>(std::max<size_t>(slots, R));
   }
   {
     const size_t G = 4 * 256;            // (CTAs of the LM-head kernel <= SMs) x 4 lane quadrants
@@ -418,65 +424,67 @@ bool encode_q_map(tidar_ctx *c, CUtensorMap *tm, const void *q, int rows) {
   return c->encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(q), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+// K or V pages [page][kv head][64][head_dim]; a load brings one page of one KV head, the 64-element halves of the head one behind the other.
 bool encode_pages_map(tidar_ctx *c, CUtensorMap *tm, const void *pool, long long n_pages) {
   const tidar_config &cf = c->cfg;
-  cuuint64_t dims[4] = {(cuuint64_t)cf.head_dim, 64, (cuuint64_t)cf.n_kv_heads, (cuuint64_t)n_pages};
-  cuuint64_t strides[3] = {(cuuint64_t)cf.head_dim * 2, (cuuint64_t)64 * cf.head_dim * 2, (cuuint64_t)cf.n_kv_heads * 64 * cf.head_dim * 2};
-  cuuint32_t box[4] = {64, 64, 1, 1}, es[4] = {1, 1, 1, 1};
-  return c->encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(pool), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+  const cuuint64_t row = (cuuint64_t)cf.head_dim * 2;
+  cuuint64_t dims[5] = {64, 64, (cuuint64_t)cf.head_dim / 64, (cuuint64_t)cf.n_kv_heads, (cuuint64_t)n_pages};
+  cuuint64_t strides[4] = {row, 128, 64 * row, (cuuint64_t)cf.n_kv_heads * 64 * row};
+  cuuint32_t box[5] = {64, 64, (cuuint32_t)cf.head_dim / 64, 1, 1}, es[5] = {1, 1, 1, 1, 1};
+  return c->encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void *>(pool), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+// Step-local K or V rows [row][kv head][head_dim]; a load brings 64 rows in the layout of a page.
 bool encode_local_map(tidar_ctx *c, CUtensorMap *tm, const void *loc, long long rows) {
   const tidar_config &cf = c->cfg;
-  cuuint64_t dims[3] = {(cuuint64_t)cf.head_dim, (cuuint64_t)cf.n_kv_heads, (cuuint64_t)rows};
-  cuuint64_t strides[2] = {(cuuint64_t)cf.head_dim * 2, (cuuint64_t)cf.n_kv_heads * cf.head_dim * 2};
-  cuuint32_t box[3] = {64, 1, 64}, es[3] = {1, 1, 1};
-  return c->encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(loc), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+  const cuuint64_t head = (cuuint64_t)cf.head_dim * 2;
+  cuuint64_t dims[4] = {64, (cuuint64_t)rows, (cuuint64_t)cf.head_dim / 64, (cuuint64_t)cf.n_kv_heads};
+  cuuint64_t strides[3] = {(cuuint64_t)cf.n_kv_heads * head, 128, head};
+  cuuint32_t box[4] = {64, 64, (cuuint32_t)cf.head_dim / 64, 1}, es[4] = {1, 1, 1, 1};
+  return c->encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(loc), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                    CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Key-range split of the attention kernel: fill the SMs (two CTAs fit on one) without giving a
-// CTA fewer than two key tiles; and once half the SMs have a CTA, not fewer than four: a CTA pays
-// ~7 us of set-up, partial-result store and merge traffic whatever its key range, while a nearly
-// empty machine (a one-slot step) is served best by as many CTAs as there are key tiles to hand
-// out.  (8B-class heads, 1 k cached positions, 72 query-tile units: 4 splits of 4-5 tiles each
-// 26.9 us per call against 29.4 with 3 splits of 6; from 4 k positions on the limit is moot.)
-int attn_key_splits(const tidar_ctx *c, int units, int key_tiles_hint) {
-  int splits = 2 * c->n_sms / std::max(units, 1);
-  splits = std::min(splits, std::max(1, key_tiles_hint / 2));
-  splits = std::max(1, std::min(splits, attn_tc::MAX_SPLITS));
-  while (splits > 1 && units * splits > c->n_sms / 2 && key_tiles_hint / splits < 4) --splits;
-  return splits;
 }
 
 struct AttnMaps { const CUtensorMap *q, *k, *v, *kloc, *vloc; int page_base_k, page_base_v; };
 
-// rows_per_group: slots per sequence (k(k+1) in a step; all rows in a first-pass chunk); <= 0: the
-// sequences' groups differ in size and the query tiles come from the mixed step's tile table.
-// key_tiles_hint: rough number of 64-key tiles per row, to size the key split.
-void launch_attention_tc(tidar_ctx *c, const AttnMaps &m, const KvGeom &g, bf16 *O, int R, int rows_per_group, int key_tiles_hint) {
+// Units (up to two query tiles of one sequence) of a pass of R rows.  rows_per_group: slots per sequence (k(k+1) in a
+// step; all rows in a first-pass chunk); <= 0: the sequences' groups differ in size and the units come from the mixed
+// step's table.  Key ranges may be split (see attn_tc::plan_block) while there are fewer than three
+// (unit, KV head) combinations for two SMs: beyond that they fill the machine evenly enough.
+// The grid is the number of items the plan may use; a CTA holds a whole SM, so up to one combination per SM it is one wave.
+attn_tc::PlanArgs attention_plan(const tidar_ctx *c, int R, int rows_per_group) {
+  const tidar_config &cf = c->cfg;
+  attn_tc::PlanArgs p{};
+  p.R = R; p.spt = 128 / (cf.n_q_heads / cf.n_kv_heads); p.Hkv = cf.n_kv_heads;
+  if (rows_per_group > 0) {
+    p.rows_per_group = rows_per_group;
+    p.units_per_group = (rows_per_group + 2 * p.spt - 1) / (2 * p.spt);
+    p.n_units = (R + rows_per_group - 1) / rows_per_group * p.units_per_group;
+  } else {
+    p.rows_per_group = R; p.units_per_group = 1;
+    p.unit_row0 = c->d_unit_row0; p.unit_rend = c->d_unit_rend; p.n_units = c->mixed_units;
+  }
+  p.n_sms = c->n_sms;
+  const int units = p.n_units * p.Hkv;
+  static_assert(attn_tc::PLAN_UNITS >= 3 * MAX_SMS / 2, "units that may be split are planned");
+  p.max_items = units <= c->n_sms ? c->n_sms / p.Hkv : 2 * units < 3 * c->n_sms ? attn_tc::SLOTS_PER_SM * c->n_sms / p.Hkv : p.n_units;
+  p.items = c->plan_items; p.tiles = c->plan_tiles;
+  return p;
+}
+
+// Attention of the pass that plan p was made for (the plan itself is in device memory by then).
+void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMaps &m, const KvGeom &g, bf16 *O) {
   const tidar_config &cf = c->cfg;
   attn_tc::Args a{};
-  a.R = R; a.rows_per_group = rows_per_group;
-  a.G = cf.n_q_heads / cf.n_kv_heads; a.Hq = cf.n_q_heads; a.Hkv = cf.n_kv_heads;
-  a.spt = 128 / a.G;
-  if (rows_per_group > 0) {
-    a.tiles_per_group = (rows_per_group + a.spt - 1) / a.spt;
-    a.n_groups = (R + rows_per_group - 1) / rows_per_group;
-    a.n_tiles = a.n_groups * a.tiles_per_group;
-  } else {                       // groups of different sizes: the tile table of the mixed step
-    a.rows_per_group = R; a.tiles_per_group = 1; a.n_groups = 1;
-    a.tile_row0 = c->d_tile_row0; a.tile_rend = c->d_tile_rend; a.n_tiles = c->mixed_tiles;
-  }
-  const int units = a.n_tiles * a.Hkv;
-  a.splits = attn_key_splits(c, units, key_tiles_hint);
-  a.seq = c->meta.seq; a.nvis = c->meta.nvis; a.loc0 = c->meta.loc0; a.nloc = c->meta.nloc;
+  a.G = cf.n_q_heads / cf.n_kv_heads; a.Hq = cf.n_q_heads; a.Hkv = cf.n_kv_heads; a.spt = p.spt;
+  a.items = p.items; a.tiles = p.tiles;
+  a.nvis = c->meta.nvis; a.loc0 = c->meta.loc0; a.nloc = c->meta.nloc;
   a.page_table = g.page_table; a.pages_per_seq = g.pages_per_seq;
   a.page_base_k = m.page_base_k; a.page_base_v = m.page_base_v;
   a.scale_log2 = 1.4426950408889634f / sqrtf((float)cf.head_dim);
   a.O = O; a.part_O = c->attn_part_O; a.part_ml = c->attn_part_ml; a.status = c->d_status;
   a.tile_count = c->count_tiles ? c->d_tl + 2 * tidar_ctx::TL_MAX : nullptr;
-  const int grid = units * a.splits;
+  const int grid = p.max_items * p.Hkv;
   {
     Launch l(c, TIDAR_TC_ATTN);
     if (cf.head_dim == 128)
@@ -484,13 +492,11 @@ void launch_attention_tc(tidar_ctx *c, const AttnMaps &m, const KvGeom &g, bf16 
     else
       launch_pdl(attn_tc::attn_tc_kernel<64>, grid, attn_tc::THREADS, attn_tc::Smem<64>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
   }
-  if (a.splits > 1) {
+  if (p.max_items > p.n_units) {
     Launch l(c, TIDAR_TC_ATTN);
-    const size_t threads = (size_t)R * cf.n_q_heads * (cf.head_dim / 4);
-    if (cf.head_dim == 128)
-      launch_after(attn_tc::attn_combine_kernel<128>, (unsigned)((threads + 255) / 256), 256, 0, c->stream, c->attn_part_O, c->attn_part_ml, a.splits, R, cf.n_q_heads, O, l.tl);
-    else
-      launch_after(attn_tc::attn_combine_kernel<64>, (unsigned)((threads + 255) / 256), 256, 0, c->stream, c->attn_part_O, c->attn_part_ml, a.splits, R, cf.n_q_heads, O, l.tl);
+    const int blocks = 2 * p.n_units * p.Hkv * (cf.head_dim / 16);
+    if (cf.head_dim == 128) launch_pdl(attn_tc::attn_combine_kernel<128>, blocks, 256, 0, c->stream, a, l.tl);
+    else launch_pdl(attn_tc::attn_combine_kernel<64>, blocks, 256, 0, c->stream, a, l.tl);
   }
 }
 
@@ -522,14 +528,16 @@ struct MixRows { int n = 0, k = 1, a0 = 0, a_seq = 0, a_j = 0, b0 = 0, b_seq = 0
 
 // head_row0: the LM head (with_head) runs on rows [head_row0, R) only, followed by the mixed rows; the
 // argmax ids and the logits dump are indexed from head_row0.
-int forward_rows(tidar_ctx *c, int R, bool with_head, int rows_per_group, int key_tiles_hint, const MixRows &mix = MixRows(), int head_row0 = 0) {
+int forward_rows(tidar_ctx *c, int R, bool with_head, int rows_per_group, const MixRows &mix = MixRows(), int head_row0 = 0) {
   const tidar_config &cf = c->cfg;
   const int d = cf.d_model, hd = cf.head_dim, Hq = cf.n_q_heads, Hkv = cf.n_kv_heads;
   const KvGeom g = geom(c);
+  const attn_tc::PlanArgs plan = cf.impl == 0 ? attention_plan(c, R, rows_per_group) : attn_tc::PlanArgs{};
   {
     Launch l(c, TIDAR_TC_ROPE);
     const int n = R * (hd / 2);
-    launch_after(rope_table_kernel, (n + 255) / 256, 256, 0, c->stream, c->meta.pos, R, hd / 2, (double)cf.rope_theta, c->rope_cos, c->rope_sin, l.tl);
+    launch_after(pass_setup_kernel, (n + 255) / 256 + (plan.tiles ? 1 : 0), 256, 0, c->stream, c->meta, R, hd / 2, (double)cf.rope_theta, c->rope_cos,
+                 c->rope_sin, plan, l.tl);
   }
   int S = 0; size_t stride = 0;          // pending partials of the previous down projection
   const bool tc = cf.impl == 0;
@@ -556,7 +564,7 @@ if (tc && c->slab_bf16)
     }
     if (tc) {
       AttnMaps am{&c->tm_q, &c->tm_kv, &c->tm_kv, &c->tm_kloc, &c->tm_vloc, (2 * l) * c->n_pages, (2 * l + 1) * c->n_pages};
-      launch_attention_tc(c, am, g, c->O, R, rows_per_group, key_tiles_hint);
+      launch_attention_tc(c, plan, am, g, c->O);
     } else {
       launch_attention(c, c->Q, Kp, Vp, g, c->Kloc, c->Vloc, c->O, R);
     }
@@ -617,6 +625,7 @@ int init_tensor_core_path(tidar_ctx *c) {
   CUDA_TRY(c, cudaGetDeviceProperties(&prop, dev));
   if (prop.major != 10) return fail(c, TIDAR_ECUDA, "the tensor-core path needs an sm_100 device, found sm_%d%d", prop.major, prop.minor);
   c->n_sms = prop.multiProcessorCount;
+  if (c->n_sms > MAX_SMS) return fail(c, TIDAR_ECUDA, "%d SMs; scratch is sized for %d", c->n_sms, MAX_SMS);
   void *fn = nullptr;
   cudaDriverEntryPointQueryResult qres;
   CUDA_TRY(c, cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres));
@@ -703,7 +712,7 @@ int ensure_pages(tidar_ctx *c, int seq, int upto_positions) {
 // k: block length of this step; ar: plain autoregressive step (the causal section alone).
 // mixed_R > 0: the listed sequences use different block lengths (layout staged in h_lay, mixed_R rows in all).
 // mixed_K: the sum of those block lengths (= verified positions, one mixed row each when beta < 1).
-int record_step(tidar_ctx *c, int n_seqs, int k, int key_tiles_hint, bool ar, int mixed_R = 0, int mixed_K = 0) {
+int record_step(tidar_ctx *c, int n_seqs, int k, bool ar, int mixed_R = 0, int mixed_K = 0) {
   const tidar_config &cf = c->cfg;
   const int n_blocks = ar ? 0 : k;
   const int T = k * (n_blocks + 1), R = mixed_R > 0 ? mixed_R : n_seqs * T;
@@ -727,7 +736,7 @@ int record_step(tidar_ctx *c, int n_seqs, int k, int key_tiles_hint, bool ar, in
     if (mixed_R > 0) { mix.n = mixed_K; mix.lay = lay; }
     else { mix.n = n_seqs * k; mix.k = k; mix.a0 = 0; mix.a_seq = T; mix.a_j = 1; mix.b0 = k; mix.b_seq = T; mix.b_j = k; }
   }
-  if (int rc = forward_rows(c, R, true, mixed_R > 0 ? 0 : T, key_tiles_hint, mix)) return rc;
+  if (int rc = forward_rows(c, R, true, mixed_R > 0 ? 0 : T, mix)) return rc;
   {
     Launch l(c, TIDAR_TC_VERIFY);
     launch_after(verify_select_kernel, n_seqs, 32, 0, c->stream, c->d_arg_idx, mix.n ? c->d_arg_idx + R : (const int32_t *)nullptr, c->d_step_seqs,
@@ -744,15 +753,13 @@ int record_step(tidar_ctx *c, int n_seqs, int k, int key_tiles_hint, bool ar, in
 
 // Every launch of a step has the same arguments from step to step (lengths, page tables, token
 // blocks and, for a step of mixed block lengths, the row layout live in device memory), except
-// for the grid sizes and the attention key split, so the step is captured once per (k, n_seqs,
-// rows, query tiles, split) and replayed.  Per-launch timing and the debug read-backs use plain
-// launches.  tiles: query tiles of the attention kernel per KV head.
-int replay_or_record_step(tidar_ctx *c, int n_seqs, int k, int hint, bool ar, int mixed_R, int tiles, int mixed_K = 0) {
+// for the grid sizes, so the step is captured once per (k, n_seqs, rows, query tiles) and replayed.  Per-launch timing and the debug read-backs use plain
+// launches.  tiles: attention units per KV head.
+int replay_or_record_step(tidar_ctx *c, int n_seqs, int k, bool ar, int mixed_R, int tiles, int mixed_K = 0) {
   const tidar_config &cf = c->cfg;
   if (cf.impl == 0 && c->graphs_ok && !c->timing && !(cf.debug & (1 | 8))) {
-    const int splits = attn_key_splits(c, tiles * cf.n_kv_heads, hint);
     tidar_ctx::StepGraph &sg = c->sg;
-    if (!sg.exec || sg.k != k || sg.ar != ar || sg.n_seqs != n_seqs || sg.splits != splits || sg.timeline != c->timeline ||
+    if (!sg.exec || sg.k != k || sg.ar != ar || sg.n_seqs != n_seqs || sg.timeline != c->timeline ||
         sg.mixed_R != mixed_R || sg.tiles != tiles || sg.mixed_K != mixed_K) {
       if (sg.exec) {
         if (!c->inflight.empty()) CUDA_TRY(c, cudaStreamSynchronize(c->stream));    // the old graph may still be running
@@ -763,7 +770,7 @@ int replay_or_record_step(tidar_ctx *c, int n_seqs, int k, int hint, bool ar, in
       int rc = TIDAR_OK;
       cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
-        rc = record_step(c, n_seqs, k, hint, ar, mixed_R, mixed_K);
+        rc = record_step(c, n_seqs, k, ar, mixed_R, mixed_K);
         e = cudaStreamEndCapture(c->stream, &graph);
       }
       if (e == cudaSuccess && rc == TIDAR_OK && graph) e = cudaGraphInstantiate(&sg.exec, graph, 0);
@@ -772,7 +779,7 @@ int replay_or_record_step(tidar_ctx *c, int n_seqs, int k, int hint, bool ar, in
         cudaGetLastError();                         // capture is not available here: plain launches from now on
         sg.exec = nullptr; c->graphs_ok = false;
       } else {
-        sg.k = k; sg.ar = ar; sg.n_seqs = n_seqs; sg.splits = splits; sg.timeline = c->timeline; sg.mixed_R = mixed_R; sg.tiles = tiles; sg.mixed_K = mixed_K;
+        sg.k = k; sg.ar = ar; sg.n_seqs = n_seqs; sg.timeline = c->timeline; sg.mixed_R = mixed_R; sg.tiles = tiles; sg.mixed_K = mixed_K;
         sg.launches = c->launches - l0;
       }
       c->launches = l0;
@@ -783,7 +790,7 @@ int replay_or_record_step(tidar_ctx *c, int n_seqs, int k, int hint, bool ar, in
       return TIDAR_OK;
     }
   }
-  return record_step(c, n_seqs, k, hint, ar, mixed_R, mixed_K);
+  return record_step(c, n_seqs, k, ar, mixed_R, mixed_K);
 }
 
 // Whether one more step may be enqueued: always when none is in flight; behind a step in flight only when
@@ -797,11 +804,11 @@ bool may_enqueue(tidar_ctx *c, bool all_forced, bool mixed) {
 
 // The step proper: its inputs from the slot's pinned staging, the kernels (replayed graph or plain
 // launches), its results into the slot's pinned buffers, and the event its waiter blocks on.
-int launch_step(tidar_ctx *c, int n_seqs, int k, int hint, bool ar, int mixed_R, int tiles, int slot, int mixed_K = 0) {
+int launch_step(tidar_ctx *c, int n_seqs, int k, bool ar, int mixed_R, int tiles, int slot, int mixed_K = 0) {
   const tidar_config &cf = c->cfg;
   CUDA_TRY(c, cudaMemcpyAsync(c->d_step_seqs, c->h_stage2[slot], n_seqs * sizeof(int), cudaMemcpyHostToDevice, c->stream));
   CUDA_TRY(c, cudaMemcpyAsync(c->d_forced, c->h_stage2[slot] + cf.max_batch, n_seqs * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  if (int rc = replay_or_record_step(c, n_seqs, k, hint, ar, mixed_R, tiles, mixed_K)) return rc;
+  if (int rc = replay_or_record_step(c, n_seqs, k, ar, mixed_R, tiles, mixed_K)) return rc;
   CUDA_TRY(c, cudaMemcpyAsync(c->h_out2[slot], c->d_out, (size_t)n_seqs * (cf.k_max + 1) * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaMemcpyAsync(c->h_status2[slot], c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaEventRecord(c->flight_done[slot], c->stream));
@@ -857,11 +864,8 @@ int enqueue_step(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int32_t *f
   const int T = ar ? 1 : k * (k + 1), R = n_seqs * T;
   const int slot = c->next_slot;
   for (int i = 0; i < n_seqs; ++i) { c->h_stage2[slot][i] = seqs[i]; c->h_stage2[slot][cf.max_batch + i] = forced ? forced[i] : 0; }
-  int min_n = 1 << 30;
-  for (int i = 0; i < n_seqs; ++i) min_n = std::min(min_n, c->seqs[seqs[i]].n);
-  const int hint = (min_n + k + 63) / 64;
-  const int spt = 128 / (cf.n_q_heads / cf.n_kv_heads);          // slots per attention query tile
-  if (int rc = launch_step(c, n_seqs, k, hint, ar, 0, n_seqs * ((T + spt - 1) / spt), slot)) return rc;
+  const int spt = 2 * (128 / (cf.n_q_heads / cf.n_kv_heads));      // slots per attention unit (two query tiles)
+  if (int rc = launch_step(c, n_seqs, k, ar, 0, n_seqs * ((T + spt - 1) / spt), slot)) return rc;
   push_flight(c, seqs, n_seqs, forced, k, nullptr, slot);
   c->last_hidden_off = 0;
   c->last_rows = R + ((cf.beta < 1.0f && !ar) ? n_seqs * k : 0); c->last_first_pos = -1;      // the mixed rows follow the slots
@@ -895,23 +899,22 @@ int enqueue_step_mixed(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int3
   }
   for (int i = 0; i < n_seqs; ++i)
     if (int rc = ensure_pages(c, seqs[i], c->seqs[seqs[i]].n + ks[i])) return rc;
-  const int mb = cf.max_batch, spt = 128 / (cf.n_q_heads / cf.n_kv_heads);
+  const int mb = cf.max_batch, spt = 2 * (128 / (cf.n_q_heads / cf.n_kv_heads));
   int32_t *hk = c->h_lay, *hoff = hk + (mb + 1), *hloc = hoff + (mb + 1), *ht0 = hloc + (mb + 1), *hte = ht0 + (c->R_head + mb);
   const int slot = c->next_slot;
-  int R = 0, loc = 0, tiles = 0, min_nk = 1 << 30, sum_k = 0;
+  int R = 0, loc = 0, tiles = 0, sum_k = 0;
   for (int i = 0; i < n_seqs; ++i) {
     const int k = ks[i], T = k * (k + 1);
     hk[i] = k; hoff[i] = R; hloc[i] = loc; sum_k += k;
     for (int r0 = R; r0 < R + T; r0 += spt) { ht0[tiles] = r0; hte[tiles] = R + T; ++tiles; }
     R += T; loc += k * k;
-    min_nk = std::min(min_nk, c->seqs[seqs[i]].n + k);
     c->h_stage2[slot][i] = seqs[i]; c->h_stage2[slot][mb + i] = forced ? forced[i] : 0;
   }
   hk[n_seqs] = 0; hoff[n_seqs] = R; hloc[n_seqs] = loc;
-  c->mixed_tiles = tiles;
+  c->mixed_units = tiles;
   // a mixed step's kernels take every per-sequence length from the staged layout: the nominal k is unused
   const int mixed_rows = cf.beta < 1.0f ? sum_k : 0;         // one mixed LM-head input row per verified position
-  if (int rc = launch_step(c, n_seqs, 0, (min_nk + 63) / 64, false, R, tiles, slot, mixed_rows)) return rc;
+  if (int rc = launch_step(c, n_seqs, 0, false, R, tiles, slot, mixed_rows)) return rc;
   push_flight(c, seqs, n_seqs, forced, 0, ks, slot);
   c->last_hidden_off = 0;
   c->last_rows = R + mixed_rows; c->last_first_pos = -1;
@@ -1072,7 +1075,7 @@ int tidar_prefill(tidar_ctx *c, int32_t seq, const int32_t *prompt, int32_t n_pr
     // logits are needed for the last prompt row and the k mask rows only; the LM head runs on the
     // trailing rows of the last chunk, as many as a decode step has (all of them for a short prompt)
     const int head_row0 = last ? std::max(0, rows + mix.n - c->R_head) : 0;
-    if (int rc = forward_rows(c, rows, last, rows, (row0 + rows / 2 + 63) / 64, mix, head_row0)) return rc;
+    if (int rc = forward_rows(c, rows, last, rows, mix, head_row0)) return rc;
     if (last) {
       Launch l(c, TIDAR_TC_VERIFY);
       prefill_finish_kernel<<<1, 32, 0, c->stream>>>(c->d_arg_idx, rlp - head_row0, (mix.n ? rows : rlp) - head_row0, k, cf.k_max, seq, n_prompt,
@@ -1189,7 +1192,7 @@ int tidar_score(tidar_ctx *c, int32_t seq, const int32_t *ids, int32_t n, float 
       Launch l(c, TIDAR_TC_EMBED);
       assemble_prefill_kernel<<<rows, 256, 0, c->stream>>>(c->meta, seq, row0, n, 0, cf.mask_token_id, c->d_prompt, c->embed, d, c->X, 0, 0ull);
     }
-    if (int rc = forward_rows(c, rows, false, rows, (row0 + rows / 2 + 63) / 64)) return rc;      // ends with the final norm in c->A
+    if (int rc = forward_rows(c, rows, false, rows)) return rc;      // ends with the final norm in c->A
     for (int v0 = 0, ci = 0; v0 < cf.vocab; v0 += c->lm_chunk, ++ci) {
       const int nc = std::min(c->lm_chunk, cf.vocab - v0);
       int S = 1; size_t stride = 0;
@@ -1415,10 +1418,12 @@ int tidar_attention(tidar_ctx *c, const void *q, const void *k_pages, const void
   if (((uintptr_t)q | (uintptr_t)k_pages | (uintptr_t)v_pages | (uintptr_t)k_local | (uintptr_t)v_local | (uintptr_t)out) % 16 ||
       ((uintptr_t)page_table | (uintptr_t)seq_len) % 4)
     return fail(c, TIDAR_EINVAL, "tensors must be 16-byte aligned (page_table and seq_len 4-byte)");
-  const int R = n_seqs * k * (k + 1);
+  const int R = n_seqs * k * (k + 1), n_max = pages_per_seq * c->cfg.page_size - k;
+  const attn_tc::PlanArgs plan = c->cfg.impl == 0 ? attention_plan(c, R, k * (k + 1)) : attn_tc::PlanArgs{};
   {
     Launch l(c, TIDAR_TC_EMBED);
-    attn_meta_kernel<<<(R + 127) / 128, 128, 0, c->stream>>>(c->meta, seq_len, k, R, pages_per_seq * c->cfg.page_size - k);
+    if (c->cfg.impl == 0) launch_pdl(attn_meta_plan_kernel, 1 + (R + 511) / 512, 512, 0, c->stream, c->meta, seq_len, k, R, n_max, plan);
+    else attn_meta_kernel<<<(R + 127) / 128, 128, 0, c->stream>>>(c->meta, seq_len, k, R, n_max);
   }
   KvGeom g{c->cfg.n_kv_heads, c->cfg.head_dim, c->cfg.page_size, pages_per_seq, page_table, n_pages};
   if (c->cfg.impl == 0) {
@@ -1427,7 +1432,7 @@ int tidar_attention(tidar_ctx *c, const void *q, const void *k_pages, const void
         !encode_local_map(c, &tkl, k_local, (long long)n_seqs * k * k) || !encode_local_map(c, &tvl, v_local, (long long)n_seqs * k * k))
       return fail(c, TIDAR_ECUDA, "cuTensorMapEncodeTiled failed for an attention operand");
     AttnMaps am{&tq, &tk, &tv, &tkl, &tvl, 0, 0};
-    launch_attention_tc(c, am, g, (bf16 *)out, R, k * (k + 1), pages_per_seq);
+    launch_attention_tc(c, plan, am, g, (bf16 *)out);
   } else {
     launch_attention(c, (const bf16 *)q, (const bf16 *)k_pages, (const bf16 *)v_pages, g, (const bf16 *)k_local, (const bf16 *)v_local,
                      (bf16 *)out, R);

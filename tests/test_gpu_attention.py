@@ -114,3 +114,15 @@ def test_attention_microbench_sizes_sampled_rows(n):
     t = Tidar(sh, pack_weights(gen_model_weights(sh), "cuda:0"), k_max=16, max_batch=1, max_seq_len=128, impl=0)
     _case_sampled(t, 128, 32, 8, 16, n, 40 + n % 97)
     t.close()
+
+
+@pytest.mark.parametrize("ns,k", [
+    ([3000, 5, 700], 4),          # one long sequence among short ones: its key range is cut into items, the others' are not
+    ([2500], 1),                  # a single query tile: more items than the page ids one warp holds at a time
+    ([2] * 200 + [300] * 30, 1),  # more (tile pair, KV head) units than three for two SMs: nothing is split
+    ([1, 0, 66] * 180, 1),        # more tile pairs than the plan ranks by length
+])
+def test_attention_work_plan(ns, k):
+    t = _ctx(64, 4, 2, 8, 32, 0)
+    _case(t, 64, 4, 2, k, ns, 31)
+    t.close()
