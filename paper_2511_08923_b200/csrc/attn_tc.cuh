@@ -283,7 +283,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   using L = Smem<HD>;
   constexpr int NH = L::NH;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  pdl_trigger();
   const int warp = sm100::warp_index(), lane = threadIdx.x & 31;
   const uint32_t smem0 = sm100::smem_u32(smem_raw);
   if (smem0 & 1023u) {                               // cannot place swizzled tiles: report, touch nothing
@@ -316,6 +315,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   const uint32_t tmem = ctl.tmem_base;
   const uint32_t tmem_S = tmem, tmem_O = tmem + 4 * PAGE;             // per stream: 2 x 64 columns of S, HD columns of O
   volatile int *abortp = &ctl.abort_flag;
+  pdl_trigger();              // not before the tensor memory is ours (see gemm_tc_kernel)
   pdl_wait();                 // everything below reads what earlier kernels of the pass wrote
   if (threadIdx.x == 0) tl_go(tl);
 

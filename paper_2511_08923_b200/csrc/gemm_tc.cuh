@@ -23,6 +23,7 @@
 #pragma once
 #include "common.cuh"
 #include "sm100_ptx.cuh"
+#include <algorithm>
 
 namespace gemm_tc {
 
@@ -37,6 +38,22 @@ constexpr int W_STAGE_BYTES = TILE_N * TILE_K * 2;
 constexpr int SMEM_BUDGET = 216 * 1024;   // dynamic shared memory for the rings; up to 9 KB of static shared memory come on top
 constexpr int TMEM_COLS = 512;
 
+// Few rows (SMALL instances: a row block of at most SMALL_ROWS).  Such a launch is bound by streaming its weights, but a
+// good part of its time used to be spent elsewhere:
+// * Before the first weights had arrived: with all of an SM's registers, a CTA could not become resident before the
+//   SM had emptied.  A SMALL CTA takes 80 registers per thread and 128 TMEM columns, so it sits beside the kernels
+//   between two projections, its ring full of weights by the time its activations are ready.
+// * Per stage: each costs its producers, the watcher and the MMA warp some 600 cycles of barrier tests and issue,
+//   three times what the MMAs of a 64-wide K block take with few rows.  A stage holds two K blocks there.
+// 1.5B-class autoregressive step of 8 rows 1.90 -> 1.75 ms, 8B-class step of 20 rows 4.2 -> 4.0 ms (the gate/up projection
+// of the former 11.4 -> 10.3 us, QKV 5.3 -> 3.4 us).  Measured and not kept: fetching weights into L2 ahead of the ring, this
+// launch's or the next projection's (2 - 8 % slower, the more the further ahead).
+constexpr int SMALL_ROWS = 96;
+__host__ __device__ constexpr int k_per_stage(bool small) { return small ? 2 : 1; }     // K blocks of 64 per stage
+constexpr int SMALL_SMEM_BUDGET = 212 * 1024;
+constexpr int MAX_STAGES = 12;      // of the weight ring (hardware barriers 1 .. 12)
+constexpr int SMALL_TMEM_COLS = 128;
+
 // MODE_SAMPLE is MODE_ARGMAX with Gumbel noise added to the tempered logits (a draw per row instead of
 // the argmax); it is a mode of its own so that the greedy LM head carries none of its registers.
 enum Mode { MODE_SLAB = 0, MODE_SWIGLU = 1, MODE_ARGMAX = 2, MODE_SAMPLE = 3 };
@@ -50,7 +67,7 @@ struct Args {
   int fused_items;          // items [0, fused_items) are whole tiles 0.. (no K split) finished by the mode's own epilogue;
                             // the rest are tiles tile_b0.. split S ways along K, written as fp32 slabs
   int tile_b0, n_tiles_b;   // first tile and tile count of the split region
-  int kb_total;             // K / 64
+  int kb_total;             // stages of K: K / 64, or half of it (rounded up) in a SMALL launch
   int w_stages, a_stages;   // depths of the weight ring (<= 8) and of the activation ring (<= w_stages)
   int box_rows, n_box;      // activation rows per TMA box, boxes per stage
   int n1, n2;               // MMA N of the two instructions (n2 may be 0)
@@ -96,25 +113,27 @@ __device__ __forceinline__ Item decode_item(const Args &g, int item) {
 // the right limit (-0) when exp(-g) overflows.
 __device__ __forceinline__ float silu_mul(float g, float u) { return __fdividef(g, 1.f + __expf(-g)) * u; }
 
-template <int MODE>
-__global__ void __launch_bounds__(THREADS, 1)
+template <int MODE, bool SMALL = false>
+__global__ void __launch_bounds__(THREADS, SMALL ? 2 : 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmA, const Args g, const TlSlot tl) {
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t w_full[8], w_empty[8], a_full[8], a_empty[8], tmem_full_bar, tmem_empty_bar;
+  __shared__ __align__(8) uint64_t w_full[MAX_STAGES], w_empty[MAX_STAGES], a_full[MAX_STAGES], a_empty[MAX_STAGES], tmem_full_bar, tmem_empty_bar;
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
   __shared__ __align__(16) uint16_t epi_stage[MODE == MODE_SWIGLU ? EPI_WARPS : 1][32][16];   // MODE_SWIGLU: two 16-column chunks per epilogue warp, [column][feature]
 
-  pdl_trigger();
+  constexpr int KPS = k_per_stage(SMALL);
+  constexpr int W_STAGE = KPS * W_STAGE_BYTES;
+  constexpr int NCH = SMALL ? SMALL_ROWS / 32 : 9;         // 16-column chunks of the accumulator per epilogue warp
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t smem0 = (sm100::smem_u32(smem_raw) + 1023u) & ~1023u;
-  const int a_stage_bytes = g.rb_rows * TILE_K * 2;                 // multiple of 1024 (rb_rows % 16 == 0)
-  const uint32_t smem_a0 = smem0 + (uint32_t)g.w_stages * W_STAGE_BYTES;   // activation ring behind the weight ring
+  const int a_stage_bytes = KPS * g.rb_rows * TILE_K * 2;           // multiple of 1024 (rb_rows % 16 == 0)
+  const uint32_t smem_a0 = smem0 + (uint32_t)g.w_stages * W_STAGE;   // activation ring behind the weight ring
   const int n_items = g.total_items();
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
-    for (int s = 0; s < 8; ++s) {
+    for (int s = 0; s < MAX_STAGES; ++s) {
       sm100::mbar_init(sm100::smem_u32(&w_full[s]), 1); sm100::mbar_init(sm100::smem_u32(&w_empty[s]), 1);
       sm100::mbar_init(sm100::smem_u32(&a_full[s]), 1); sm100::mbar_init(sm100::smem_u32(&a_empty[s]), 1);
     }
@@ -124,13 +143,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   }
   if (warp == 1) {
     __syncwarp();
-    sm100::tmem_alloc(sm100::smem_u32(&tmem_base_slot), TMEM_COLS);
+    sm100::tmem_alloc(sm100::smem_u32(&tmem_base_slot), SMALL ? SMALL_TMEM_COLS : TMEM_COLS);
     sm100::tmem_relinquish();
   }
   sm100::tc_fence_before();
   __syncthreads();
   sm100::tc_fence_after();
   const uint32_t tmem_acc = tmem_base_slot;
+  // Only now may the next kernel's CTAs be scheduled: one that got in before this CTA had its tensor memory could take
+  // it, and would keep it while it waits for this kernel.
+  pdl_trigger();
   volatile int *abortp = &abort_flag;
 
   // The epilogue warps hold the whole accumulator (144 registers per thread) next to their
@@ -141,7 +163,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   // the register budget of that code.)
 
   if (warp < ROLE_WARPS) {
-  sm100::setmaxnreg_dec<ROLE_REGS>();
+  if constexpr (!SMALL) sm100::setmaxnreg_dec<ROLE_REGS>();
   if (warp == 0) {
     // ===================== weight producer =====================
     if (lane == 0) {
@@ -155,8 +177,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         for (int kb = w.kb0; kb < w.kb1; ++kb) {
           if (!sm100::mbar_wait(sm100::smem_u32(&w_empty[s]), ph ^ 1u, abortp)) { ok = false; break; }
           const uint32_t fb = sm100::smem_u32(&w_full[s]);
-          sm100::mbar_expect_tx(fb, (uint32_t)W_STAGE_BYTES);
-          sm100::tma_load_2d(smem0 + (uint32_t)s * W_STAGE_BYTES, &tmW, fb, kb * TILE_K, w.tile * TILE_N, pol_w);
+          sm100::mbar_expect_tx(fb, (uint32_t)W_STAGE);
+          if constexpr (SMALL) sm100::tma_load_3d(smem0 + (uint32_t)s * W_STAGE, &tmW, fb, 0, w.tile * TILE_N, kb * KPS, pol_w);
+          else sm100::tma_load_2d(smem0 + (uint32_t)s * W_STAGE, &tmW, fb, kb * TILE_K, w.tile * TILE_N, pol_w);
           if (++s == g.w_stages) { s = 0; ph ^= 1u; }
         }
       }
@@ -176,6 +199,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           const uint32_t fb = sm100::smem_u32(&a_full[s]);
           const uint32_t sa = smem_a0 + (uint32_t)s * a_stage_bytes;
           sm100::mbar_expect_tx(fb, (uint32_t)a_stage_bytes);
+          if constexpr (SMALL) sm100::tma_load_3d(sa, &tmA, fb, 0, w.rb * g.rb_rows, kb * KPS, pol_a);
+          else
           for (int b = 0; b < g.n_box; ++b)
             sm100::tma_load_2d(sa + (uint32_t)(b * g.box_rows * TILE_K * 2), &tmA, fb, kb * TILE_K, w.rb * g.rb_rows + b * g.box_rows, pol_a);
           if (++s == g.a_stages) { s = 0; ph ^= 1u; }
@@ -198,7 +223,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // and the status word reports the failure.
     const uint32_t idesc1 = sm100::make_idesc_bf16(TILE_N, g.n1), idesc2 = sm100::make_idesc_bf16(TILE_N, g.n2 ? g.n2 : 16);
     const uint64_t wdesc0 = sm100::make_desc_sw128(smem0), adesc0 = sm100::make_desc_sw128(smem_a0);   // stage 0 of each ring
-    const uint64_t wstage16 = (uint64_t)(W_STAGE_BYTES >> 4), astage16 = (uint64_t)(a_stage_bytes >> 4);
+    const uint64_t wstage16 = (uint64_t)(W_STAGE >> 4), astage16 = (uint64_t)(a_stage_bytes >> 4);
     const uint64_t a2_off16 = (uint64_t)(g.n1 * 8);
     const uint32_t tmem_acc2 = tmem_acc + (uint32_t)g.n1;
     const bool two = g.n2 != 0;
@@ -212,7 +237,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         sm100::named_bar_sync(1u + (uint32_t)s, 64);
         sm100::tc_fence_after();
         if (lane == 0) {
-          if (two) {
+          if constexpr (SMALL) {
+            const uint64_t a_kb16 = (uint64_t)(g.rb_rows * 8);         // the stage's second K block, 16-byte units
+#pragma unroll
+            for (int kk = 0; kk < KPS * TILE_K / 16; ++kk) {
+              sm100::mma_bf16_ss(tmem_acc, wd + (kk / 4) * (W_STAGE_BYTES >> 4) + 2 * (kk % 4), ad + (kk / 4) * a_kb16 + 2 * (kk % 4), idesc1, acc);
+              acc = 1u;
+            }
+          } else if (two) {
             const uint64_t ad2 = ad + a2_off16;
 #pragma unroll
             for (int kk = 0; kk < TILE_K / 16; ++kk) {
@@ -267,7 +299,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     }
   }
   } else {
-    sm100::setmaxnreg_inc<EPI_REGS>();
+    if constexpr (!SMALL) sm100::setmaxnreg_inc<EPI_REGS>();
     // ===================== epilogue =====================
     pdl_wait();
     const int q = warp & 3;                      // TMEM lane quadrant this warp may read
@@ -357,12 +389,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // brings the code in; g.warm_epilogue is a run-time value so that both walks share one copy.
     // A fused item that is its CTA's last one takes a third route: nobody waits for the accumulator, so it
     // stays in tensor memory and a loop of a few hundred instructions takes 32 columns per round (the
-    // 1.5B-class gate/up projection, one item per CTA, ends 4 us earlier than with the long code).
-    bool dry = (MODE == MODE_SWIGLU) && g.warm_epilogue != 0 && (int)(blockIdx.x + gridDim.x) < n_items;
+    // 1.5B-class gate/up projection, one item per CTA, ends 4 us earlier than with the long code).  With few rows
+    // every fused item goes that way: it is one or two rounds.
+    bool dry = (MODE == MODE_SWIGLU) && !SMALL && g.warm_epilogue != 0 && (int)(blockIdx.x + gridDim.x) < n_items;
     for (int item = blockIdx.x; item < n_items && ok;) {
       const Item w = decode_item<MODE>(g, item);
       const int split = w.split, tile = w.tile, rb = w.rb;
-      if (MODE == MODE_SWIGLU && w.fused && item + (int)gridDim.x >= n_items) {
+      if (MODE == MODE_SWIGLU && w.fused && (SMALL || item + (int)gridDim.x >= n_items)) {
         if (!sm100::mbar_wait(sm100::smem_u32(&tmem_full_bar), it & 1u, abortp)) { ok = false; break; }
         sm100::tc_fence_after();
         const uint32_t t0 = tmem_acc + ((uint32_t)(q * 32) << 16) + (uint32_t)c_begin;
@@ -382,13 +415,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         item += gridDim.x; ++it;
         continue;
       }
-      uint32_t v[9][16];
+      uint32_t v[NCH][16];
       if (!dry) {
         if (!sm100::mbar_wait(sm100::smem_u32(&tmem_full_bar), it & 1u, abortp)) { ok = false; break; }
         sm100::tc_fence_after();
         const uint32_t t0 = tmem_acc + ((uint32_t)(q * 32) << 16) + (uint32_t)c_begin;
 #pragma unroll
-        for (int i = 0; i < 9; ++i)
+        for (int i = 0; i < NCH; ++i)
           if (i * 16 < ncols) sm100::tmem_ld16(t0 + i * 16, v[i]);
         sm100::tmem_wait_ld();
         sm100::tc_fence_before();
@@ -410,7 +443,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           float *p = reinterpret_cast<float *>(g.out) + (long long)split * g.slab_stride + nc + (long long)r_base * g.ldo;
           const int rows_left = n_ok ? R_live - r_base : 0;
 #pragma unroll
-          for (int i = 0; i < 9; ++i) {
+          for (int i = 0; i < NCH; ++i) {
             if (i * 16 < ncols) {
 #pragma unroll
               for (int j = 0; j < 16; ++j) {
@@ -425,7 +458,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           bf16 *o = reinterpret_cast<bf16 *>(g.out) + (long long)split * g.slab_stride + (nc & ~1);
           const bool odd = lane & 1;
 #pragma unroll
-          for (int i = 0; i < 9; ++i) {
+          for (int i = 0; i < NCH; ++i) {
             if (i * 16 < ncols) {
 #pragma unroll
               for (int j = 0; j < 16; j += 2) {
@@ -442,16 +475,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
             }
           }
         }
-      } else if (MODE == MODE_SWIGLU) {
+      } else if (MODE == MODE_SWIGLU && !SMALL) {
         // Register-staged walk over the whole accumulator, two 16-column chunks per pass.
 #pragma unroll
-        for (int ip = 0; ip < 5; ++ip) {
+        for (int ip = 0; ip < (NCH + 1) / 2; ++ip) {
           if (ip * 32 < ncols) {
-            const bool second = (2 * ip + 1) < 9 && (2 * ip + 1) * 16 < ncols;      // warp-uniform
-            swiglu_pass(v[2 * ip], v[(2 * ip + 1) < 9 ? 2 * ip + 1 : 8], second, r_base + ip * 32, R_live, tile);
+            const bool second = (2 * ip + 1) < NCH && (2 * ip + 1) * 16 < ncols;    // warp-uniform
+            swiglu_pass(v[2 * ip], v[(2 * ip + 1) < NCH ? 2 * ip + 1 : NCH - 1], second, r_base + ip * 32, R_live, tile);
           }
         }
-      } else {
+      } else if (MODE == MODE_ARGMAX || MODE == MODE_SAMPLE) {
         // Per column: best (value, index) over the 32 features of this warp, folded into a
         // running best over all tiles this CTA processes.  The 32 lanes x 32 columns of a
         // group are reduced by recursive halving: in the step with stride h a lane keeps the
@@ -463,7 +496,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         const int my_idx = (n_ok ? g.col0 + n : 0x7fffffff);
         if (g.dump && n_ok) {
 #pragma unroll
-          for (int i = 0; i < 9; ++i)
+          for (int i = 0; i < NCH; ++i)
             if (i * 16 < ncols) {
 #pragma unroll
               for (int j = 0; j < 16; ++j) {
@@ -473,13 +506,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
             }
         }
 #pragma unroll
-        for (int grp = 0; grp < 5; ++grp) {
+        for (int grp = 0; grp < (NCH + 1) / 2; ++grp) {
           if (grp * 32 < ncols) {
             float val[32]; int idx[32];
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
               const int i = grp * 2 + (j >> 4);
-              float x = (i < 9 && i * 16 < ncols) ? __uint_as_float(v[i < 9 ? i : 8][j & 15]) : -INFINITY;
+              float x = (i < NCH && i * 16 < ncols) ? __uint_as_float(v[i < NCH ? i : NCH - 1][j & 15]) : -INFINITY;
               if (MODE == MODE_SAMPLE) {
                 const int r = r_base + grp * 32 + j;
                 if (r < g.R && n_ok) x = x * g.inv_temp + gumbel_noise(g.skey[r], (uint32_t)my_idx);
@@ -526,7 +559,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   if (warp == 1) {
     __syncwarp();
     sm100::tc_fence_after();
-    sm100::tmem_dealloc(tmem_acc, TMEM_COLS);
+    sm100::tmem_dealloc(tmem_acc, SMALL ? SMALL_TMEM_COLS : TMEM_COLS);
   }
   if (threadIdx.x == 0) tl_end(tl);
 }
@@ -547,6 +580,17 @@ inline CUresult encode_2d(EncodeTiledFn fn, CUtensorMap *tm, const void *base, u
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
+// The same matrix for SMALL launches: box = two 64-column blocks of box_rows rows, one block behind the other (a last block
+// that does not exist reads as zero).
+inline CUresult encode_2d_small(EncodeTiledFn fn, CUtensorMap *tm, const void *base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+  cuuint64_t dims[3] = {(cuuint64_t)TILE_K, rows, cols / TILE_K};
+  cuuint64_t strides[2] = {cols * 2, TILE_K * 2};
+  cuuint32_t box[3] = {(cuuint32_t)TILE_K, box_rows, (cuuint32_t)k_per_stage(true)};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+}
+
 // Row-block geometry for R activation rows.
 inline void plan_rows(int R, Args &a, int max_rows = MAX_ROWS) {
   a.n_rb = (R + max_rows - 1) / max_rows;
@@ -563,18 +607,28 @@ inline void plan_rows(int R, Args &a, int max_rows = MAX_ROWS) {
   if (a.w_stages < 3) a.w_stages = 3;
   while (a.a_stages < a.w_stages && (a.a_stages + 1) * a_stage + a.w_stages * W_STAGE_BYTES <= SMEM_BUDGET) a.a_stages++;
 }
-inline size_t smem_bytes(const Args &a) { return (size_t)a.w_stages * W_STAGE_BYTES + (size_t)a.a_stages * (a.rb_rows * TILE_K * 2) + 1024; }
+// Ring depths of a SMALL launch whose CTAs read n stages each: no more than n (the next projection's CTA may then sit
+// on the same SM), at most five of the weights (24 MB in flight over the machine; the 8B-class step of 20 rows takes
+// 4.0 ms with five, 4.05 with four, 4.5 with two and a half).
+inline void plan_stages_small(Args &a, int n) {
+  const int kps = k_per_stage(true), a_stage = kps * a.rb_rows * TILE_K * 2;
+  a.a_stages = std::max(2, std::min(4, n));
+  a.w_stages = std::max(2, std::min({5, (SMALL_SMEM_BUDGET - a.a_stages * a_stage) / (kps * W_STAGE_BYTES), n}));
+}
+inline size_t smem_bytes(const Args &a, bool small) {
+  return (size_t)k_per_stage(small) * ((size_t)a.w_stages * W_STAGE_BYTES + (size_t)a.a_stages * (a.rb_rows * TILE_K * 2)) + 1024;
+}
 
 // K splits: fill the SMs with whole waves of equally sized items, keeping at least
 // min_kb K blocks per item.
-inline int plan_splits(int n_items_unsplit, int kb_total, int n_sms, int max_splits, int min_kb) {
+inline int plan_splits(int n_items_unsplit, int kb_total, int n_sms, int max_splits, int min_kb, double item_cost = 3.0) {
   int best = 1; double best_eff = 0.0;
   for (int s = 1; s <= max_splits; ++s) {
     if (s > 1 && kb_total / s < min_kb) break;
     const long long items = (long long)n_items_unsplit * s;
     const long long waves = (items + n_sms - 1) / n_sms;
     // time ~ waves * (k blocks per item + fixed per-item cost in k-block units)
-    const double per_item = (double)((kb_total + s - 1) / s) + 3.0;
+    const double per_item = (double)((kb_total + s - 1) / s) + item_cost;
     const double eff = ((double)n_items_unsplit * kb_total) / ((double)waves * n_sms * per_item);
     if (eff > best_eff + 1e-9) { best_eff = eff; best = s; }
   }

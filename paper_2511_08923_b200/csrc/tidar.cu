@@ -60,7 +60,8 @@ struct tidar_ctx {
   int mixed_units = 0;             // attention units of the current mixed step
   float *d_run_max = nullptr, *d_run_sum = nullptr, *d_tgt_logit = nullptr, *d_logprob = nullptr;   // likelihood scoring, per row
   int32_t *d_target = nullptr;
-  std::vector<CUtensorMap> tm_lm_chunks;   // the LM head in vocabulary chunks of lm_chunk rows (scoring)
+  struct WMap { CUtensorMap full, small; };   // a weight matrix for the full and the SMALL instances of the projection kernel
+  std::vector<WMap> tm_lm_chunks;   // the LM head in vocabulary chunks of lm_chunk rows (scoring)
   int32_t *d_seq_len = nullptr, *d_block = nullptr, *d_page_table = nullptr, *d_step_seqs = nullptr, *d_forced = nullptr,
           *d_step_n = nullptr, *d_step_L = nullptr, *d_out = nullptr, *d_prompt = nullptr, *d_arg_idx = nullptr;
   float *X = nullptr, *partials = nullptr, *rope_cos = nullptr, *rope_sin = nullptr, *d_arg_val = nullptr,
@@ -85,9 +86,9 @@ struct tidar_ctx {
   int next_slot = 0;
   // tensor-core path
   gemm_tc::EncodeTiledFn encode = nullptr;
-  std::vector<CUtensorMap> tm_wqkv, tm_wo, tm_wgu, tm_wdown;
-  CUtensorMap tm_lm;
-  struct AMap { const void *p; int rows, cols, box; CUtensorMap tm; };
+  std::vector<WMap> tm_wqkv, tm_wo, tm_wgu, tm_wdown;
+  WMap tm_lm;
+  struct AMap { const void *p; int rows, cols, box; bool small; CUtensorMap tm; };
   std::vector<AMap> amaps;
   CUtensorMap tm_q, tm_kv, tm_kloc, tm_vloc;
   float *attn_part_O = nullptr; float2 *attn_part_ml = nullptr;
@@ -229,34 +230,21 @@ void layout(tidar_ctx &x, void *arena, size_t *bytes) {
   *bytes = align_up(cv.off, 256);
 }
 
-// Two ways to launch a kernel of the step.  launch_pdl: with programmatic stream serialization,
-// the kernel may be scheduled while the previous kernel of the stream is still running and
-// synchronises itself with pdl_wait(); only kernels that call pdl_wait() before touching
-// produced data may be launched this way.  It pays for kernels with a heavy prologue (the
-// projections: tensor-memory allocation, barriers, the weight ring filling; attention).
-// launch_after: an ordinary dependency.  The small kernels gain nothing from starting early,
-// and their CTAs waiting on the SMs only take resources from the kernel that is still
-// running: a chain of small kernels in a graph costs ~1 us per kernel either way (1.5B-class
-// step 2.57 -> 2.51 ms, k = 1 step 1.71 -> 1.59 ms with the small kernels launched this way).
-// Their pdl_wait() / pdl_trigger() are no-ops then, apart from letting the NEXT kernel start
-// early.
+// A kernel of a pass is launched with programmatic stream serialization: it may be scheduled while the previous
+// kernel of the stream is still running and synchronises itself with pdl_wait(); only kernels that call
+// pdl_wait() before they touch produced data may be launched this way.  Between a projection and the small kernel
+// behind it (norm, RoPE) an ordinary dependency costs 2.3 - 4 us, this one 1.0 - 1.5.  What makes it pay is that the
+// kernels fit beside one another: all ask for the same split of the SM's memory (an SM changes its split only when it is
+// empty; see init_tensor_core_path).
 template <typename... KP, typename... AP>
-inline void launch_with(bool programmatic, void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, AP &&...args) {
+inline void launch_pdl(void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, AP &&...args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at; cfg.numAttrs = programmatic ? 1 : 0;
+  cfg.attrs = at; cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kernel, KP(std::forward<AP>(args))...);
-}
-template <typename... KP, typename... AP>
-inline void launch_pdl(void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, AP &&...args) {
-  launch_with(true, kernel, grid, block, smem, st, std::forward<AP>(args)...);
-}
-template <typename... KP, typename... AP>
-inline void launch_after(void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, AP &&...args) {
-  launch_with(false, kernel, grid, block, smem, st, std::forward<AP>(args)...);
 }
 
 // ---- launch bookkeeping -----------------------------------------------------
@@ -307,32 +295,36 @@ KvGeom geom(const tidar_ctx *c) {
 }
 
 // ---- projections --------------------------------------------------------------
+bool encode_weights(tidar_ctx *c, tidar_ctx::WMap *tm, const void *p, int rows, int cols) {
+  return gemm_tc::encode_2d(c->encode, &tm->full, p, (uint64_t)rows, (uint64_t)cols, gemm_tc::TILE_N) == CUDA_SUCCESS &&
+         gemm_tc::encode_2d_small(c->encode, &tm->small, p, (uint64_t)rows, (uint64_t)cols, gemm_tc::TILE_N) == CUDA_SUCCESS;
+}
 // Tensor map of an activation matrix [rows][cols] (bf16) with a box of `box` rows; cached.
-const CUtensorMap *act_map(tidar_ctx *c, const void *p, int rows, int cols, int box) {
-  for (auto &m : c->amaps) if (m.p == p && m.rows == rows && m.cols == cols && m.box == box) return &m.tm;
-  tidar_ctx::AMap m{p, rows, cols, box, {}};
-  if (gemm_tc::encode_2d(c->encode, &m.tm, p, (uint64_t)rows, (uint64_t)cols, (uint32_t)box) != CUDA_SUCCESS) return nullptr;
+const CUtensorMap *act_map(tidar_ctx *c, const void *p, int rows, int cols, int box, bool small) {
+  for (auto &m : c->amaps) if (m.p == p && m.rows == rows && m.cols == cols && m.box == box && m.small == small) return &m.tm;
+  tidar_ctx::AMap m{p, rows, cols, box, small, {}};
+  if ((small ? gemm_tc::encode_2d_small : gemm_tc::encode_2d)(c->encode, &m.tm, p, (uint64_t)rows, (uint64_t)cols, (uint32_t)box) != CUDA_SUCCESS) return nullptr;
   if (c->amaps.size() > 256) c->amaps.erase(c->amaps.begin());
   c->amaps.push_back(m);
   return &c->amaps.back().tm;
 }
 
-// Tensor-core projection.  A [a_rows][K] (first R rows used), W described by tmW ([N][K]).
-//   MODE_SLAB  : S split-K partial slabs of fp32 [R][N] into c->partials (S chosen here)
-//   MODE_SWIGLU: bf16 c->H [R][N/2]
-//   MODE_ARGMAX: candidates for argmax_merge_kernel (+ optional logits dump)
-int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const CUtensorMap &tmW, int R, int N, int K, int cls,
-                   int *S_out, size_t *stride_out, float *slab_out = nullptr, int force_S = 0) {
+// Whether a projection runs as a SMALL instance (the LM head's argmax epilogue needs the registers of the full one).
+bool small_gemm(int mode, int R) { return R <= gemm_tc::SMALL_ROWS && (mode == gemm_tc::MODE_SLAB || mode == gemm_tc::MODE_SWIGLU); }
+
+// Work of a tensor-core projection of R rows: row blocks, K splits, which tiles finish in the fused epilogue.
+gemm_tc::Args plan_gemm(const tidar_ctx *c, int mode, int R, int N, int K, int force_S = 0) {
   gemm_tc::Args a{};
   a.R = R; a.N = N; a.K = K;
   gemm_tc::plan_rows(R, a);
   a.n_tiles = (N + gemm_tc::TILE_N - 1) / gemm_tc::TILE_N;
-  a.kb_total = K / gemm_tc::TILE_K;
+  const bool small = small_gemm(mode, R);
+  const int kps = gemm_tc::k_per_stage(small);
+  a.kb_total = (K / gemm_tc::TILE_K + kps - 1) / kps;
   a.S = 1; a.fused_items = 0; a.tile_b0 = 0; a.n_tiles_b = 0;
-  int rem_tiles = 0;
   if (mode == gemm_tc::MODE_SLAB) {
     a.n_tiles_b = a.n_tiles;
-    a.S = force_S > 0 ? std::min(force_S, a.kb_total) : gemm_tc::plan_splits(a.n_rb * a.n_tiles, a.kb_total, c->n_sms, c->S_max, 4);
+    a.S = force_S > 0 ? std::min(force_S, a.kb_total) : gemm_tc::plan_splits(a.n_rb * a.n_tiles, a.kb_total, c->n_sms, c->S_max, 4 / kps, 3.0 / kps);
     // One row block of up to 288 rows, or two of half the rows?  Two halves fetch every weight tile
     // twice (the second time from L2: ~0.37 instead of 0.46 us per K block of an item, but twice as
     // many K blocks per item once the SMs are full), while a CTA's slab store, which its SM cannot
@@ -350,10 +342,9 @@ int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const CUte
       };
       if (cost(h, 0.37, 1.7) < cost(a, 0.46, 3.3)) a = h;
     }
-    a.out = slab_out ? (void *)slab_out : (void *)c->partials; a.ldo = N; a.slab_stride = (long long)R * N;
-    a.slab_bf16 = (slab_out || !c->slab_bf16) ? 0 : 1;   // an explicit output buffer always gets exact fp32 slabs
+    a.ldo = N; a.slab_stride = (long long)R * N;
   } else if (mode == gemm_tc::MODE_SWIGLU) {
-    a.H = c->H; a.ldh = N / 2;
+    a.ldh = N / 2;
     a.fused_items = a.n_rb * a.n_tiles;
     // more tiles than SMs: whole waves of tiles finish in the fused epilogue; the tiles of the
     // last, partial wave are split along K so that they also fill the machine, and are finished
@@ -361,39 +352,65 @@ int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const CUte
     if (a.n_rb == 1 && a.n_tiles > c->n_sms && a.n_tiles % c->n_sms) {
       const int full = a.n_tiles / c->n_sms * c->n_sms;
       const int rem = a.n_tiles - full;
-      const int S2 = std::min({c->n_sms / rem, a.kb_total / 4, c->S_max});
+      const int S2 = std::min({c->n_sms / rem, a.kb_total * kps / 4, c->S_max});
       if (S2 >= 2 && (size_t)S2 * R * rem * gemm_tc::TILE_N <= c->partials_cap) {
-        rem_tiles = rem;
         a.fused_items = full; a.tile_b0 = full; a.n_tiles_b = rem; a.S = S2;
-        a.out = c->partials; a.ldo = rem * gemm_tc::TILE_N; a.slab_stride = (long long)R * a.ldo; a.slab_bf16 = c->slab_bf16 ? 1 : 0;
+        a.ldo = rem * gemm_tc::TILE_N; a.slab_stride = (long long)R * a.ldo;
       }
     }
   } else {
     a.fused_items = a.n_rb * a.n_tiles;
-    a.cand_val = c->cand_val; a.cand_idx = c->cand_idx; a.cand_ld = c->n_sms * 4; a.dump = c->dbg_logits; a.ld_dump = c->cfg.vocab; a.col0 = 0;
+  }
+  return a;
+}
+
+// Tensor-core projection.  A [a_rows][K] (first R rows used), W described by tmW ([N][K]).
+//   MODE_SLAB  : S split-K partial slabs of fp32 [R][N] into c->partials (S chosen here)
+//   MODE_SWIGLU: bf16 c->H [R][N/2]
+//   MODE_ARGMAX: candidates for argmax_merge_kernel (+ optional logits dump)
+int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const tidar_ctx::WMap &tmW, int R, int N, int K, int cls,
+                   int *S_out, size_t *stride_out, float *slab_out = nullptr, int force_S = 0) {
+  gemm_tc::Args a = plan_gemm(c, mode, R, N, K, force_S);
+  const bool small = small_gemm(mode, R);
+  const int rem_tiles = mode == gemm_tc::MODE_SWIGLU ? a.n_tiles_b : 0;
+  if (mode == gemm_tc::MODE_SLAB) {
+    a.out = slab_out ? (void *)slab_out : (void *)c->partials;
+    a.slab_bf16 = (slab_out || !c->slab_bf16) ? 0 : 1;   // an explicit output buffer always gets exact fp32 slabs
+  } else if (mode == gemm_tc::MODE_SWIGLU) {
+    a.H = c->H;
+    a.out = c->partials; a.slab_bf16 = c->slab_bf16 ? 1 : 0;
+  } else {
+    a.cand_val = c->cand_val; a.cand_idx = c->cand_idx; a.cand_ld = (a.n_rb == 1 ? std::min(a.fused_items, c->n_sms) : c->n_sms) * 4; a.dump = c->dbg_logits; a.ld_dump = c->cfg.vocab; a.col0 = 0;
     a.inv_temp = c->cfg.temperature > 0.f ? 1.0f / c->cfg.temperature : 0.f; a.skey = c->meta.skey + c->head_row0;
   }
   a.status = c->d_status;
   a.warm_epilogue = mode == gemm_tc::MODE_SWIGLU ? 1 : 0;
-  const CUtensorMap *tmA = act_map(c, A, a_rows, K, a.box_rows);
+  const CUtensorMap *tmA = act_map(c, A, a_rows, K, a.box_rows, small);
   if (!tmA) return fail(c, TIDAR_ECUDA, "cuTensorMapEncodeTiled failed for an activation matrix (%d x %d, box %d)", a_rows, K, a.box_rows);
   const int items = a.total_items();
   const int grid = std::min(items, c->n_sms);
-  const size_t smem = gemm_tc::smem_bytes(a);
+  if (small) {
+    int kb = 0;
+    for (int i = 0; i < items; i += grid) kb += i < a.fused_items ? a.kb_total : (a.kb_total + a.S - 1) / a.S;
+    gemm_tc::plan_stages_small(a, kb);
+  }
+  const size_t smem = gemm_tc::smem_bytes(a, small);
   Launch l(c, cls);
-  if (mode == gemm_tc::MODE_SLAB) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB>, grid, gemm_tc::THREADS, smem, c->stream, tmW, *tmA, a, l.tl);
-  else if (mode == gemm_tc::MODE_SWIGLU) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU>, grid, gemm_tc::THREADS, smem, c->stream, tmW, *tmA, a, l.tl);
-  else if (a.inv_temp > 0.f) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SAMPLE>, grid, gemm_tc::THREADS, smem, c->stream, tmW, *tmA, a, l.tl);
-  else launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_ARGMAX>, grid, gemm_tc::THREADS, smem, c->stream, tmW, *tmA, a, l.tl);
+  if (small && mode == gemm_tc::MODE_SLAB) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB, true>, grid, gemm_tc::THREADS, smem, c->stream, tmW.small, *tmA, a, l.tl);
+  else if (small) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU, true>, grid, gemm_tc::THREADS, smem, c->stream, tmW.small, *tmA, a, l.tl);
+  else if (mode == gemm_tc::MODE_SLAB) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
+  else if (mode == gemm_tc::MODE_SWIGLU) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
+  else if (a.inv_temp > 0.f) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SAMPLE>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
+  else launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_ARGMAX>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
   if (rem_tiles) {
     const int nf = (N - a.tile_b0 * gemm_tc::TILE_N) / 2;          // features of the split tiles
     const size_t n = (size_t)R * nf;
     Launch lf(c, cls);
     if (c->slab_bf16)
-      launch_after(swiglu_slab_kernel<bf16>, (unsigned)((n / 2 + 255) / 256), 256, 0, c->stream, (const bf16 *)c->partials, a.S, (size_t)a.slab_stride, R, a.ldo, nf,
+      launch_pdl(swiglu_slab_kernel<bf16>, (unsigned)((n / 2 + 255) / 256), 256, 0, c->stream, (const bf16 *)c->partials, a.S, (size_t)a.slab_stride, R, a.ldo, nf,
                                                                            a.tile_b0 * gemm_tc::TILE_N / 2, a.ldh, c->H, lf.tl);
     else
-      launch_after(swiglu_slab_kernel<float>, (unsigned)((n / 2 + 255) / 256), 256, 0, c->stream, (const float *)c->partials, a.S, (size_t)a.slab_stride, R, a.ldo, nf,
+      launch_pdl(swiglu_slab_kernel<float>, (unsigned)((n / 2 + 255) / 256), 256, 0, c->stream, (const float *)c->partials, a.S, (size_t)a.slab_stride, R, a.ldo, nf,
                                                                            a.tile_b0 * gemm_tc::TILE_N / 2, a.ldh, c->H, lf.tl);
   }
   if (S_out) *S_out = a.S;
@@ -404,7 +421,7 @@ int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const CUte
 enum Proj { P_QKV, P_O, P_GU, P_DOWN };
 
 // out = A[R][K] * W[N][K]^T as S split-K partial slabs of fp32 [R][N] (replay: S = 1).
-int gemm_partials(tidar_ctx *c, const bf16 *A, int a_rows, const bf16 *W, const CUtensorMap *tmW, int R, int N, int K, float *out,
+int gemm_partials(tidar_ctx *c, const bf16 *A, int a_rows, const bf16 *W, const tidar_ctx::WMap *tmW, int R, int N, int K, float *out,
                   int *S_out, size_t *stride_out, int cls) {
   if (c->cfg.impl == 0) return gemm_tc_launch(c, gemm_tc::MODE_SLAB, A, a_rows, *tmW, R, N, K, cls, S_out, stride_out);
   Launch l(c, cls);
@@ -516,9 +533,9 @@ void launch_norm(tidar_ctx *c, int R, const float *partials, int S, size_t strid
   Launch l(c, TIDAR_TC_NORM);
   const int d = c->cfg.d_model;
   if (c->cfg.impl == 0 && c->slab_bf16)
-    launch_after(rmsnorm_reduce_kernel<512, bf16>, R, 512, d * sizeof(float), c->stream, c->X, (const bf16 *)partials, S, stride, gain, c->cfg.rms_eps, d, c->A, l.tl);
+    launch_pdl(rmsnorm_reduce_kernel<512, bf16>, R, 512, d * sizeof(float), c->stream, c->X, (const bf16 *)partials, S, stride, gain, c->cfg.rms_eps, d, c->A, l.tl);
   else
-    launch_after(rmsnorm_reduce_kernel<512, float>, R, 512, d * sizeof(float), c->stream, c->X, partials, S, stride, gain, c->cfg.rms_eps, d, c->A, l.tl);
+    launch_pdl(rmsnorm_reduce_kernel<512, float>, R, 512, d * sizeof(float), c->stream, c->X, partials, S, stride, gain, c->cfg.rms_eps, d, c->A, l.tl);
 }
 
 // The transformer stack over R assembled rows (metadata and X already filled).
@@ -536,7 +553,7 @@ int forward_rows(tidar_ctx *c, int R, bool with_head, int rows_per_group, const 
   {
     Launch l(c, TIDAR_TC_ROPE);
     const int n = R * (hd / 2);
-    launch_after(pass_setup_kernel, (n + 255) / 256 + (plan.tiles ? 1 : 0), 256, 0, c->stream, c->meta, R, hd / 2, (double)cf.rope_theta, c->rope_cos,
+    launch_pdl(pass_setup_kernel, (n + 255) / 256 + (plan.tiles ? 1 : 0), 256, 0, c->stream, c->meta, R, hd / 2, (double)cf.rope_theta, c->rope_cos,
                  c->rope_sin, plan, l.tl);
   }
   int S = 0; size_t stride = 0;          // pending partials of the previous down projection
@@ -556,10 +573,10 @@ int forward_rows(tidar_ctx *c, int R, bool with_head, int rows_per_group, const 
       const bf16 *bias_l = c->bqkv.empty() ? nullptr : c->bqkv[l], *qn_l = c->q_norm.empty() ? nullptr : c->q_norm[l],
                  *kn_l = c->k_norm.empty() ? nullptr : c->k_norm[l];
 if (tc && c->slab_bf16)
-        launch_after(rope_kv_kernel<bf16>, dim3(R, rope_chunks), 256, 0, c->stream, (const bf16 *)c->partials, S, stride, Hq, Hkv, hd, c->meta, c->rope_cos,
+        launch_pdl(rope_kv_kernel<bf16>, dim3(R, rope_chunks), 256, 0, c->stream, (const bf16 *)c->partials, S, stride, Hq, Hkv, hd, c->meta, c->rope_cos,
                                                                       c->rope_sin, g, c->Q, Kp, Vp, c->Kloc, c->Vloc, bias_l, qn_l, kn_l, cf.rms_eps, ll.tl);
       else
-        launch_after(rope_kv_kernel<float>, dim3(R, rope_chunks), 256, 0, c->stream, c->partials, S, stride, Hq, Hkv, hd, c->meta, c->rope_cos,
+        launch_pdl(rope_kv_kernel<float>, dim3(R, rope_chunks), 256, 0, c->stream, c->partials, S, stride, Hq, Hkv, hd, c->meta, c->rope_cos,
                                                                       c->rope_sin, g, c->Q, Kp, Vp, c->Kloc, c->Vloc, bias_l, qn_l, kn_l, cf.rms_eps, ll.tl);
     }
     if (tc) {
@@ -586,7 +603,7 @@ if (tc && c->slab_bf16)
                                 cudaMemcpyDeviceToDevice, c->stream));
   if (with_head && mix.n > 0) {            // rows R .. R + mix.n - 1 of the LM head's input
     Launch lm(c, TIDAR_TC_NORM);
-    launch_after(mix_rows_kernel, mix.n, 256, 0, c->stream, c->A, d, cf.beta, mix.k, mix.a0, mix.a_seq, mix.a_j, mix.b0, mix.b_seq, mix.b_j, mix.lay, R,
+    launch_pdl(mix_rows_kernel, mix.n, 256, 0, c->stream, c->A, d, cf.beta, mix.k, mix.a0, mix.a_seq, mix.a_j, mix.b0, mix.b_seq, mix.b_j, mix.lay, R,
                  cf.temperature > 0.f ? c->meta.skey : (uint32_t *)nullptr, lm.tl);
     R += mix.n;
   }
@@ -596,11 +613,13 @@ if (tc && c->slab_bf16)
   const int Rh = R - head_row0;
   if (with_head && Rh > c->R_head) return fail(c, TIDAR_ECAPACITY, "%d rows for the LM head exceed the context's %d", Rh, c->R_head);
   if (with_head && tc) {
-    const int G = c->n_sms * 4;          // upper bound of (CTAs of the LM-head kernel) x 4 lane quadrants
-    CUDA_TRY(c, cudaMemsetAsync(c->cand_idx, 0xff, (size_t)G * Rh * sizeof(int32_t), c->stream));
+    // with one row block every CTA leaves a candidate for every row; with several it may meet only some of them
+    const bool one_block = Rh <= gemm_tc::MAX_ROWS;
+    const int G = (one_block ? std::min((cf.vocab + gemm_tc::TILE_N - 1) / gemm_tc::TILE_N, c->n_sms) : c->n_sms) * 4;
+    if (!one_block) CUDA_TRY(c, cudaMemsetAsync(c->cand_idx, 0xff, (size_t)G * Rh * sizeof(int32_t), c->stream));
     if ((rc = gemm_tc_launch(c, gemm_tc::MODE_ARGMAX, Ah, RA - head_row0, c->tm_lm, Rh, cf.vocab, d, TIDAR_TC_LMHEAD, nullptr, nullptr))) return rc;
     Launch ll(c, TIDAR_TC_LMHEAD);
-    launch_after(argmax_merge_kernel, (Rh * 32 + 255) / 256, 256, 0, c->stream, c->cand_val, c->cand_idx, G, Rh, c->d_arg_val, c->d_arg_idx, ll.tl);
+    launch_pdl(argmax_merge_kernel, (Rh * 32 + 255) / 256, 256, 0, c->stream, c->cand_val, c->cand_idx, G, Rh, c->d_arg_val, c->d_arg_idx, ll.tl);
   } else if (with_head) {
     for (int v0 = 0; v0 < cf.vocab; v0 += c->lm_chunk) {
       const int nc = std::min(c->lm_chunk, cf.vocab - v0);
@@ -632,9 +651,7 @@ int init_tensor_core_path(tidar_ctx *c) {
   if (!fn || qres != cudaDriverEntryPointSuccess) return fail(c, TIDAR_ECUDA, "cuTensorMapEncodeTiled is not available in this driver");
   c->encode = (gemm_tc::EncodeTiledFn)fn;
   const int d = cf.d_model, qo = cf.n_q_heads * cf.head_dim;
-  auto enc = [&](CUtensorMap *tm, const void *p, int rows, int cols) {
-    return gemm_tc::encode_2d(c->encode, tm, p, (uint64_t)rows, (uint64_t)cols, gemm_tc::TILE_N) == CUDA_SUCCESS;
-  };
+  auto enc = [&](tidar_ctx::WMap *tm, const void *p, int rows, int cols) { return encode_weights(c, tm, p, rows, cols); };
   c->tm_wqkv.resize(cf.n_layers); c->tm_wo.resize(cf.n_layers); c->tm_wgu.resize(cf.n_layers); c->tm_wdown.resize(cf.n_layers);
   bool ok = enc(&c->tm_lm, c->lm_head, cf.vocab, d);
   c->tm_lm_chunks.resize((cf.vocab + c->lm_chunk - 1) / c->lm_chunk);
@@ -659,7 +676,21 @@ int init_tensor_core_path(tidar_ctx *c) {
     CUDA_TRY(c, cudaFuncSetAttribute(attn_tc::attn_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_tc::Smem<128>::TOTAL));
     CUDA_TRY(c, cudaFuncSetAttribute(attn_tc::attn_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_tc::Smem<64>::TOTAL));
   }
-  const int max_smem = gemm_tc::SMEM_BUDGET + 1024;
+  {
+    auto max_smem_split = [&](const void *f) { return cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared); };
+    const void *kernels[] = {(const void *)assemble_step_kernel, (const void *)pass_setup_kernel, (const void *)attn_meta_plan_kernel,
+                             (const void *)rmsnorm_reduce_kernel<512, float>, (const void *)rmsnorm_reduce_kernel<512, bf16>,
+                             (const void *)rope_kv_kernel<float>, (const void *)rope_kv_kernel<bf16>,
+                             (const void *)swiglu_slab_kernel<float>, (const void *)swiglu_slab_kernel<bf16>,
+                             (const void *)attn_tc::attn_combine_kernel<128>, (const void *)attn_tc::attn_combine_kernel<64>,
+                             (const void *)mix_rows_kernel, (const void *)argmax_merge_kernel, (const void *)verify_select_kernel, (const void *)kv_commit_kernel};
+    for (const void *f : kernels) CUDA_TRY(c, max_smem_split(f));
+  }
+  const int max_smem = gemm_tc::SMEM_BUDGET + 1024, small_smem = gemm_tc::SMALL_SMEM_BUDGET + 1024;
+  CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, small_smem));
+  CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, small_smem));
+  CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+  CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_ARGMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
@@ -727,7 +758,7 @@ int record_step(tidar_ctx *c, int n_seqs, int k, bool ar, int mixed_R = 0, int m
   }
   {
     Launch l(c, TIDAR_TC_EMBED);
-    launch_after(assemble_step_kernel, R, 256, 0, c->stream, c->meta, c->d_step_seqs, c->d_seq_len, c->d_block, c->d_blk_len, k, n_blocks, lay, cf.k_max,
+    launch_pdl(assemble_step_kernel, R, 256, 0, c->stream, c->meta, c->d_step_seqs, c->d_seq_len, c->d_block, c->d_blk_len, k, n_blocks, lay, cf.k_max,
                cf.mask_token_id, c->d_step_n, c->embed, cf.d_model, c->X, cf.temperature > 0.f ? 1 : 0, (unsigned long long)cf.sample_seed, l.tl);
   }
   // beta < 1: the verified prediction of causal slot j mixes its row with the first slot of block j
@@ -739,12 +770,12 @@ int record_step(tidar_ctx *c, int n_seqs, int k, bool ar, int mixed_R = 0, int m
   if (int rc = forward_rows(c, R, true, mixed_R > 0 ? 0 : T, mix)) return rc;
   {
     Launch l(c, TIDAR_TC_VERIFY);
-    launch_after(verify_select_kernel, n_seqs, 32, 0, c->stream, c->d_arg_idx, mix.n ? c->d_arg_idx + R : (const int32_t *)nullptr, c->d_step_seqs,
+    launch_pdl(verify_select_kernel, n_seqs, 32, 0, c->stream, c->d_arg_idx, mix.n ? c->d_arg_idx + R : (const int32_t *)nullptr, c->d_step_seqs,
                c->d_forced, k, n_blocks, lay, cf.k_max, c->d_block, c->d_blk_len, c->d_step_L, c->d_out, l.tl);
   }
   {
     Launch l(c, TIDAR_TC_VERIFY);
-    launch_after(kv_commit_kernel, dim3(n_seqs, cf.n_layers), 128, 0, c->stream, c->d_step_seqs, c->d_step_n, c->d_step_L, c->d_seq_len, k, lay.k,
+    launch_pdl(kv_commit_kernel, dim3(n_seqs, cf.n_layers), 128, 0, c->stream, c->d_step_seqs, c->d_step_n, c->d_step_L, c->d_seq_len, k, lay.k,
                (cf.debug >> 1) & 1, geom(c), c->kv, c->pool_stride, l.tl);
   }
   CUDA_TRY(c, cudaGetLastError());
@@ -1384,8 +1415,8 @@ int tidar_gemm(tidar_ctx *c, const void *A, const void *W, int32_t R, int32_t N,
   if (need > c->partials_cap) return fail(c, TIDAR_ECAPACITY, "R*N*splits = %zu floats exceed the context's scratch (%zu)", need, c->partials_cap);
   int S = 1; size_t stride = 0;
   if (c->cfg.impl == 0) {
-    CUtensorMap tmW;
-    if (gemm_tc::encode_2d(c->encode, &tmW, W, (uint64_t)N, (uint64_t)K, gemm_tc::TILE_N) != CUDA_SUCCESS)
+    tidar_ctx::WMap tmW;
+    if (!encode_weights(c, &tmW, W, N, K))
       return fail(c, TIDAR_ECUDA, "cuTensorMapEncodeTiled failed for W");
     if (int rc = gemm_tc_launch(c, gemm_tc::MODE_SLAB, (const bf16 *)A, R, tmW, R, N, K, TIDAR_TC_GEMM, &S, &stride, c->partials, splits)) return rc;
   } else {

@@ -58,6 +58,16 @@ def test_gemm_matches_definition(ctx, R, N, K):
     assert np.abs(b - c).max() <= TOL
 
 
+@pytest.mark.parametrize("R", [1, 16, 17, 48, 95, 96, 97])
+@pytest.mark.parametrize("N,K", [(130, 64), (1100, 704), (640, 2048)])
+def test_gemm_few_rows(ctx, R, N, K):
+    """Around the largest row count of the few-rows instance; its stages hold two 64-wide K blocks, the last of which
+    may not exist (K = 64, 704)."""
+    a = _run(ctx, R, N, K, 0, 300 + R)
+    b = _run(ctx, R, N, K, 1, 300 + R)
+    assert np.abs(a - b).max() <= TOL
+
+
 def test_gemm_rejects_bad_arguments(ctx):
     from paper_2511_08923_b200 import TidarError
     A = torch.zeros(4, 100, dtype=torch.bfloat16, device="cuda:0")
