@@ -75,6 +75,7 @@ struct PlanArgs {
   int spt;                  // slots per query tile = 128 / G
   int Hkv;
   int n_sms, max_items;     // items a pass may have; n_units = every unit is one item
+  int max_pieces;           // items a tile or pair may have (1: nothing is split, the merge kernel is not launched)
   Item *items; Tile *tiles; // out: [max_items] (unused ones are zero), [2 n_units] (only where items may be split)
 };
 
@@ -216,7 +217,7 @@ __device__ inline void plan_block(const PlanArgs &p, ROW row_keys) {
       items += __shfl_xor_sync(0xffffffffu, items, o); live += __shfl_xor_sync(0xffffffffu, live, o); most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
       us_sum += __shfl_xor_sync(0xffffffffu, us_sum, o); us_max = fmaxf(us_max, __shfl_xor_sync(0xffffffffu, us_max, o));
     }
-    if (live_cnd && sub == 0 && items <= p.max_items && most <= MAX_SPLITS) {
+    if (live_cnd && sub == 0 && items <= p.max_items && most <= p.max_pieces) {
       float us = us_max;
       if (items * p.Hkv > p.n_sms) us = fmaxf(us, p.Hkv * us_sum / p.n_sms + 0.5f * us_max);
       if (items > live) us += MERGE + 0.3f * items / live;
@@ -663,19 +664,30 @@ attn_combine_kernel(const Args a, TlSlot tl) {
     const float2 *ml = a.part_ml + part * 128 + m;
     const float4 *po = reinterpret_cast<const float4 *>(a.part_O) + part * (HD / 4) * 128 + (size_t)cg * 2 * 128 + m;
     const size_t ml_step = (size_t)a.Hkv * 2 * 128, po_step = (size_t)a.Hkv * 2 * (HD / 4) * 128;
-    float M = -INFINITY;
-#pragma unroll 4
-    for (int s = 0; s < t.n_items; ++s) M = fmaxf(M, ml[s * ml_step].x);
-    float den = 0.f;
+    // four partial results at a time, all their loads before the first use; the running sum is rescaled when the maximum rises
+    float M = -INFINITY, den = 0.f;
     float acc[8] = {};
-#pragma unroll 4
-    for (int s = 0; s < t.n_items; ++s) {
-      const float2 v = ml[s * ml_step];
-      const float4 x = po[s * po_step], y = po[s * po_step + 128];
-      const float wgt = (v.x == -INFINITY) ? 0.f : exp2f(v.x - M);
-      den += wgt * v.y;
-      acc[0] = fmaf(wgt, x.x, acc[0]); acc[1] = fmaf(wgt, x.y, acc[1]); acc[2] = fmaf(wgt, x.z, acc[2]); acc[3] = fmaf(wgt, x.w, acc[3]);
-      acc[4] = fmaf(wgt, y.x, acc[4]); acc[5] = fmaf(wgt, y.y, acc[5]); acc[6] = fmaf(wgt, y.z, acc[6]); acc[7] = fmaf(wgt, y.w, acc[7]);
+    for (int s0 = 0; s0 < t.n_items; s0 += 4) {
+      float2 v[4]; float4 x[4], y[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        v[u] = make_float2(-INFINITY, 0.f);
+        x[u] = y[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (s0 + u < t.n_items) { v[u] = ml[(s0 + u) * ml_step]; x[u] = po[(s0 + u) * po_step]; y[u] = po[(s0 + u) * po_step + 128]; }
+      }
+      const float M_new = fmaxf(fmaxf(M, fmaxf(v[0].x, v[1].x)), fmaxf(v[2].x, v[3].x));
+      const float keep = M == -INFINITY ? 0.f : exp2f(M - M_new);
+      M = M_new;
+      den *= keep;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[j] *= keep;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float wgt = v[u].x == -INFINITY ? 0.f : exp2f(v[u].x - M);
+        den += wgt * v[u].y;
+        acc[0] = fmaf(wgt, x[u].x, acc[0]); acc[1] = fmaf(wgt, x[u].y, acc[1]); acc[2] = fmaf(wgt, x[u].z, acc[2]); acc[3] = fmaf(wgt, x[u].w, acc[3]);
+        acc[4] = fmaf(wgt, y[u].x, acc[4]); acc[5] = fmaf(wgt, y[u].y, acc[5]); acc[6] = fmaf(wgt, y[u].z, acc[6]); acc[7] = fmaf(wgt, y[u].w, acc[7]);
+      }
     }
     const float inv = 1.f / den;
     __nv_bfloat162 h0 = __floats2bfloat162_rn(acc[0] * inv, acc[1] * inv), h1 = __floats2bfloat162_rn(acc[2] * inv, acc[3] * inv),

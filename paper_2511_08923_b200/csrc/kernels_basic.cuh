@@ -14,6 +14,25 @@ template <> __device__ __forceinline__ float4 load4<bf16>(const bf16 *p) {
   return make_float4(a.x, a.y, b.x, b.y);
 }
 
+// v += the S (at most MAX_SLABS) partial sums at p, p + stride, ..., in that order.  AT_ONCE loads are issued before their
+// first addition: with one load per turn of a loop over S, the kernels that read slabs spent most of their time waiting
+// (norm 3.6 -> 2.0 us at 272 rows of 1536).
+constexpr int MAX_SLABS = 8;
+template <int AT_ONCE, typename SLAB>
+__device__ __forceinline__ void add_slabs(float4 &v, const SLAB *__restrict__ p, int S, size_t stride) {
+#pragma unroll
+  for (int s0 = 0; s0 < MAX_SLABS; s0 += AT_ONCE) {
+    if (s0 >= S) break;
+    float4 q[AT_ONCE];
+#pragma unroll
+    for (int u = 0; u < AT_ONCE; ++u)
+      if (s0 + u < S) q[u] = load4<SLAB>(p + (s0 + u) * stride);
+#pragma unroll
+    for (int u = 0; u < AT_ONCE; ++u)
+      if (s0 + u < S) { v.x += q[u].x; v.y += q[u].y; v.z += q[u].z; v.w += q[u].w; }
+  }
+}
+
 // One embedding row (bf16, d a multiple of 8) -> fp32, 16-byte loads.
 __device__ __forceinline__ void embed_row_to_f32(const bf16 *__restrict__ e, float *__restrict__ x, int d) {
   for (int c = threadIdx.x * 8; c < d; c += blockDim.x * 8) {
@@ -43,6 +62,37 @@ __device__ __forceinline__ void embed_row_to_f32(const bf16 *__restrict__ e, flo
 // ---------------------------------------------------------------------------
 struct StepLayout { const int32_t *k, *off, *loc; int n_seqs; };     // per listed sequence; k == null: uniform
 
+// A step's exchange with the host goes through pinned host memory that the kernels read and write themselves: two slots,
+// used in turn (a second step may be enqueued while the first runs).  turn: device word, the number of steps run.
+// (Four small copies around the kernels cost a one-sequence step of the tiny model 40 of its 160 us.)
+struct StepIo {
+  int32_t *turn, *blocks_done, *status;                      // device
+  const int32_t *in[2];                                      // [2][max_batch]: listed sequences, forced lengths
+  int32_t *out[2];                                           // [n_seqs][k_max + 1]: L, tokens
+  int32_t *done[2];                                          // [0] = turn + 1 once the slot's results are there, [1] = status
+  int32_t max_batch;
+};
+
+// The step's inputs to device memory, and for a step of mixed block lengths its layout (n_head > 0): h_lay holds n_head ints and
+// two tables of cap entries, n_units of them in use, in the same order as the device arrays at lay.  One block.
+__global__ void __launch_bounds__(256) stage_step_kernel(StepIo io, int n_seqs, int32_t *__restrict__ step_seqs, int32_t *__restrict__ forced,
+                                                         const int32_t *__restrict__ h_lay, int32_t *__restrict__ lay, int n_head, int cap, int n_units, TlSlot tl) {
+  pdl_trigger();
+  pdl_wait();
+  if (threadIdx.x == 0) tl_go(tl);
+  const int32_t *in = io.in[*io.turn & 1];
+  for (int i = threadIdx.x; i < n_seqs; i += blockDim.x) {
+    const int a = in[i], b = in[io.max_batch + i];
+    step_seqs[i] = a; forced[i] = b;
+  }
+  if (n_head > 0)
+    for (int i = threadIdx.x; i < n_head + 2 * n_units; i += blockDim.x) {
+      const int j = i - n_head, at = j < n_units ? i : i + cap - n_units;
+      lay[at] = h_lay[at];
+    }
+  if (threadIdx.x == 0) tl_end(tl);
+}
+
 __global__ void assemble_step_kernel(RowMeta m, const int32_t *__restrict__ step_seqs, const int32_t *__restrict__ seq_len,
                                      const int32_t *__restrict__ block_ids, const int32_t *__restrict__ blk_len, int k, int n_blocks,
                                      StepLayout lay, int k_max, int mask_id,
@@ -53,6 +103,15 @@ __global__ void assemble_step_kernel(RowMeta m, const int32_t *__restrict__ step
   if (threadIdx.x == 0) tl_go(tl);
   const int r = blockIdx.x;
   int s, slot, loc_base;
+  if (lay.k && r >= lay.off[lay.n_seqs]) {       // a row that only fills the last 16 rows up: no sequence, no K/V, seen by nothing
+    if (threadIdx.x == 0) {
+      m.seq[r] = 0; m.ids[r] = mask_id; m.pos[r] = 0; m.nvis[r] = 0; m.loc0[r] = 0; m.nloc[r] = 0; m.cache_pos[r] = -1; m.local_idx[r] = -1;
+      if (sampling) m.skey[r] = 0;
+      tl_end(tl);
+    }
+    for (int c = threadIdx.x; c < d; c += blockDim.x) X[(size_t)r * d + c] = 0.f;
+    return;
+  }
   if (lay.k) {                                   // per-sequence block lengths: find the sequence this row belongs to
     s = 0;
     while (s + 1 < lay.n_seqs && r >= lay.off[s + 1]) ++s;
@@ -160,28 +219,36 @@ __global__ void __launch_bounds__(256) pass_setup_kernel(RowMeta m, int R, int h
 // ---------------------------------------------------------------------------
 // Residual update + RMSNorm.  X (fp32 residual stream) += sum over the S split-K
 // partial results of the previous projection (fixed order: deterministic), then
-// A = bf16(X * rsqrt(mean(X^2) + eps) * gain).  One block per row.
+// A = bf16(X * rsqrt(mean(X^2) + eps) * gain).  One block per row; a thread keeps NV
+// groups of four columns in registers (NV * 4 * THREADS >= d).
 // ---------------------------------------------------------------------------
-template <int THREADS, typename SLAB>
+template <int THREADS, int NV, typename SLAB>
 __global__ void __launch_bounds__(THREADS)
 rmsnorm_reduce_kernel(float *__restrict__ X, const SLAB *__restrict__ partials, int S, size_t partial_stride,
                       const bf16 *__restrict__ gain, float eps, int d, bf16 *__restrict__ A, TlSlot tl) {
   pdl_trigger();
-  pdl_wait();
-  if (threadIdx.x == 0) tl_go(tl);
-  extern __shared__ float row[];
   __shared__ float red[THREADS / 32];
   const int r = blockIdx.x;
-  float ss = 0.f;
+  uint2 gb[NV];                                  // weights: no need to wait for the previous kernel
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int c = (i * THREADS + threadIdx.x) * 4;
+    gb[i] = c < d ? *reinterpret_cast<const uint2 *>(gain + c) : make_uint2(0u, 0u);
+  }
+  pdl_wait();
+  if (threadIdx.x == 0) tl_go(tl);
   float *xr = X + (size_t)r * d;
-  for (int c = threadIdx.x * 4; c < d; c += THREADS * 4) {
-    float4 v = *reinterpret_cast<const float4 *>(xr + c);
-    for (int s = 0; s < S; ++s) {
-      const float4 p = load4<SLAB>(partials + s * partial_stride + (size_t)r * d + c);
-      v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
+  float4 v[NV];
+  float ss = 0.f;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int c = (i * THREADS + threadIdx.x) * 4;
+    v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (c < d) {
+      v[i] = *reinterpret_cast<const float4 *>(xr + c);
+      add_slabs<MAX_SLABS>(v[i], partials + (size_t)r * d + c, S, partial_stride);
     }
-    *reinterpret_cast<float4 *>(row + c) = v;
-    ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+    ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
   }
   ss = warp_sum(ss);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
@@ -190,14 +257,16 @@ rmsnorm_reduce_kernel(float *__restrict__ X, const SLAB *__restrict__ partials, 
 #pragma unroll
   for (int i = 0; i < THREADS / 32; ++i) tot += red[i];
   const float inv = rsqrtf(tot / (float)d + eps);
-  for (int c = threadIdx.x * 4; c < d; c += THREADS * 4) {
-    const float4 v = *reinterpret_cast<const float4 *>(row + c);
-    if (S > 0) *reinterpret_cast<float4 *>(xr + c) = v;
-    const uint2 gb = *reinterpret_cast<const uint2 *>(gain + c);
-    const float2 g0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gb.x)), g1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gb.y));
-    __nv_bfloat162 o0 = __floats2bfloat162_rn(v.x * inv * g0.x, v.y * inv * g0.y), o1 = __floats2bfloat162_rn(v.z * inv * g1.x, v.w * inv * g1.y);
-    uint2 ob; ob.x = *reinterpret_cast<uint32_t *>(&o0); ob.y = *reinterpret_cast<uint32_t *>(&o1);
-    *reinterpret_cast<uint2 *>(A + (size_t)r * d + c) = ob;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int c = (i * THREADS + threadIdx.x) * 4;
+    if (c < d) {
+      if (S > 0) *reinterpret_cast<float4 *>(xr + c) = v[i];
+      const float2 g0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gb[i].x)), g1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gb[i].y));
+      __nv_bfloat162 o0 = __floats2bfloat162_rn(v[i].x * inv * g0.x, v[i].y * inv * g0.y), o1 = __floats2bfloat162_rn(v[i].z * inv * g1.x, v[i].w * inv * g1.y);
+      uint2 ob; ob.x = *reinterpret_cast<uint32_t *>(&o0); ob.y = *reinterpret_cast<uint32_t *>(&o1);
+      *reinterpret_cast<uint2 *>(A + (size_t)r * d + c) = ob;
+    }
   }
   if (threadIdx.x == 0) tl_end(tl);
 }
@@ -232,11 +301,20 @@ rope_kv_kernel(const SLAB *__restrict__ partials, int S, size_t partial_stride, 
     const int h = u / upr, i = (u % upr) * 4;
     const size_t base = (size_t)r * N + (size_t)h * hd + i;
     float4 x1 = make_float4(0.f, 0.f, 0.f, 0.f), x2 = x1;
-    for (int s = 0; s < S; ++s) {
-      const float4 a = load4<SLAB>(partials + s * partial_stride + base);
-      const float4 b = load4<SLAB>(partials + s * partial_stride + base + half);
-      x1.x += a.x; x1.y += a.y; x1.z += a.z; x1.w += a.w;
-      x2.x += b.x; x2.y += b.y; x2.z += b.z; x2.w += b.w;
+    // (both halves' loads together: two chains of additions)
+#pragma unroll
+    for (int s0 = 0; s0 < MAX_SLABS; s0 += 4) {
+      if (s0 >= S) break;
+      float4 q1[4], q2[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (s0 + t < S) { q1[t] = load4<SLAB>(partials + (s0 + t) * partial_stride + base); q2[t] = load4<SLAB>(partials + (s0 + t) * partial_stride + base + half); }
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        if (s0 + t < S) {
+          x1.x += q1[t].x; x1.y += q1[t].y; x1.z += q1[t].z; x1.w += q1[t].w;
+          x2.x += q2[t].x; x2.y += q2[t].y; x2.z += q2[t].z; x2.w += q2[t].w;
+        }
     }
     if (bias) {
       const uint2 b1 = *reinterpret_cast<const uint2 *>(bias + (size_t)h * hd + i), b2 = *reinterpret_cast<const uint2 *>(bias + (size_t)h * hd + i + half);
@@ -267,6 +345,7 @@ rope_kv_kernel(const SLAB *__restrict__ partials, int S, size_t partial_stride, 
     } else {
       const bool isk = h < Hq + Hkv;
       const int kvh = isk ? h - Hq : h - Hq - Hkv;
+      if (cp < 0 && li < 0) continue;
       if (cp >= 0) dst = (isk ? Kpool : Vpool) + kv_row_offset(g, seq, cp, kvh);
       else dst = (isk ? Kloc : Vloc) + ((size_t)li * Hkv + kvh) * hd;
       rotate = isk;
@@ -311,10 +390,7 @@ __global__ void swiglu_slab_kernel(const SLAB *__restrict__ slabs, int S, size_t
   if (t >= (size_t)R * nf2) { if (threadIdx.x == 0) tl_end(tl); return; }
   const int r = (int)(t / nf2), f = (int)(t % nf2) * 2;
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);                      // gate f, up f, gate f+1, up f+1
-  for (int s = 0; s < S; ++s) {
-    const float4 v = load4<SLAB>(slabs + s * stride + (size_t)r * ld + 2 * f);
-    acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
-  }
+  add_slabs<4>(acc, slabs + (size_t)r * ld + 2 * f, S, stride);
   __nv_bfloat162 o = __floats2bfloat162_rn(__fdividef(acc.x, 1.f + __expf(-acc.x)) * acc.y, __fdividef(acc.z, 1.f + __expf(-acc.z)) * acc.w);
   *reinterpret_cast<__nv_bfloat162 *>(H + (size_t)r * ldh + f0 + f) = o;
   if (threadIdx.x == 0) tl_end(tl);
@@ -403,16 +479,21 @@ __global__ void slab_sum_kernel(const float *__restrict__ in, int S, size_t stri
 //   forced value;  emitted = block[1..L-1], target_{L-1};
 //   next block = target_{L-1}, then the argmax of mask slots (L-1, 1..k-1); with no mask
 //   blocks (plain autoregressive step, k = 1) the next block is target_0 alone.
+// Commits as well (paper Section 3.3): the causal slots' K/V are in the cache at n..n+k-1, committing L of them is
+// n <- n + L.  The last block to finish hands the results over: everything a step wrote is visible to the host
+// once it reads the slot's new turn number.
 // ---------------------------------------------------------------------------
 __global__ void verify_select_kernel(const int32_t *__restrict__ arg_ids, const int32_t *__restrict__ tgt_ids,
                                      const int32_t *__restrict__ step_seqs,
                                      const int32_t *__restrict__ forced, int k, int n_blocks, StepLayout lay, int k_max,
-                                     int32_t *__restrict__ block_ids, int32_t *__restrict__ blk_len, int32_t *__restrict__ step_L,
-                                     int32_t *__restrict__ out /*[n_seqs][k_max+1]*/, TlSlot tl) {
+                                     int32_t *__restrict__ block_ids, int32_t *__restrict__ blk_len, const int32_t *__restrict__ step_n,
+                                     int32_t *__restrict__ step_L, int32_t *__restrict__ seq_len, StepIo io, TlSlot tl) {
   pdl_trigger();
   pdl_wait();
   if (threadIdx.x == 0) tl_go(tl);
   const int s = blockIdx.x, lane = threadIdx.x;
+  const int turn = *io.turn;
+  int32_t *out = io.out[turn & 1];                // [n_seqs][k_max+1]
   if (lay.k) { k = lay.k[s]; n_blocks = k; }
   const int T = k * (n_blocks + 1);
   const int seq = step_seqs[s];
@@ -438,7 +519,16 @@ __global__ void verify_select_kernel(const int32_t *__restrict__ arg_ids, const 
     out[(size_t)s * (k_max + 1) + 1 + lane] = lane < L - 1 ? shifted : (lane == L - 1 ? t_last : -1);
     blk[lane] = lane == 0 ? t_last : next_draft;
   }
-  if (lane == 0) { out[(size_t)s * (k_max + 1)] = L; step_L[s] = L; blk_len[seq] = n_blocks > 0 ? k : 1; tl_end(tl); }
+  if (lane == 0) { out[(size_t)s * (k_max + 1)] = L; step_L[s] = L; seq_len[seq] = step_n[s] + L; blk_len[seq] = n_blocks > 0 ? k : 1; tl_end(tl); }
+  __threadfence_system();
+  __syncwarp();
+  if (lane == 0 && atomicAdd(io.blocks_done, 1) == (int)gridDim.x - 1) {
+    *io.blocks_done = 0; *io.turn = turn + 1;
+    volatile int32_t *done = io.done[turn & 1];
+    done[1] = *(volatile int32_t *)io.status;
+    __threadfence_system();
+    done[0] = turn + 1;
+  }
 }
 
 // Verification by a mix of the autoregressive and the diffusion prediction (paper Section 4.4.3:
@@ -527,25 +617,22 @@ __global__ void score_finish_kernel(const float *__restrict__ run_max, const flo
 // mixes it with the first mask row when beta < 1).
 __global__ void prefill_finish_kernel(const int32_t *__restrict__ arg_ids, int row_last_prompt, int row_first, int k, int k_max, int seq,
                                       int n_prompt, int32_t *__restrict__ block_ids, int32_t *__restrict__ blk_len,
-                                      int32_t *__restrict__ seq_len, int32_t *__restrict__ out) {
+                                      int32_t *__restrict__ seq_len, const int32_t *status, int32_t *out /*pinned: first token, status*/) {
   const int i = threadIdx.x;
   if (i < k) block_ids[(size_t)seq * k_max + i] = i == 0 ? arg_ids[row_first] : arg_ids[row_last_prompt + 1 + i];
-  if (i == 0) { seq_len[seq] = n_prompt; blk_len[seq] = k; out[0] = arg_ids[row_first]; }
+  if (i == 0) { seq_len[seq] = n_prompt; blk_len[seq] = k; out[0] = arg_ids[row_first]; out[1] = *(volatile const int32_t *)status; }
 }
 
 // ---------------------------------------------------------------------------
-// KV commit / evict (paper Section 3.3): the k causal slots' K/V were written to
-// the cache at positions n..n+k-1 during the pass; committing L of them is
-// n <- n + L, after which positions n+L..n+k-1 are dead and get overwritten by the
-// next step.  With poison != 0 the dead slots are filled, in every layer, with the
+// KV eviction check (debug): after a step has committed L of its k causal slots, positions n+L..n+k-1 are dead and
+// get overwritten by the next step.  This fills them, in every layer, with the
 // largest finite bf16 (3.4e38), so that any later use of evicted data with a non-zero
 // weight would surface as inf/NaN or a wild value.  (Not NaN itself: the tensor-core
 // attention loads whole 64-position pages and multiplies the masked positions' V rows
 // by an exact zero, which must stay zero.)  Grid (n_seqs, n_layers).
 // ---------------------------------------------------------------------------
-__global__ void kv_commit_kernel(const int32_t *__restrict__ step_seqs, const int32_t *__restrict__ step_n,
-                                 const int32_t *__restrict__ step_L, int32_t *__restrict__ seq_len, int k, const int32_t *__restrict__ step_k,
-                                 int poison, KvGeom g, bf16 *__restrict__ kv_base, size_t pool_stride, TlSlot tl) {
+__global__ void kv_poison_kernel(const int32_t *__restrict__ step_seqs, const int32_t *__restrict__ step_n, const int32_t *__restrict__ step_L, int k,
+                                 const int32_t *__restrict__ step_k, KvGeom g, bf16 *__restrict__ kv_base, size_t pool_stride, TlSlot tl) {
   pdl_trigger();
   pdl_wait();
   if (threadIdx.x == 0) tl_go(tl);
@@ -553,8 +640,6 @@ __global__ void kv_commit_kernel(const int32_t *__restrict__ step_seqs, const in
   if (step_k) k = step_k[s];
   const int seq = step_seqs[s];
   const int n = step_n[s], L = step_L[s];
-  if (l == 0 && threadIdx.x == 0) seq_len[seq] = n + L;
-  if (!poison) { if (threadIdx.x == 0) tl_end(tl); return; }
   bf16 *Kp = kv_base + (size_t)(2 * l) * pool_stride, *Vp = Kp + pool_stride;
   const int per = g.n_kv_heads * g.head_dim;
   const bf16 nanv = __ushort_as_bfloat16((unsigned short)0x7f7f);

@@ -1,7 +1,10 @@
 // C-ABI entry points and per-step orchestration of the TiDAR decode path.
 #include "../../include/tidar.h"
 
+#include <immintrin.h>
+
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -18,6 +21,7 @@
 
 namespace {
 
+constexpr int NORM_SMEM = 200 * 1024;  // shared memory of an SM that the norm kernel's blocks may claim between them
 constexpr int MAX_SMS = 160;      // scratch is sized for this many (a B200 has 148)
 
 std::string g_init_error;
@@ -63,7 +67,7 @@ struct tidar_ctx {
   struct WMap { CUtensorMap full, small; };   // a weight matrix for the full and the SMALL instances of the projection kernel
   std::vector<WMap> tm_lm_chunks;   // the LM head in vocabulary chunks of lm_chunk rows (scoring)
   int32_t *d_seq_len = nullptr, *d_block = nullptr, *d_page_table = nullptr, *d_step_seqs = nullptr, *d_forced = nullptr,
-          *d_step_n = nullptr, *d_step_L = nullptr, *d_out = nullptr, *d_prompt = nullptr, *d_arg_idx = nullptr;
+          *d_step_n = nullptr, *d_step_L = nullptr, *d_prompt = nullptr, *d_arg_idx = nullptr;
   float *X = nullptr, *partials = nullptr, *rope_cos = nullptr, *rope_sin = nullptr, *d_arg_val = nullptr,
         *dbg_hidden = nullptr, *dbg_logits = nullptr;
   bf16 *A = nullptr, *Q = nullptr, *Kloc = nullptr, *Vloc = nullptr, *O = nullptr, *H = nullptr, *dbg_kv = nullptr;
@@ -78,12 +82,11 @@ struct tidar_ctx {
   // Steps that have been enqueued and not yet waited for, oldest first.  Two may be in flight when every
   // acceptance length is forced (the host then knows the lengths without reading the device): the second
   // is enqueued while the first runs, so the device never waits for the host between steps.
-  struct Flight { std::vector<int> seqs, ks; int k = 0, slot = 0; bool counted = false; };
+  struct Flight { std::vector<int> seqs, ks; int k = 0, turn = 0; bool counted = false; };
   std::deque<Flight> inflight;
-  cudaEvent_t flight_done[2] = {nullptr, nullptr};
-  int32_t *h_out2[2] = {nullptr, nullptr}, *h_stage2[2] = {nullptr, nullptr}, *h_status2[2] = {nullptr, nullptr};   // pinned, one set per slot
+  int32_t *h_out2[2] = {nullptr, nullptr}, *h_stage2[2] = {nullptr, nullptr}, *h_done2[2] = {nullptr, nullptr};     // pinned, one set per slot (see StepIo)
   int32_t *h_page_table = nullptr;   // pinned mirror of the page table: the source of its (asynchronous) updates
-  int next_slot = 0;
+  int turn = 0;                      // steps enqueued so far; step i uses slot i & 1
   // tensor-core path
   gemm_tc::EncodeTiledFn encode = nullptr;
   std::vector<WMap> tm_wqkv, tm_wo, tm_wgu, tm_wdown;
@@ -94,8 +97,18 @@ struct tidar_ctx {
   float *attn_part_O = nullptr; float2 *attn_part_ml = nullptr;
   attn_tc::Item *plan_items = nullptr; attn_tc::Tile *plan_tiles = nullptr;       // attention work plan of the current pass
   int n_sms = 0;
-  // the launches of one decode step as an executable graph, valid for one (k, n_seqs)
-  struct StepGraph { int k = 0, n_seqs = 0, mixed_R = 0, tiles = 0, mixed_K = 0; bool ar = false, timeline = false; cudaGraphExec_t exec = nullptr; int64_t launches = 0; } sg;
+  // the launches of one decode step as an executable graph, valid for one key; the most recently used ones are kept
+  struct StepKey {
+    int k = 0, n_seqs = 0, mixed_R = 0, units = 0, mixed_K = 0; bool ar = false, timeline = false, count_tiles = false, split = false;
+    bool operator==(const StepKey &o) const {
+      return k == o.k && n_seqs == o.n_seqs && mixed_R == o.mixed_R && units == o.units && mixed_K == o.mixed_K && ar == o.ar && timeline == o.timeline &&
+             count_tiles == o.count_tiles && split == o.split;
+    }
+  };
+  struct StepGraph { StepKey key; cudaGraphExec_t exec = nullptr; int64_t launches = 0; };
+  static constexpr size_t MAX_GRAPHS = 16;
+  std::deque<StepGraph> graphs;      // most recently used first
+  bool split_keys = true;            // attention key ranges of the current pass may be cut (see attention_plan)
   bool graphs_ok = true;
   bool slab_bf16 = false;          // split-K partial sums of the step in bf16 instead of fp32 (config debug bit 2)
   int32_t *d_status = nullptr, *cand_idx = nullptr;
@@ -171,7 +184,7 @@ void layout(tidar_ctx &x, void *arena, size_t *bytes) {
   x.n_qkv = (c.n_q_heads + 2 * c.n_kv_heads) * c.head_dim;
   x.pool_stride = (size_t)x.n_pages * c.n_kv_heads * c.page_size * c.head_dim;
   x.lm_chunk = std::min(c.vocab, 16384);
-  x.S_max = c.impl == 0 ? 8 : 4;
+  x.S_max = c.impl == 0 ? MAX_SLABS : 4;
   const size_t R = x.R_cap;
   const size_t widest = std::max<size_t>({(size_t)x.S_max * x.n_qkv, (size_t)x.S_max * c.d_model, (size_t)2 * c.d_ffn,
                                           (size_t)x.lm_chunk});
@@ -195,7 +208,6 @@ void layout(tidar_ctx &x, void *arena, size_t *bytes) {
   x.d_page_table = cv.take<int32_t>((size_t)c.max_batch * x.pages_per_seq);
   x.d_step_seqs = cv.take<int32_t>(c.max_batch); x.d_forced = cv.take<int32_t>(c.max_batch);
   x.d_step_n = cv.take<int32_t>(c.max_batch); x.d_step_L = cv.take<int32_t>(c.max_batch);
-  x.d_out = cv.take<int32_t>((size_t)c.max_batch * (c.k_max + 1));
   x.d_prompt = cv.take<int32_t>(c.max_seq_len);
   x.d_arg_idx = cv.take<int32_t>(R); x.d_arg_val = cv.take<float>(R);
   x.d_status = cv.take<int32_t>(64);
@@ -468,6 +480,7 @@ struct AttnMaps { const CUtensorMap *q, *k, *v, *kloc, *vloc; int page_base_k, p
 // step; all rows in a first-pass chunk); <= 0: the sequences' groups differ in size and the units come from the mixed
 // step's table.  Key ranges may be split (see attn_tc::plan_block) while there are fewer than three
 // (unit, KV head) combinations for two SMs: beyond that they fill the machine evenly enough.
+// c->split_keys == false: no key range of the pass is long enough to be worth cutting (see may_split).
 // The grid is the number of items the plan may use; a CTA holds a whole SM, so up to one combination per SM it is one wave.
 attn_tc::PlanArgs attention_plan(const tidar_ctx *c, int R, int rows_per_group) {
   const tidar_config &cf = c->cfg;
@@ -485,9 +498,15 @@ attn_tc::PlanArgs attention_plan(const tidar_ctx *c, int R, int rows_per_group) 
   const int units = p.n_units * p.Hkv;
   static_assert(attn_tc::PLAN_UNITS >= 3 * MAX_SMS / 2, "units that may be split are planned");
   p.max_items = units <= c->n_sms ? c->n_sms / p.Hkv : 2 * units < 3 * c->n_sms ? attn_tc::SLOTS_PER_SM * c->n_sms / p.Hkv : p.n_units;
+  p.max_pieces = attn_tc::MAX_SPLITS;
+  if (!c->split_keys) { p.max_pieces = 1; p.max_items = 2 * units <= c->n_sms ? 2 * p.n_units : p.n_units; }
   p.items = c->plan_items; p.tiles = c->plan_tiles;
   return p;
 }
+
+// Whether a pass whose rows see at most n_keys positions may cut key ranges.  A cut costs a partial result's store and the merge
+// kernel, about 5 us, and saves half of 0.56 us per page at best.
+bool may_split(int n_keys) { return n_keys > 12 * attn_tc::PAGE; }
 
 // Attention of the pass that plan p was made for (the plan itself is in device memory by then).
 void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMaps &m, const KvGeom &g, bf16 *O) {
@@ -509,7 +528,7 @@ void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMap
     else
       launch_pdl(attn_tc::attn_tc_kernel<64>, grid, attn_tc::THREADS, attn_tc::Smem<64>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
   }
-  if (p.max_items > p.n_units) {
+  if (p.max_items > p.n_units && p.max_pieces > 1) {
     Launch l(c, TIDAR_TC_ATTN);
     const int blocks = 2 * p.n_units * p.Hkv * (cf.head_dim / 16);
     if (cf.head_dim == 128) launch_pdl(attn_tc::attn_combine_kernel<128>, blocks, 256, 0, c->stream, a, l.tl);
@@ -529,13 +548,24 @@ void launch_attention(tidar_ctx *c, const bf16 *Q, const bf16 *Kp, const bf16 *V
 }
 
 // partials: split-K slabs of the previous projection, bf16 on the tensor-core path, fp32 on the replay path
-void launch_norm(tidar_ctx *c, int R, const float *partials, int S, size_t stride, const bf16 *gain) {
+template <typename SLAB>
+void launch_norm_as(tidar_ctx *c, int R, const SLAB *partials, int S, size_t stride, const bf16 *gain) {
   Launch l(c, TIDAR_TC_NORM);
-  const int d = c->cfg.d_model;
-  if (c->cfg.impl == 0 && c->slab_bf16)
-    launch_pdl(rmsnorm_reduce_kernel<512, bf16>, R, 512, d * sizeof(float), c->stream, c->X, (const bf16 *)partials, S, stride, gain, c->cfg.rms_eps, d, c->A, l.tl);
-  else
-    launch_pdl(rmsnorm_reduce_kernel<512, float>, R, 512, d * sizeof(float), c->stream, c->X, partials, S, stride, gain, c->cfg.rms_eps, d, c->A, l.tl);
+  const int d = c->cfg.d_model, nv = (d + 2047) / 2048;
+  // Behind a projection of many rows the blocks would all crowd onto the SMs that run out of work first (5.6 instead of
+  // 3.6 us at 272 rows); claiming a share of the shared memory spreads them evenly.  With few rows they must leave room
+  // for the next projection's CTAs.
+  const int per_sm = c->cfg.impl == 0 ? (R + c->n_sms - 1) / c->n_sms : 0;
+  const size_t smem = R > gemm_tc::SMALL_ROWS && per_sm <= 4 && per_sm > 0 ? (size_t)(NORM_SMEM / per_sm) & ~(size_t)1023 : 0;
+  auto go = [&](auto kernel) { launch_pdl(kernel, R, 512, smem, c->stream, c->X, partials, S, stride, gain, c->cfg.rms_eps, d, c->A, l.tl); };
+  if (nv <= 1) go(rmsnorm_reduce_kernel<512, 1, SLAB>);
+  else if (nv <= 2) go(rmsnorm_reduce_kernel<512, 2, SLAB>);
+  else if (nv <= 3) go(rmsnorm_reduce_kernel<512, 3, SLAB>);
+  else go(rmsnorm_reduce_kernel<512, 6, SLAB>);
+}
+void launch_norm(tidar_ctx *c, int R, const float *partials, int S, size_t stride, const bf16 *gain) {
+  if (c->cfg.impl == 0 && c->slab_bf16) launch_norm_as<bf16>(c, R, (const bf16 *)partials, S, stride, gain);
+  else launch_norm_as<float>(c, R, partials, S, stride, gain);
 }
 
 // The transformer stack over R assembled rows (metadata and X already filled).
@@ -679,12 +709,16 @@ int init_tensor_core_path(tidar_ctx *c) {
   {
     auto max_smem_split = [&](const void *f) { return cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared); };
     const void *kernels[] = {(const void *)assemble_step_kernel, (const void *)pass_setup_kernel, (const void *)attn_meta_plan_kernel,
-                             (const void *)rmsnorm_reduce_kernel<512, float>, (const void *)rmsnorm_reduce_kernel<512, bf16>,
+                             (const void *)rmsnorm_reduce_kernel<512, 1, float>, (const void *)rmsnorm_reduce_kernel<512, 1, bf16>,
+                             (const void *)rmsnorm_reduce_kernel<512, 2, float>, (const void *)rmsnorm_reduce_kernel<512, 2, bf16>,
+                             (const void *)rmsnorm_reduce_kernel<512, 3, float>, (const void *)rmsnorm_reduce_kernel<512, 3, bf16>,
+                             (const void *)rmsnorm_reduce_kernel<512, 6, float>, (const void *)rmsnorm_reduce_kernel<512, 6, bf16>,
                              (const void *)rope_kv_kernel<float>, (const void *)rope_kv_kernel<bf16>,
                              (const void *)swiglu_slab_kernel<float>, (const void *)swiglu_slab_kernel<bf16>,
                              (const void *)attn_tc::attn_combine_kernel<128>, (const void *)attn_tc::attn_combine_kernel<64>,
-                             (const void *)mix_rows_kernel, (const void *)argmax_merge_kernel, (const void *)verify_select_kernel, (const void *)kv_commit_kernel};
+                             (const void *)mix_rows_kernel, (const void *)argmax_merge_kernel, (const void *)verify_select_kernel, (const void *)stage_step_kernel};
     for (const void *f : kernels) CUDA_TRY(c, max_smem_split(f));
+    for (int i = 3; i < 11; ++i) CUDA_TRY(c, cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, NORM_SMEM));
   }
   const int max_smem = gemm_tc::SMEM_BUDGET + 1024, small_smem = gemm_tc::SMALL_SMEM_BUDGET + 1024;
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, small_smem));
@@ -698,8 +732,11 @@ int init_tensor_core_path(tidar_ctx *c) {
   return TIDAR_OK;
 }
 
-// Reads the device status word (already copied to pinned memory by the caller's
-// synchronised copy) and turns a device-side timeout into an error code.
+int device_timeout(tidar_ctx *c, int st) {
+  return fail(c, TIDAR_EDEVICE_TIMEOUT, "a bounded device-side wait gave up (status %d); results of this call are invalid", st);
+}
+
+// Reads the device status word and turns a device-side timeout into an error code.
 int check_device_status(tidar_ctx *c) {
   if (c->cfg.impl != 0) return TIDAR_OK;
   int st = 0;
@@ -707,7 +744,7 @@ int check_device_status(tidar_ctx *c) {
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   if (st) {
     cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
-    return fail(c, TIDAR_EDEVICE_TIMEOUT, "a bounded device-side wait gave up (status %d); results of this call are invalid", st);
+    return device_timeout(c, st);
   }
   return TIDAR_OK;
 }
@@ -739,22 +776,35 @@ int ensure_pages(tidar_ctx *c, int seq, int upto_positions) {
   return TIDAR_OK;
 }
 
-// Enqueues the kernels of one decode step (its inputs are already in d_step_seqs / d_forced).
-// k: block length of this step; ar: plain autoregressive step (the causal section alone).
-// mixed_R > 0: the listed sequences use different block lengths (layout staged in h_lay, mixed_R rows in all).
-// mixed_K: the sum of those block lengths (= verified positions, one mixed row each when beta < 1).
-int record_step(tidar_ctx *c, int n_seqs, int k, bool ar, int mixed_R = 0, int mixed_K = 0) {
+StepIo step_io(const tidar_ctx *c) {
+  StepIo io;
+  io.turn = c->d_status + 16; io.blocks_done = c->d_status + 32; io.status = c->d_status;
+  for (int sl = 0; sl < 2; ++sl) { io.in[sl] = c->h_stage2[sl]; io.out[sl] = c->h_out2[sl]; io.done[sl] = c->h_done2[sl]; }
+  io.max_batch = c->cfg.max_batch;
+  return io;
+}
+
+// Enqueues the kernels of one decode step (its inputs are in the slot's pinned staging).
+// key.k: block length of this step; key.ar: plain autoregressive step (the causal section alone).
+// key.mixed_R > 0: the listed sequences use different block lengths (layout staged in h_lay, mixed_R rows in all).
+// key.mixed_K: the sum of those block lengths (= verified positions, one mixed row each when beta < 1).
+int record_step(tidar_ctx *c, const tidar_ctx::StepKey &key) {
   const tidar_config &cf = c->cfg;
-  const int n_blocks = ar ? 0 : k;
-  const int T = k * (n_blocks + 1), R = mixed_R > 0 ? mixed_R : n_seqs * T;
+  const int n_seqs = key.n_seqs, k = key.k, n_blocks = key.ar ? 0 : k;
+  const int T = k * (n_blocks + 1), R = key.mixed_R > 0 ? key.mixed_R : n_seqs * T;
   StepLayout lay{nullptr, nullptr, nullptr, n_seqs};
-  if (mixed_R > 0) {
-    CUDA_TRY(c, cudaMemcpyAsync(c->d_step_k, c->h_lay, c->lay_ints * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    lay.k = c->d_step_k; lay.off = c->d_step_off; lay.loc = c->d_step_loc;
-  }
+  if (key.mixed_R > 0) { lay.k = c->d_step_k; lay.off = c->d_step_off; lay.loc = c->d_step_loc; }
+  c->split_keys = key.split;
+  c->mixed_units = key.units;
   if (c->timeline) {
     c->tl_n = 0; c->tl_cls.clear();
     CUDA_TRY(c, cudaMemsetAsync(c->d_tl, 0, 2 * tidar_ctx::TL_MAX * sizeof(unsigned long long), c->stream));
+  }
+  const StepIo io = step_io(c);
+  {
+    Launch l(c, TIDAR_TC_EMBED);
+    launch_pdl(stage_step_kernel, 1, 256, 0, c->stream, io, n_seqs, c->d_step_seqs, c->d_forced, c->h_lay, c->d_step_k,
+               key.mixed_R > 0 ? 3 * (cf.max_batch + 1) : 0, c->R_head + cf.max_batch, key.units, l.tl);
   }
   {
     Launch l(c, TIDAR_TC_EMBED);
@@ -763,65 +813,77 @@ int record_step(tidar_ctx *c, int n_seqs, int k, bool ar, int mixed_R = 0, int m
   }
   // beta < 1: the verified prediction of causal slot j mixes its row with the first slot of block j
   MixRows mix;
-  if (cf.beta < 1.0f && !ar) {
-    if (mixed_R > 0) { mix.n = mixed_K; mix.lay = lay; }
+  if (cf.beta < 1.0f && !key.ar) {
+    if (key.mixed_R > 0) { mix.n = key.mixed_K; mix.lay = lay; }
     else { mix.n = n_seqs * k; mix.k = k; mix.a0 = 0; mix.a_seq = T; mix.a_j = 1; mix.b0 = k; mix.b_seq = T; mix.b_j = k; }
   }
-  if (int rc = forward_rows(c, R, true, mixed_R > 0 ? 0 : T, mix)) return rc;
+  if (int rc = forward_rows(c, R, true, key.mixed_R > 0 ? 0 : T, mix)) return rc;
   {
     Launch l(c, TIDAR_TC_VERIFY);
     launch_pdl(verify_select_kernel, n_seqs, 32, 0, c->stream, c->d_arg_idx, mix.n ? c->d_arg_idx + R : (const int32_t *)nullptr, c->d_step_seqs,
-               c->d_forced, k, n_blocks, lay, cf.k_max, c->d_block, c->d_blk_len, c->d_step_L, c->d_out, l.tl);
+               c->d_forced, k, n_blocks, lay, cf.k_max, c->d_block, c->d_blk_len, c->d_step_n, c->d_step_L, c->d_seq_len, io, l.tl);
   }
-  {
+  if (cf.debug & 2) {
     Launch l(c, TIDAR_TC_VERIFY);
-    launch_pdl(kv_commit_kernel, dim3(n_seqs, cf.n_layers), 128, 0, c->stream, c->d_step_seqs, c->d_step_n, c->d_step_L, c->d_seq_len, k, lay.k,
-               (cf.debug >> 1) & 1, geom(c), c->kv, c->pool_stride, l.tl);
+    launch_pdl(kv_poison_kernel, dim3(n_seqs, cf.n_layers), 128, 0, c->stream, c->d_step_seqs, c->d_step_n, c->d_step_L, k, lay.k, geom(c), c->kv,
+               c->pool_stride, l.tl);
   }
   CUDA_TRY(c, cudaGetLastError());
   return TIDAR_OK;
 }
 
-// Every launch of a step has the same arguments from step to step (lengths, page tables, token
+bool use_graphs(const tidar_ctx *c) { return c->cfg.impl == 0 && c->graphs_ok && !c->timing && !(c->cfg.debug & (1 | 8)); }
+
+void drop_graphs(tidar_ctx *c, size_t keep) {
+  while (c->graphs.size() > keep) {
+    cudaStreamSynchronize(c->stream);               // it may still be running
+    cudaGraphExecDestroy(c->graphs.back().exec);
+    c->graphs.pop_back();
+  }
+}
+
+// The step proper.  Every launch of a step has the same arguments from step to step (lengths, page tables, token
 // blocks and, for a step of mixed block lengths, the row layout live in device memory), except
-// for the grid sizes, so the step is captured once per (k, n_seqs, rows, query tiles) and replayed.  Per-launch timing and the debug read-backs use plain
-// launches.  tiles: attention units per KV head.
-int replay_or_record_step(tidar_ctx *c, int n_seqs, int k, bool ar, int mixed_R, int tiles, int mixed_K = 0) {
-  const tidar_config &cf = c->cfg;
-  if (cf.impl == 0 && c->graphs_ok && !c->timing && !(cf.debug & (1 | 8))) {
-    tidar_ctx::StepGraph &sg = c->sg;
-    if (!sg.exec || sg.k != k || sg.ar != ar || sg.n_seqs != n_seqs || sg.timeline != c->timeline ||
-        sg.mixed_R != mixed_R || sg.tiles != tiles || sg.mixed_K != mixed_K) {
-      if (sg.exec) {
-        if (!c->inflight.empty()) CUDA_TRY(c, cudaStreamSynchronize(c->stream));    // the old graph may still be running
-        cudaGraphExecDestroy(sg.exec); sg.exec = nullptr;
-      }
+// for the grid sizes, so the step is captured once per key and replayed.  Per-launch timing and the debug read-backs
+// use plain launches.  key.units: attention units per KV head.
+int launch_step(tidar_ctx *c, tidar_ctx::StepKey key) {
+  key.timeline = c->timeline; key.count_tiles = c->count_tiles;
+  if (use_graphs(c)) {
+    auto it = std::find_if(c->graphs.begin(), c->graphs.end(), [&](const tidar_ctx::StepGraph &g) { return g.key == key; });
+    if (it == c->graphs.end()) {
+      drop_graphs(c, tidar_ctx::MAX_GRAPHS - 1);
+      tidar_ctx::StepGraph sg;
+      sg.key = key;
       const int64_t l0 = c->launches;
       cudaGraph_t graph = nullptr;
       int rc = TIDAR_OK;
       cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
       if (e == cudaSuccess) {
-        rc = record_step(c, n_seqs, k, ar, mixed_R, mixed_K);
+        rc = record_step(c, key);
         e = cudaStreamEndCapture(c->stream, &graph);
       }
       if (e == cudaSuccess && rc == TIDAR_OK && graph) e = cudaGraphInstantiate(&sg.exec, graph, 0);
       if (graph) cudaGraphDestroy(graph);
+      sg.launches = c->launches - l0;
+      c->launches = l0;
       if (e != cudaSuccess || rc != TIDAR_OK || !sg.exec) {
         cudaGetLastError();                         // capture is not available here: plain launches from now on
-        sg.exec = nullptr; c->graphs_ok = false;
+        c->graphs_ok = false;
       } else {
-        sg.k = k; sg.ar = ar; sg.n_seqs = n_seqs; sg.timeline = c->timeline; sg.mixed_R = mixed_R; sg.tiles = tiles; sg.mixed_K = mixed_K;
-        sg.launches = c->launches - l0;
+        c->graphs.push_front(sg);
       }
-      c->launches = l0;
+    } else if (it != c->graphs.begin()) {
+      const tidar_ctx::StepGraph sg = *it;
+      c->graphs.erase(it);
+      c->graphs.push_front(sg);
     }
-    if (sg.exec) {
-      CUDA_TRY(c, cudaGraphLaunch(sg.exec, c->stream));
-      c->launches += sg.launches;
+    if (c->graphs_ok) {
+      CUDA_TRY(c, cudaGraphLaunch(c->graphs.front().exec, c->stream));
+      c->launches += c->graphs.front().launches;
       return TIDAR_OK;
     }
   }
-  return record_step(c, n_seqs, k, ar, mixed_R, mixed_K);
+  return record_step(c, key);
 }
 
 // Whether one more step may be enqueued: always when none is in flight; behind a step in flight only when
@@ -833,31 +895,17 @@ bool may_enqueue(tidar_ctx *c, bool all_forced, bool mixed) {
   return c->inflight.front().counted && c->inflight.front().ks.empty();
 }
 
-// The step proper: its inputs from the slot's pinned staging, the kernels (replayed graph or plain
-// launches), its results into the slot's pinned buffers, and the event its waiter blocks on.
-int launch_step(tidar_ctx *c, int n_seqs, int k, bool ar, int mixed_R, int tiles, int slot, int mixed_K = 0) {
-  const tidar_config &cf = c->cfg;
-  CUDA_TRY(c, cudaMemcpyAsync(c->d_step_seqs, c->h_stage2[slot], n_seqs * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  CUDA_TRY(c, cudaMemcpyAsync(c->d_forced, c->h_stage2[slot] + cf.max_batch, n_seqs * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  if (int rc = replay_or_record_step(c, n_seqs, k, ar, mixed_R, tiles, mixed_K)) return rc;
-  CUDA_TRY(c, cudaMemcpyAsync(c->h_out2[slot], c->d_out, (size_t)n_seqs * (cf.k_max + 1) * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  CUDA_TRY(c, cudaMemcpyAsync(c->h_status2[slot], c->d_status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  CUDA_TRY(c, cudaEventRecord(c->flight_done[slot], c->stream));
-  return TIDAR_OK;
-}
-
 // Book-keeping of an enqueued step.  With every length forced the host advances the sequences now.
-void push_flight(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int32_t *forced, int k, const int32_t *ks, int slot) {
+void push_flight(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int32_t *forced, int k, const int32_t *ks) {
   tidar_ctx::Flight f;
   f.seqs.assign(seqs, seqs + n_seqs);
   if (ks) f.ks.assign(ks, ks + n_seqs);
-  f.k = k; f.slot = slot;
+  f.k = k; f.turn = c->turn++;
   f.counted = forced != nullptr;
   for (int i = 0; i < n_seqs && f.counted; ++i) f.counted = forced[i] > 0;
   if (f.counted)
     for (int i = 0; i < n_seqs; ++i) { c->seqs[seqs[i]].n += forced[i]; c->seqs[seqs[i]].k = ks ? ks[i] : k; }
   c->inflight.push_back(std::move(f));
-  c->next_slot ^= 1;
 }
 
 // k_step: block length of this step (0 = the one the sequences' last pass left, which must then be
@@ -893,11 +941,17 @@ int enqueue_step(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int32_t *f
     if (rc) return rc;
   }
   const int T = ar ? 1 : k * (k + 1), R = n_seqs * T;
-  const int slot = c->next_slot;
-  for (int i = 0; i < n_seqs; ++i) { c->h_stage2[slot][i] = seqs[i]; c->h_stage2[slot][cf.max_batch + i] = forced ? forced[i] : 0; }
+  const int slot = c->turn & 1;
+  int max_n = 0;
+  for (int i = 0; i < n_seqs; ++i) {
+    c->h_stage2[slot][i] = seqs[i]; c->h_stage2[slot][cf.max_batch + i] = forced ? forced[i] : 0;
+    max_n = std::max(max_n, c->seqs[seqs[i]].n);
+  }
   const int spt = 2 * (128 / (cf.n_q_heads / cf.n_kv_heads));      // slots per attention unit (two query tiles)
-  if (int rc = launch_step(c, n_seqs, k, ar, 0, n_seqs * ((T + spt - 1) / spt), slot)) return rc;
-  push_flight(c, seqs, n_seqs, forced, k, nullptr, slot);
+  tidar_ctx::StepKey key;
+  key.k = k; key.n_seqs = n_seqs; key.ar = ar; key.units = n_seqs * ((T + spt - 1) / spt); key.split = may_split(max_n);
+  if (int rc = launch_step(c, key)) return rc;
+  push_flight(c, seqs, n_seqs, forced, k, nullptr);
   c->last_hidden_off = 0;
   c->last_rows = R + ((cf.beta < 1.0f && !ar) ? n_seqs * k : 0); c->last_first_pos = -1;      // the mixed rows follow the slots
   // the host tracks lengths without reading the device when L is forced
@@ -907,8 +961,8 @@ int enqueue_step(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int32_t *f
 // A step in which listed sequence i uses block length ks[i] (Section 5: the block length follows the
 // compute profile; nothing in the method ties the sequences of a batch to one length).  Equal lengths
 // take the ordinary path; different lengths run over R = sum k_i (k_i + 1) rows with a per-sequence
-// row layout and an attention tile table (one captured graph serves every step with the same
-// number of sequences, rows and query tiles).
+// row layout and an attention unit table (one captured graph serves every step with the same
+// number of sequences, row blocks of 16 and units).
 int enqueue_step_mixed(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int32_t *ks, const int32_t *forced) {
   const tidar_config &cf = c->cfg;
   if (!seqs || !ks || n_seqs < 1 || n_seqs > cf.max_batch) return fail(c, TIDAR_EINVAL, "n_seqs must be in [1, max_batch]");
@@ -932,21 +986,31 @@ int enqueue_step_mixed(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int3
     if (int rc = ensure_pages(c, seqs[i], c->seqs[seqs[i]].n + ks[i])) return rc;
   const int mb = cf.max_batch, spt = 2 * (128 / (cf.n_q_heads / cf.n_kv_heads));
   int32_t *hk = c->h_lay, *hoff = hk + (mb + 1), *hloc = hoff + (mb + 1), *ht0 = hloc + (mb + 1), *hte = ht0 + (c->R_head + mb);
-  const int slot = c->next_slot;
-  int R = 0, loc = 0, tiles = 0, sum_k = 0;
+  const int slot = c->turn & 1;
+  int max_n = 0, R = 0, loc = 0, tiles = 0, sum_k = 0;
   for (int i = 0; i < n_seqs; ++i) {
     const int k = ks[i], T = k * (k + 1);
     hk[i] = k; hoff[i] = R; hloc[i] = loc; sum_k += k;
     for (int r0 = R; r0 < R + T; r0 += spt) { ht0[tiles] = r0; hte[tiles] = R + T; ++tiles; }
     R += T; loc += k * k;
     c->h_stage2[slot][i] = seqs[i]; c->h_stage2[slot][mb + i] = forced ? forced[i] : 0;
+    max_n = std::max(max_n, c->seqs[seqs[i]].n);
   }
   hk[n_seqs] = 0; hoff[n_seqs] = R; hloc[n_seqs] = loc;
-  c->mixed_units = tiles;
   // a mixed step's kernels take every per-sequence length from the staged layout: the nominal k is unused
+  tidar_ctx::StepKey key;
+  key.n_seqs = n_seqs; key.mixed_R = R; key.units = tiles; key.split = may_split(max_n);
   const int mixed_rows = cf.beta < 1.0f ? sum_k : 0;         // one mixed LM-head input row per verified position
-  if (int rc = launch_step(c, n_seqs, 0, false, R, tiles, slot, mixed_rows)) return rc;
-  push_flight(c, seqs, n_seqs, forced, 0, ks, slot);
+  key.mixed_K = mixed_rows;
+  // Steps of nearly the same size share one captured graph: rows are filled up to a multiple of 16 (the projections' row
+  // blocks are that anyway) and units to a multiple of 4 with ones that have no rows.
+  if (cf.impl == 0 && mixed_rows == 0) {
+    key.mixed_R = (R + 15) / 16 * 16;
+    for (; tiles % 4 && tiles < c->R_head + mb; ++tiles) ht0[tiles] = hte[tiles] = 0;
+    key.units = tiles;
+  }
+  if (int rc = launch_step(c, key)) return rc;
+  push_flight(c, seqs, n_seqs, forced, 0, ks);
   c->last_hidden_off = 0;
   c->last_rows = R + mixed_rows; c->last_first_pos = -1;
   return TIDAR_OK;
@@ -957,16 +1021,30 @@ int finish_step(tidar_ctx *c, int32_t *out_tokens, int32_t *out_n) {
   if (c->inflight.empty()) return fail(c, TIDAR_EINVAL, "no step in flight");
   tidar_ctx::Flight f = std::move(c->inflight.front());
   c->inflight.pop_front();
-  CUDA_TRY(c, cudaEventSynchronize(c->flight_done[f.slot]));
+  const int slot = f.turn & 1;
+  if (c->timing || c->timeline || (c->cfg.debug & 2)) CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  // The step's last kernel writes its turn number behind the results (see StepIo).  The stream is asked now and then
+  // only, in case the kernels failed.
+  const volatile int32_t *done = c->h_done2[slot];
+  for (uint32_t polls = 1; done[0] != f.turn + 1; ++polls) {
+    if ((polls & 0x3fff) == 0) {
+      const cudaError_t e = cudaStreamQuery(c->stream);
+      if (e == cudaErrorNotReady) continue;
+      CUDA_TRY(c, e);
+      if (done[0] != f.turn + 1) return fail(c, TIDAR_ECUDA, "the step's kernels ended without results");
+    }
+    _mm_pause();
+  }
+  std::atomic_thread_fence(std::memory_order_acquire);
   if (c->timing) collect_timing(c);
   if (c->timeline) collect_timeline(c);
-  if (c->h_status2[f.slot][0]) {
+  if (done[1]) {
     // The step's kernels have already rewritten the device-side lengths and blocks of the listed
     // sequences from invalid results: their state is lost, and so is that of a step enqueued behind
     // it.  Release them all; a new first pass is needed.
-    const int st = c->h_status2[f.slot][0];
+    const int st = done[1];
     cudaStreamSynchronize(c->stream);
-    c->h_status2[0][0] = 0; c->h_status2[1][0] = 0; cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
+    cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
     for (int q : f.seqs) release_sequence(c, q);
     for (auto &g : c->inflight) for (int q : g.seqs) release_sequence(c, q);
     c->inflight.clear();
@@ -974,7 +1052,7 @@ int finish_step(tidar_ctx *c, int32_t *out_tokens, int32_t *out_n) {
                                           "listed sequences were released (prefill them again)", st);
   }
   const int km = c->cfg.k_max;
-  const int32_t *res = c->h_out2[f.slot];
+  const int32_t *res = c->h_out2[slot];
   for (size_t i = 0; i < f.seqs.size(); ++i) {
     const int L = res[i * (km + 1)];
     if (!f.counted) {
@@ -1044,7 +1122,7 @@ int tidar_init(const tidar_config *cfg, const tidar_weights *w, void *arena, siz
   for (int i = 0; i < c->n_pages; ++i) c->free_pages[i] = i;
   uint32_t st = 0x9e3779b9u;
   for (int i = c->n_pages - 1; i > 0; --i) { st = st * 1664525u + 1013904223u; std::swap(c->free_pages[i], c->free_pages[(st >> 8) % (i + 1)]); }
-  // one pinned block: first-pass result | per slot: step results, staged inputs, status | mixed-step layout | page-table mirror
+  // one pinned block: first-pass result | per slot: step results, staged inputs, turn and status | mixed-step layout | page-table mirror
   const size_t n_out = (size_t)cfg->max_batch * (cfg->k_max + 1), n_stage = 2 * (size_t)cfg->max_batch, n_pt = (size_t)cfg->max_batch * c->pages_per_seq;
   cudaError_t e = cudaHostAlloc((void **)&c->h_pinned, (n_out + 2 * (n_out + n_stage + 16) + c->lay_ints + n_pt) * sizeof(int), cudaHostAllocDefault);
   if (e != cudaSuccess) { delete c; return fail(nullptr, TIDAR_ECUDA, "cudaHostAlloc: %s", cudaGetErrorString(e)); }
@@ -1053,17 +1131,13 @@ int tidar_init(const tidar_config *cfg, const tidar_weights *w, void *arena, siz
     for (int sl = 0; sl < 2; ++sl) {
       c->h_out2[sl] = p; p += n_out;
       c->h_stage2[sl] = p; p += n_stage;
-      c->h_status2[sl] = p; p += 16;
-      c->h_status2[sl][0] = 0;
+      c->h_done2[sl] = p; p += 16;
+      c->h_done2[sl][0] = c->h_done2[sl][1] = 0;
     }
     c->h_lay = p; p += c->lay_ints;
     c->h_page_table = p;
     std::memset(c->h_page_table, 0, n_pt * sizeof(int));
   }
-  for (int sl = 0; sl < 2; ++sl)
-    if (cudaEventCreateWithFlags(&c->flight_done[sl], cudaEventDisableTiming) != cudaSuccess) {
-      cudaFreeHost(c->h_pinned); delete c; return fail(nullptr, TIDAR_ECUDA, "cudaEventCreate failed");
-    }
   e = cudaMemsetAsync(c->d_seq_len, 0, cfg->max_batch * sizeof(int), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_status, 0, 64 * sizeof(int), c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_page_table, 0, (size_t)cfg->max_batch * c->pages_per_seq * sizeof(int), c->stream);
@@ -1105,21 +1179,24 @@ int tidar_prefill(tidar_ctx *c, int32_t seq, const int32_t *prompt, int32_t n_pr
     if (last && cf.beta < 1.0f) { mix.n = 1; mix.k = 1; mix.a0 = rlp; mix.b0 = rlp + 1; }
     // logits are needed for the last prompt row and the k mask rows only; the LM head runs on the
     // trailing rows of the last chunk, as many as a decode step has (all of them for a short prompt)
+    c->split_keys = may_split(row0 + rows);
     const int head_row0 = last ? std::max(0, rows + mix.n - c->R_head) : 0;
     if (int rc = forward_rows(c, rows, last, rows, mix, head_row0)) return rc;
     if (last) {
       Launch l(c, TIDAR_TC_VERIFY);
       prefill_finish_kernel<<<1, 32, 0, c->stream>>>(c->d_arg_idx, rlp - head_row0, (mix.n ? rows : rlp) - head_row0, k, cf.k_max, seq, n_prompt,
-                                                     c->d_block, c->d_blk_len, c->d_seq_len, c->d_out);
+                                                     c->d_block, c->d_blk_len, c->d_seq_len, c->d_status, c->h_pinned);
       c->last_rows = rows - head_row0; c->last_first_pos = row0 + head_row0; c->last_hidden_off = head_row0;
     }
     row0 += rows;
   }
-  CUDA_TRY(c, cudaMemcpyAsync(c->h_pinned, c->d_out, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  CUDA_TRY(c, cudaGetLastError());
   if (c->timing) collect_timing(c);
-  if (int rc = check_device_status(c)) { release_sequence(c, seq); return rc; }
+  if (const int st = c->h_pinned[1]) {
+    cudaMemsetAsync(c->d_status, 0, sizeof(int), c->stream);
+    release_sequence(c, seq);
+    return device_timeout(c, st);
+  }
   s.n = n_prompt; s.active = true;
   if (out_first) *out_first = c->h_pinned[0];
   return TIDAR_OK;
@@ -1223,6 +1300,7 @@ int tidar_score(tidar_ctx *c, int32_t seq, const int32_t *ids, int32_t n, float 
       Launch l(c, TIDAR_TC_EMBED);
       assemble_prefill_kernel<<<rows, 256, 0, c->stream>>>(c->meta, seq, row0, n, 0, cf.mask_token_id, c->d_prompt, c->embed, d, c->X, 0, 0ull);
     }
+    c->split_keys = may_split(row0 + rows);
     if (int rc = forward_rows(c, rows, false, rows)) return rc;      // ends with the final norm in c->A
     for (int v0 = 0, ci = 0; v0 < cf.vocab; v0 += c->lm_chunk, ++ci) {
       const int nc = std::min(c->lm_chunk, cf.vocab - v0);
@@ -1252,8 +1330,7 @@ int tidar_free(tidar_ctx *c) {
   if (!c) return TIDAR_EINVAL;
   cudaStreamSynchronize(c->stream);
   for (auto &t : c->timed) { cudaEventDestroy(t.a); cudaEventDestroy(t.b); }
-  if (c->sg.exec) cudaGraphExecDestroy(c->sg.exec);
-  for (int sl = 0; sl < 2; ++sl) if (c->flight_done[sl]) cudaEventDestroy(c->flight_done[sl]);
+  drop_graphs(c, 0);
   if (c->h_pinned) cudaFreeHost(c->h_pinned);
   delete c;
   return TIDAR_OK;
@@ -1372,7 +1449,6 @@ int tidar_debug_count_attention_tiles(tidar_ctx *c, int32_t on, uint64_t *visite
     *visited = v;
   }
   CUDA_TRY(c, cudaMemset(ctr, 0, sizeof(unsigned long long)));
-  if ((on != 0) != c->count_tiles && c->sg.exec) { cudaGraphExecDestroy(c->sg.exec); c->sg.exec = nullptr; }   // the flag is baked into the graph
   c->count_tiles = on != 0;
   return TIDAR_OK;
 }
@@ -1450,6 +1526,7 @@ int tidar_attention(tidar_ctx *c, const void *q, const void *k_pages, const void
       ((uintptr_t)page_table | (uintptr_t)seq_len) % 4)
     return fail(c, TIDAR_EINVAL, "tensors must be 16-byte aligned (page_table and seq_len 4-byte)");
   const int R = n_seqs * k * (k + 1), n_max = pages_per_seq * c->cfg.page_size - k;
+  c->split_keys = may_split(pages_per_seq * c->cfg.page_size);       // the lengths themselves are on the device
   const attn_tc::PlanArgs plan = c->cfg.impl == 0 ? attention_plan(c, R, k * (k + 1)) : attn_tc::PlanArgs{};
   {
     Launch l(c, TIDAR_TC_EMBED);
