@@ -6,37 +6,46 @@
 // A decode step has only k*(k+1) token slots per sequence (paper Section 3.3 footnote),
 // so every projection is a GEMM with a small row count and a weight matrix that is read
 // exactly once: the regime in which, by the paper's argument, extra token slots are nearly free
-// (Section 1; figure "Latency Scaling").  The kernel therefore puts the WEIGHT rows on the 128 TMEM lanes (the MMA M
+// (Section 1; figure "Latency Scaling").  The kernel therefore puts the WEIGHT rows on the TMEM lanes (the MMA M
 // dimension) and the activation rows on the MMA N dimension (up to 288 = two instructions
 // of up to 144 columns), so no tensor-core work is wasted on padding rows.
 //
-// Work item = (row block, 128-row weight tile, K split).  Persistent CTAs, one per SM, loop
+// PAIR instances: two CTAs (a cluster) share one MMA of M = 256.  Each holds its own 128-row weight tile and HALF of the
+// activation rows, and gets the accumulator of its own tile, all columns.  What bounds the main loop of many
+// rows is shared memory: for 272 rows a lone CTA reads 66 KB of operands and has 51 KB written to it per 64-wide K
+// block, 916 cycles at 128 B per cycle against 544 cycles of MMAs (measured: 811 - 867); half the activations
+// leaves 49 + 33 KB, 640 cycles.
+// SMALL instances: few rows, see below.
+//
+// Work item = (row block, weight tile or pair of tiles, K split).  Persistent CTAs, one per SM, loop
 // over items.  Warp roles:
-//   warp 0      streams the weight tiles by TMA into a deep ring of shared-memory stages (a
-//               tile comes from HBM and takes > 1 us to arrive);
-//   warp 3      streams the wide activation tiles (from L2) into a ring of three stages;
-//   warp 1      issues the MMAs into one fp32 accumulator in TMEM;
+//   warp 0      streams the weight tiles by TMA into a ring of stages (a tile comes from HBM and takes > 1 us to arrive);
+//   warp 3      streams the activation tiles (from L2) into the same stages;
+//   warp 1      issues the MMAs into one fp32 accumulator in TMEM (even CTA of a pair);
 //   warp 2      watches the stages' mbarriers on behalf of warp 1, which must not touch the
-//               memory pipeline between its MMAs, and releases it through hardware barriers;
+//               memory pipeline between its MMAs, and releases it through hardware barriers (even CTA);
 //   warps 4-11  drain the accumulator into registers (which frees it for the next item at
 //               once) and run the epilogue from registers while the next item's MMAs proceed.
 #pragma once
+#include <algorithm>
+
 #include "common.cuh"
 #include "sm100_ptx.cuh"
-#include <algorithm>
 
 namespace gemm_tc {
 
 constexpr int TILE_N = 128;         // weight rows per tile (TMEM lanes)
 constexpr int TILE_K = 64;          // bf16 elements per 128-byte swizzled row
-constexpr int MAX_ROWS = 288;       // activation rows per row block (2 x 144 TMEM columns)
+constexpr int MAX_ROWS = 288;       // activation rows of a single row block (2 x 144 TMEM columns)
+constexpr int BLOCK_ROWS = 256;     // activation rows per row block when there are several (one instruction)
 constexpr int EPI_WARPS = 8;
 constexpr int ROLE_WARPS = 4;      // warpgroup 0: weight producer, MMA issuer, stage watcher, activation producer
 constexpr int THREADS = 32 * (ROLE_WARPS + EPI_WARPS);
 constexpr int ROLE_REGS = 56, EPI_REGS = 224;   // registers per thread after the split: 128 * 56 + 256 * 224 <= 64 K
 constexpr int W_STAGE_BYTES = TILE_N * TILE_K * 2;
-constexpr int SMEM_BUDGET = 216 * 1024;   // dynamic shared memory for the rings; up to 9 KB of static shared memory come on top
+constexpr int SMEM_BUDGET = 212 * 1024;   // dynamic shared memory for the ring; up to 9 KB of static shared memory come on top
 constexpr int TMEM_COLS = 512;
+constexpr int MAX_STAGES = 12;     // of the ring (hardware barriers 1 .. 12)
 
 // Few rows (SMALL instances: a row block of at most SMALL_ROWS).  Such a launch is bound by streaming its weights, but a
 // good part of its time used to be spent elsewhere:
@@ -49,27 +58,26 @@ constexpr int TMEM_COLS = 512;
 // of the former 11.4 -> 10.3 us, QKV 5.3 -> 3.4 us).  Measured and not kept: fetching weights into L2 ahead of the ring, this
 // launch's or the next projection's (2 - 8 % slower, the more the further ahead).
 constexpr int SMALL_ROWS = 96;
-__host__ __device__ constexpr int k_per_stage(bool small) { return small ? 2 : 1; }     // K blocks of 64 per stage
-constexpr int SMALL_SMEM_BUDGET = 212 * 1024;
-constexpr int MAX_STAGES = 12;      // of the weight ring (hardware barriers 1 .. 12)
 constexpr int SMALL_TMEM_COLS = 128;
+__host__ __device__ constexpr int k_per_stage(bool small) { return small ? 2 : 1; }     // K blocks of 64 per stage
+__host__ __device__ constexpr int tile_rows(bool small) { return small ? TILE_N : 2 * TILE_N; }   // weight rows of an item
 
 // MODE_SAMPLE is MODE_ARGMAX with Gumbel noise added to the tempered logits (a draw per row instead of
 // the argmax); it is a mode of its own so that the greedy LM head carries none of its registers.
 enum Mode { MODE_SLAB = 0, MODE_SWIGLU = 1, MODE_ARGMAX = 2, MODE_SAMPLE = 3 };
 
+// A "tile" below is what an item covers: tile_rows(small) weight rows.
 struct Args {
   int R, N, K;              // activation rows in use, output features, input features
   int rb_rows;              // rows per row block: multiple of 16, 16..288
   int n_rb;                 // row blocks
-  int n_tiles;              // ceil(N / 128)
+  int n_tiles;              // ceil(N / tile rows)
   int S;                    // K splits of the split region
   int fused_items;          // items [0, fused_items) are whole tiles 0.. (no K split) finished by the mode's own epilogue;
                             // the rest are tiles tile_b0.. split S ways along K, written as fp32 slabs
   int tile_b0, n_tiles_b;   // first tile and tile count of the split region
   int kb_total;             // stages of K: K / 64, or half of it (rounded up) in a SMALL launch
-  int w_stages, a_stages;   // depths of the weight ring (<= 8) and of the activation ring (<= w_stages)
-  int box_rows, n_box;      // activation rows per TMA box, boxes per stage
+  int stages;               // depth of the ring (<= MAX_STAGES)
   int n1, n2;               // MMA N of the two instructions (n2 may be 0)
   // MODE_SLAB: out[split][r][n], fp32 or (slab_bf16) bf16; strides in elements
   void *out; long long slab_stride; int ldo; int slab_bf16;
@@ -113,41 +121,44 @@ __device__ __forceinline__ Item decode_item(const Args &g, int item) {
 // the right limit (-0) when exp(-g) overflows.
 __device__ __forceinline__ float silu_mul(float g, float u) { return __fdividef(g, 1.f + __expf(-g)) * u; }
 
+// PAIR: two CTAs share an item (see the head of this file); otherwise SMALL.
 template <int MODE, bool SMALL = false>
 __global__ void __launch_bounds__(THREADS, SMALL ? 2 : 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmA, const Args g, const TlSlot tl) {
+  constexpr bool PAIR = !SMALL;
+  constexpr int KPS = k_per_stage(SMALL);
+  constexpr int NCH = SMALL ? SMALL_ROWS / 32 : 9;         // 16-column chunks of the accumulator per epilogue warp
   extern __shared__ uint8_t smem_raw[];
-  __shared__ __align__(8) uint64_t w_full[MAX_STAGES], w_empty[MAX_STAGES], a_full[MAX_STAGES], a_empty[MAX_STAGES], tmem_full_bar, tmem_empty_bar;
+  __shared__ __align__(8) uint64_t full[MAX_STAGES], empty[MAX_STAGES], tmem_full_bar, tmem_empty_bar;
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
   __shared__ __align__(16) uint16_t epi_stage[MODE == MODE_SWIGLU ? EPI_WARPS : 1][32][16];   // MODE_SWIGLU: two 16-column chunks per epilogue warp, [column][feature]
 
-  constexpr int KPS = k_per_stage(SMALL);
-  constexpr int W_STAGE = KPS * W_STAGE_BYTES;
-  constexpr int NCH = SMALL ? SMALL_ROWS / 32 : 9;         // 16-column chunks of the accumulator per epilogue warp
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = PAIR ? (int)sm100::cluster_rank() : 0;
+  const int worker = PAIR ? blockIdx.x >> 1 : blockIdx.x, n_workers = PAIR ? gridDim.x >> 1 : gridDim.x;
   const uint32_t smem0 = (sm100::smem_u32(smem_raw) + 1023u) & ~1023u;
-  const int a_stage_bytes = KPS * g.rb_rows * TILE_K * 2;           // multiple of 1024 (rb_rows % 16 == 0)
-  const uint32_t smem_a0 = smem0 + (uint32_t)g.w_stages * W_STAGE;   // activation ring behind the weight ring
+  // A stage: KPS weight blocks [128][64], then KPS activation blocks [a_rows][64] (a_rows multiple of 8: whole swizzle atoms).
+  const int a_rows = PAIR ? g.rb_rows >> 1 : g.rb_rows;
+  const uint32_t a_block = (uint32_t)(a_rows * TILE_K * 2);
+  const uint32_t stage_bytes = KPS * (W_STAGE_BYTES + a_block);
   const int n_items = g.total_items();
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
-    for (int s = 0; s < MAX_STAGES; ++s) {
-      sm100::mbar_init(sm100::smem_u32(&w_full[s]), 1); sm100::mbar_init(sm100::smem_u32(&w_empty[s]), 1);
-      sm100::mbar_init(sm100::smem_u32(&a_full[s]), 1); sm100::mbar_init(sm100::smem_u32(&a_empty[s]), 1);
-    }
+    for (int s = 0; s < MAX_STAGES; ++s) { sm100::mbar_init(sm100::smem_u32(&full[s]), 1); sm100::mbar_init(sm100::smem_u32(&empty[s]), 1); }
     sm100::mbar_init(sm100::smem_u32(&tmem_full_bar), 1);
-    sm100::mbar_init(sm100::smem_u32(&tmem_empty_bar), EPI_WARPS);
+    sm100::mbar_init(sm100::smem_u32(&tmem_empty_bar), PAIR ? 2 * EPI_WARPS : EPI_WARPS);
     sm100::fence_mbar_init();
   }
   if (warp == 1) {
     __syncwarp();
-    sm100::tmem_alloc(sm100::smem_u32(&tmem_base_slot), SMALL ? SMALL_TMEM_COLS : TMEM_COLS);
-    sm100::tmem_relinquish();
+    if constexpr (PAIR) { sm100::tmem_alloc_pair(sm100::smem_u32(&tmem_base_slot), TMEM_COLS); sm100::tmem_relinquish_pair(); }
+    else { sm100::tmem_alloc(sm100::smem_u32(&tmem_base_slot), SMALL_TMEM_COLS); sm100::tmem_relinquish(); }
   }
   sm100::tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) sm100::cluster_sync();     // the other CTA's barriers exist
   sm100::tc_fence_after();
   const uint32_t tmem_acc = tmem_base_slot;
   // Only now may the next kernel's CTAs be scheduled: one that got in before this CTA had its tensor memory could take
@@ -164,53 +175,40 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 
   if (warp < ROLE_WARPS) {
   if constexpr (!SMALL) sm100::setmaxnreg_dec<ROLE_REGS>();
-  if (warp == 0) {
-    // ===================== weight producer =====================
+  if (warp == 0 || warp == 3) {
+    // ===================== weight producer (warp 0), activation producer (warp 3) =====================
+    // Both fill the same stages.  A stage's bytes (of both CTAs of a pair) are counted on the even CTA's barrier, where the weight
+    // producer announces them; loads that complete before the announcement are no problem, the phase needs its arrival too.
+    // Weights are never written by a kernel, so their producer does not wait for the previous kernel:
+    // the ring fills while that kernel is still finishing.
     if (lane == 0) {
-      sm100::prefetch_tensormap(&tmW);
-      const uint64_t pol_w = sm100::policy_evict_first();
+      const bool is_w = warp == 0;
+      sm100::prefetch_tensormap(is_w ? &tmW : &tmA);
+      const uint64_t pol = is_w ? sm100::policy_evict_first() : sm100::policy_evict_last();
       int s = 0; uint32_t ph = 0; bool ok = true;
-      // Weights are never written by a kernel, so nothing here waits for the previous kernel:
-      // the ring fills while that kernel is still finishing.
-      for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
+      if (!is_w) {
+        pdl_wait();                      // the activations are the previous kernel's output
+        tl_go(tl);
+      }
+      for (int item = worker; item < n_items && ok; item += n_workers) {
         const Item w = decode_item<MODE>(g, item);
+        const int row = is_w ? (PAIR ? (w.tile * 2 + rank) * TILE_N : w.tile * TILE_N) : w.rb * g.rb_rows + rank * a_rows;
+        const CUtensorMap *tm = is_w ? &tmW : &tmA;
         for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          if (!sm100::mbar_wait(sm100::smem_u32(&w_empty[s]), ph ^ 1u, abortp)) { ok = false; break; }
-          const uint32_t fb = sm100::smem_u32(&w_full[s]);
-          sm100::mbar_expect_tx(fb, (uint32_t)W_STAGE);
-          if constexpr (SMALL) sm100::tma_load_3d(smem0 + (uint32_t)s * W_STAGE, &tmW, fb, 0, w.tile * TILE_N, kb * KPS, pol_w);
-          else sm100::tma_load_2d(smem0 + (uint32_t)s * W_STAGE, &tmW, fb, kb * TILE_K, w.tile * TILE_N, pol_w);
-          if (++s == g.w_stages) { s = 0; ph ^= 1u; }
+          if (!sm100::mbar_wait(sm100::smem_u32(&empty[s]), ph ^ 1u, abortp)) { ok = false; break; }
+          const uint32_t fb = sm100::smem_u32(&full[s]);
+          const uint32_t dst = smem0 + (uint32_t)s * stage_bytes + (is_w ? 0u : (uint32_t)(KPS * W_STAGE_BYTES));
+          if (is_w && rank == 0) sm100::mbar_expect_tx(fb, (PAIR ? 2u : 1u) * stage_bytes);
+          if constexpr (PAIR) sm100::tma_load_2d_pair(dst, tm, sm100::cluster_addr(fb, 0), kb * TILE_K, row, pol);
+          else sm100::tma_load_3d(dst, tm, fb, 0, row, kb * KPS, pol);
+          if (++s == g.stages) { s = 0; ph ^= 1u; }
         }
       }
     }
-  } else if (warp == 3) {
-    // ===================== activation producer =====================
-    if (lane == 0) {
-      sm100::prefetch_tensormap(&tmA);
-      const uint64_t pol_a = sm100::policy_evict_last();
-      int s = 0; uint32_t ph = 0; bool ok = true;
-      pdl_wait();                      // the activations are the previous kernel's output
-      tl_go(tl);
-      for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
-        const Item w = decode_item<MODE>(g, item);
-        for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          if (!sm100::mbar_wait(sm100::smem_u32(&a_empty[s]), ph ^ 1u, abortp)) { ok = false; break; }
-          const uint32_t fb = sm100::smem_u32(&a_full[s]);
-          const uint32_t sa = smem_a0 + (uint32_t)s * a_stage_bytes;
-          sm100::mbar_expect_tx(fb, (uint32_t)a_stage_bytes);
-          if constexpr (SMALL) sm100::tma_load_3d(sa, &tmA, fb, 0, w.rb * g.rb_rows, kb * KPS, pol_a);
-          else
-          for (int b = 0; b < g.n_box; ++b)
-            sm100::tma_load_2d(sa + (uint32_t)(b * g.box_rows * TILE_K * 2), &tmA, fb, kb * TILE_K, w.rb * g.rb_rows + b * g.box_rows, pol_a);
-          if (++s == g.a_stages) { s = 0; ph ^= 1u; }
-        }
-      }
-    }
-  } else if (warp == 1) {
+  } else if (warp == 1 && rank == 0) {
     // ===================== MMA issuer =====================
     // One thread issues every MMA, and it issues them barely faster than the tensor pipe
-    // retires them, so nothing else may sit in its instruction stream: a test of an mbarrier
+    // retires them (59 cycles each, 50 more per commit), so nothing else may sit in its instruction stream: a test of an mbarrier
     // (any access through the memory pipeline) completes only once the MMAs queued before it
     // have gone out, and the pipe runs dry for ~250 cycles per K block.  The watcher warp
     // therefore does the mbarrier waits and releases this warp through one hardware barrier
@@ -221,64 +219,59 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // happens elsewhere, one barrier operation each per K block, so neither can be left
     // waiting for the other; after a failed wait the MMAs read stale tiles, which is harmless,
     // and the status word reports the failure.
-    const uint32_t idesc1 = sm100::make_idesc_bf16(TILE_N, g.n1), idesc2 = sm100::make_idesc_bf16(TILE_N, g.n2 ? g.n2 : 16);
-    const uint64_t wdesc0 = sm100::make_desc_sw128(smem0), adesc0 = sm100::make_desc_sw128(smem_a0);   // stage 0 of each ring
-    const uint64_t wstage16 = (uint64_t)(W_STAGE >> 4), astage16 = (uint64_t)(a_stage_bytes >> 4);
-    const uint64_t a2_off16 = (uint64_t)(g.n1 * 8);
+    constexpr int M = PAIR ? 2 * TILE_N : TILE_N;
+    const uint32_t idesc1 = sm100::make_idesc_bf16(M, g.n1), idesc2 = sm100::make_idesc_bf16(M, g.n2 ? g.n2 : 16);
+    const uint64_t wdesc0 = sm100::make_desc_sw128(smem0), adesc0 = sm100::make_desc_sw128(smem0 + KPS * W_STAGE_BYTES);   // stage 0
+    const uint64_t stage16 = (uint64_t)(stage_bytes >> 4), a_block16 = (uint64_t)(a_block >> 4);
+    const uint64_t a2_off16 = (uint64_t)((PAIR ? g.n1 >> 1 : g.n1) * 8);
     const uint32_t tmem_acc2 = tmem_acc + (uint32_t)g.n1;
     const bool two = g.n2 != 0;
-    int s = 0, sa = 0;
+    auto mma = [](uint32_t d, uint64_t wd, uint64_t ad, uint32_t idesc, uint32_t acc) {
+      if constexpr (PAIR) sm100::mma_bf16_ss_pair(d, wd, ad, idesc, acc); else sm100::mma_bf16_ss(d, wd, ad, idesc, acc);
+    };
+    auto commit = [](uint32_t bar) { if constexpr (PAIR) sm100::mma_commit_pair(bar); else sm100::mma_commit(bar); };
+    int s = 0;
     uint64_t wd = wdesc0, ad = adesc0;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+    for (int item = worker; item < n_items; item += n_workers) {
       const Item w = decode_item<MODE>(g, item);
-      const int kb0 = w.kb0, kb1 = w.kb1;
       uint32_t acc = 0u;                 // the watcher's first release of an item also says that the accumulator is free
-      for (int kb = kb0; kb < kb1; ++kb) {
+      for (int kb = w.kb0; kb < w.kb1; ++kb) {
         sm100::named_bar_sync(1u + (uint32_t)s, 64);
         sm100::tc_fence_after();
         if (lane == 0) {
-          if constexpr (SMALL) {
-            const uint64_t a_kb16 = (uint64_t)(g.rb_rows * 8);         // the stage's second K block, 16-byte units
-#pragma unroll
-            for (int kk = 0; kk < KPS * TILE_K / 16; ++kk) {
-              sm100::mma_bf16_ss(tmem_acc, wd + (kk / 4) * (W_STAGE_BYTES >> 4) + 2 * (kk % 4), ad + (kk / 4) * a_kb16 + 2 * (kk % 4), idesc1, acc);
-              acc = 1u;
-            }
-          } else if (two) {
+          if (PAIR && two) {
             const uint64_t ad2 = ad + a2_off16;
 #pragma unroll
             for (int kk = 0; kk < TILE_K / 16; ++kk) {
-              sm100::mma_bf16_ss(tmem_acc, wd + 2 * kk, ad + 2 * kk, idesc1, acc);
-              sm100::mma_bf16_ss(tmem_acc2, wd + 2 * kk, ad2 + 2 * kk, idesc2, acc);
+              mma(tmem_acc, wd + 2 * kk, ad + 2 * kk, idesc1, acc);
+              mma(tmem_acc2, wd + 2 * kk, ad2 + 2 * kk, idesc2, acc);
               acc = 1u;
             }
           } else {
 #pragma unroll
-            for (int kk = 0; kk < TILE_K / 16; ++kk) {
-              sm100::mma_bf16_ss(tmem_acc, wd + 2 * kk, ad + 2 * kk, idesc1, acc);
+            for (int kk = 0; kk < KPS * TILE_K / 16; ++kk) {
+              mma(tmem_acc, wd + (kk / 4) * (W_STAGE_BYTES >> 4) + 2 * (kk % 4), ad + (kk / 4) * a_block16 + 2 * (kk % 4), idesc1, acc);
               acc = 1u;
             }
           }
-          sm100::mma_commit(sm100::smem_u32(&w_empty[s]));       // both stages reusable once these MMAs have read them
-          sm100::mma_commit(sm100::smem_u32(&a_empty[sa]));
+          commit(sm100::smem_u32(&empty[s]));       // the stage is reusable once these MMAs have read it
         }
         __syncwarp();
-        wd += wstage16; ad += astage16;
-        if (++s == g.w_stages) { s = 0; wd = wdesc0; }
-        if (++sa == g.a_stages) { sa = 0; ad = adesc0; }
+        wd += stage16; ad += stage16;
+        if (++s == g.stages) { s = 0; wd = wdesc0; ad = adesc0; }
       }
-      if (lane == 0) sm100::mma_commit(sm100::smem_u32(&tmem_full_bar));
+      if (lane == 0) commit(sm100::smem_u32(&tmem_full_bar));
       __syncwarp();
     }
-  } else if (warp == 2) {
+  } else if (warp == 2 && rank == 0) {
     // ===================== stage watcher =====================
     // Waits (bounded) for the accumulator to be drained and for each stage's loads to land,
     // then arrives on the stage's hardware barrier.  A stage's barrier cannot be arrived on
     // twice before the MMA warp has passed it: the second landing needs the producer's refill,
     // which needs the MMA warp's commit for the first.  After a failed wait that argument no
     // longer holds, so from then on the watcher meets the MMA warp at every barrier instead.
-    int s = 0, sa = 0; uint32_t ph = 0, pha = 0, it = 0; bool failed = false;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++it) {
+    int s = 0; uint32_t ph = 0, it = 0; bool failed = false;
+    for (int item = worker; item < n_items; item += n_workers, ++it) {
       const Item w = decode_item<MODE>(g, item);
       if (!failed) {
         bool ok = true;
@@ -288,13 +281,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       for (int kb = w.kb0; kb < w.kb1; ++kb) {
         if (!failed) {
           bool ok = true;
-          if (lane == 0) ok = sm100::mbar_wait(sm100::smem_u32(&w_full[s]), ph, abortp) && sm100::mbar_wait(sm100::smem_u32(&a_full[sa]), pha, abortp);
+          if (lane == 0) ok = sm100::mbar_wait(sm100::smem_u32(&full[s]), ph, abortp);
           failed = !__shfl_sync(0xffffffffu, ok, 0);
         }
         if (!failed) sm100::named_bar_arrive(1u + (uint32_t)s, 64);
         else sm100::named_bar_sync(1u + (uint32_t)s, 64);
-        if (++s == g.w_stages) { s = 0; ph ^= 1u; }
-        if (++sa == g.a_stages) { sa = 0; pha ^= 1u; }
+        if (++s == g.stages) { s = 0; ph ^= 1u; }
       }
     }
   }
@@ -308,6 +300,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     const int c_begin = half ? hc : 0;
     const int c_end = half ? g.rb_rows : (hc < g.rb_rows ? hc : g.rb_rows);
     const int ncols = c_end - c_begin;           // multiple of 16, <= 144
+    // Row of the block that accumulator column c (a multiple of 8, or any column of its group of 8) belongs to.  With two instructions over
+    // a pair, the first takes the first n1 / 2 of each CTA's rows and the second the rest.
+    const int h1 = g.n1 >> 1, h2 = g.n2 >> 1;
+    auto col_row = [&](int c) {
+      if (!PAIR || h2 == 0) return c;
+      return c < h1 ? c : c < 2 * h1 ? c + h2 : c < 2 * h1 + h2 ? c - h1 : c;
+    };
+    const uint32_t drained_bar = PAIR ? sm100::cluster_addr(sm100::smem_u32(&tmem_empty_bar), 0) : sm100::smem_u32(&tmem_empty_bar);
+    auto drained = [&]() {                       // the accumulator may be overwritten
+      sm100::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) { if constexpr (PAIR) sm100::mbar_arrive_cluster(drained_bar); else sm100::mbar_arrive(drained_bar); }
+    };
     uint32_t it = 0; bool ok = true;
     // MODE_ARGMAX: running best of column c_begin + 32*slot + lane, and the row block it belongs to
     float best_v[5]; int best_i[5]; int cur_rb = -1;
@@ -318,7 +323,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 #pragma unroll
       for (int k = 0; k < 5; ++k) {
         const int cidx = k * 32 + lane;
-        const int r = cur_rb * g.rb_rows + c_begin + cidx;
+        const int r = cur_rb * g.rb_rows + col_row(c_begin + cidx);
         if (cidx < ncols && r < g.R) {
           const long long o = (long long)r * g.cand_ld + (blockIdx.x * 4 + q);
           g.cand_val[o] = best_v[k]; g.cand_idx[o] = best_i[k] == 0x7fffffff ? -1 : best_i[k];
@@ -334,12 +339,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // row with one 16-byte store: 2-byte stores from each lane took 18 us per tile.
     // All exchanges first, then sixteen independent silu chains (one chain at a time is bound by
     // instruction latency: 16 us per tile instead of 2), then the turn through shared memory.
-    // c0 / c1: the two chunks (c1 only if second); row0: output row of c0's first column.
-    auto swiglu_pass = [&](const uint32_t (&c0)[16], const uint32_t (&c1)[16], bool second, int row0, int R_live, int tile) {
+    // c0 / c1: the two chunks (c1 only if second); col0: accumulator column of c0's first; row_block: first row of the block;
+    // n0: first weight row of the tile.
+    auto swiglu_pass = [&](const uint32_t (&c0)[16], const uint32_t (&c1)[16], bool second, int col0, int row_block, int R_live, int n0) {
       const bool odd = lane & 1;
       uint16_t (*stage)[16] = epi_stage[MODE == MODE_SWIGLU ? warp - ROLE_WARPS : 0];
       const int srow = lane >> 1, sf = (lane & 1) * 8;
-      const int f0 = ((tile * TILE_N + q * 32) >> 1) + sf;          // first of this lane's 8 features
+      const int f0 = ((n0 + q * 32) >> 1) + sf;          // first of this lane's 8 features
       const int n_feat = g.N >> 1;
       float h[2][8];
 #pragma unroll
@@ -367,7 +373,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       for (int c = 0; c < 2; ++c)
         if (c == 0 || second) {
           const uint4 packed = *reinterpret_cast<const uint4 *>(&stage[c * 16 + srow][sf]);
-          const int r = row0 + c * 16 + srow;
+          const int r = row_block + col_row(col0 + c * 16 + srow);
           if (r < R_live) {
             bf16 *dst = g.H + (long long)r * g.ldh + f0;
             if (f0 + 8 <= n_feat && (g.ldh & 7) == 0) {
@@ -391,15 +397,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // stays in tensor memory and a loop of a few hundred instructions takes 32 columns per round (the
     // 1.5B-class gate/up projection, one item per CTA, ends 4 us earlier than with the long code).  With few rows
     // every fused item goes that way: it is one or two rounds.
-    bool dry = (MODE == MODE_SWIGLU) && !SMALL && g.warm_epilogue != 0 && (int)(blockIdx.x + gridDim.x) < n_items;
-    for (int item = blockIdx.x; item < n_items && ok;) {
+    bool dry = (MODE == MODE_SWIGLU) && !SMALL && g.warm_epilogue != 0 && worker + n_workers < n_items;
+    for (int item = worker; item < n_items && ok;) {
       const Item w = decode_item<MODE>(g, item);
-      const int split = w.split, tile = w.tile, rb = w.rb;
-      if (MODE == MODE_SWIGLU && w.fused && (SMALL || item + (int)gridDim.x >= n_items)) {
+      const int split = w.split, rb = w.rb, row_block = rb * g.rb_rows;
+      const int n0 = (PAIR ? w.tile * 2 + rank : w.tile) * TILE_N;      // first weight row of this CTA's tile
+      if (MODE == MODE_SWIGLU && w.fused && (SMALL || item + n_workers >= n_items)) {
         if (!sm100::mbar_wait(sm100::smem_u32(&tmem_full_bar), it & 1u, abortp)) { ok = false; break; }
         sm100::tc_fence_after();
         const uint32_t t0 = tmem_acc + ((uint32_t)(q * 32) << 16) + (uint32_t)c_begin;
-        const int row_first = rb * g.rb_rows + c_begin;
 #pragma unroll 1
         for (int cc = 0; cc < ncols; cc += 32) {
           uint32_t c0[16], c1[16];
@@ -407,12 +413,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           sm100::tmem_ld16(t0 + cc, c0);
           if (second) sm100::tmem_ld16(t0 + cc + 16, c1);
           sm100::tmem_wait_ld();
-          swiglu_pass(c0, c1, second, row_first + cc, g.R, tile);
+          swiglu_pass(c0, c1, second, c_begin + cc, row_block, g.R, n0);
         }
-        sm100::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) sm100::mbar_arrive(sm100::smem_u32(&tmem_empty_bar));
-        item += gridDim.x; ++it;
+        drained();
+        item += n_workers; ++it;
         continue;
       }
       uint32_t v[NCH][16];
@@ -424,31 +428,33 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         for (int i = 0; i < NCH; ++i)
           if (i * 16 < ncols) sm100::tmem_ld16(t0 + i * 16, v[i]);
         sm100::tmem_wait_ld();
-        sm100::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) sm100::mbar_arrive(sm100::smem_u32(&tmem_empty_bar));   // accumulator free for the next item
+        drained();                                       // accumulator free for the next item
       }                                                  // (dry: v holds whatever the registers held; nothing of it is stored)
       const int R_live = dry ? 0 : g.R;                  // rows this walk may store
 
-      const int n = tile * TILE_N + q * 32 + lane;       // this thread's output feature
-      const int r_base = rb * g.rb_rows + c_begin;
+      const int n = n0 + q * 32 + lane;                  // this thread's output feature
       if (MODE == MODE_SLAB || !w.fused) {
         // split-K partial sums; columns are counted from the first tile of the split region
-        const int nc = n - g.tile_b0 * TILE_N;
+        const int nc = n - g.tile_b0 * tile_rows(SMALL);
         const bool n_ok = n < g.N;
         if (!g.slab_bf16) {
-          // One running pointer and a bound counted from this thread's first row: with the address
+          // One running pointer and a bound counted from the first row of eight: with the address
           // and the row test recomputed per store (r * ldo, r < R) the same 144 stores take 1.65 times
           // as long (19.5 instead of 32 bytes per cycle and SM, the rate the L2 takes stores at).
-          float *p = reinterpret_cast<float *>(g.out) + (long long)split * g.slab_stride + nc + (long long)r_base * g.ldo;
-          const int rows_left = n_ok ? R_live - r_base : 0;
+          float *out = reinterpret_cast<float *>(g.out) + (long long)split * g.slab_stride + nc;
 #pragma unroll
           for (int i = 0; i < NCH; ++i) {
             if (i * 16 < ncols) {
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                if (i * 16 + j < rows_left) *p = __uint_as_float(v[i][j]);
-                p += g.ldo;
+              for (int h = 0; h < 2; ++h) {
+                const int r0 = row_block + col_row(c_begin + i * 16 + h * 8);
+                float *p = out + (long long)r0 * g.ldo;
+                const int rows_left = n_ok ? R_live - r0 : 0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  if (j < rows_left) *p = __uint_as_float(v[i][h * 8 + j]);
+                  p += g.ldo;
+                }
               }
             }
           }
@@ -466,7 +472,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
                 const uint32_t recv = __shfl_xor_sync(0xffffffffu, send, 1);
                 const float lo = __uint_as_float(odd ? recv : v[i][j]);          // feature n & ~1
                 const float hi = __uint_as_float(odd ? v[i][j + 1] : recv);      // feature n | 1
-                const int r = r_base + i * 16 + j + (odd ? 1 : 0);
+                const int r = row_block + col_row(c_begin + i * 16 + j) + (odd ? 1 : 0);
                 if (n_ok && r < R_live) {
                   __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
                   *reinterpret_cast<__nv_bfloat162 *>(o + (long long)r * g.ldo) = h2;
@@ -481,7 +487,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         for (int ip = 0; ip < (NCH + 1) / 2; ++ip) {
           if (ip * 32 < ncols) {
             const bool second = (2 * ip + 1) < NCH && (2 * ip + 1) * 16 < ncols;    // warp-uniform
-            swiglu_pass(v[2 * ip], v[(2 * ip + 1) < NCH ? 2 * ip + 1 : NCH - 1], second, r_base + ip * 32, R_live, tile);
+            swiglu_pass(v[2 * ip], v[(2 * ip + 1) < NCH ? 2 * ip + 1 : NCH - 1], second, c_begin + ip * 32, row_block, R_live, n0);
           }
         }
       } else if (MODE == MODE_ARGMAX || MODE == MODE_SAMPLE) {
@@ -500,7 +506,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
             if (i * 16 < ncols) {
 #pragma unroll
               for (int j = 0; j < 16; ++j) {
-                const int r = r_base + i * 16 + j;
+                const int r = row_block + col_row(c_begin + i * 16 + j);
                 if (r < g.R) g.dump[(long long)r * g.ld_dump + n] = __uint_as_float(v[i][j]);
               }
             }
@@ -514,7 +520,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
               const int i = grp * 2 + (j >> 4);
               float x = (i < NCH && i * 16 < ncols) ? __uint_as_float(v[i < NCH ? i : NCH - 1][j & 15]) : -INFINITY;
               if (MODE == MODE_SAMPLE) {
-                const int r = r_base + grp * 32 + j;
+                const int r = row_block + col_row(c_begin + grp * 32 + j);
                 if (r < g.R && n_ok) x = x * g.inv_temp + gumbel_noise(g.skey[r], (uint32_t)my_idx);
               }
               const bool ok_v = n_ok && (x == x);
@@ -541,7 +547,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         }
       }
       if (dry) dry = false;                              // the same item again, for real
-      else { item += gridDim.x; ++it; }
+      else { item += n_workers; ++it; }
     }
     if (MODE == MODE_ARGMAX || MODE == MODE_SAMPLE) flush_best();
   }
@@ -556,10 +562,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
     __syncthreads();
   }
+  if constexpr (PAIR) sm100::cluster_sync();     // nothing of the other CTA refers to this one any more
   if (warp == 1) {
     __syncwarp();
     sm100::tc_fence_after();
-    sm100::tmem_dealloc(tmem_acc, SMALL ? SMALL_TMEM_COLS : TMEM_COLS);
+    if constexpr (PAIR) sm100::tmem_dealloc_pair(tmem_acc, TMEM_COLS); else sm100::tmem_dealloc(tmem_acc, SMALL_TMEM_COLS);
   }
   if (threadIdx.x == 0) tl_end(tl);
 }
@@ -593,31 +600,22 @@ inline CUresult encode_2d_small(EncodeTiledFn fn, CUtensorMap *tm, const void *b
 
 // Row-block geometry for R activation rows.
 inline void plan_rows(int R, Args &a, int max_rows = MAX_ROWS) {
-  a.n_rb = (R + max_rows - 1) / max_rows;
+  a.n_rb = R <= max_rows ? 1 : (R + BLOCK_ROWS - 1) / BLOCK_ROWS;
+  if (max_rows < BLOCK_ROWS) a.n_rb = (R + max_rows - 1) / max_rows;
   const int per = (R + a.n_rb - 1) / a.n_rb;
   a.rb_rows = (per + 15) / 16 * 16;
-  if (a.rb_rows <= 256) { a.box_rows = a.rb_rows; a.n_box = 1; a.n1 = a.rb_rows; a.n2 = 0; }
-  else { a.box_rows = a.rb_rows / 2; a.n_box = 2; a.n1 = ((a.rb_rows / 2 + 15) / 16) * 16; a.n2 = a.rb_rows - a.n1; }
-  // Three activation stages keep that ring a K block ahead of the MMAs; the weight ring gets
-  // the rest of the budget.  Small row blocks get equally deep rings.
-  const int a_stage = a.rb_rows * TILE_K * 2;
-  a.a_stages = 3;
-  a.w_stages = (SMEM_BUDGET - a.a_stages * a_stage) / W_STAGE_BYTES;
-  if (a.w_stages > 8) a.w_stages = 8;
-  if (a.w_stages < 3) a.w_stages = 3;
-  while (a.a_stages < a.w_stages && (a.a_stages + 1) * a_stage + a.w_stages * W_STAGE_BYTES <= SMEM_BUDGET) a.a_stages++;
+  a.n1 = a.rb_rows; a.n2 = 0;
+  if (a.rb_rows > 256) { a.n1 = ((a.rb_rows / 2 + 15) / 16) * 16; a.n2 = a.rb_rows - a.n1; }
 }
-// Ring depths of a SMALL launch whose CTAs read n stages each: no more than n (the next projection's CTA may then sit
-// on the same SM), at most five of the weights (24 MB in flight over the machine; the 8B-class step of 20 rows takes
-// 4.0 ms with five, 4.05 with four, 4.5 with two and a half).
-inline void plan_stages_small(Args &a, int n) {
-  const int kps = k_per_stage(true), a_stage = kps * a.rb_rows * TILE_K * 2;
-  a.a_stages = std::max(2, std::min(4, n));
-  a.w_stages = std::max(2, std::min({5, (SMALL_SMEM_BUDGET - a.a_stages * a_stage) / (kps * W_STAGE_BYTES), n}));
+inline int stage_bytes(const Args &a, bool small) { return k_per_stage(small) * (W_STAGE_BYTES + (small ? a.rb_rows : a.rb_rows / 2) * TILE_K * 2); }
+// Depth of the ring of a launch whose CTAs read n stages each.  A SMALL launch takes no more than n (the next projection's
+// CTA may then sit on the same SM) and at most five (24 MB of weights in flight over the machine; the 8B-class step of
+// 20 rows takes 4.0 ms with five, 4.05 with four, 4.5 with two and a half).
+inline void plan_stages(Args &a, int n, bool small) {
+  const int fit = SMEM_BUDGET / stage_bytes(a, small);
+  a.stages = small ? std::max(2, std::min({5, fit, n})) : std::min(fit, MAX_STAGES);
 }
-inline size_t smem_bytes(const Args &a, bool small) {
-  return (size_t)k_per_stage(small) * ((size_t)a.w_stages * W_STAGE_BYTES + (size_t)a.a_stages * (a.rb_rows * TILE_K * 2)) + 1024;
-}
+inline size_t smem_bytes(const Args &a, bool small) { return (size_t)a.stages * stage_bytes(a, small) + 1024; }
 
 // K splits: fill the SMs with whole waves of equally sized items, keeping at least
 // min_kb K blocks per item.

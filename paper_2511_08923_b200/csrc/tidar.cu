@@ -249,14 +249,20 @@ void layout(tidar_ctx &x, void *arena, size_t *bytes) {
 // kernels fit beside one another: all ask for the same split of the SM's memory (an SM changes its split only when it is
 // empty; see init_tensor_core_path).
 template <typename... KP, typename... AP>
-inline void launch_pdl(void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, AP &&...args) {
+inline void launch_pdl_cluster(unsigned cluster, void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, AP &&...args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at; cfg.numAttrs = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = cluster > 1 ? 2 : 1;
   cudaLaunchKernelEx(&cfg, kernel, KP(std::forward<AP>(args))...);
+}
+template <typename... KP, typename... AP>
+inline void launch_pdl(void (*kernel)(KP...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, AP &&...args) {
+  launch_pdl_cluster(1, kernel, grid, block, smem, st, std::forward<AP>(args)...);
 }
 
 // ---- launch bookkeeping -----------------------------------------------------
@@ -322,6 +328,11 @@ const CUtensorMap *act_map(tidar_ctx *c, const void *p, int rows, int cols, int 
 }
 
 // Whether a projection runs as a SMALL instance (the LM head's argmax epilogue needs the registers of the full one).
+// CTAs of the LM head, each of which leaves four candidates per row (with several row blocks it may meet only some of the rows).
+int lm_head_ctas(const tidar_ctx *c, int R, int vocab) {
+  const int pairs = c->n_sms / 2, tiles = (vocab + gemm_tc::tile_rows(false) - 1) / gemm_tc::tile_rows(false);
+  return 2 * (R <= gemm_tc::MAX_ROWS ? std::min(tiles, pairs) : pairs);
+}
 bool small_gemm(int mode, int R) { return R <= gemm_tc::SMALL_ROWS && (mode == gemm_tc::MODE_SLAB || mode == gemm_tc::MODE_SWIGLU); }
 
 // Work of a tensor-core projection of R rows: row blocks, K splits, which tiles finish in the fused epilogue.
@@ -329,27 +340,27 @@ gemm_tc::Args plan_gemm(const tidar_ctx *c, int mode, int R, int N, int K, int f
   gemm_tc::Args a{};
   a.R = R; a.N = N; a.K = K;
   gemm_tc::plan_rows(R, a);
-  a.n_tiles = (N + gemm_tc::TILE_N - 1) / gemm_tc::TILE_N;
   const bool small = small_gemm(mode, R);
-  const int kps = gemm_tc::k_per_stage(small);
+  const int kps = gemm_tc::k_per_stage(small), tile = gemm_tc::tile_rows(small);
+  const int workers = small ? c->n_sms : c->n_sms / 2;             // CTAs, or pairs of CTAs, that work on items
+  a.n_tiles = (N + tile - 1) / tile;
   a.kb_total = (K / gemm_tc::TILE_K + kps - 1) / kps;
   a.S = 1; a.fused_items = 0; a.tile_b0 = 0; a.n_tiles_b = 0;
   if (mode == gemm_tc::MODE_SLAB) {
     a.n_tiles_b = a.n_tiles;
-    a.S = force_S > 0 ? std::min(force_S, a.kb_total) : gemm_tc::plan_splits(a.n_rb * a.n_tiles, a.kb_total, c->n_sms, c->S_max, 4 / kps, 3.0 / kps);
+    a.S = force_S > 0 ? std::min(force_S, a.kb_total) : gemm_tc::plan_splits(a.n_rb * a.n_tiles, a.kb_total, workers, c->S_max, 4 / kps, 3.0 / kps);
     // One row block of up to 288 rows, or two of half the rows?  Two halves fetch every weight tile
-    // twice (the second time from L2: ~0.37 instead of 0.46 us per K block of an item, but twice as
-    // many K blocks per item once the SMs are full), while a CTA's slab store, which its SM cannot
+    // twice (the second time from L2), while a CTA's slab store, which its SM cannot
     // push out faster than ~42 GB/s, shrinks from 3.3 to 1.7 us and fewer slabs are left for the
-    // consumer.  Halves win when an item has few K blocks (the 1.5B-class shapes: step -6.5 %), one
-    // block when it has many (the 8B-class shapes: halves cost +4 %).
+    // consumer.  Halves win when an item has few K blocks (the 1.5B-class shapes), one
+    // block when it has many (the 8B-class shapes).
     if (force_S <= 0 && a.n_rb == 1 && R > gemm_tc::MAX_ROWS / 2) {
       gemm_tc::Args h = a;
       gemm_tc::plan_rows(R, h, gemm_tc::MAX_ROWS / 2);
-      h.S = gemm_tc::plan_splits(h.n_rb * h.n_tiles, h.kb_total, c->n_sms, c->S_max, 4);
+      h.S = gemm_tc::plan_splits(h.n_rb * h.n_tiles, h.kb_total, workers, c->S_max, 4);
       auto cost = [&](const gemm_tc::Args &x, double us_per_kb, double us_store) {
         const long long items = (long long)x.n_rb * x.n_tiles * x.S;
-        const long long waves = (items + c->n_sms - 1) / c->n_sms;
+        const long long waves = (items + workers - 1) / workers;
         return waves * ((x.kb_total + x.S - 1) / x.S * us_per_kb + 1.5) + us_store + 0.5 * x.S;
       };
       if (cost(h, 0.37, 1.7) < cost(a, 0.46, 3.3)) a = h;
@@ -361,13 +372,13 @@ gemm_tc::Args plan_gemm(const tidar_ctx *c, int mode, int R, int N, int K, int f
     // more tiles than SMs: whole waves of tiles finish in the fused epilogue; the tiles of the
     // last, partial wave are split along K so that they also fill the machine, and are finished
     // from fp32 slabs by swiglu_slab_kernel
-    if (a.n_rb == 1 && a.n_tiles > c->n_sms && a.n_tiles % c->n_sms) {
-      const int full = a.n_tiles / c->n_sms * c->n_sms;
+    if (a.n_rb == 1 && a.n_tiles > workers && a.n_tiles % workers) {
+      const int full = a.n_tiles / workers * workers;
       const int rem = a.n_tiles - full;
-      const int S2 = std::min({c->n_sms / rem, a.kb_total * kps / 4, c->S_max});
-      if (S2 >= 2 && (size_t)S2 * R * rem * gemm_tc::TILE_N <= c->partials_cap) {
+      const int S2 = std::min({workers / rem, a.kb_total * kps / 4, c->S_max});
+      if (S2 >= 2 && (size_t)S2 * R * rem * tile <= c->partials_cap) {
         a.fused_items = full; a.tile_b0 = full; a.n_tiles_b = rem; a.S = S2;
-        a.ldo = rem * gemm_tc::TILE_N; a.slab_stride = (long long)R * a.ldo;
+        a.ldo = rem * tile; a.slab_stride = (long long)R * a.ldo;
       }
     }
   } else {
@@ -392,38 +403,39 @@ int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const tida
     a.H = c->H;
     a.out = c->partials; a.slab_bf16 = c->slab_bf16 ? 1 : 0;
   } else {
-    a.cand_val = c->cand_val; a.cand_idx = c->cand_idx; a.cand_ld = (a.n_rb == 1 ? std::min(a.fused_items, c->n_sms) : c->n_sms) * 4; a.dump = c->dbg_logits; a.ld_dump = c->cfg.vocab; a.col0 = 0;
+    a.cand_val = c->cand_val; a.cand_idx = c->cand_idx; a.cand_ld = lm_head_ctas(c, R, N) * 4; a.dump = c->dbg_logits; a.ld_dump = c->cfg.vocab; a.col0 = 0;
     a.inv_temp = c->cfg.temperature > 0.f ? 1.0f / c->cfg.temperature : 0.f; a.skey = c->meta.skey + c->head_row0;
   }
   a.status = c->d_status;
   a.warm_epilogue = mode == gemm_tc::MODE_SWIGLU ? 1 : 0;
-  const CUtensorMap *tmA = act_map(c, A, a_rows, K, a.box_rows, small);
-  if (!tmA) return fail(c, TIDAR_ECUDA, "cuTensorMapEncodeTiled failed for an activation matrix (%d x %d, box %d)", a_rows, K, a.box_rows);
+  const int box = small ? a.rb_rows : a.rb_rows / 2;
+  const CUtensorMap *tmA = act_map(c, A, a_rows, K, box, small);
+  if (!tmA) return fail(c, TIDAR_ECUDA, "cuTensorMapEncodeTiled failed for an activation matrix (%d x %d, box %d)", a_rows, K, box);
   const int items = a.total_items();
-  const int grid = std::min(items, c->n_sms);
-  if (small) {
-    int kb = 0;
-    for (int i = 0; i < items; i += grid) kb += i < a.fused_items ? a.kb_total : (a.kb_total + a.S - 1) / a.S;
-    gemm_tc::plan_stages_small(a, kb);
+  const int workers = std::min(items, small ? c->n_sms : c->n_sms / 2), grid = small ? workers : 2 * workers;
+  {
+    int n = 0;                                   // stages the first worker's items have
+    for (int i = 0; i < items; i += workers) n += i < a.fused_items ? a.kb_total : (a.kb_total + a.S - 1) / a.S;
+    gemm_tc::plan_stages(a, n, small);
   }
   const size_t smem = gemm_tc::smem_bytes(a, small);
   Launch l(c, cls);
   if (small && mode == gemm_tc::MODE_SLAB) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB, true>, grid, gemm_tc::THREADS, smem, c->stream, tmW.small, *tmA, a, l.tl);
   else if (small) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU, true>, grid, gemm_tc::THREADS, smem, c->stream, tmW.small, *tmA, a, l.tl);
-  else if (mode == gemm_tc::MODE_SLAB) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
-  else if (mode == gemm_tc::MODE_SWIGLU) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
-  else if (a.inv_temp > 0.f) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SAMPLE>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
-  else launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_ARGMAX>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
+  else if (mode == gemm_tc::MODE_SLAB) launch_pdl_cluster(2, gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
+  else if (mode == gemm_tc::MODE_SWIGLU) launch_pdl_cluster(2, gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
+  else if (a.inv_temp > 0.f) launch_pdl_cluster(2, gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SAMPLE>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
+  else launch_pdl_cluster(2, gemm_tc::gemm_tc_kernel<gemm_tc::MODE_ARGMAX>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
   if (rem_tiles) {
-    const int nf = (N - a.tile_b0 * gemm_tc::TILE_N) / 2;          // features of the split tiles
+    const int f0 = a.tile_b0 * gemm_tc::tile_rows(small) / 2, nf = N / 2 - f0;          // features of the split tiles
     const size_t n = (size_t)R * nf;
     Launch lf(c, cls);
     if (c->slab_bf16)
       launch_pdl(swiglu_slab_kernel<bf16>, (unsigned)((n / 2 + 255) / 256), 256, 0, c->stream, (const bf16 *)c->partials, a.S, (size_t)a.slab_stride, R, a.ldo, nf,
-                                                                           a.tile_b0 * gemm_tc::TILE_N / 2, a.ldh, c->H, lf.tl);
+                                                                           f0, a.ldh, c->H, lf.tl);
     else
       launch_pdl(swiglu_slab_kernel<float>, (unsigned)((n / 2 + 255) / 256), 256, 0, c->stream, (const float *)c->partials, a.S, (size_t)a.slab_stride, R, a.ldo, nf,
-                                                                           a.tile_b0 * gemm_tc::TILE_N / 2, a.ldh, c->H, lf.tl);
+                                                                           f0, a.ldh, c->H, lf.tl);
   }
   if (S_out) *S_out = a.S;
   if (stride_out) *stride_out = (size_t)R * N;
@@ -645,7 +657,7 @@ if (tc && c->slab_bf16)
   if (with_head && tc) {
     // with one row block every CTA leaves a candidate for every row; with several it may meet only some of them
     const bool one_block = Rh <= gemm_tc::MAX_ROWS;
-    const int G = (one_block ? std::min((cf.vocab + gemm_tc::TILE_N - 1) / gemm_tc::TILE_N, c->n_sms) : c->n_sms) * 4;
+    const int G = lm_head_ctas(c, Rh, cf.vocab) * 4;
     if (!one_block) CUDA_TRY(c, cudaMemsetAsync(c->cand_idx, 0xff, (size_t)G * Rh * sizeof(int32_t), c->stream));
     if ((rc = gemm_tc_launch(c, gemm_tc::MODE_ARGMAX, Ah, RA - head_row0, c->tm_lm, Rh, cf.vocab, d, TIDAR_TC_LMHEAD, nullptr, nullptr))) return rc;
     Launch ll(c, TIDAR_TC_LMHEAD);
@@ -720,9 +732,9 @@ int init_tensor_core_path(tidar_ctx *c) {
     for (const void *f : kernels) CUDA_TRY(c, max_smem_split(f));
     for (int i = 3; i < 11; ++i) CUDA_TRY(c, cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, NORM_SMEM));
   }
-  const int max_smem = gemm_tc::SMEM_BUDGET + 1024, small_smem = gemm_tc::SMALL_SMEM_BUDGET + 1024;
-  CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, small_smem));
-  CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, small_smem));
+  const int max_smem = gemm_tc::SMEM_BUDGET + 1024;
+  CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
+  CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU, true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
