@@ -134,7 +134,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   __shared__ int abort_flag;
   __shared__ __align__(16) uint16_t epi_stage[MODE == MODE_SWIGLU ? EPI_WARPS : 1][32][16];   // MODE_SWIGLU: two 16-column chunks per epilogue warp, [column][feature]
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = sm100::warp_index(), lane = threadIdx.x & 31;
   const int rank = PAIR ? (int)sm100::cluster_rank() : 0;
   const int worker = PAIR ? blockIdx.x >> 1 : blockIdx.x, n_workers = PAIR ? gridDim.x >> 1 : gridDim.x;
   const uint32_t smem0 = (sm100::smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -181,34 +181,38 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // producer announces them; loads that complete before the announcement are no problem, the phase needs its arrival too.
     // Weights are never written by a kernel, so their producer does not wait for the previous kernel:
     // the ring fills while that kernel is still finishing.
-    if (lane == 0) {
-      const bool is_w = warp == 0;
-      sm100::prefetch_tensormap(is_w ? &tmW : &tmA);
-      const uint64_t pol = is_w ? sm100::policy_evict_first() : sm100::policy_evict_last();
-      int s = 0; uint32_t ph = 0; bool ok = true;
-      if (!is_w) {
-        pdl_wait();                      // the activations are the previous kernel's output
-        tl_go(tl);
-      }
-      for (int item = worker; item < n_items && ok; item += n_workers) {
-        const Item w = decode_item<MODE>(g, item);
-        const int row = is_w ? (PAIR ? (w.tile * 2 + rank) * TILE_N : w.tile * TILE_N) : w.rb * g.rb_rows + rank * a_rows;
-        const CUtensorMap *tm = is_w ? &tmW : &tmA;
-        for (int kb = w.kb0; kb < w.kb1; ++kb) {
-          if (!sm100::mbar_wait(sm100::smem_u32(&empty[s]), ph ^ 1u, abortp)) { ok = false; break; }
+    // (The whole warp walks the schedule and one elected lane issues: see the MMA issuer.)
+    const bool is_w = warp == 0;
+    const CUtensorMap *tm = is_w ? &tmW : &tmA;
+    if (lane == 0) sm100::prefetch_tensormap(tm);
+    const uint64_t pol = is_w ? sm100::policy_evict_first() : sm100::policy_evict_last();
+    int s = 0; uint32_t ph = 0; bool ok = true;
+    if (!is_w) {
+      pdl_wait();                      // the activations are the previous kernel's output
+      if (lane == 0) tl_go(tl);
+    }
+    for (int item = worker; item < n_items && ok; item += n_workers) {
+      const Item w = decode_item<MODE>(g, item);
+      const int row = is_w ? (PAIR ? (w.tile * 2 + rank) * TILE_N : w.tile * TILE_N) : w.rb * g.rb_rows + rank * a_rows;
+      for (int kb = w.kb0; kb < w.kb1; ++kb) {
+        if (!__all_sync(0xffffffffu, sm100::mbar_wait(sm100::smem_u32(&empty[s]), ph ^ 1u, abortp))) { ok = false; break; }
+        if (sm100::elect_one()) {
           const uint32_t fb = sm100::smem_u32(&full[s]);
           const uint32_t dst = smem0 + (uint32_t)s * stage_bytes + (is_w ? 0u : (uint32_t)(KPS * W_STAGE_BYTES));
           if (is_w && rank == 0) sm100::mbar_expect_tx(fb, (PAIR ? 2u : 1u) * stage_bytes);
           if constexpr (PAIR) sm100::tma_load_2d_pair(dst, tm, sm100::cluster_addr(fb, 0), kb * TILE_K, row, pol);
           else sm100::tma_load_3d(dst, tm, fb, 0, row, kb * KPS, pol);
-          if (++s == g.stages) { s = 0; ph ^= 1u; }
         }
+        __syncwarp();
+        if (++s == g.stages) { s = 0; ph ^= 1u; }
       }
     }
   } else if (warp == 1 && rank == 0) {
     // ===================== MMA issuer =====================
-    // One thread issues every MMA, and it issues them barely faster than the tensor pipe
-    // retires them (59 cycles each, 50 more per commit), so nothing else may sit in its instruction stream: a test of an mbarrier
+    // One thread issues every MMA.  The whole warp runs the loop, with a warp index that the compiler can see is uniform, and elects the
+    // thread: with the operands in uniform registers an MMA issues in 59 cycles, behind a plain test of the lane
+    // index in 90 (a K block of 272 rows: 715 instead of 543 cycles).  That is barely faster than the tensor pipe
+    // retires them, so nothing else may sit in this instruction stream: a test of an mbarrier
     // (any access through the memory pipeline) completes only once the MMAs queued before it
     // have gone out, and the pipe runs dry for ~250 cycles per K block.  The watcher warp
     // therefore does the mbarrier waits and releases this warp through one hardware barrier
@@ -238,7 +242,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       for (int kb = w.kb0; kb < w.kb1; ++kb) {
         sm100::named_bar_sync(1u + (uint32_t)s, 64);
         sm100::tc_fence_after();
-        if (lane == 0) {
+        if (sm100::elect_one()) {
           if (PAIR && two) {
             const uint64_t ad2 = ad + a2_off16;
 #pragma unroll
@@ -257,10 +261,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           commit(sm100::smem_u32(&empty[s]));       // the stage is reusable once these MMAs have read it
         }
         __syncwarp();
+        acc = 1u;
         wd += stage16; ad += stage16;
         if (++s == g.stages) { s = 0; wd = wdesc0; ad = adesc0; }
       }
-      if (lane == 0) commit(sm100::smem_u32(&tmem_full_bar));
+      if (sm100::elect_one()) commit(sm100::smem_u32(&tmem_full_bar));
       __syncwarp();
     }
   } else if (warp == 2 && rank == 0) {
