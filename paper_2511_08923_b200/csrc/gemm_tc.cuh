@@ -80,7 +80,9 @@ struct Args {
   int stages;               // depth of the ring (<= MAX_STAGES)
   int n1, n2;               // MMA N of the two instructions (n2 may be 0)
   // MODE_SLAB: out[split][r][n], fp32 or (slab_bf16) bf16; strides in elements
-  void *out; long long slab_stride; int ldo; int slab_bf16;
+  // accumulate (S = 1 only): out is added to instead of written; every element has one writer, so the result does not
+  // depend on any order
+  void *out; long long slab_stride; int ldo; int slab_bf16, accumulate;
   // MODE_SWIGLU: weight rows interleave (gate f, up f); H[r][f] = silu(gate) * up, bf16
   bf16 *H; int ldh;
   // MODE_ARGMAX: per (CTA, lane quadrant) candidates, [R][cand_ld >= gridDim*4] (index -1 = none; the
@@ -442,7 +444,22 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         // split-K partial sums; columns are counted from the first tile of the split region
         const int nc = n - g.tile_b0 * tile_rows(SMALL);
         const bool n_ok = n < g.N;
-        if (!g.slab_bf16) {
+        if (g.accumulate) {
+          float *out = reinterpret_cast<float *>(g.out) + nc;
+#pragma unroll
+          for (int i = 0; i < NCH; ++i) {
+            if (i * 16 < ncols) {
+              const int r0 = row_block + c_begin + i * 16;             // (one instruction per block: columns are rows in order)
+              float *p = out + (long long)r0 * g.ldo;
+              const int rows_left = n_ok ? R_live - r0 : 0;
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                if (j < rows_left) atomicAdd(p, __uint_as_float(v[i][j]));
+                p += g.ldo;
+              }
+            }
+          }
+        } else if (!g.slab_bf16) {
           // One running pointer and a bound counted from the first row of eight: with the address
           // and the row test recomputed per store (r * ldo, r < R) the same 144 stores take 1.65 times
           // as long (19.5 instead of 32 bytes per cycle and SM, the rate the L2 takes stores at).
@@ -622,19 +639,31 @@ inline void plan_stages(Args &a, int n, bool small) {
 }
 inline size_t smem_bytes(const Args &a, bool small) { return (size_t)a.stages * stage_bytes(a, small) + 1024; }
 
-// K splits: fill the SMs with whole waves of equally sized items, keeping at least
-// min_kb K blocks per item.
-inline int plan_splits(int n_items_unsplit, int kb_total, int n_sms, int max_splits, int min_kb, double item_cost = 3.0) {
+// K splits of one row block: fill the workers (CTAs, or pairs) with whole waves of equally sized items, keeping at least
+// min_kb stages per item; item_cost: fixed cost of an item in stages.
+inline int plan_splits(int n_items_unsplit, int kb_total, int workers, int max_splits, int min_kb, double item_cost) {
   int best = 1; double best_eff = 0.0;
   for (int s = 1; s <= max_splits; ++s) {
     if (s > 1 && kb_total / s < min_kb) break;
     const long long items = (long long)n_items_unsplit * s;
-    const long long waves = (items + n_sms - 1) / n_sms;
-    // time ~ waves * (k blocks per item + fixed per-item cost in k-block units)
-    const double per_item = (double)((kb_total + s - 1) / s) + item_cost;
-    const double eff = ((double)n_items_unsplit * kb_total) / ((double)waves * n_sms * per_item);
+    const long long waves = (items + workers - 1) / workers;
+    const double eff = ((double)n_items_unsplit * kb_total) / ((double)waves * workers * ((double)((kb_total + s - 1) / s) + item_cost));
     if (eff > best_eff + 1e-9) { best_eff = eff; best = s; }
   }
+  return best;
+}
+// The same for several row blocks, where slabs are large: the split with the least estimated time.  Whole waves of items;
+// per stage of K 2.15 cycles per row at 1.75 GHz; 1 us to hand an accumulator over; and S slabs of R x N floats written, and
+// read again by the next kernel.  (Chosen for whole waves alone, the O projection of 1152 rows was split 4 ways and a
+// 4 k first pass spent 85 us per norm on slabs, 30 now.)
+inline int plan_splits_blocks(const Args &a, int workers, int max_splits, int min_kb) {
+  auto us = [&](int S) {
+    const long long items = (long long)a.n_rb * a.n_tiles * S, waves = (items + workers - 1) / workers;
+    return (double)waves * (((a.kb_total + S - 1) / S) * ((2.15 * a.rb_rows + 50.0) / 1750.0) + 1.0) + S * ((double)a.R * a.N * 6.0 / 5.0e6);
+  };
+  int best = 1;
+  for (int s = 2; s <= max_splits && a.kb_total / s >= min_kb; ++s)
+    if (us(s) < us(best) - 1e-9) best = s;
   return best;
 }
 

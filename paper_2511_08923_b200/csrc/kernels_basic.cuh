@@ -18,10 +18,10 @@ template <> __device__ __forceinline__ float4 load4<bf16>(const bf16 *p) {
 // first addition: with one load per turn of a loop over S, the kernels that read slabs spent most of their time waiting
 // (norm 3.6 -> 2.0 us at 272 rows of 1536).
 constexpr int MAX_SLABS = 8;
-template <int AT_ONCE, typename SLAB>
+template <int AT_ONCE, int MOST = MAX_SLABS, typename SLAB>
 __device__ __forceinline__ void add_slabs(float4 &v, const SLAB *__restrict__ p, int S, size_t stride) {
 #pragma unroll
-  for (int s0 = 0; s0 < MAX_SLABS; s0 += AT_ONCE) {
+  for (int s0 = 0; s0 < MOST; s0 += AT_ONCE) {
     if (s0 >= S) break;
     float4 q[AT_ONCE];
 #pragma unroll
@@ -222,8 +222,9 @@ __global__ void __launch_bounds__(256) pass_setup_kernel(RowMeta m, int R, int h
 // A = bf16(X * rsqrt(mean(X^2) + eps) * gain).  One block per row; a thread keeps NV
 // groups of four columns in registers (NV * 4 * THREADS >= d).
 // ---------------------------------------------------------------------------
-template <int THREADS, int NV, typename SLAB>
-__global__ void __launch_bounds__(THREADS)
+// SLABS: the most partial results there can be (1 or MAX_SLABS: with one, four blocks of a many-row pass fit on an SM).
+template <int THREADS, int NV, int SLABS, typename SLAB>
+__global__ void __launch_bounds__(THREADS, SLABS == 1 && NV <= 2 ? 4 : 1)
 rmsnorm_reduce_kernel(float *__restrict__ X, const SLAB *__restrict__ partials, int S, size_t partial_stride,
                       const bf16 *__restrict__ gain, float eps, int d, bf16 *__restrict__ A, TlSlot tl) {
   pdl_trigger();
@@ -246,7 +247,7 @@ rmsnorm_reduce_kernel(float *__restrict__ X, const SLAB *__restrict__ partials, 
     v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (c < d) {
       v[i] = *reinterpret_cast<const float4 *>(xr + c);
-      add_slabs<MAX_SLABS>(v[i], partials + (size_t)r * d + c, S, partial_stride);
+      add_slabs<SLABS, SLABS>(v[i], partials + (size_t)r * d + c, S, partial_stride);
     }
     ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
   }

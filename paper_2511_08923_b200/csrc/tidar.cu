@@ -348,16 +348,17 @@ gemm_tc::Args plan_gemm(const tidar_ctx *c, int mode, int R, int N, int K, int f
   a.S = 1; a.fused_items = 0; a.tile_b0 = 0; a.n_tiles_b = 0;
   if (mode == gemm_tc::MODE_SLAB) {
     a.n_tiles_b = a.n_tiles;
-    a.S = force_S > 0 ? std::min(force_S, a.kb_total) : gemm_tc::plan_splits(a.n_rb * a.n_tiles, a.kb_total, workers, c->S_max, 4 / kps, 3.0 / kps);
+    a.S = force_S > 0 ? std::min(force_S, a.kb_total) : a.n_rb > 1 ? gemm_tc::plan_splits_blocks(a, workers, c->S_max, 4)
+                      : gemm_tc::plan_splits(a.n_tiles, a.kb_total, workers, c->S_max, 4 / kps, 3.0 / kps);
     // One row block of up to 288 rows, or two of half the rows?  Two halves fetch every weight tile
     // twice (the second time from L2), while a CTA's slab store, which its SM cannot
-    // push out faster than ~42 GB/s, shrinks from 3.3 to 1.7 us and fewer slabs are left for the
+    // push out faster than ~42 GB/s, shrinks by half and fewer slabs are left for the
     // consumer.  Halves win when an item has few K blocks (the 1.5B-class shapes), one
     // block when it has many (the 8B-class shapes).
     if (force_S <= 0 && a.n_rb == 1 && R > gemm_tc::MAX_ROWS / 2) {
       gemm_tc::Args h = a;
       gemm_tc::plan_rows(R, h, gemm_tc::MAX_ROWS / 2);
-      h.S = gemm_tc::plan_splits(h.n_rb * h.n_tiles, h.kb_total, workers, c->S_max, 4);
+      h.S = gemm_tc::plan_splits(h.n_rb * h.n_tiles, h.kb_total, workers, c->S_max, 4, 3.0);
       auto cost = [&](const gemm_tc::Args &x, double us_per_kb, double us_store) {
         const long long items = (long long)x.n_rb * x.n_tiles * x.S;
         const long long waves = (items + workers - 1) / workers;
@@ -388,17 +389,19 @@ gemm_tc::Args plan_gemm(const tidar_ctx *c, int mode, int R, int N, int K, int f
 }
 
 // Tensor-core projection.  A [a_rows][K] (first R rows used), W described by tmW ([N][K]).
-//   MODE_SLAB  : S split-K partial slabs of fp32 [R][N] into c->partials (S chosen here)
+//   MODE_SLAB  : S split-K partial slabs of fp32 [R][N] into c->partials (S chosen here); with `residual` [R][N] given and
+//                nothing split, the result is added to it instead and *S_out is 0
 //   MODE_SWIGLU: bf16 c->H [R][N/2]
 //   MODE_ARGMAX: candidates for argmax_merge_kernel (+ optional logits dump)
 int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const tidar_ctx::WMap &tmW, int R, int N, int K, int cls,
-                   int *S_out, size_t *stride_out, float *slab_out = nullptr, int force_S = 0) {
+                   int *S_out, size_t *stride_out, float *slab_out = nullptr, int force_S = 0, float *residual = nullptr) {
   gemm_tc::Args a = plan_gemm(c, mode, R, N, K, force_S);
   const bool small = small_gemm(mode, R);
   const int rem_tiles = mode == gemm_tc::MODE_SWIGLU ? a.n_tiles_b : 0;
   if (mode == gemm_tc::MODE_SLAB) {
     a.out = slab_out ? (void *)slab_out : (void *)c->partials;
     a.slab_bf16 = (slab_out || !c->slab_bf16) ? 0 : 1;   // an explicit output buffer always gets exact fp32 slabs
+    if (residual && a.S == 1 && a.n2 == 0 && !a.slab_bf16) { a.out = residual; a.accumulate = 1; }
   } else if (mode == gemm_tc::MODE_SWIGLU) {
     a.H = c->H;
     a.out = c->partials; a.slab_bf16 = c->slab_bf16 ? 1 : 0;
@@ -437,7 +440,7 @@ int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const tida
       launch_pdl(swiglu_slab_kernel<float>, (unsigned)((n / 2 + 255) / 256), 256, 0, c->stream, (const float *)c->partials, a.S, (size_t)a.slab_stride, R, a.ldo, nf,
                                                                            f0, a.ldh, c->H, lf.tl);
   }
-  if (S_out) *S_out = a.S;
+  if (S_out) *S_out = a.accumulate ? 0 : a.S;
   if (stride_out) *stride_out = (size_t)R * N;
   return TIDAR_OK;
 }
@@ -446,8 +449,8 @@ enum Proj { P_QKV, P_O, P_GU, P_DOWN };
 
 // out = A[R][K] * W[N][K]^T as S split-K partial slabs of fp32 [R][N] (replay: S = 1).
 int gemm_partials(tidar_ctx *c, const bf16 *A, int a_rows, const bf16 *W, const tidar_ctx::WMap *tmW, int R, int N, int K, float *out,
-                  int *S_out, size_t *stride_out, int cls) {
-  if (c->cfg.impl == 0) return gemm_tc_launch(c, gemm_tc::MODE_SLAB, A, a_rows, *tmW, R, N, K, cls, S_out, stride_out);
+                  int *S_out, size_t *stride_out, int cls, float *residual = nullptr) {
+  if (c->cfg.impl == 0) return gemm_tc_launch(c, gemm_tc::MODE_SLAB, A, a_rows, *tmW, R, N, K, cls, S_out, stride_out, nullptr, 0, residual);
   Launch l(c, cls);
   dim3 grid((N + 63) / 64, (R + 63) / 64);
   gemm_replay_kernel<<<grid, 256, 0, c->stream>>>(A, K, W, K, out, N, R, N, K);
@@ -570,10 +573,14 @@ void launch_norm_as(tidar_ctx *c, int R, const SLAB *partials, int S, size_t str
   const int per_sm = c->cfg.impl == 0 ? (R + c->n_sms - 1) / c->n_sms : 0;
   const size_t smem = R > gemm_tc::SMALL_ROWS && per_sm <= 4 && per_sm > 0 ? (size_t)(NORM_SMEM / per_sm) & ~(size_t)1023 : 0;
   auto go = [&](auto kernel) { launch_pdl(kernel, R, 512, smem, c->stream, c->X, partials, S, stride, gain, c->cfg.rms_eps, d, c->A, l.tl); };
-  if (nv <= 1) go(rmsnorm_reduce_kernel<512, 1, SLAB>);
-  else if (nv <= 2) go(rmsnorm_reduce_kernel<512, 2, SLAB>);
-  else if (nv <= 3) go(rmsnorm_reduce_kernel<512, 3, SLAB>);
-  else go(rmsnorm_reduce_kernel<512, 6, SLAB>);
+  auto by_width = [&](auto slabs) {
+    constexpr int SL = decltype(slabs)::value;
+    if (nv <= 1) go(rmsnorm_reduce_kernel<512, 1, SL, SLAB>);
+    else if (nv <= 2) go(rmsnorm_reduce_kernel<512, 2, SL, SLAB>);
+    else if (nv <= 3) go(rmsnorm_reduce_kernel<512, 3, SL, SLAB>);
+    else go(rmsnorm_reduce_kernel<512, 6, SL, SLAB>);
+  };
+  if (S <= 1) by_width(std::integral_constant<int, 1>()); else by_width(std::integral_constant<int, MAX_SLABS>());
 }
 void launch_norm(tidar_ctx *c, int R, const float *partials, int S, size_t stride, const bf16 *gain) {
   if (c->cfg.impl == 0 && c->slab_bf16) launch_norm_as<bf16>(c, R, (const bf16 *)partials, S, stride, gain);
@@ -627,7 +634,7 @@ if (tc && c->slab_bf16)
     } else {
       launch_attention(c, c->Q, Kp, Vp, g, c->Kloc, c->Vloc, c->O, R);
     }
-    if ((rc = gemm_partials(c, c->O, RA, c->wo[l], tc ? &c->tm_wo[l] : nullptr, R, d, Hq * hd, c->partials, &S, &stride, TIDAR_TC_GEMM))) return rc;
+    if ((rc = gemm_partials(c, c->O, RA, c->wo[l], tc ? &c->tm_wo[l] : nullptr, R, d, Hq * hd, c->partials, &S, &stride, TIDAR_TC_GEMM, c->X))) return rc;
     launch_norm(c, R, c->partials, S, stride, c->ffn_norm[l]);
     if (tc) {
       if ((rc = gemm_tc_launch(c, gemm_tc::MODE_SWIGLU, c->A, RA, c->tm_wgu[l], R, 2 * cf.d_ffn, d, TIDAR_TC_GEMM, nullptr, nullptr))) return rc;
@@ -637,7 +644,7 @@ if (tc && c->slab_bf16)
       const size_t n = (size_t)R * cf.d_ffn;
       swiglu_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(c->partials, R, cf.d_ffn, c->H);
     }
-    if ((rc = gemm_partials(c, c->H, RA, c->wdown[l], tc ? &c->tm_wdown[l] : nullptr, R, d, cf.d_ffn, c->partials, &S, &stride, TIDAR_TC_GEMM))) return rc;
+    if ((rc = gemm_partials(c, c->H, RA, c->wdown[l], tc ? &c->tm_wdown[l] : nullptr, R, d, cf.d_ffn, c->partials, &S, &stride, TIDAR_TC_GEMM, c->X))) return rc;
   }
   launch_norm(c, R, c->partials, S, stride, c->final_norm);
   if (c->dbg_hidden)
@@ -721,16 +728,20 @@ int init_tensor_core_path(tidar_ctx *c) {
   {
     auto max_smem_split = [&](const void *f) { return cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared); };
     const void *kernels[] = {(const void *)assemble_step_kernel, (const void *)pass_setup_kernel, (const void *)attn_meta_plan_kernel,
-                             (const void *)rmsnorm_reduce_kernel<512, 1, float>, (const void *)rmsnorm_reduce_kernel<512, 1, bf16>,
-                             (const void *)rmsnorm_reduce_kernel<512, 2, float>, (const void *)rmsnorm_reduce_kernel<512, 2, bf16>,
-                             (const void *)rmsnorm_reduce_kernel<512, 3, float>, (const void *)rmsnorm_reduce_kernel<512, 3, bf16>,
-                             (const void *)rmsnorm_reduce_kernel<512, 6, float>, (const void *)rmsnorm_reduce_kernel<512, 6, bf16>,
+                             (const void *)rmsnorm_reduce_kernel<512, 1, 1, float>, (const void *)rmsnorm_reduce_kernel<512, 1, 1, bf16>,
+                             (const void *)rmsnorm_reduce_kernel<512, 2, 1, float>, (const void *)rmsnorm_reduce_kernel<512, 2, 1, bf16>,
+                             (const void *)rmsnorm_reduce_kernel<512, 3, 1, float>, (const void *)rmsnorm_reduce_kernel<512, 3, 1, bf16>,
+                             (const void *)rmsnorm_reduce_kernel<512, 6, 1, float>, (const void *)rmsnorm_reduce_kernel<512, 6, 1, bf16>,
+                             (const void *)rmsnorm_reduce_kernel<512, 1, MAX_SLABS, float>, (const void *)rmsnorm_reduce_kernel<512, 1, MAX_SLABS, bf16>,
+                             (const void *)rmsnorm_reduce_kernel<512, 2, MAX_SLABS, float>, (const void *)rmsnorm_reduce_kernel<512, 2, MAX_SLABS, bf16>,
+                             (const void *)rmsnorm_reduce_kernel<512, 3, MAX_SLABS, float>, (const void *)rmsnorm_reduce_kernel<512, 3, MAX_SLABS, bf16>,
+                             (const void *)rmsnorm_reduce_kernel<512, 6, MAX_SLABS, float>, (const void *)rmsnorm_reduce_kernel<512, 6, MAX_SLABS, bf16>,
                              (const void *)rope_kv_kernel<float>, (const void *)rope_kv_kernel<bf16>,
                              (const void *)swiglu_slab_kernel<float>, (const void *)swiglu_slab_kernel<bf16>,
                              (const void *)attn_tc::attn_combine_kernel<128>, (const void *)attn_tc::attn_combine_kernel<64>,
                              (const void *)mix_rows_kernel, (const void *)argmax_merge_kernel, (const void *)verify_select_kernel, (const void *)stage_step_kernel};
     for (const void *f : kernels) CUDA_TRY(c, max_smem_split(f));
-    for (int i = 3; i < 11; ++i) CUDA_TRY(c, cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, NORM_SMEM));
+    for (int i = 3; i < 19; ++i) CUDA_TRY(c, cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, NORM_SMEM));
   }
   const int max_smem = gemm_tc::SMEM_BUDGET + 1024;
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
