@@ -622,8 +622,8 @@ inline CUresult encode_2d_small(EncodeTiledFn fn, CUtensorMap *tm, const void *b
 
 // Row-block geometry for R activation rows.
 inline void plan_rows(int R, Args &a, int max_rows = MAX_ROWS) {
-  a.n_rb = R <= max_rows ? 1 : (R + BLOCK_ROWS - 1) / BLOCK_ROWS;
-  if (max_rows < BLOCK_ROWS) a.n_rb = (R + max_rows - 1) / max_rows;
+  const int block = std::min(max_rows, BLOCK_ROWS);
+  a.n_rb = R <= max_rows ? 1 : (R + block - 1) / block;
   const int per = (R + a.n_rb - 1) / a.n_rb;
   a.rb_rows = (per + 15) / 16 * 16;
   a.n1 = a.rb_rows; a.n2 = 0;

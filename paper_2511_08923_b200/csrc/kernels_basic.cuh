@@ -282,8 +282,10 @@ rmsnorm_reduce_kernel(float *__restrict__ X, const SLAB *__restrict__ partials, 
 // bias [(Hq+2Hkv)*hd] added to the projection; qn / kn [hd]: RMSNorm over each Q / K head's
 // dimensions before the rotation (the hd/8 threads of a head reduce with shuffles).
 // ---------------------------------------------------------------------------
-template <typename SLAB>
-__global__ void __launch_bounds__(256)
+// SLABS: the most partial results there can be (1 or MAX_SLABS: with one, and few registers, a pass of many rows keeps
+// three times as many loads in flight).
+template <int SLABS, typename SLAB>
+__global__ void __launch_bounds__(256, SLABS == 1 ? 6 : 3)
 rope_kv_kernel(const SLAB *__restrict__ partials, int S, size_t partial_stride, int Hq, int Hkv, int hd,
                RowMeta m, const float *__restrict__ cs, const float *__restrict__ sn, KvGeom g,
                bf16 *__restrict__ Q, bf16 *__restrict__ Kpool, bf16 *__restrict__ Vpool,
@@ -304,14 +306,15 @@ rope_kv_kernel(const SLAB *__restrict__ partials, int S, size_t partial_stride, 
     float4 x1 = make_float4(0.f, 0.f, 0.f, 0.f), x2 = x1;
     // (both halves' loads together: two chains of additions)
 #pragma unroll
-    for (int s0 = 0; s0 < MAX_SLABS; s0 += 4) {
+    for (int s0 = 0; s0 < SLABS; s0 += 4) {
       if (s0 >= S) break;
-      float4 q1[4], q2[4];
+      constexpr int AT_ONCE = SLABS < 4 ? SLABS : 4;
+      float4 q1[AT_ONCE], q2[AT_ONCE];
 #pragma unroll
-      for (int t = 0; t < 4; ++t)
+      for (int t = 0; t < AT_ONCE; ++t)
         if (s0 + t < S) { q1[t] = load4<SLAB>(partials + (s0 + t) * partial_stride + base); q2[t] = load4<SLAB>(partials + (s0 + t) * partial_stride + base + half); }
 #pragma unroll
-      for (int t = 0; t < 4; ++t)
+      for (int t = 0; t < AT_ONCE; ++t)
         if (s0 + t < S) {
           x1.x += q1[t].x; x1.y += q1[t].y; x1.z += q1[t].z; x1.w += q1[t].w;
           x2.x += q2[t].x; x2.y += q2[t].y; x2.z += q2[t].z; x2.w += q2[t].w;

@@ -327,20 +327,28 @@ const CUtensorMap *act_map(tidar_ctx *c, const void *p, int rows, int cols, int 
   return &c->amaps.back().tm;
 }
 
-// Whether a projection runs as a SMALL instance (the LM head's argmax epilogue needs the registers of the full one).
 // CTAs of the LM head, each of which leaves four candidates per row (with several row blocks it may meet only some of the rows).
 int lm_head_ctas(const tidar_ctx *c, int R, int vocab) {
   const int pairs = c->n_sms / 2, tiles = (vocab + gemm_tc::tile_rows(false) - 1) / gemm_tc::tile_rows(false);
   return 2 * (R <= gemm_tc::MAX_ROWS ? std::min(tiles, pairs) : pairs);
 }
-bool small_gemm(int mode, int R) { return R <= gemm_tc::SMALL_ROWS && (mode == gemm_tc::MODE_SLAB || mode == gemm_tc::MODE_SWIGLU); }
+// Whether a projection runs as a SMALL instance (the LM head's argmax epilogue needs the registers of the full one).  Up to one
+// block of SMALL_ROWS rows always.  Up to one block's worth of rows (MAX_ROWS), as several blocks of 96, where the weight
+// matrix is small: such a launch is all start-up and slab store, both of which a SMALL CTA, which sits beside the kernels in
+// front of it, hides better, and re-reading a few MB of weights per block from L2 costs less.  (1.5B-class step at 272 rows, its
+// projections of 2.4 - 13.8 M weights: 2.18 -> 1.96 ms; 8B-class, from 16.8 M weights on: 1 % slower that way; the fused
+// gate/up projection of 27.5 M weights: 12 % of the step slower.)
+bool small_gemm(int mode, int R, int N, int K) {
+  if (mode != gemm_tc::MODE_SLAB && mode != gemm_tc::MODE_SWIGLU) return false;
+  return R <= gemm_tc::SMALL_ROWS || (mode == gemm_tc::MODE_SLAB && R <= gemm_tc::MAX_ROWS && (long long)N * K <= 15000000);
+}
 
 // Work of a tensor-core projection of R rows: row blocks, K splits, which tiles finish in the fused epilogue.
 gemm_tc::Args plan_gemm(const tidar_ctx *c, int mode, int R, int N, int K, int force_S = 0) {
   gemm_tc::Args a{};
   a.R = R; a.N = N; a.K = K;
-  gemm_tc::plan_rows(R, a);
-  const bool small = small_gemm(mode, R);
+  const bool small = small_gemm(mode, R, N, K);
+  gemm_tc::plan_rows(R, a, small ? gemm_tc::SMALL_ROWS : gemm_tc::MAX_ROWS);
   const int kps = gemm_tc::k_per_stage(small), tile = gemm_tc::tile_rows(small);
   const int workers = small ? c->n_sms : c->n_sms / 2;             // CTAs, or pairs of CTAs, that work on items
   a.n_tiles = (N + tile - 1) / tile;
@@ -348,24 +356,8 @@ gemm_tc::Args plan_gemm(const tidar_ctx *c, int mode, int R, int N, int K, int f
   a.S = 1; a.fused_items = 0; a.tile_b0 = 0; a.n_tiles_b = 0;
   if (mode == gemm_tc::MODE_SLAB) {
     a.n_tiles_b = a.n_tiles;
-    a.S = force_S > 0 ? std::min(force_S, a.kb_total) : a.n_rb > 1 ? gemm_tc::plan_splits_blocks(a, workers, c->S_max, 4)
-                      : gemm_tc::plan_splits(a.n_tiles, a.kb_total, workers, c->S_max, 4 / kps, 3.0 / kps);
-    // One row block of up to 288 rows, or two of half the rows?  Two halves fetch every weight tile
-    // twice (the second time from L2), while a CTA's slab store, which its SM cannot
-    // push out faster than ~42 GB/s, shrinks by half and fewer slabs are left for the
-    // consumer.  Halves win when an item has few K blocks (the 1.5B-class shapes), one
-    // block when it has many (the 8B-class shapes).
-    if (force_S <= 0 && a.n_rb == 1 && R > gemm_tc::MAX_ROWS / 2) {
-      gemm_tc::Args h = a;
-      gemm_tc::plan_rows(R, h, gemm_tc::MAX_ROWS / 2);
-      h.S = gemm_tc::plan_splits(h.n_rb * h.n_tiles, h.kb_total, workers, c->S_max, 4, 3.0);
-      auto cost = [&](const gemm_tc::Args &x, double us_per_kb, double us_store) {
-        const long long items = (long long)x.n_rb * x.n_tiles * x.S;
-        const long long waves = (items + workers - 1) / workers;
-        return waves * ((x.kb_total + x.S - 1) / x.S * us_per_kb + 1.5) + us_store + 0.5 * x.S;
-      };
-      if (cost(h, 0.37, 1.7) < cost(a, 0.46, 3.3)) a = h;
-    }
+    a.S = force_S > 0 ? std::min(force_S, a.kb_total) : a.n_rb > 1 && !small ? gemm_tc::plan_splits_blocks(a, workers, c->S_max, 4)
+                      : gemm_tc::plan_splits(a.n_rb * a.n_tiles, a.kb_total, workers, c->S_max, 4 / kps, 3.0 / kps);
     a.ldo = N; a.slab_stride = (long long)R * N;
   } else if (mode == gemm_tc::MODE_SWIGLU) {
     a.ldh = N / 2;
@@ -396,7 +388,7 @@ gemm_tc::Args plan_gemm(const tidar_ctx *c, int mode, int R, int N, int K, int f
 int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const tidar_ctx::WMap &tmW, int R, int N, int K, int cls,
                    int *S_out, size_t *stride_out, float *slab_out = nullptr, int force_S = 0, float *residual = nullptr) {
   gemm_tc::Args a = plan_gemm(c, mode, R, N, K, force_S);
-  const bool small = small_gemm(mode, R);
+  const bool small = small_gemm(mode, R, N, K);
   const int rem_tiles = mode == gemm_tc::MODE_SWIGLU ? a.n_tiles_b : 0;
   if (mode == gemm_tc::MODE_SLAB) {
     a.out = slab_out ? (void *)slab_out : (void *)c->partials;
@@ -621,12 +613,13 @@ int forward_rows(tidar_ctx *c, int R, bool with_head, int rows_per_group, const 
       const int rope_chunks = ((Hq + 2 * Hkv) * (hd / 8) + 255) / 256;
       const bf16 *bias_l = c->bqkv.empty() ? nullptr : c->bqkv[l], *qn_l = c->q_norm.empty() ? nullptr : c->q_norm[l],
                  *kn_l = c->k_norm.empty() ? nullptr : c->k_norm[l];
-if (tc && c->slab_bf16)
-        launch_pdl(rope_kv_kernel<bf16>, dim3(R, rope_chunks), 256, 0, c->stream, (const bf16 *)c->partials, S, stride, Hq, Hkv, hd, c->meta, c->rope_cos,
-                                                                      c->rope_sin, g, c->Q, Kp, Vp, c->Kloc, c->Vloc, bias_l, qn_l, kn_l, cf.rms_eps, ll.tl);
-      else
-        launch_pdl(rope_kv_kernel<float>, dim3(R, rope_chunks), 256, 0, c->stream, c->partials, S, stride, Hq, Hkv, hd, c->meta, c->rope_cos,
-                                                                      c->rope_sin, g, c->Q, Kp, Vp, c->Kloc, c->Vloc, bias_l, qn_l, kn_l, cf.rms_eps, ll.tl);
+      auto rope = [&](auto kernel, auto *partials) {
+        launch_pdl(kernel, dim3(R, rope_chunks), 256, 0, c->stream, partials, S, stride, Hq, Hkv, hd, c->meta, c->rope_cos, c->rope_sin, g, c->Q, Kp, Vp,
+                   c->Kloc, c->Vloc, bias_l, qn_l, kn_l, cf.rms_eps, ll.tl);
+      };
+      if (tc && c->slab_bf16) rope(rope_kv_kernel<MAX_SLABS, bf16>, (const bf16 *)c->partials);
+      else if (S <= 1) rope(rope_kv_kernel<1, float>, (const float *)c->partials);
+      else rope(rope_kv_kernel<MAX_SLABS, float>, (const float *)c->partials);
     }
     if (tc) {
       AttnMaps am{&c->tm_q, &c->tm_kv, &c->tm_kv, &c->tm_kloc, &c->tm_vloc, (2 * l) * c->n_pages, (2 * l + 1) * c->n_pages};
@@ -689,10 +682,11 @@ int init_tensor_core_path(tidar_ctx *c) {
   const tidar_config &cf = c->cfg;
   int dev = 0;
   CUDA_TRY(c, cudaGetDevice(&dev));
-  cudaDeviceProp prop;
-  CUDA_TRY(c, cudaGetDeviceProperties(&prop, dev));
-  if (prop.major != 10) return fail(c, TIDAR_ECUDA, "the tensor-core path needs an sm_100 device, found sm_%d%d", prop.major, prop.minor);
-  c->n_sms = prop.multiProcessorCount;
+  int major = 0, minor = 0;                       // (cudaGetDeviceProperties takes milliseconds)
+  CUDA_TRY(c, cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev));
+  CUDA_TRY(c, cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev));
+  CUDA_TRY(c, cudaDeviceGetAttribute(&c->n_sms, cudaDevAttrMultiProcessorCount, dev));
+  if (major != 10) return fail(c, TIDAR_ECUDA, "the tensor-core path needs an sm_100 device, found sm_%d%d", major, minor);
   if (c->n_sms > MAX_SMS) return fail(c, TIDAR_ECUDA, "%d SMs; scratch is sized for %d", c->n_sms, MAX_SMS);
   void *fn = nullptr;
   cudaDriverEntryPointQueryResult qres;
@@ -736,7 +730,7 @@ int init_tensor_core_path(tidar_ctx *c) {
                              (const void *)rmsnorm_reduce_kernel<512, 2, MAX_SLABS, float>, (const void *)rmsnorm_reduce_kernel<512, 2, MAX_SLABS, bf16>,
                              (const void *)rmsnorm_reduce_kernel<512, 3, MAX_SLABS, float>, (const void *)rmsnorm_reduce_kernel<512, 3, MAX_SLABS, bf16>,
                              (const void *)rmsnorm_reduce_kernel<512, 6, MAX_SLABS, float>, (const void *)rmsnorm_reduce_kernel<512, 6, MAX_SLABS, bf16>,
-                             (const void *)rope_kv_kernel<float>, (const void *)rope_kv_kernel<bf16>,
+                             (const void *)rope_kv_kernel<1, float>, (const void *)rope_kv_kernel<MAX_SLABS, float>, (const void *)rope_kv_kernel<MAX_SLABS, bf16>,
                              (const void *)swiglu_slab_kernel<float>, (const void *)swiglu_slab_kernel<bf16>,
                              (const void *)attn_tc::attn_combine_kernel<128>, (const void *)attn_tc::attn_combine_kernel<64>,
                              (const void *)mix_rows_kernel, (const void *)argmax_merge_kernel, (const void *)verify_select_kernel, (const void *)stage_step_kernel};

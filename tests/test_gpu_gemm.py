@@ -68,6 +68,15 @@ def test_gemm_few_rows(ctx, R, N, K):
     assert np.abs(a - b).max() <= TOL
 
 
+@pytest.mark.parametrize("R", [97, 144, 256, 257, 288, 289])
+def test_gemm_cta_pairs(ctx, R):
+    """A weight matrix too large for the few-rows instance: one instruction (up to 256 rows), two (up to 288), several
+    row blocks; an odd number of 128-row weight tiles with a ragged end."""
+    a = _run(ctx, R, 2430, 6400, 0, 400 + R)
+    b = _run(ctx, R, 2430, 6400, 3, 400 + R)
+    assert np.abs(a - b).max() <= TOL
+
+
 def test_gemm_rejects_bad_arguments(ctx):
     from paper_2511_08923_b200 import TidarError
     A = torch.zeros(4, 100, dtype=torch.bfloat16, device="cuda:0")
