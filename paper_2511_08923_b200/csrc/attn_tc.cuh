@@ -144,10 +144,9 @@ __device__ inline void plan_block(const PlanArgs &p, ROW row_keys) {
   __shared__ float ent_us[3 * PLAN_UNITS];             // units, then tiles
   __shared__ short ent_n[2 * PLAN_UNITS], order_s[2 * PLAN_UNITS], place_s[2 * PLAN_UNITS];
   __shared__ int longest_us[2];                        // longest unit / tile, as float bits
-  __shared__ unsigned long long best;
+  __shared__ unsigned long long best[32];              // per warp (64-bit atomics in shared memory would take turns)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
   const bool planned = p.n_units <= PLAN_UNITS, splits = p.max_items > p.n_units;
-  if (threadIdx.x == 0) best = ~0ull;
   if (threadIdx.x < 2) longest_us[threadIdx.x] = 0;
   __syncthreads();
   for (int u = warp; u < p.n_units; u += n_warps) {
@@ -217,14 +216,21 @@ __device__ inline void plan_block(const PlanArgs &p, ROW row_keys) {
       items += __shfl_xor_sync(0xffffffffu, items, o); live += __shfl_xor_sync(0xffffffffu, live, o); most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
       us_sum += __shfl_xor_sync(0xffffffffu, us_sum, o); us_max = fmaxf(us_max, __shfl_xor_sync(0xffffffffu, us_max, o));
     }
-    if (live_cnd && sub == 0 && items <= p.max_items && most <= p.max_pieces) {
+    unsigned long long mine = ~0ull;
+    if (live_cnd && items <= p.max_items && most <= p.max_pieces) {
       float us = us_max;
       if (items * p.Hkv > p.n_sms) us = fmaxf(us, p.Hkv * us_sum / p.n_sms + 0.5f * us_max);
       if (items > live) us += MERGE + 0.3f * items / live;
-      atomicMin(&best, ((unsigned long long)__float_as_uint(us) << 32) | (unsigned)cnd);     // us > 0: its bits order like its value
+      mine = ((unsigned long long)__float_as_uint(us) << 32) | (unsigned)cnd;                // us > 0: its bits order like its value
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mine = min(mine, __shfl_xor_sync(0xffffffffu, mine, o));
+    if (lane == 0) best[warp] = mine;
     __syncthreads();
-    if (best != ~0ull) { const int c = (int)(best & 0xffffffffu); paired = c < CAND; limit = limit_of(c); }
+    mine = lane < n_warps ? best[lane] : ~0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mine = min(mine, __shfl_xor_sync(0xffffffffu, mine, o));
+    if (mine != ~0ull) { const int c = (int)(mine & 0xffffffffu); paired = c < CAND; limit = limit_of(c); }
   }
   const int n_ent = paired ? p.n_units : 2 * p.n_units, e0 = paired ? 0 : p.n_units;
   for (int e = threadIdx.x; e < n_ent; e += blockDim.x) {
