@@ -90,6 +90,9 @@ struct Args {
   bf16 *O;                                   // [R][Hq*hd]
   float *part_O;                             // [CTA][tile of the pair][hd / 4][128 rows][4]: a warp's stores are contiguous
   float2 *part_ml;                           // [CTA][tile of the pair][128 rows] (reference max, sum)
+  // early: plan, row metadata and page table were written before the kernel in front of this one started, and that one lets its
+  // successor in only once its own predecessors are complete, so they are read ahead of pdl_wait()
+  int early;
   int *status;
   unsigned long long *tile_count;            // diagnostics: += steps this CTA computes (null = off)
 };
@@ -323,8 +326,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   const uint32_t tmem_S = tmem, tmem_O = tmem + 4 * PAGE;             // per stream: 2 x 64 columns of S, HD columns of O
   volatile int *abortp = &ctl.abort_flag;
   pdl_trigger();              // not before the tensor memory is ours (see gemm_tc_kernel)
-  pdl_wait();                 // everything below reads what earlier kernels of the pass wrote
-  if (threadIdx.x == 0) tl_go(tl);
+  if (!a.early) pdl_wait();
 
   // ---- which work item (every thread reads it: no barrier before the first loads go out) ----
   const int kvh = blockIdx.x % a.Hkv, item_no = blockIdx.x / a.Hkv;
@@ -343,6 +345,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     if (np > 0) {
       const bool is_k = warp == 0;
       const uint64_t pol = sm100::policy_evict_last();
+      const int32_t *table = a.page_table + (size_t)item.seq * a.pages_per_seq;
+      const int n_table = min(item.n_cache_pages, item.p_end) - p_begin;         // pages of this item that the table backs
+      int cur = lane < n_table ? table[p_begin + lane] : 0, next = 0;
+      pdl_wait();                                      // Q, K and V are the previous kernel's output
+      if (threadIdx.x == 0) tl_go(tl);
       if (!is_k && sm100::elect_one()) {
         const uint32_t qb = sm100::smem_u32(&ctl.q_full);
         sm100::mbar_expect_tx(qb, (uint32_t)(NH * rows_used * 128 * (pair ? 2 : 1)));
@@ -350,9 +357,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
           for (int h = 0; h < NH; ++h)
             sm100::tma_load_3d(smem0 + L::Q_OFF + t * L::Q_BYTES + h * (128 * 128), &tmQ, qb, h * 64, kvh * a.G, row0 + t * a.spt, pol);
       }
-      const int32_t *table = a.page_table + (size_t)item.seq * a.pages_per_seq;
-      const int n_table = min(item.n_cache_pages, item.p_end) - p_begin;         // pages of this item that the table backs
-      int cur = lane < n_table ? table[p_begin + lane] : 0, next = 0;
       const CUtensorMap *tm = is_k ? &tmK : &tmV, *tm_loc = is_k ? &tmKloc : &tmVloc;
       const int base = is_k ? a.page_base_k : a.page_base_v;
       const uint32_t full0 = sm100::smem_u32(is_k ? ctl.k_full : ctl.v_full), empty0 = sm100::smem_u32(is_k ? ctl.k_empty : ctl.v_empty);
@@ -551,6 +555,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       l_run = l_run * alpha + (sa + sb);
     }
     // ---- output: O is complete once the last P V has finished ----
+    pdl_wait();                                          // (long over; the stores below must not overtake it formally either)
     if (ok && nj > 1) ok = wait_s(nj);                   // (P V of the last step but one; in order, so that the parity wait below is unambiguous)
     if (ok && nj > 0) ok = wait_s(nj + 1);
     sm100::tc_fence_after();
@@ -658,13 +663,14 @@ template <int HD>
 __global__ void __launch_bounds__(256)
 attn_combine_kernel(const Args a, TlSlot tl) {
   pdl_trigger();
-  pdl_wait();
-  if (threadIdx.x == 0) tl_go(tl);
+  if (!a.early) pdl_wait();
   constexpr int BLOCKS = HD / 16;
   const int w = blockIdx.x / BLOCKS, kvh = w % a.Hkv;
   const int cg = (blockIdx.x % BLOCKS) * 2 + (threadIdx.x >> 7), m = threadIdx.x & 127;
   const Tile t = a.tiles[w / a.Hkv];
   const int slot = t.row0 + m / a.G;
+  pdl_wait();
+  if (threadIdx.x == 0) tl_go(tl);
   if (t.n_items > 1 && m < a.spt * a.G && slot < t.row_end) {
     const size_t part = ((size_t)t.item0 * a.Hkv + kvh) * 2 + t.sub;
     const float2 *ml = a.part_ml + part * 128 + m;

@@ -291,8 +291,8 @@ rope_kv_kernel(const SLAB *__restrict__ partials, int S, size_t partial_stride, 
                bf16 *__restrict__ Q, bf16 *__restrict__ Kpool, bf16 *__restrict__ Vpool,
                bf16 *__restrict__ Kloc, bf16 *__restrict__ Vloc,
                const bf16 *__restrict__ bias, const bf16 *__restrict__ qn, const bf16 *__restrict__ kn, float eps, TlSlot tl) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();             // in this order: the attention kernel relies on it (see attn_tc::Args::early)
   if (threadIdx.x == 0) tl_go(tl);
   // a work unit is 4 consecutive dims i..i+3 of the first half of one
   // head together with their rotation partners i+hd/2..

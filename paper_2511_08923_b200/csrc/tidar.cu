@@ -515,8 +515,8 @@ attn_tc::PlanArgs attention_plan(const tidar_ctx *c, int R, int rows_per_group) 
 // kernel, about 5 us, and saves half of 0.56 us per page at best.
 bool may_split(int n_keys) { return n_keys > 12 * attn_tc::PAGE; }
 
-// Attention of the pass that plan p was made for (the plan itself is in device memory by then).
-void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMaps &m, const KvGeom &g, bf16 *O) {
+// Attention of the pass that plan p was made for (the plan itself is in device memory by then).  early: see attn_tc::Args.
+void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMaps &m, const KvGeom &g, bf16 *O, bool early) {
   const tidar_config &cf = c->cfg;
   attn_tc::Args a{};
   a.G = cf.n_q_heads / cf.n_kv_heads; a.Hq = cf.n_q_heads; a.Hkv = cf.n_kv_heads; a.spt = p.spt;
@@ -525,6 +525,7 @@ void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMap
   a.page_table = g.page_table; a.pages_per_seq = g.pages_per_seq;
   a.page_base_k = m.page_base_k; a.page_base_v = m.page_base_v;
   a.scale_log2 = 1.4426950408889634f / sqrtf((float)cf.head_dim);
+  a.early = early ? 1 : 0;
   a.O = O; a.part_O = c->attn_part_O; a.part_ml = c->attn_part_ml; a.status = c->d_status;
   a.tile_count = c->count_tiles ? c->d_tl + 2 * tidar_ctx::TL_MAX : nullptr;
   const int grid = p.max_items * p.Hkv;
@@ -623,7 +624,7 @@ int forward_rows(tidar_ctx *c, int R, bool with_head, int rows_per_group, const 
     }
     if (tc) {
       AttnMaps am{&c->tm_q, &c->tm_kv, &c->tm_kv, &c->tm_kloc, &c->tm_vloc, (2 * l) * c->n_pages, (2 * l + 1) * c->n_pages};
-      launch_attention_tc(c, plan, am, g, c->O);
+      launch_attention_tc(c, plan, am, g, c->O, true);          // behind the RoPE kernel
     } else {
       launch_attention(c, c->Q, Kp, Vp, g, c->Kloc, c->Vloc, c->O, R);
     }
@@ -1557,7 +1558,7 @@ int tidar_attention(tidar_ctx *c, const void *q, const void *k_pages, const void
         !encode_local_map(c, &tkl, k_local, (long long)n_seqs * k * k) || !encode_local_map(c, &tvl, v_local, (long long)n_seqs * k * k))
       return fail(c, TIDAR_ECUDA, "cuTensorMapEncodeTiled failed for an attention operand");
     AttnMaps am{&tq, &tk, &tv, &tkl, &tvl, 0, 0};
-    launch_attention_tc(c, plan, am, g, (bf16 *)out);
+    launch_attention_tc(c, plan, am, g, (bf16 *)out, false);   // behind the kernel that makes the plan
   } else {
     launch_attention(c, (const bf16 *)q, (const bf16 *)k_pages, (const bf16 *)v_pages, g, (const bf16 *)k_local, (const bf16 *)v_local,
                      (bf16 *)out, R);
