@@ -449,13 +449,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 #pragma unroll
           for (int i = 0; i < NCH; ++i) {
             if (i * 16 < ncols) {
-              const int r0 = row_block + c_begin + i * 16;             // (one instruction per block: columns are rows in order)
-              float *p = out + (long long)r0 * g.ldo;
-              const int rows_left = n_ok ? R_live - r0 : 0;
 #pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                if (j < rows_left) atomicAdd(p, __uint_as_float(v[i][j]));
-                p += g.ldo;
+              for (int h = 0; h < 2; ++h) {
+                const int r0 = row_block + col_row(c_begin + i * 16 + h * 8);
+                float *p = out + (long long)r0 * g.ldo;
+                const int rows_left = n_ok ? R_live - r0 : 0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  if (j < rows_left) atomicAdd(p, __uint_as_float(v[i][h * 8 + j]));
+                  p += g.ldo;
+                }
               }
             }
           }
@@ -620,11 +623,10 @@ inline CUresult encode_2d_small(EncodeTiledFn fn, CUtensorMap *tm, const void *b
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
-// Row-block geometry for R activation rows.
-inline void plan_rows(int R, Args &a, int max_rows = MAX_ROWS) {
-  const int block = std::min(max_rows, BLOCK_ROWS);
-  a.n_rb = R <= max_rows ? 1 : (R + block - 1) / block;
-  const int per = (R + a.n_rb - 1) / a.n_rb;
+// Row-block geometry for R activation rows in n_rb blocks.
+inline void plan_rows(int R, Args &a, int n_rb) {
+  a.n_rb = n_rb;
+  const int per = (R + n_rb - 1) / n_rb;
   a.rb_rows = (per + 15) / 16 * 16;
   a.n1 = a.rb_rows; a.n2 = 0;
   if (a.rb_rows > 256) { a.n1 = ((a.rb_rows / 2 + 15) / 16) * 16; a.n2 = a.rb_rows - a.n1; }
@@ -652,19 +654,24 @@ inline int plan_splits(int n_items_unsplit, int kb_total, int workers, int max_s
   }
   return best;
 }
-// The same for several row blocks, where slabs are large: the split with the least estimated time.  Whole waves of items;
+// The same for several row blocks, where slabs are large: blocks and split with the least estimated time.  Whole waves of items;
 // per stage of K 2.15 cycles per row at 1.75 GHz; 1 us to hand an accumulator over; and S slabs of R x N floats written, and
-// read again by the next kernel.  (Chosen for whole waves alone, the O projection of 1152 rows was split 4 ways and a
-// 4 k first pass spent 85 us per norm on slabs, 30 now.)
-inline int plan_splits_blocks(const Args &a, int workers, int max_splits, int min_kb) {
-  auto us = [&](int S) {
-    const long long items = (long long)a.n_rb * a.n_tiles * S, waves = (items + workers - 1) / workers;
-    return (double)waves * (((a.kb_total + S - 1) / S) * ((2.15 * a.rb_rows + 50.0) / 1750.0) + 1.0) + S * ((double)a.R * a.N * 6.0 / 5.0e6);
-  };
-  int best = 1;
-  for (int s = 2; s <= max_splits && a.kb_total / s >= min_kb; ++s)
-    if (us(s) < us(best) - 1e-9) best = s;
-  return best;
+// read again by the next kernel (max_splits = 0: no slabs, nothing is split).  Blocks take one instruction (up to 256 rows) or two (288):
+// fewer blocks where that saves a wave.  (Chosen for whole waves alone, the O projection of 1152 rows was split 4 ways and a
+// 4 k first pass spent 85 us per norm on slabs, 30 now.  1152 rows, 8B-class: O and its norm take 47 + 23 us as five blocks of 240 rows
+// in two splits and 38 + 5.5 us as four of 288, unsplit; down and its norm 103 + 29 and 91 + 5.5 us.)
+inline void plan_blocks(Args &a, int workers, int max_splits, int min_kb) {
+  double best = 1e30;
+  Args pick = a;
+  for (int block : {BLOCK_ROWS, MAX_ROWS}) {
+    plan_rows(a.R, a, (a.R + block - 1) / block);
+    for (int S = 1; S == 1 || (S <= max_splits && a.kb_total / S >= min_kb); ++S) {
+      const long long items = (long long)a.n_rb * a.n_tiles * S, waves = (items + workers - 1) / workers;
+      const double us = (double)waves * (((a.kb_total + S - 1) / S) * ((2.15 * a.rb_rows + 50.0) / 1750.0) + 1.0) + (max_splits ? S * ((double)a.R * a.N * 6.0 / 5.0e6) : 0.0);
+      if (us < best - 1e-9) { best = us; pick = a; pick.S = S; }
+    }
+  }
+  a = pick;
 }
 
 }  // namespace gemm_tc

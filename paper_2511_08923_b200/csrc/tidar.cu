@@ -348,15 +348,18 @@ gemm_tc::Args plan_gemm(const tidar_ctx *c, int mode, int R, int N, int K, int f
   gemm_tc::Args a{};
   a.R = R; a.N = N; a.K = K;
   const bool small = small_gemm(mode, R, N, K);
-  gemm_tc::plan_rows(R, a, small ? gemm_tc::SMALL_ROWS : gemm_tc::MAX_ROWS);
+  const int max_rows = small ? gemm_tc::SMALL_ROWS : gemm_tc::MAX_ROWS;
+  gemm_tc::plan_rows(R, a, (R + max_rows - 1) / max_rows);
   const int kps = gemm_tc::k_per_stage(small), tile = gemm_tc::tile_rows(small);
   const int workers = small ? c->n_sms : c->n_sms / 2;             // CTAs, or pairs of CTAs, that work on items
   a.n_tiles = (N + tile - 1) / tile;
   a.kb_total = (K / gemm_tc::TILE_K + kps - 1) / kps;
   a.S = 1; a.fused_items = 0; a.tile_b0 = 0; a.n_tiles_b = 0;
+  const bool blocks = a.n_rb > 1 && !small;
+  if (blocks) gemm_tc::plan_blocks(a, workers, mode == gemm_tc::MODE_SLAB ? c->S_max : 0, 4);
   if (mode == gemm_tc::MODE_SLAB) {
     a.n_tiles_b = a.n_tiles;
-    a.S = force_S > 0 ? std::min(force_S, a.kb_total) : a.n_rb > 1 && !small ? gemm_tc::plan_splits_blocks(a, workers, c->S_max, 4)
+    a.S = force_S > 0 ? std::min(force_S, a.kb_total) : blocks ? a.S
                       : gemm_tc::plan_splits(a.n_rb * a.n_tiles, a.kb_total, workers, c->S_max, 4 / kps, 3.0 / kps);
     a.ldo = N; a.slab_stride = (long long)R * N;
   } else if (mode == gemm_tc::MODE_SWIGLU) {
@@ -393,7 +396,7 @@ int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const tida
   if (mode == gemm_tc::MODE_SLAB) {
     a.out = slab_out ? (void *)slab_out : (void *)c->partials;
     a.slab_bf16 = (slab_out || !c->slab_bf16) ? 0 : 1;   // an explicit output buffer always gets exact fp32 slabs
-    if (residual && a.S == 1 && a.n2 == 0 && !a.slab_bf16) { a.out = residual; a.accumulate = 1; }
+    if (residual && a.S == 1 && !a.slab_bf16) { a.out = residual; a.accumulate = 1; }
   } else if (mode == gemm_tc::MODE_SWIGLU) {
     a.H = c->H;
     a.out = c->partials; a.slab_bf16 = c->slab_bf16 ? 1 : 0;

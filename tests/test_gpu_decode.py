@@ -1,5 +1,6 @@
 """CUDA path vs oracle on the decode step, through the C ABI (needs a B200)."""
 import itertools
+from dataclasses import replace
 
 import numpy as np
 import pytest
@@ -430,6 +431,27 @@ def test_long_first_pass_in_one_chunk(tiny, impl):
     np.testing.assert_array_equal(outs[0][1][0][0], outs[1][1][0][0]); np.testing.assert_array_equal(outs[0][1][0][1], outs[1][1][0][1])
     if top1_margin(fo.logits[n - 1]) > MARGIN:
         assert outs[0][0] == outs[1][0] == c
+
+
+@pytest.mark.parametrize("n", [1025, 1100, 1152])
+def test_first_pass_in_blocks_of_two_instructions(n):
+    """Rows for which four blocks of up to 288 rows need one wave of a 3840-wide projection and five blocks of up to 256 need two:
+    the result, unsplit, is added to the residual stream from accumulators that two instructions filled.  Against the replay kernels."""
+    sh, _ = make_model("tiny")
+    sh = replace(sh, d_model=3840, n_layers=1, n_q_heads=2, n_kv_heads=1, head_dim=64, d_ffn=128)
+    wt = gen_model_weights_(sh)
+    k = sh.k
+    prompt = prompt_ids(sh, n - k, seed=5)
+    hidden = []
+    for impl in IMPLS:
+        t = _gpu(sh, wt, impl, max_seq_len=1280, prefill_rows=1152)
+        t.prefill(0, prompt, k)
+        n_rows, _ = t.last_rows()
+        hidden.append([t.hidden(l, 0, n_rows) for l in range(2)])
+        _close(t)
+    np.testing.assert_array_equal(hidden[0][0], hidden[1][0])
+    assert np.abs(hidden[0][1] - hidden[1][1]).max() <= TOL_LOGITS
+    assert np.abs(hidden[0][1] - hidden[0][0]).max() > 3 * TOL_LOGITS          # the layer adds something
 
 
 def test_two_steps_in_flight_match_one_at_a_time():
