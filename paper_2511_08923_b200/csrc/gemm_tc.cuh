@@ -64,7 +64,10 @@ __host__ __device__ constexpr int tile_rows(bool small) { return small ? TILE_N 
 
 // MODE_SAMPLE is MODE_ARGMAX with Gumbel noise added to the tempered logits (a draw per row instead of
 // the argmax); it is a mode of its own so that the greedy LM head carries none of its registers.
-enum Mode { MODE_SLAB = 0, MODE_SWIGLU = 1, MODE_ARGMAX = 2, MODE_SAMPLE = 3 };
+// MODE_LSE (likelihood scoring): the logits never leave the chip; each warp of each tile leaves, per row, the maximum of its 32 logits and
+// the sum of their exponentials below it, and the lane that owns a row's target id leaves that logit.  No state is carried from
+// tile to tile, so the row block varies fastest as in the projections and a weight tile is read once from HBM.
+enum Mode { MODE_SLAB = 0, MODE_SWIGLU = 1, MODE_ARGMAX = 2, MODE_SAMPLE = 3, MODE_LSE = 4 };
 
 // A "tile" below is what an item covers: tile_rows(small) weight rows.
 struct Args {
@@ -91,11 +94,15 @@ struct Args {
   // MODE_SAMPLE: the compared value is logit * inv_temp + Gumbel noise of (skey[row], id),
   // i.e. a draw from softmax(logits / temperature) per row (see gumbel_noise); the dump keeps the raw logits
   float inv_temp; const uint32_t *skey;
+  // MODE_LSE: (max, sum) of lse_parts(N) groups of 32 ids, [group][R]; the target id of each row, and its logit
+  float2 *lse; const int32_t *target; float *tgt_logit;
   int warm_epilogue;        // MODE_SWIGLU: walk through the epilogue once before the first accumulator is ready (see the kernel)
   int *status;              // device word set to 1 when a bounded wait gave up
   __host__ __device__ int tile_b0_or_all() const { return n_tiles_b ? tile_b0 : n_tiles; }   // tiles per row block in the fused region
   __host__ __device__ int total_items() const { return fused_items + n_rb * n_tiles_b * S; }
 };
+
+__host__ __device__ inline int lse_parts(int N) { return (N + tile_rows(false) - 1) / tile_rows(false) * (tile_rows(false) / 32); }
 
 struct Item { int rb, tile, split, kb0, kb1; bool fused; };
 // Item order.  With several row blocks (a long first pass) the row block varies fastest: the CTAs
@@ -445,18 +452,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         const int nc = n - g.tile_b0 * tile_rows(SMALL);
         const bool n_ok = n < g.N;
         if (g.accumulate) {
+          constexpr int RUN = SMALL ? 16 : 8;            // columns that are consecutive rows
           float *out = reinterpret_cast<float *>(g.out) + nc;
 #pragma unroll
           for (int i = 0; i < NCH; ++i) {
             if (i * 16 < ncols) {
 #pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                const int r0 = row_block + col_row(c_begin + i * 16 + h * 8);
+              for (int h = 0; h < 16; h += RUN) {
+                const int r0 = row_block + col_row(c_begin + i * 16 + h);
                 float *p = out + (long long)r0 * g.ldo;
                 const int rows_left = n_ok ? R_live - r0 : 0;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  if (j < rows_left) atomicAdd(p, __uint_as_float(v[i][h * 8 + j]));
+                for (int j = 0; j < RUN; ++j) {
+                  if (j < rows_left) atomicAdd(p, __uint_as_float(v[i][h + j]));
                   p += g.ldo;
                 }
               }
@@ -568,6 +576,50 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
               }
             }
             if (val[0] > best_v[grp] || (val[0] == best_v[grp] && idx[0] < best_i[grp])) { best_v[grp] = val[0]; best_i[grp] = idx[0]; }
+          }
+        }
+      }
+      else if (MODE == MODE_LSE) {
+        const bool n_ok = n < g.N;
+        float2 *out = g.lse + (long long)((n0 + q * 32) >> 5) * g.R;
+#pragma unroll
+        for (int grp = 0; grp < (NCH + 1) / 2; ++grp) {
+          if (grp * 32 < ncols) {
+            // lane l finishes column 32 * grp + l
+            const int r = row_block + col_row(c_begin + grp * 32 + lane);
+            const bool live = grp * 32 + lane < ncols && r < g.R;
+            float val[32], mx[32];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              const int i = grp * 2 + (j >> 4);
+              val[j] = n_ok && i < NCH && i * 16 < ncols ? __uint_as_float(v[i < NCH ? i : NCH - 1][j & 15]) : -INFINITY;
+              mx[j] = val[j];
+            }
+            const int tg = live ? g.target[r] - (n0 + q * 32) : -1;
+            for (uint32_t hit = __ballot_sync(0xffffffffu, tg >= 0 && tg < 32); hit; hit &= hit - 1) {      // (rare)
+              const int j = __ffs(hit) - 1, owner = __shfl_sync(0xffffffffu, tg, j), row = __shfl_sync(0xffffffffu, r, j);
+              float x = 0.f;
+#pragma unroll
+              for (int jj = 0; jj < 32; ++jj) if (jj == j) x = val[jj];
+              if (lane == owner) g.tgt_logit[row] = x;
+            }
+            // maximum and sum over the lanes by recursive halving, as in MODE_ARGMAX
+#pragma unroll
+            for (int h = 16; h >= 1; h >>= 1) {
+              const bool up = lane & h;
+#pragma unroll
+              for (int j = 0; j < h; ++j) mx[j] = fmaxf(up ? mx[j + h] : mx[j], __shfl_xor_sync(0xffffffffu, up ? mx[j] : mx[j + h], h));
+            }
+            const float ref = mx[0] == -INFINITY ? 0.f : mx[0];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) val[j] = __expf(val[j] - __shfl_sync(0xffffffffu, ref, j));
+#pragma unroll
+            for (int h = 16; h >= 1; h >>= 1) {
+              const bool up = lane & h;
+#pragma unroll
+              for (int j = 0; j < h; ++j) val[j] = (up ? val[j + h] : val[j]) + __shfl_xor_sync(0xffffffffu, up ? val[j] : val[j + h], h);
+            }
+            if (live) out[r] = make_float2(mx[0], val[0]);
           }
         }
       }

@@ -615,6 +615,38 @@ __global__ void score_finish_kernel(const float *__restrict__ run_max, const flo
   if (r < R) logprob[r] = tgt_logit[r] - (run_max[r] + logf(run_sum[r]));
 }
 
+// The same from per-group (max, sum) pairs [parts][R]; 16 rows per block, 32 threads share a row's groups (fixed order).
+__global__ void __launch_bounds__(512)
+score_merge_kernel(const float2 *__restrict__ lse, int parts, const float *__restrict__ tgt_logit, int R, float *__restrict__ logprob) {
+  __shared__ float2 red[32][16];
+  const int i = threadIdx.x & 15, sub = threadIdx.x >> 4, r = blockIdx.x * 16 + i;
+  float M = -INFINITY, sum = 0.f;
+  pdl_wait();
+  if (r < R) {
+    for (int p0 = sub; p0 < parts; p0 += 32 * 8) {
+      float2 v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = p0 + u * 32 < parts ? lse[(size_t)(p0 + u * 32) * R + r] : make_float2(-INFINITY, 0.f);
+      float m = M;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) m = fmaxf(m, v[u].x);
+      const float ref = m == -INFINITY ? 0.f : m;
+      sum *= __expf(M - ref);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) sum += v[u].y * __expf(v[u].x - ref);
+      M = m;
+    }
+  }
+  red[sub][i] = make_float2(M, sum);
+  __syncthreads();
+  if (sub == 0 && r < R) {
+    for (int s = 1; s < 32; ++s) M = fmaxf(M, red[s][i].x);
+    sum = 0.f;
+    for (int s = 0; s < 32; ++s) sum += red[s][i].y * __expf(red[s][i].x - M);
+    logprob[r] = tgt_logit[r] - (M + logf(sum));
+  }
+}
+
 // First-pass finish: settled token = argmax of the last prompt row; drafts = argmax
 // of mask rows 1..k-1 (paper Section 3.2, start of generation).
 // row_first: the row whose argmax is the settled token (the last prompt row, or the extra row that

@@ -65,7 +65,6 @@ struct tidar_ctx {
   float *d_run_max = nullptr, *d_run_sum = nullptr, *d_tgt_logit = nullptr, *d_logprob = nullptr;   // likelihood scoring, per row
   int32_t *d_target = nullptr;
   struct WMap { CUtensorMap full, small; };   // a weight matrix for the full and the SMALL instances of the projection kernel
-  std::vector<WMap> tm_lm_chunks;   // the LM head in vocabulary chunks of lm_chunk rows (scoring)
   int32_t *d_seq_len = nullptr, *d_block = nullptr, *d_page_table = nullptr, *d_step_seqs = nullptr, *d_forced = nullptr,
           *d_step_n = nullptr, *d_step_L = nullptr, *d_prompt = nullptr, *d_arg_idx = nullptr;
   float *X = nullptr, *partials = nullptr, *rope_cos = nullptr, *rope_sin = nullptr, *d_arg_val = nullptr,
@@ -187,7 +186,7 @@ void layout(tidar_ctx &x, void *arena, size_t *bytes) {
   x.S_max = c.impl == 0 ? MAX_SLABS : 4;
   const size_t R = x.R_cap;
   const size_t widest = std::max<size_t>({(size_t)x.S_max * x.n_qkv, (size_t)x.S_max * c.d_model, (size_t)2 * c.d_ffn,
-                                          (size_t)x.lm_chunk});
+                                          (size_t)x.lm_chunk, (size_t)2 * gemm_tc::lse_parts(c.vocab)});
   x.partial_stride = 0;  // set per projection
   Carver cv(arena);
   x.kv = cv.take<bf16>((size_t)c.n_layers * 2 * x.pool_stride);
@@ -388,8 +387,10 @@ gemm_tc::Args plan_gemm(const tidar_ctx *c, int mode, int R, int N, int K, int f
 //                nothing split, the result is added to it instead and *S_out is 0
 //   MODE_SWIGLU: bf16 c->H [R][N/2]
 //   MODE_ARGMAX: candidates for argmax_merge_kernel (+ optional logits dump)
+//   MODE_LSE   : pieces of the rows' log-sum-exp in c->partials for score_merge_kernel, and the logits of `target` [R]
 int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const tidar_ctx::WMap &tmW, int R, int N, int K, int cls,
-                   int *S_out, size_t *stride_out, float *slab_out = nullptr, int force_S = 0, float *residual = nullptr) {
+                   int *S_out, size_t *stride_out, float *slab_out = nullptr, int force_S = 0, float *residual = nullptr,
+                   const int32_t *target = nullptr) {
   gemm_tc::Args a = plan_gemm(c, mode, R, N, K, force_S);
   const bool small = small_gemm(mode, R, N, K);
   const int rem_tiles = mode == gemm_tc::MODE_SWIGLU ? a.n_tiles_b : 0;
@@ -400,6 +401,8 @@ int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const tida
   } else if (mode == gemm_tc::MODE_SWIGLU) {
     a.H = c->H;
     a.out = c->partials; a.slab_bf16 = c->slab_bf16 ? 1 : 0;
+  } else if (mode == gemm_tc::MODE_LSE) {
+    a.lse = reinterpret_cast<float2 *>(c->partials); a.target = target; a.tgt_logit = c->d_tgt_logit;
   } else {
     a.cand_val = c->cand_val; a.cand_idx = c->cand_idx; a.cand_ld = lm_head_ctas(c, R, N) * 4; a.dump = c->dbg_logits; a.ld_dump = c->cfg.vocab; a.col0 = 0;
     a.inv_temp = c->cfg.temperature > 0.f ? 1.0f / c->cfg.temperature : 0.f; a.skey = c->meta.skey + c->head_row0;
@@ -422,6 +425,7 @@ int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const tida
   else if (small) launch_pdl(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU, true>, grid, gemm_tc::THREADS, smem, c->stream, tmW.small, *tmA, a, l.tl);
   else if (mode == gemm_tc::MODE_SLAB) launch_pdl_cluster(2, gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
   else if (mode == gemm_tc::MODE_SWIGLU) launch_pdl_cluster(2, gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
+  else if (mode == gemm_tc::MODE_LSE) launch_pdl_cluster(2, gemm_tc::gemm_tc_kernel<gemm_tc::MODE_LSE>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
   else if (a.inv_temp > 0.f) launch_pdl_cluster(2, gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SAMPLE>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
   else launch_pdl_cluster(2, gemm_tc::gemm_tc_kernel<gemm_tc::MODE_ARGMAX>, grid, gemm_tc::THREADS, smem, c->stream, tmW.full, *tmA, a, l.tl);
   if (rem_tiles) {
@@ -701,11 +705,6 @@ int init_tensor_core_path(tidar_ctx *c) {
   auto enc = [&](tidar_ctx::WMap *tm, const void *p, int rows, int cols) { return encode_weights(c, tm, p, rows, cols); };
   c->tm_wqkv.resize(cf.n_layers); c->tm_wo.resize(cf.n_layers); c->tm_wgu.resize(cf.n_layers); c->tm_wdown.resize(cf.n_layers);
   bool ok = enc(&c->tm_lm, c->lm_head, cf.vocab, d);
-  c->tm_lm_chunks.resize((cf.vocab + c->lm_chunk - 1) / c->lm_chunk);
-  for (size_t ci = 0; ci < c->tm_lm_chunks.size() && ok; ++ci) {
-    const int v0 = (int)ci * c->lm_chunk;
-    ok = enc(&c->tm_lm_chunks[ci], c->lm_head + (size_t)v0 * d, std::min(c->lm_chunk, cf.vocab - v0), d);
-  }
   for (int l = 0; l < cf.n_layers && ok; ++l)
     ok = enc(&c->tm_wqkv[l], c->wqkv[l], c->n_qkv, d) && enc(&c->tm_wo[l], c->wo[l], d, qo) &&
          enc(&c->tm_wgu[l], c->wgu[l], 2 * cf.d_ffn, d) && enc(&c->tm_wdown[l], c->wdown[l], d, cf.d_ffn);
@@ -749,6 +748,7 @@ int init_tensor_core_path(tidar_ctx *c) {
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_ARGMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
+  CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_LSE>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SAMPLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
   return TIDAR_OK;
 }
@@ -1323,18 +1323,21 @@ int tidar_score(tidar_ctx *c, int32_t seq, const int32_t *ids, int32_t n, float 
     }
     c->split_keys = may_split(row0 + rows);
     if (int rc = forward_rows(c, rows, false, rows)) return rc;      // ends with the final norm in c->A
-    for (int v0 = 0, ci = 0; v0 < cf.vocab; v0 += c->lm_chunk, ++ci) {
-      const int nc = std::min(c->lm_chunk, cf.vocab - v0);
-      int S = 1; size_t stride = 0;
-      if (cf.impl == 0) {
-        if (int rc = gemm_tc_launch(c, gemm_tc::MODE_SLAB, c->A, c->R_cap, c->tm_lm_chunks[ci], rows, nc, d, TIDAR_TC_LMHEAD, &S, &stride, c->partials, 1)) return rc;
-      } else {
-        if (int rc = gemm_partials(c, c->A, c->R_cap, c->lm_head + (size_t)v0 * d, nullptr, rows, nc, d, c->partials, &S, &stride, TIDAR_TC_LMHEAD)) return rc;
-      }
+    const int32_t *target = c->d_prompt + row0 + 1;
+    if (cf.impl == 0) {
+      // (Through fp32 logits in 16384-id chunks, each reduced by a kernel of its own, 1776 rows of a 1536-wide 152 k vocabulary took 1.39 ms;
+      // this way 0.63, 1.3 PFLOP/s.)
+      if (int rc = gemm_tc_launch(c, gemm_tc::MODE_LSE, c->A, c->R_cap, c->tm_lm, rows, cf.vocab, d, TIDAR_TC_LMHEAD, nullptr, nullptr, nullptr, 0, nullptr, target)) return rc;
       Launch ll(c, TIDAR_TC_LMHEAD);
-      score_chunk_kernel<<<rows, 256, 0, c->stream>>>(c->partials, nc, nc, v0, v0 == 0, c->d_prompt + row0 + 1, c->d_run_max, c->d_run_sum, c->d_tgt_logit);
-    }
-    {
+      launch_pdl(score_merge_kernel, (rows + 15) / 16, 512, 0, c->stream, (const float2 *)c->partials, gemm_tc::lse_parts(cf.vocab), c->d_tgt_logit, rows, c->d_logprob);
+    } else {
+      for (int v0 = 0; v0 < cf.vocab; v0 += c->lm_chunk) {
+        const int nc = std::min(c->lm_chunk, cf.vocab - v0);
+        int S = 1; size_t stride = 0;
+        if (int rc = gemm_partials(c, c->A, c->R_cap, c->lm_head + (size_t)v0 * d, nullptr, rows, nc, d, c->partials, &S, &stride, TIDAR_TC_LMHEAD)) return rc;
+        Launch ll(c, TIDAR_TC_LMHEAD);
+        score_chunk_kernel<<<rows, 256, 0, c->stream>>>(c->partials, nc, nc, v0, v0 == 0, target, c->d_run_max, c->d_run_sum, c->d_tgt_logit);
+      }
       Launch ll(c, TIDAR_TC_LMHEAD);
       score_finish_kernel<<<(rows + 127) / 128, 128, 0, c->stream>>>(c->d_run_max, c->d_run_sum, c->d_tgt_logit, rows, c->d_logprob);
     }

@@ -94,6 +94,23 @@ def test_likelihood_scoring_matches_causal_log_softmax(tiny, impl):
         _close(t)
 
 
+@pytest.mark.parametrize("n,vocab", [(2, 129), (34, 257), (290, 2000), (578, 1100)])
+def test_scoring_without_logits_matches_the_replay_kernels(n, vocab):
+    """The LM head that keeps only (max, sum) pairs and the target's logit: one row, one and two instructions, several row blocks; ragged last
+    tiles; targets at both ends of the vocabulary."""
+    sh, wt = make_model("tiny", vocab=vocab)
+    ids = prompt_ids(sh, n, seed=n)
+    ids[1] = vocab - 1
+    ids[n // 2 + 1:n // 2 + 2] = 0
+    got = []
+    from paper_2511_08923_b200 import Tidar, pack_weights
+    for impl in IMPLS:
+        t = Tidar(sh, pack_weights(wt, "cuda:0"), k_max=4, max_batch=1, max_seq_len=1024, debug=0, impl=impl, guard_bytes=64 * 1024, prefill_rows=640)
+        got.append(t.score(0, ids))
+        _close(t)
+    assert np.abs(got[0] - got[1]).max() <= TOL_LOGITS
+
+
 def test_autoregressive_mode_at_the_benchmark_widths():
     """The one-slot step and the scoring pass at the 8B-class widths (two layers, 8192-entry vocabulary so
     that the oracle stays fast): one-row projections (a 16-row MMA block), 4096-wide rows, 32 / 8 heads.
