@@ -21,7 +21,7 @@
 // What bounds it: shared memory.  A step's operands are 64 KB read (Q 32, K 16, V 16) and up to 32 KB written by
 // the loads, 500 - 750 cycles at 128 B per cycle against 512 cycles of MMAs (a product with N = 64 takes 48 cycles, not
 // 32, for the 6 KB it reads); a step takes 0.53 - 0.56 us, 0.93 - 0.98 kcycles, on an SM.  Whole calls, 32/8
-// heads of 128, 272 rows, 1 k / 4 k / 16 k / 32 k cached positions: 22.6 / 33 / 85 / 156 us; the kernel before this one
+// heads of 128, 272 rows, 1 k / 4 k / 16 k / 32 k cached positions: 22.0 / 32.7 / 82 / 148 us; the kernel before this one
 // (two CTAs per SM, one tile and one stream each, the same split for every sequence) took 26.4 / 40 / 97 / 197 us.
 //   PAIR of tiles: A and B are two query tiles, each K/V page serves both: half the loads, and 80
 //     instead of 96 KB through shared memory per step.

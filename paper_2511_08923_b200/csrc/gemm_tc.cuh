@@ -37,7 +37,7 @@ namespace gemm_tc {
 constexpr int TILE_N = 128;         // weight rows per tile (TMEM lanes)
 constexpr int TILE_K = 64;          // bf16 elements per 128-byte swizzled row
 constexpr int MAX_ROWS = 288;       // activation rows of a single row block (2 x 144 TMEM columns)
-constexpr int BLOCK_ROWS = 256;     // activation rows per row block when there are several (one instruction)
+constexpr int BLOCK_ROWS = 256;     // activation rows of a row block that one instruction covers (see plan_blocks)
 constexpr int EPI_WARPS = 8;
 constexpr int ROLE_WARPS = 4;      // warpgroup 0: weight producer, MMA issuer, stage watcher, activation producer
 constexpr int THREADS = 32 * (ROLE_WARPS + EPI_WARPS);
