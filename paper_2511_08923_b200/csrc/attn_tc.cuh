@@ -141,7 +141,7 @@ struct RowKeys { int nvis, loc0, nloc, seq; };
 
 template <typename ROW>
 __device__ inline void plan_block(const PlanArgs &p, ROW row_keys) {
-  struct Keys { short n_cache, n_pages; int loc_lo; };
+  struct Keys { int n_cache, n_pages, loc_lo; };       // (a sequence of more than 32767 pages fits a B200)
   __shared__ Keys keys[3][PLAN_UNITS];                 // tile 0, tile 1, the unit
   __shared__ int unit_row0[PLAN_UNITS], unit_rend[PLAN_UNITS], unit_seq[PLAN_UNITS];
   __shared__ float ent_us[3 * PLAN_UNITS];             // units, then tiles
@@ -179,7 +179,7 @@ __device__ inline void plan_block(const PlanArgs &p, ROW row_keys) {
       const bool two = row0 + p.spt < row_end;
       const int n_cache = (nv + PAGE - 1) / PAGE, n_pages = n_cache + (h > l ? (h - l + PAGE - 1) / PAGE : 0);
       if (planned) {
-        keys[lane][u] = Keys{(short)n_cache, (short)n_pages, l};
+        keys[lane][u] = Keys{n_cache, n_pages, l};
         const float us = n_pages * (lane == 2 && two ? PAIR_PAGE : SINGLE_PAGE);
         ent_us[lane == 2 ? u : p.n_units + 2 * u + lane] = us;
         atomicMax(&longest_us[lane == 2 ? 0 : 1], __float_as_int(us));
@@ -279,7 +279,7 @@ __device__ inline void plan_block(const PlanArgs &p, ROW row_keys) {
       Item it{};
       it.row0 = unit_row0[u] + (paired ? 0 : (e & 1) * p.spt); it.row_end = unit_rend[u]; it.seq = unit_seq[u];
       it.n_cache_pages = k.n_cache; it.loc_lo = k.loc_lo;
-      it.p_begin = k.n_pages * j / n; it.p_end = k.n_pages * (j + 1) / n;
+      it.p_begin = (int)((long long)k.n_pages * j / n); it.p_end = (int)((long long)k.n_pages * (j + 1) / n);
       it.pair = paired && unit_row0[u] + p.spt < unit_rend[u]; it.split = n > 1;
       p.items[place_s[e] + j] = it;
     }

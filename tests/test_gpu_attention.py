@@ -126,3 +126,42 @@ def test_attention_work_plan(ns, k):
     t = _ctx(64, 4, 2, 8, 32, 0)
     _case(t, 64, 4, 2, k, ns, 31)
     t.close()
+
+
+def test_attention_beyond_32767_pages():
+    """One sequence of 32770 pages.  Scores are small (weights within e^+-0.4 of each other) and V rises with the position, so that the output
+    says which part of the cache was attended to: 0.5 for all of it.  Bound: bf16 rounding of the output, 2^-9 x 0.5, of V (the same,
+    averaged over two million positions) and of P (the same): 4e-3 is four times their sum."""
+    n, k, hq, hd, dev = 32769 * 64 + 30, 2, 2, 64, "cuda:0"
+    pages = (n + k + 63) // 64
+    t = _ctx(hd, hq, 1, k, 1, 0)
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(7)
+
+    def rnd(*shape):
+        return torch.randn(*shape, device=dev, dtype=torch.bfloat16, generator=gen)
+    q, kp = rnd(k * (k + 1), hq, hd) * 0.1, rnd(pages, 1, 64, hd)
+    ramp = torch.arange(pages * 64, device=dev, dtype=torch.float32) / n
+    vp = ramp.to(torch.bfloat16).view(pages, 1, 64, 1).expand(pages, 1, 64, hd).contiguous()
+    kl, vl = rnd(k * k, 1, hd), rnd(k * k, 1, hd)
+    table = torch.randperm(pages, device=dev, generator=gen)
+    kp2, vp2 = torch.empty_like(kp), torch.empty_like(vp)
+    kp2[table], vp2[table] = kp, vp                     # position p lies in page table[p / 64]
+    out = torch.full((k * (k + 1), hq * hd), float("nan"), dtype=torch.bfloat16, device=dev)
+    t.attention(q, kp2, vp2, table.to(torch.int32).view(1, pages), torch.tensor([n], dtype=torch.int32, device=dev), kl, vl, out, 1, k)
+    t.sync()
+    got = out.float().view(k * (k + 1), hq, hd)
+    keys, vals = kp.view(-1, hd)[:n + k].float(), vp.view(-1, hd)[:n + k, 0].double()
+    for r in range(k * (k + 1)):
+        b = (r - k) // k
+        seen = n + r + 1 if r < k else n + b + 1
+        for h in range(hq):
+            s = keys[:seen] @ q[r, h].float() / hd ** 0.5
+            if r >= k:
+                s = torch.cat([s, kl[b * k:(b + 1) * k, 0].float() @ q[r, h].float() / hd ** 0.5])
+            w = torch.softmax(s.double(), 0)
+            want = w[:seen] @ vals[:seen]
+            if r >= k:
+                want = want + w[seen:] @ vl[b * k:(b + 1) * k, 0].double()
+            assert (got[r, h].double() - want).abs().max() <= 4e-3, (r, h)
+    t.close()
