@@ -69,7 +69,7 @@ struct StepIo {
   int32_t *turn, *blocks_done, *status;                      // device
   const int32_t *in[2];                                      // [2][max_batch]: listed sequences, forced lengths
   int32_t *out[2];                                           // [n_seqs][k_max + 1]: L, tokens
-  int32_t *done[2];                                          // [0] = turn + 1 once the slot's results are there, [1] = status
+  int32_t *done[2];                                          // [0] = turn + 1 (the step ran to its end), [1] = status
   int32_t max_batch;
 };
 
@@ -484,8 +484,7 @@ __global__ void slab_sum_kernel(const float *__restrict__ in, int S, size_t stri
 //   next block = target_{L-1}, then the argmax of mask slots (L-1, 1..k-1); with no mask
 //   blocks (plain autoregressive step, k = 1) the next block is target_0 alone.
 // Commits as well (paper Section 3.3): the causal slots' K/V are in the cache at n..n+k-1, committing L of them is
-// n <- n + L.  The last block to finish hands the results over: everything a step wrote is visible to the host
-// once it reads the slot's new turn number.
+// n <- n + L.  The last block to finish closes the step: it moves the turn on and leaves turn number and status with the results.
 // ---------------------------------------------------------------------------
 __global__ void verify_select_kernel(const int32_t *__restrict__ arg_ids, const int32_t *__restrict__ tgt_ids,
                                      const int32_t *__restrict__ step_seqs,

@@ -1,10 +1,7 @@
 // C-ABI entry points and per-step orchestration of the TiDAR decode path.
 #include "../../include/tidar.h"
 
-#include <immintrin.h>
-
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -83,6 +80,7 @@ struct tidar_ctx {
   // is enqueued while the first runs, so the device never waits for the host between steps.
   struct Flight { std::vector<int> seqs, ks; int k = 0, turn = 0; bool counted = false; };
   std::deque<Flight> inflight;
+  cudaEvent_t flight_done[2] = {nullptr, nullptr};  // recorded behind the kernels of a slot's step
   int32_t *h_out2[2] = {nullptr, nullptr}, *h_stage2[2] = {nullptr, nullptr}, *h_done2[2] = {nullptr, nullptr};     // pinned, one set per slot (see StepIo)
   int32_t *h_page_table = nullptr;   // pinned mirror of the page table: the source of its (asynchronous) updates
   int turn = 0;                      // steps enqueued so far; step i uses slot i & 1
@@ -972,6 +970,7 @@ int enqueue_step(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int32_t *f
   tidar_ctx::StepKey key;
   key.k = k; key.n_seqs = n_seqs; key.ar = ar; key.units = n_seqs * ((T + spt - 1) / spt); key.split = may_split(max_n);
   if (int rc = launch_step(c, key)) return rc;
+  CUDA_TRY(c, cudaEventRecord(c->flight_done[slot], c->stream));
   push_flight(c, seqs, n_seqs, forced, k, nullptr);
   c->last_hidden_off = 0;
   c->last_rows = R + ((cf.beta < 1.0f && !ar) ? n_seqs * k : 0); c->last_first_pos = -1;      // the mixed rows follow the slots
@@ -1031,6 +1030,7 @@ int enqueue_step_mixed(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int3
     key.units = tiles;
   }
   if (int rc = launch_step(c, key)) return rc;
+  CUDA_TRY(c, cudaEventRecord(c->flight_done[slot], c->stream));
   push_flight(c, seqs, n_seqs, forced, 0, ks);
   c->last_hidden_off = 0;
   c->last_rows = R + mixed_rows; c->last_first_pos = -1;
@@ -1043,20 +1043,11 @@ int finish_step(tidar_ctx *c, int32_t *out_tokens, int32_t *out_n) {
   tidar_ctx::Flight f = std::move(c->inflight.front());
   c->inflight.pop_front();
   const int slot = f.turn & 1;
-  if (c->timing || c->timeline || (c->cfg.debug & 2)) CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  // The step's last kernel writes its turn number behind the results (see StepIo).  The stream is asked now and then
-  // only, in case the kernels failed.
-  const volatile int32_t *done = c->h_done2[slot];
-  for (uint32_t polls = 1; done[0] != f.turn + 1; ++polls) {
-    if ((polls & 0x3fff) == 0) {
-      const cudaError_t e = cudaStreamQuery(c->stream);
-      if (e == cudaErrorNotReady) continue;
-      CUDA_TRY(c, e);
-      if (done[0] != f.turn + 1) return fail(c, TIDAR_ECUDA, "the step's kernels ended without results");
-    }
-    _mm_pause();
-  }
-  std::atomic_thread_fence(std::memory_order_acquire);
+  // Everything up to the step is complete when this returns, as the caller is promised (the results, which the step's last kernel writes to
+  // pinned memory, arrive a moment earlier).
+  CUDA_TRY(c, cudaEventSynchronize(c->flight_done[slot]));
+  const int32_t *done = c->h_done2[slot];
+  if (done[0] != f.turn + 1) return fail(c, TIDAR_ECUDA, "the step's kernels ended without results");
   if (c->timing) collect_timing(c);
   if (c->timeline) collect_timeline(c);
   if (done[1]) {
@@ -1164,6 +1155,11 @@ int tidar_init(const tidar_config *cfg, const tidar_weights *w, void *arena, siz
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_page_table, 0, (size_t)cfg->max_batch * c->pages_per_seq * sizeof(int), c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) { cudaFreeHost(c->h_pinned); delete c; return fail(nullptr, TIDAR_ECUDA, "arena set-up: %s", cudaGetErrorString(e)); }
+  for (cudaEvent_t &ev : c->flight_done)
+    if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
+      if (c->flight_done[0]) cudaEventDestroy(c->flight_done[0]);
+      cudaFreeHost(c->h_pinned); delete c; return fail(nullptr, TIDAR_ECUDA, "cudaEventCreate failed");
+    }
   *out = c;
   return TIDAR_OK;
 }
@@ -1355,6 +1351,7 @@ int tidar_free(tidar_ctx *c) {
   cudaStreamSynchronize(c->stream);
   for (auto &t : c->timed) { cudaEventDestroy(t.a); cudaEventDestroy(t.b); }
   drop_graphs(c, 0);
+  for (cudaEvent_t ev : c->flight_done) cudaEventDestroy(ev);
   if (c->h_pinned) cudaFreeHost(c->h_pinned);
   delete c;
   return TIDAR_OK;

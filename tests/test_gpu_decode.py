@@ -15,12 +15,13 @@ pytestmark = pytest.mark.gpu
 IMPLS = [0, 1]
 
 
-def _gpu(sh, wt, impl, k_max=None, debug=1, max_batch=1, max_seq_len=512, prefill_rows=0):
+def _gpu(sh, wt, impl, k_max=None, debug=1, max_batch=1, max_seq_len=512, prefill_rows=0, stream=None):
     """A context whose arena is followed by 64 KiB of sentinel bytes; _close() checks them."""
     from paper_2511_08923_b200 import Tidar, pack_weights
     packed = pack_weights(wt, "cuda:0")
+    torch.cuda.synchronize()                        # the weights were packed on the default stream
     return Tidar(sh, packed, k_max=k_max or sh.k, max_batch=max_batch, max_seq_len=max_seq_len, debug=debug, impl=impl,
-                 guard_bytes=64 * 1024, prefill_rows=prefill_rows)
+                 guard_bytes=64 * 1024, prefill_rows=prefill_rows, stream=stream)
 
 
 def _close(t):
@@ -452,6 +453,30 @@ def test_first_pass_in_blocks_of_two_instructions(n):
     np.testing.assert_array_equal(hidden[0][0], hidden[1][0])
     assert np.abs(hidden[0][1] - hidden[1][1]).max() <= TOL_LOGITS
     assert np.abs(hidden[0][1] - hidden[0][0]).max() > 3 * TOL_LOGITS          # the layer adds something
+
+
+@pytest.mark.parametrize("own_stream", [False, True])
+def test_steps_return_with_the_stream_idle(own_stream):
+    """A first pass, a step and the last step waited for leave nothing running on the context's stream."""
+    sh, wt = make_model("tiny")
+    stream = torch.cuda.Stream() if own_stream else None
+    t = _gpu(sh, wt, 0, debug=0, stream=stream)
+    seen = stream or torch.cuda.default_stream()
+    t.prefill(0, prompt_ids(sh), sh.k)
+    assert seen.query()
+    for i in range(60):
+        t.step([0], forced=[1 + i % 2])
+        assert seen.query(), i
+    for i in range(20):
+        t.step_async([0], [1])
+        t.step_async([0], [2])
+        t.step_wait()
+        t.step_wait()
+        assert seen.query(), i
+    for i in range(20):
+        t.ar_step([0])
+        assert seen.query(), i
+    _close(t)
 
 
 def test_two_steps_in_flight_match_one_at_a_time():
