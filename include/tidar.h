@@ -286,7 +286,7 @@ int tidar_debug_count_attention_tiles(tidar_ctx *ctx, int32_t on, uint64_t *visi
  * the latest moment one finished (%globaltimer).  After the step, class_ms[cls] is the sum of
  * (end - start) over the launches of a class (TIDAR_TC_*), *busy_ms the sum over all launches
  * and *span_ms the time from the first start to the last end.  Costs two atomics per CTA;
- * switching it on or off re-captures the step's graph.  impl 0 only.                    */
+ * steps with it have captured graphs of their own.  impl 0 only.                        */
 int tidar_debug_set_timeline(tidar_ctx *ctx, int32_t on);
 int tidar_debug_get_timeline(tidar_ctx *ctx, float *class_ms /*host,[TIDAR_TC_COUNT]*/, float *busy_ms /*host, or NULL*/,
                              float *span_ms /*host, or NULL*/);

@@ -102,7 +102,7 @@ struct tidar_ctx {
              count_tiles == o.count_tiles && split == o.split;
     }
   };
-  struct StepGraph { StepKey key; cudaGraphExec_t exec = nullptr; int64_t launches = 0; };
+  struct StepGraph { StepKey key; cudaGraphExec_t exec = nullptr; int64_t launches = 0; std::vector<int> tl_cls; };   // tl_cls: of its timeline slots
   static constexpr size_t MAX_GRAPHS = 16;
   std::deque<StepGraph> graphs;      // most recently used first
   bool split_keys = true;            // attention key ranges of the current pass may be cut (see attention_plan)
@@ -883,6 +883,7 @@ int launch_step(tidar_ctx *c, tidar_ctx::StepKey key) {
       }
       if (e == cudaSuccess && rc == TIDAR_OK && graph) e = cudaGraphInstantiate(&sg.exec, graph, 0);
       if (graph) cudaGraphDestroy(graph);
+      if (key.timeline) sg.tl_cls = c->tl_cls;
       sg.launches = c->launches - l0;
       c->launches = l0;
       if (e != cudaSuccess || rc != TIDAR_OK || !sg.exec) {
@@ -897,8 +898,10 @@ int launch_step(tidar_ctx *c, tidar_ctx::StepKey key) {
       c->graphs.push_front(sg);
     }
     if (c->graphs_ok) {
-      CUDA_TRY(c, cudaGraphLaunch(c->graphs.front().exec, c->stream));
-      c->launches += c->graphs.front().launches;
+      const tidar_ctx::StepGraph &sg = c->graphs.front();
+      CUDA_TRY(c, cudaGraphLaunch(sg.exec, c->stream));
+      c->launches += sg.launches;
+      if (key.timeline) { c->tl_cls = sg.tl_cls; c->tl_n = (int)sg.tl_cls.size(); }      // (another step may have been recorded since)
       return TIDAR_OK;
     }
   }

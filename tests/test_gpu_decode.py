@@ -479,6 +479,22 @@ def test_steps_return_with_the_stream_idle(own_stream):
     _close(t)
 
 
+def test_timeline_of_a_replayed_step_is_its_own():
+    """Two kept graphs with different launch lists (a long context adds the merge of split key ranges in every layer): replaying the first
+    after the second was recorded still attributes every launch of the first to its class."""
+    sh, wt = make_model("tiny")
+    t = _gpu(sh, wt, 0, debug=0, max_batch=2, max_seq_len=1024, stream=torch.cuda.Stream())
+    t.prefill(0, prompt_ids(sh, 64), sh.k)
+    t.prefill(1, prompt_ids(sh, 900), sh.k)
+    t.set_timeline(True)
+    for seq in (0, 1, 0, 1, 0):
+        t.step([seq])
+        tl = t.timeline()
+        assert all(tl[c] > 0 for c in ("embed", "norm", "gemm", "rope", "attn", "lmhead", "verify")), (seq, tl)
+        assert tl["busy"] == pytest.approx(sum(v for c, v in tl.items() if c not in ("busy", "span")), rel=1e-4)
+    _close(t)
+
+
 def test_two_steps_in_flight_match_one_at_a_time():
     """tidar_step_async accepts a second step while the first is in flight (forced lengths): the results,
     handed out oldest first, the blocks and the cached K/V are bit-identical to the same steps run one at a
