@@ -27,7 +27,10 @@
  *     instance through PyTorch), keeps them alive until tidar_free and must
  *     not touch the arena while the context exists.
  *   - All work is enqueued on the CUDA stream given to tidar_init.  tidar_prefill
- *     and tidar_step synchronise that stream before they return the tokens.
+ *     and tidar_step synchronise that stream before they return the tokens.  On a stream
+ *     that the caller created, a step is captured once per shape and replayed as one graph
+ *     launch; on the default stream (NULL), which CUDA does not let be captured, the same
+ *     kernels are launched one by one.
  *   - A context is not synchronised between host threads: one thread at a time may call
  *     into it (different contexts are independent).
  *   - There is no CPU fallback: without a CUDA device tidar_init fails.
@@ -290,6 +293,10 @@ int tidar_debug_count_attention_tiles(tidar_ctx *ctx, int32_t on, uint64_t *visi
 int tidar_debug_set_timeline(tidar_ctx *ctx, int32_t on);
 int tidar_debug_get_timeline(tidar_ctx *ctx, float *class_ms /*host,[TIDAR_TC_COUNT]*/, float *busy_ms /*host, or NULL*/,
                              float *span_ms /*host, or NULL*/);
+/* How steps were launched since tidar_init: steps captured into a graph, steps launched as a graph (the
+ * captured ones included; all others ran as plain launches), and graphs kept at the moment (the most
+ * recently used shapes, 16 at most).  Any pointer may be NULL.                            */
+int tidar_debug_graph_stats(const tidar_ctx *ctx, int64_t *captured /*host*/, int64_t *launched /*host*/, int32_t *kept /*host*/);
 /* Exercises the bounded wait the tensor-core kernels are built on: enqueues a one-thread kernel
  * that waits, for at most limit_polls polls (a few milliseconds at 2^14), on a barrier that
  * nothing arrives on, gives up and sets the status word.  tidar_sync then returns

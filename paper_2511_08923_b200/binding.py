@@ -93,6 +93,7 @@ def load(rebuild: bool = False) -> C.CDLL:
         "tidar_debug_wait_probe": (C.c_int, [ctxp, I32]),
         "tidar_debug_count_attention_tiles": (C.c_int, [ctxp, I32, P(C.c_uint64)]),
         "tidar_debug_set_timeline": (C.c_int, [ctxp, I32]),
+        "tidar_debug_graph_stats": (C.c_int, [ctxp, P(C.c_int64), P(C.c_int64), P(I32)]),
         "tidar_debug_get_timeline": (C.c_int, [ctxp, P(C.c_float), P(C.c_float), P(C.c_float)]),
     }
     for name, (res, args) in sig.items():
@@ -343,6 +344,12 @@ class Tidar:
         v = C.c_uint64(0)
         self._check(self.lib.tidar_debug_count_attention_tiles(self.ctx, int(on), C.byref(v)))
         return int(v.value)
+
+    def graph_stats(self):
+        """(steps captured into a graph, steps launched as a graph, graphs kept): see tidar_debug_graph_stats."""
+        captured, launched, kept = C.c_int64(0), C.c_int64(0), C.c_int32(0)
+        self._check(self.lib.tidar_debug_graph_stats(self.ctx, C.byref(captured), C.byref(launched), C.byref(kept)))
+        return int(captured.value), int(launched.value), int(kept.value)
 
     def set_timeline(self, on: bool):
         self._check(self.lib.tidar_debug_set_timeline(self.ctx, int(on)))

@@ -106,7 +106,8 @@ struct tidar_ctx {
   static constexpr size_t MAX_GRAPHS = 16;
   std::deque<StepGraph> graphs;      // most recently used first
   bool split_keys = true;            // attention key ranges of the current pass may be cut (see attention_plan)
-  bool graphs_ok = true;
+  bool graphs_ok = true;             // steps can be captured on this stream (the legacy default stream refuses it)
+  int64_t graphs_captured = 0, graphs_launched = 0;
   bool slab_bf16 = false;          // split-K partial sums of the step in bf16 instead of fp32 (config debug bit 2)
   int32_t *d_status = nullptr, *cand_idx = nullptr;
   float *cand_val = nullptr;
@@ -863,8 +864,8 @@ void drop_graphs(tidar_ctx *c, size_t keep) {
 
 // The step proper.  Every launch of a step has the same arguments from step to step (lengths, page tables, token
 // blocks and, for a step of mixed block lengths, the row layout live in device memory), except
-// for the grid sizes, so the step is captured once per key and replayed.  Per-launch timing and the debug read-backs
-// use plain launches.  key.units: attention units per KV head.
+// for the grid sizes, so on a stream of the caller's the step is captured once per key and replayed.  The legacy default
+// stream, which cannot be captured, per-launch timing and the debug read-backs use plain launches of the same kernels.  key.units: attention units per KV head.
 int launch_step(tidar_ctx *c, tidar_ctx::StepKey key) {
   key.timeline = c->timeline; key.count_tiles = c->count_tiles;
   if (use_graphs(c)) {
@@ -891,6 +892,7 @@ int launch_step(tidar_ctx *c, tidar_ctx::StepKey key) {
         c->graphs_ok = false;
       } else {
         c->graphs.push_front(sg);
+        c->graphs_captured++;
       }
     } else if (it != c->graphs.begin()) {
       const tidar_ctx::StepGraph sg = *it;
@@ -901,6 +903,7 @@ int launch_step(tidar_ctx *c, tidar_ctx::StepKey key) {
       const tidar_ctx::StepGraph &sg = c->graphs.front();
       CUDA_TRY(c, cudaGraphLaunch(sg.exec, c->stream));
       c->launches += sg.launches;
+      c->graphs_launched++;
       if (key.timeline) { c->tl_cls = sg.tl_cls; c->tl_n = (int)sg.tl_cls.size(); }      // (another step may have been recorded since)
       return TIDAR_OK;
     }
@@ -1026,8 +1029,9 @@ int enqueue_step_mixed(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int3
   const int mixed_rows = cf.beta < 1.0f ? sum_k : 0;         // one mixed LM-head input row per verified position
   key.mixed_K = mixed_rows;
   // Steps of nearly the same size share one captured graph: rows are filled up to a multiple of 16 (the projections' row
-  // blocks are that anyway) and units to a multiple of 4 with ones that have no rows.
-  if (cf.impl == 0 && mixed_rows == 0) {
+  // blocks are that anyway) and units to a multiple of 4 with ones that have no rows.  (Also under debug bit 3, so that it differs in
+  // the launch mode alone.)
+  if (cf.impl == 0 && mixed_rows == 0 && c->graphs_ok) {
     key.mixed_R = (R + 15) / 16 * 16;
     for (; tiles % 4 && tiles < c->R_head + mb; ++tiles) ht0[tiles] = hte[tiles] = 0;
     key.units = tiles;
@@ -1108,6 +1112,7 @@ int tidar_init(const tidar_config *cfg, const tidar_weights *w, void *arena, siz
   c->cfg = *cfg;
   c->slab_bf16 = (cfg->debug & 4) != 0;
   c->stream = (cudaStream_t)cuda_stream;
+  c->graphs_ok = c->stream != nullptr && c->stream != cudaStreamLegacy;
   size_t need = 0;
   layout(*c, arena, &need);
   if (need > arena_bytes) { delete c; return fail(nullptr, TIDAR_ENOMEM, "arena has %zu bytes, %zu needed", arena_bytes, need); }
@@ -1489,6 +1494,14 @@ int tidar_debug_get_timeline(tidar_ctx *c, float *class_ms, float *busy_ms, floa
   for (int i = 0; i < TIDAR_TC_COUNT; ++i) class_ms[i] = c->tl_class_ms[i];
   if (busy_ms) *busy_ms = c->tl_busy_ms;
   if (span_ms) *span_ms = c->tl_span_ms;
+  return TIDAR_OK;
+}
+
+int tidar_debug_graph_stats(const tidar_ctx *c, int64_t *captured, int64_t *launched, int32_t *kept) {
+  if (!c) return TIDAR_EINVAL;
+  if (captured) *captured = c->graphs_captured;
+  if (launched) *launched = c->graphs_launched;
+  if (kept) *kept = (int32_t)c->graphs.size();
   return TIDAR_OK;
 }
 

@@ -315,9 +315,9 @@ def test_graph_replay_plain_launches_and_replay_kernels_agree(name):
     """The benchmark times the captured-graph path with programmatic dependent launches; the
     logits / hidden-state comparisons run with plain launches.  The same teacher-forced steps
     through (a) graph replay, (b) plain launches and (c) the fp32 CUDA-core kernels must give
-    identical acceptance lengths, tokens and next blocks, and (a) and (b) bit-identical cached
-    K/V in every layer (same kernels, same order: a kernel that read its input before the
-    previous kernel finished would show here)."""
+    identical acceptance lengths, tokens and next blocks, and (a), (b) and the plain launches of a context on the
+    default stream bit-identical cached K/V in every layer (same kernels, same order: a kernel that read its
+    input before the previous kernel finished would show here)."""
     from dataclasses import replace
     if name == "tiny":
         sh, k, n_prompt = CONFIGS_["tiny"], 4, 64
@@ -328,8 +328,8 @@ def test_graph_replay_plain_launches_and_replay_kernels_agree(name):
     prompt = prompt_ids(sh, n_prompt)
     forced = [3, k, 1, k // 2, 2]
     runs = {}
-    for tag, impl, debug in (("graph", 0, 0), ("plain", 0, 8), ("replay", 1, 0)):
-        t = _gpu(sh, wt, impl, k_max=k, debug=debug, max_seq_len=n_prompt + 8 * k + 64)
+    for tag, impl, debug in (("graph", 0, 0), ("plain", 0, 8), ("default stream", 0, 0), ("replay", 1, 0)):
+        t = _gpu(sh, wt, impl, k_max=k, debug=debug, max_seq_len=n_prompt + 8 * k + 64, stream=None if tag == "default stream" else torch.cuda.Stream())
         rec = [t.prefill(0, prompt, k)]
         blocks = [t.get_block(0, k)]
         for f in forced:
@@ -339,13 +339,15 @@ def test_graph_replay_plain_launches_and_replay_kernels_agree(name):
             rec.append((toks[0], L[0]))
             blocks.append(t.get_block(0, k))
         n = t.seq_len(0)
+        assert t.graph_stats() == ((1, len(forced), 1) if tag == "graph" else (0, 0, 0))
         kv = [t.kv(0, l, 0, n) for l in range(sh.n_layers)] if impl == 0 else None
         runs[tag] = {"rec": rec, "blocks": blocks, "kv": kv, "n": n, "launches": t.launch_count()}
         _close(t)
-    assert runs["graph"]["rec"] == runs["plain"]["rec"] and runs["graph"]["blocks"] == runs["plain"]["blocks"]
-    assert runs["graph"]["n"] == runs["plain"]["n"]
-    for (k0, v0), (k1, v1) in zip(runs["graph"]["kv"], runs["plain"]["kv"]):
-        np.testing.assert_array_equal(k0, k1); np.testing.assert_array_equal(v0, v1)
+    for tag in ("plain", "default stream"):
+        assert runs["graph"]["rec"] == runs[tag]["rec"] and runs["graph"]["blocks"] == runs[tag]["blocks"]
+        assert runs["graph"]["n"] == runs[tag]["n"] and runs["graph"]["launches"] == runs[tag]["launches"]
+        for (k0, v0), (k1, v1) in zip(runs["graph"]["kv"], runs[tag]["kv"]):
+            np.testing.assert_array_equal(k0, k1); np.testing.assert_array_equal(v0, v1)
     # the CUDA-core kernels round differently: tokens can only differ on a near-tie, which the
     # tiny model's margins make rare; lengths are forced, so the shapes must match exactly
     assert [r[1] for r in runs["replay"]["rec"][1:]] == [r[1] for r in runs["graph"]["rec"][1:]]
@@ -477,6 +479,30 @@ def test_steps_return_with_the_stream_idle(own_stream):
         t.ar_step([0])
         assert seen.query(), i
     _close(t)
+
+
+def test_kept_graphs_are_reused_and_replaced():
+    """More step shapes than a context keeps graphs for, met in an order that re-uses some and drops others: TiDAR steps of six block lengths and AR
+    steps for one to three sequences, over short and long contexts.  Same results as the same steps launched kernel by kernel."""
+    sh, wt = make_model("tiny")
+    shapes = [(q, k) for q in ([0], [0, 1], [0, 1, 2], [2]) for k in (0, 1, 2, 3, 5, 8)]      # k = 0: an AR step
+    order = shapes[:12] + shapes[8:14] + shapes[:4] + shapes[12:] + shapes[10:]
+    runs = {}
+    for tag, debug in (("graph", 0), ("plain", 8)):
+        t = _gpu(sh, wt, 0, k_max=8, debug=debug, max_batch=3, max_seq_len=1280, stream=torch.cuda.Stream())
+        rec = [t.prefill(q, prompt_ids(sh, n, seed=sh.seed + q), 8) for q, n in enumerate((40, 90, 850))]
+        for q, k in order:
+            rec.append(t.step_k(q, k, forced=[1 + (k + i) % k for i in range(len(q))]) if k else t.ar_step(q))
+        runs[tag] = rec, [[t.get_block(q, 1) for q in range(3)]] + [t.kv(q, l, 0, t.seq_len(q)) for q in range(3) for l in range(sh.n_layers)], t.launch_count()
+        captured, launched, kept = t.graph_stats()
+        if tag == "plain":
+            assert (captured, launched, kept) == (0, 0, 0)
+        else:
+            assert launched == len(order) and kept == 16 and len(shapes) < captured < len(order), captured     # some came back, some had been dropped
+        _close(t)
+    assert runs["graph"][0] == runs["plain"][0] and runs["graph"][1][0] == runs["plain"][1][0] and runs["graph"][2] == runs["plain"][2]
+    for a, b in zip(runs["graph"][1][1:], runs["plain"][1][1:]):
+        np.testing.assert_array_equal(a[0], b[0]); np.testing.assert_array_equal(a[1], b[1])
 
 
 def test_timeline_of_a_replayed_step_is_its_own():

@@ -4,7 +4,7 @@ from dataclasses import replace
 
 import numpy as np
 import pytest
-import torch  # noqa: F401
+import torch
 
 from oracle import tidar_oracle as O
 from tests.helpers import MARGIN, TOL_LOGITS, check_rows, make_model, oracle_cfg, prompt_ids, top1_margin
@@ -14,10 +14,12 @@ pytestmark = pytest.mark.gpu
 IMPLS = [0, 1]
 
 
-def _gpu(sh, wt, impl, k_max, debug=0, max_batch=1, max_seq_len=512, beta=1.0):
+def _gpu(sh, wt, impl, k_max, debug=0, max_batch=1, max_seq_len=512, beta=1.0, stream=None):
     from paper_2511_08923_b200 import Tidar, pack_weights
-    return Tidar(sh, pack_weights(wt, "cuda:0"), k_max=k_max, max_batch=max_batch, max_seq_len=max_seq_len, debug=debug, impl=impl,
-                 guard_bytes=64 * 1024, beta=beta)
+    packed = pack_weights(wt, "cuda:0")
+    torch.cuda.synchronize()                        # the weights were packed on the default stream
+    return Tidar(sh, packed, k_max=k_max, max_batch=max_batch, max_seq_len=max_seq_len, debug=debug, impl=impl,
+                 guard_bytes=64 * 1024, beta=beta, stream=stream)
 
 
 def _close(t):
@@ -311,17 +313,19 @@ def test_mixed_block_lengths_keep_the_autoregressive_continuation(tiny, impl):
 
 def test_mixed_step_graph_replay_matches_plain_launches():
     """A step of mixed block lengths replays one captured graph for every length vector with the same
-    row and tile count ((3, 4, 2) and (2, 3, 4) here, the layout living in device memory); the same
-    teacher-forced steps launched kernel by kernel give identical tokens and bit-identical cached K/V."""
+    number of 16-row blocks and of tile pairs up to a multiple of four ((3, 4, 2), (2, 3, 4) and (3, 4, 1), which has four rows
+    fewer, here; the layout lives in device memory); the same teacher-forced steps launched kernel by kernel
+    give identical tokens and bit-identical cached K/V."""
     from dataclasses import replace as _r
     from tidar_synth import CONFIGS as CONFIGS_, gen_model_weights as gen_model_weights_
     sh = _r(CONFIGS_["8b"].reduced(2), vocab=8192)
     wt = gen_model_weights_(sh)
     prompts = [prompt_ids(sh, n=150 + 37 * q, seed=sh.seed + q) for q in range(3)]
-    plan = [([3, 4, 2], [2, 1, 2]), ([2, 3, 4], [1, 3, 4]), ([3, 4, 2], [3, 2, 1]), ([4, 4, 4], [4, 1, 2]), ([4, 2, 3], [2, 2, 3])]
+    plan = [([3, 4, 2], [2, 1, 2]), ([2, 3, 4], [1, 3, 4]), ([3, 4, 2], [3, 2, 1]), ([4, 4, 4], [4, 1, 2]), ([4, 2, 3], [2, 2, 3]), ([3, 4, 1], [3, 4, 1]),
+            ([2, 3, 4], [2, 1, 3])]
     runs = {}
     for tag, debug in (("graph", 0), ("plain", 8)):
-        t = _gpu(sh, wt, 0, k_max=4, debug=debug, max_batch=3, max_seq_len=512)
+        t = _gpu(sh, wt, 0, k_max=4, debug=debug, max_batch=3, max_seq_len=512, stream=torch.cuda.Stream())
         rec = [t.prefill(q, p, 4) for q, p in enumerate(prompts)]
         blocks = [[t.get_block(q, 4) for q in range(3)]]
         l0 = t.launch_count()
@@ -331,6 +335,7 @@ def test_mixed_step_graph_replay_matches_plain_launches():
                     t.set_block(q, runs["graph"]["blocks"][i][q])
             rec.append(t.step_ks([0, 1, 2], ks, forced))
             blocks.append([t.get_block(q, ks[q]) + [0] * (4 - ks[q]) for q in range(3)])
+        assert t.graph_stats() == ((2, len(plan), 2) if tag == "graph" else (0, 0, 0))      # the mixed steps share one, the equal lengths have the other
         kv = [[t.kv(q, l, 0, t.seq_len(q)) for l in range(sh.n_layers)] for q in range(3)]
         runs[tag] = {"rec": rec, "blocks": blocks, "kv": kv, "launches": t.launch_count() - l0}
         _close(t)
