@@ -279,7 +279,7 @@ __device__ inline void plan_block(const PlanArgs &p, ROW row_keys) {
       Item it{};
       it.row0 = unit_row0[u] + (paired ? 0 : (e & 1) * p.spt); it.row_end = unit_rend[u]; it.seq = unit_seq[u];
       it.n_cache_pages = k.n_cache; it.loc_lo = k.loc_lo;
-      it.p_begin = (int)((long long)k.n_pages * j / n); it.p_end = (int)((long long)k.n_pages * (j + 1) / n);
+      it.p_begin = k.n_pages * j / n; it.p_end = k.n_pages * (j + 1) / n;      // (2^31 positions are 2^25 pages, in at most 2^5 pieces)
       it.pair = paired && unit_row0[u] + p.spt < unit_rend[u]; it.split = n > 1;
       p.items[place_s[e] + j] = it;
     }
