@@ -51,8 +51,8 @@
 namespace attn_tc {
 
 constexpr int PAGE = 64;             // keys per step (= page size)
-constexpr int STAGES = 5;            // K pages and V pages in flight, each
-constexpr int THREADS = 384;         // warp 0: K loads, 1: MMA, 2: watcher, 3: Q and V loads; warps 4..7 / 8..11: softmax of stream A / B
+// warp 0: K loads, 1: MMA, 2: watcher, 3: Q and V loads; warps 4..7 / 8..11: softmax of stream A / B
+__host__ __device__ constexpr int threads(int streams) { return 128 + 128 * streams; }
 constexpr int MAX_SPLITS = 32;       // items per tile
 constexpr int SLOTS_PER_SM = 2;      // partial results that fit the scratch = grid of a pass whose key ranges may be split
 constexpr float RAISE_THRESHOLD = 8.f;   // log2 units
@@ -93,30 +93,33 @@ struct Args {
   // early: plan, row metadata and page table were written before the kernel in front of this one started, and that one lets its
   // successor in only once its own predecessors are complete, so they are read ahead of pdl_wait()
   int early;
+  // Stand-alone calls without a plan (items = null; DIRECT instances): what a CTA works out its item and its rows' keys from.
+  struct { const int32_t *seq_len; int k, n_max; int per_group, pieces; } direct;    // query tiles per sequence, items per tile at most
   int *status;
   unsigned long long *tile_count;            // diagnostics: += steps this CTA computes (null = off)
 };
 
 // Shared memory of one CTA; everything is dynamic so that the 1024-byte alignment the
 // swizzled tiles need costs no padding (the kernel checks the base address).
-template <int HD>
+template <int HD, int STREAMS = 2>
 struct Smem {
+  static constexpr int K_STAGES = STREAMS == 2 ? 5 : 3, V_STAGES = STREAMS == 2 ? 5 : 2;     // pages in flight (one stream: two CTAs fit an SM)
   static constexpr int NH = HD / 64;                 // 64-element halves of a head
   static constexpr int Q_BYTES = 128 * HD * 2;       // one query tile
   static constexpr int KV_BYTES = PAGE * HD * 2;
   static constexpr int Q_OFF = 0;
-  static constexpr int K_OFF = Q_OFF + 2 * Q_BYTES;
-  static constexpr int V_OFF = K_OFF + STAGES * KV_BYTES;
-  static constexpr int BAR_OFF = V_OFF + STAGES * KV_BYTES;      // mbarriers and a few words
+  static constexpr int K_OFF = Q_OFF + STREAMS * Q_BYTES;
+  static constexpr int V_OFF = K_OFF + K_STAGES * KV_BYTES;
+  static constexpr int BAR_OFF = V_OFF + V_STAGES * KV_BYTES;    // mbarriers and a few words
   static constexpr int TOTAL = BAR_OFF + 512;
   static constexpr int XCHG_OFF = K_OFF;             // single tile: the streams' results, [stream][hd / 8][128 rows][4] floats; (max, sum) behind them
   static constexpr int XCHG_ML_OFF = XCHG_OFF + 128 * HD * 4;
-  static constexpr int TMEM_COLS = 512;              // 2 streams x (2 x 64 (S) + HD (O)), rounded up to a power of two
+  static constexpr int TMEM_COLS = 256 * STREAMS;    // per stream 2 x 64 (S) + HD (O), rounded up to a power of two
 };
 static_assert(Smem<128>::XCHG_ML_OFF + 2 * 128 * 8 <= Smem<128>::BAR_OFF && Smem<64>::XCHG_ML_OFF + 2 * 128 * 8 <= Smem<64>::BAR_OFF, "exchange area fits the K/V rings");
 
 struct Ctl {                                         // lives at Smem::BAR_OFF
-  uint64_t q_full, k_full[STAGES], k_empty[STAGES], v_full[STAGES], v_empty[STAGES], s_full[2][2], p_full[2][2];
+  uint64_t q_full, k_full[5], k_empty[5], v_full[5], v_empty[5], s_full[2][2], p_full[2][2];
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -286,11 +289,49 @@ __device__ inline void plan_block(const PlanArgs &p, ROW row_keys) {
   }
 }
 
-template <int HD>
-__global__ void __launch_bounds__(THREADS, 1)
+// What row r of a stand-alone call sees (the slot layout of a step of equal block lengths k).  seq_len comes from the caller: it is
+// clamped to [0, n_max] (the positions the page table can back minus the k causal slots), so that no row looks past the table.
+__device__ __forceinline__ RowKeys step_row_keys(const int32_t *__restrict__ seq_len, int k, int n_max, int r) {
+  const int T = k * (k + 1);
+  const int s = r / T, slot = r % T;
+  const int n = min(max(seq_len[s], 0), n_max);
+  if (slot < k) return RowKeys{n + slot + 1, 0, 0, s};
+  const int b = (slot - k) / k;
+  return RowKeys{n + b + 1, s * k * k + b * k, k, s};
+}
+
+// Query tile number `tile` of a stand-alone call that has no plan, with its whole key range, as an item.
+__device__ __forceinline__ Item direct_tile(const Args &a, int tile) {
+  const int k = a.direct.k, T = k * (k + 1), s = tile / a.direct.per_group, first = tile % a.direct.per_group * a.spt;
+  const int last = min(first + a.spt, T) - 1;                    // its slots
+  // the causal slots see more the later they come, the mask blocks too, and the last causal slot sees what the last block sees
+  const RowKeys most = step_row_keys(a.direct.seq_len, k, a.direct.n_max, s * T + (first < k ? min(last, k - 1) : last));
+  Item it{};
+  it.row0 = s * T + first; it.row_end = (s + 1) * T; it.seq = s;
+  it.p_end = it.n_cache_pages = (most.nvis + PAGE - 1) / PAGE;
+  if (last >= k) {
+    it.loc_lo = s * k * k + (max(first, k) - k) / k * k;
+    it.p_end += (s * k * k + ((last - k) / k + 1) * k - it.loc_lo + PAGE - 1) / PAGE;
+  }
+  return it;
+}
+// Items that a tile of n_pages pages is cut into (three pages at least: see attention_direct), out of the places it has.
+__device__ __forceinline__ int direct_pieces(const Args &a, int n_pages) { return max(1, min(a.direct.pieces, n_pages / 3)); }
+__device__ __forceinline__ Item direct_item(const Args &a, int e) {
+  Item it = direct_tile(a, e / a.direct.pieces);
+  const int j = e % a.direct.pieces, n = direct_pieces(a, it.p_end), n_pages = it.p_end;
+  it.split = n > 1;
+  it.p_begin = j < n ? n_pages * j / n : 0; it.p_end = j < n ? n_pages * (j + 1) / n : 0;      // a place that is not used has no pages
+  return it;
+}
+
+// STREAMS = 1: one tile and one stream per CTA and two CTAs per SM, which fill each other's latencies as two streams do.  It serves calls that are
+// one wave that way and two otherwise (see attention_direct for both sides' figures).  DIRECT: no plan, see direct_item.
+template <int HD, int STREAMS, bool DIRECT>
+__global__ void __launch_bounds__(threads(STREAMS), 3 - STREAMS)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                const __grid_constant__ CUtensorMap tmKloc, const __grid_constant__ CUtensorMap tmVloc, const Args a, const TlSlot tl) {
-  using L = Smem<HD>;
+  using L = Smem<HD, STREAMS>;
   constexpr int NH = L::NH;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const int warp = sm100::warp_index(), lane = threadIdx.x & 31;
@@ -306,11 +347,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   if (threadIdx.x == 0) {
     ctl.abort_flag = 0;
     sm100::mbar_init(sm100::smem_u32(&ctl.q_full), 1);
-    for (int s = 0; s < STAGES; ++s) {
-      sm100::mbar_init(sm100::smem_u32(&ctl.k_full[s]), 1); sm100::mbar_init(sm100::smem_u32(&ctl.k_empty[s]), 1);
-      sm100::mbar_init(sm100::smem_u32(&ctl.v_full[s]), 1); sm100::mbar_init(sm100::smem_u32(&ctl.v_empty[s]), 1);
-    }
-    for (int t = 0; t < 2; ++t)
+    for (int s = 0; s < L::K_STAGES; ++s) { sm100::mbar_init(sm100::smem_u32(&ctl.k_full[s]), 1); sm100::mbar_init(sm100::smem_u32(&ctl.k_empty[s]), 1); }
+    for (int s = 0; s < L::V_STAGES; ++s) { sm100::mbar_init(sm100::smem_u32(&ctl.v_full[s]), 1); sm100::mbar_init(sm100::smem_u32(&ctl.v_empty[s]), 1); }
+    for (int t = 0; t < STREAMS; ++t)
       for (int b = 0; b < 2; ++b) { sm100::mbar_init(sm100::smem_u32(&ctl.s_full[t][b]), 1); sm100::mbar_init(sm100::smem_u32(&ctl.p_full[t][b]), 4); }
     sm100::fence_mbar_init();
   }
@@ -323,17 +362,20 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   __syncthreads();
   sm100::tc_fence_after();
   const uint32_t tmem = ctl.tmem_base;
-  const uint32_t tmem_S = tmem, tmem_O = tmem + 4 * PAGE;             // per stream: 2 x 64 columns of S, HD columns of O
+  const uint32_t tmem_S = tmem, tmem_O = tmem + STREAMS * 2 * PAGE;   // per stream: 2 x 64 columns of S, HD columns of O
   volatile int *abortp = &ctl.abort_flag;
   pdl_trigger();              // not before the tensor memory is ours (see gemm_tc_kernel)
-  if (!a.early) pdl_wait();
+  if (DIRECT || !a.early) pdl_wait();
 
   // ---- which work item (every thread reads it: no barrier before the first loads go out) ----
   const int kvh = blockIdx.x % a.Hkv, item_no = blockIdx.x / a.Hkv;
-  const Item item = a.items[item_no];                                  // all zero where the grid is larger than the plan: nothing to do
+  const Item item = DIRECT ? direct_item(a, item_no) : a.items[item_no];   // all zero where the grid is larger than the plan: nothing to do
   const int row0 = item.row0, p_begin = item.p_begin, np = item.p_end - item.p_begin;
-  const bool pair = item.pair != 0;
-  const int ahead = pair ? 2 : 4;                                      // pages whose scores are computed ahead: two steps of every stream
+  const bool pair = STREAMS == 2 && item.pair != 0;
+  const bool shared = STREAMS == 1 || pair;                            // every stream takes every page; otherwise two streams take them in turn
+  const int ahead = shared ? 2 : 4;                                    // pages whose scores are computed ahead: two steps of every stream
+  auto stream0 = [&](int p) { return shared ? 0 : p & 1; };            // streams [stream0(p), stream1(p)) take page p
+  auto stream1 = [&](int p) { return pair ? 2 : stream0(p) + 1; };
   if (threadIdx.x == 0 && a.tile_count && np > 0) atomicAdd(a.tile_count, (unsigned long long)np * (pair ? 2 : 1));
 
   if (warp == 0 || warp == 3) {
@@ -376,7 +418,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
           else sm100::tma_load_4d(dst, tm_loc, fb, 0, item.loc_lo + (p_begin + p - item.n_cache_pages) * PAGE, 0, kvh, pol);
         }
         __syncwarp();
-        if (++s == STAGES) { s = 0; ph ^= 1u; }
+        if (++s == (is_k ? L::K_STAGES : L::V_STAGES)) { s = 0; ph ^= 1u; }
       }
     }
   } else if (warp == 1) {
@@ -401,8 +443,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       sm100::named_bar_sync(9u + (uint32_t)p, 64);
       sm100::tc_fence_after();
       if (sm100::elect_one()) {
-        for (int t = pair ? 0 : p & 1; t < (pair ? 2 : (p & 1) + 1); ++t) {
-          const int b = pair ? p : p >> 1;
+        for (int t = stream0(p); t < stream1(p); ++t) {
+          const int b = shared ? p : p >> 1;
           issue_qk(t, b, p);
           sm100::mma_commit(sm100::smem_u32(&ctl.s_full[t][b]));
         }
@@ -410,11 +452,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       }
       __syncwarp();
     }
-    int sv = 0, sk = ahead % STAGES;                   // ring stages of V(p) and K(p + ahead)
+    int sv = 0, sk = ahead % L::K_STAGES;              // ring stages of V(p) and K(p + ahead)
     for (int p = 0; p < np; ++p) {
-      const int j = pair ? p : p >> 1, b = j & 1;
+      const int j = shared ? p : p >> 1, b = j & 1;
       const uint64_t vd = v_desc0 + (uint64_t)sv * KV16;
-      for (int t = pair ? 0 : p & 1; t < (pair ? 2 : (p & 1) + 1); ++t) {
+      for (int t = stream0(p); t < stream1(p); ++t) {
         const bool last_stream = !pair || t == 1;
         sm100::named_bar_sync(1u + (uint32_t)(t * 2 + b), 64);
         sm100::tc_fence_after();
@@ -432,8 +474,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         }
         __syncwarp();
       }
-      if (++sv == STAGES) sv = 0;
-      if (++sk == STAGES) sk = 0;
+      if (++sv == L::V_STAGES) sv = 0;
+      if (++sk == L::K_STAGES) sk = 0;
     }
   } else if (warp == 2) {
     // ===================== watcher =====================
@@ -454,28 +496,32 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     };
     for (int p = 0; p < min(ahead, np); ++p)
       release(9u + (uint32_t)p, sm100::smem_u32(&ctl.k_full[p]), 0, p ? 0u : sm100::smem_u32(&ctl.q_full), 0, 0u, 0);
-    int sv = 0, sk = ahead % STAGES; uint32_t phv = 0, phk = (uint32_t)(ahead / STAGES) & 1u;
+    int sv = 0, sk = ahead % L::K_STAGES; uint32_t phv = 0, phk = (uint32_t)(ahead / L::K_STAGES) & 1u;
     for (int p = 0; p < np; ++p) {
-      const int j = pair ? p : p >> 1, b = j & 1;
-      for (int t = pair ? 0 : p & 1; t < (pair ? 2 : (p & 1) + 1); ++t) {
+      const int j = shared ? p : p >> 1, b = j & 1;
+      for (int t = stream0(p); t < stream1(p); ++t) {
         const bool first_stream = !pair || t == 0;
         release(1u + (uint32_t)(t * 2 + b), sm100::smem_u32(&ctl.p_full[t][b]), (uint32_t)(j >> 1) & 1u, first_stream ? sm100::smem_u32(&ctl.v_full[sv]) : 0u, phv,
                 first_stream && p + ahead < np ? sm100::smem_u32(&ctl.k_full[sk]) : 0u, phk);
       }
-      if (++sv == STAGES) { sv = 0; phv ^= 1u; }
-      if (++sk == STAGES) { sk = 0; phk ^= 1u; }
+      if (++sv == L::V_STAGES) { sv = 0; phv ^= 1u; }
+      if (++sk == L::K_STAGES) { sk = 0; phk ^= 1u; }
     }
   } else if (warp >= 4) {
     // ===================== softmax =====================
     const int t = (warp - 4) >> 2;                       // stream
     const int tile = pair ? t : 0;
     const int my_row = (warp & 3) * 32 + lane;           // this thread's MMA row = TMEM lane
-    const int nj = pair ? np : (np + 1 - t) >> 1;        // steps of this stream
+    const int nj = shared ? np : (np + 1 - t) >> 1;      // steps of this stream
     // (a row without a slot sees everything, so that its warp does not mask page after page for it)
     int my_slot = -1, my_nvis = 0x7fffffff, my_loc0 = item.loc_lo, my_nloc = 1 << 30;
     {
       const int pr = row0 + tile * a.spt + my_row / a.G;
-      if (my_row < rows_used && pr < item.row_end) { my_slot = pr; my_nvis = a.nvis[pr]; my_nloc = a.nloc[pr]; my_loc0 = a.loc0[pr]; }
+      if (my_row < rows_used && pr < item.row_end) {
+        my_slot = pr;
+        if constexpr (DIRECT) { const RowKeys w = step_row_keys(a.direct.seq_len, a.direct.k, a.direct.n_max, pr); my_nvis = w.nvis; my_nloc = w.nloc; my_loc0 = w.loc0; }
+        else { my_nvis = a.nvis[pr]; my_nloc = a.nloc[pr]; my_loc0 = a.loc0[pr]; }
+      }
     }
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t s_addr0 = tmem_S + (uint32_t)(t * 2 * PAGE) + lane_addr, o_addr = tmem_O + (uint32_t)(t * HD) + lane_addr;
@@ -497,7 +543,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       // Visible keys of the page for my row: [lo, hi) in page-local indices.  Masking is skipped
       // for pages that are visible in full (all cached pages but the last ones of a row).
       {
-        const int p = p_begin + (pair ? j : 2 * j + t);
+        const int p = p_begin + (shared ? j : 2 * j + t);
         int lo = 0, hi = 0;
         if (p < item.n_cache_pages) hi = my_nvis - p * PAGE;
         else if (my_nloc > 0) { lo = my_loc0 - (item.loc_lo + (p - item.n_cache_pages) * PAGE); hi = lo + my_nloc; }
@@ -587,7 +633,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 #pragma unroll
       for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(w[i]);
     };
-    if (pair) {
+    if (shared) {
       if (ok && nj > 0) {
         const float inv = item.split ? 1.f : 1.f / l_run;
 #pragma unroll
@@ -659,15 +705,21 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 // Merge the partial results of the query tiles that were split: O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s.
 // HD / 16 blocks of 256 threads per (query tile, KV head); a thread takes 8 columns of one MMA row, neighbouring
 // threads neighbouring rows, which is how the partial results lie in memory.
-template <int HD>
+template <int HD, bool DIRECT>
 __global__ void __launch_bounds__(256)
 attn_combine_kernel(const Args a, TlSlot tl) {
   pdl_trigger();
-  if (!a.early) pdl_wait();
+  if (DIRECT || !a.early) pdl_wait();
   constexpr int BLOCKS = HD / 16;
   const int w = blockIdx.x / BLOCKS, kvh = w % a.Hkv;
   const int cg = (blockIdx.x % BLOCKS) * 2 + (threadIdx.x >> 7), m = threadIdx.x & 127;
-  const Tile t = a.tiles[w / a.Hkv];
+  Tile t{};
+  if constexpr (DIRECT) {
+    const Item it = direct_tile(a, w / a.Hkv);
+    t.row0 = it.row0; t.row_end = it.row_end; t.n_items = direct_pieces(a, it.p_end); t.item0 = w / a.Hkv * a.direct.pieces;
+  } else {
+    t = a.tiles[w / a.Hkv];
+  }
   const int slot = t.row0 + m / a.G;
   pdl_wait();
   if (threadIdx.x == 0) tl_go(tl);

@@ -165,31 +165,21 @@ __global__ void assemble_prefill_kernel(RowMeta m, int seq, int row0, int n_prom
   embed_row_to_f32(embed + (size_t)id * d, X + (size_t)r * d, d);
 }
 
-// What row r of the stand-alone attention entry points sees (same slot layout as a step).
-// seq_len comes from the caller: it is clamped to [0, n_max] (n_max = the positions the page
-// table can back minus the k causal slots), so that no row looks past the table.
-__device__ __forceinline__ attn_tc::RowKeys attn_row_keys(const int32_t *__restrict__ seq_len, int k, int n_max, int r) {
-  const int T = k * (k + 1);
-  const int s = r / T, slot = r % T;
-  const int n = min(max(seq_len[s], 0), n_max);
-  if (slot < k) return attn_tc::RowKeys{n + slot + 1, 0, 0, s};
-  const int b = (slot - k) / k;
-  return attn_tc::RowKeys{n + b + 1, s * k * k + b * k, k, s};
-}
+// Row metadata of the stand-alone attention entry points.
 __global__ void attn_meta_kernel(RowMeta m, const int32_t *__restrict__ seq_len, int k, int R, int n_max) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= R) return;
-  const attn_tc::RowKeys w = attn_row_keys(seq_len, k, n_max, r);
+  const attn_tc::RowKeys w = attn_tc::step_row_keys(seq_len, k, n_max, r);
   m.seq[r] = w.seq; m.nvis[r] = w.nvis; m.loc0[r] = w.loc0; m.nloc[r] = w.nloc;
 }
 // The same for the tensor-core attention kernel, with its work plan (the first block).
 __global__ void __launch_bounds__(512) attn_meta_plan_kernel(RowMeta m, const int32_t *__restrict__ seq_len, int k, int R, int n_max, attn_tc::PlanArgs plan) {
   pdl_trigger();
   pdl_wait();
-  if (blockIdx.x == 0) { attn_tc::plan_block(plan, [&](int r) { return attn_row_keys(seq_len, k, n_max, r); }); return; }
+  if (blockIdx.x == 0) { attn_tc::plan_block(plan, [&](int r) { return attn_tc::step_row_keys(seq_len, k, n_max, r); }); return; }
   const int r = (blockIdx.x - 1) * blockDim.x + threadIdx.x;
   if (r >= R) return;
-  const attn_tc::RowKeys w = attn_row_keys(seq_len, k, n_max, r);
+  const attn_tc::RowKeys w = attn_tc::step_row_keys(seq_len, k, n_max, r);
   m.seq[r] = w.seq; m.nvis[r] = w.nvis; m.loc0[r] = w.loc0; m.nloc[r] = w.nloc;
 }
 

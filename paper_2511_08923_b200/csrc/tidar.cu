@@ -521,33 +521,66 @@ attn_tc::PlanArgs attention_plan(const tidar_ctx *c, int R, int rows_per_group) 
 // kernel, about 5 us, and saves half of 0.56 us per page at best.
 bool may_split(int n_keys) { return n_keys > 12 * attn_tc::PAGE; }
 
-// Attention of the pass that plan p was made for (the plan itself is in device memory by then).  early: see attn_tc::Args.
-void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMaps &m, const KvGeom &g, bf16 *O, bool early) {
+attn_tc::Args attention_args(const tidar_ctx *c, const AttnMaps &m, const KvGeom &g, bf16 *O) {
   const tidar_config &cf = c->cfg;
   attn_tc::Args a{};
-  a.G = cf.n_q_heads / cf.n_kv_heads; a.Hq = cf.n_q_heads; a.Hkv = cf.n_kv_heads; a.spt = p.spt;
-  a.items = p.items; a.tiles = p.tiles;
+  a.G = cf.n_q_heads / cf.n_kv_heads; a.Hq = cf.n_q_heads; a.Hkv = cf.n_kv_heads; a.spt = 128 / a.G;
   a.nvis = c->meta.nvis; a.loc0 = c->meta.loc0; a.nloc = c->meta.nloc;
   a.page_table = g.page_table; a.pages_per_seq = g.pages_per_seq;
   a.page_base_k = m.page_base_k; a.page_base_v = m.page_base_v;
   a.scale_log2 = 1.4426950408889634f / sqrtf((float)cf.head_dim);
-  a.early = early ? 1 : 0;
   a.O = O; a.part_O = c->attn_part_O; a.part_ml = c->attn_part_ml; a.status = c->d_status;
   a.tile_count = c->count_tiles ? c->d_tl + 2 * tidar_ctx::TL_MAX : nullptr;
-  const int grid = p.max_items * p.Hkv;
-  {
-    Launch l(c, TIDAR_TC_ATTN);
-    if (cf.head_dim == 128)
-      launch_pdl(attn_tc::attn_tc_kernel<128>, grid, attn_tc::THREADS, attn_tc::Smem<128>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
-    else
-      launch_pdl(attn_tc::attn_tc_kernel<64>, grid, attn_tc::THREADS, attn_tc::Smem<64>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
-  }
-  if (p.max_items > p.n_units && p.max_pieces > 1) {
-    Launch l(c, TIDAR_TC_ATTN);
-    const int blocks = 2 * p.n_units * p.Hkv * (cf.head_dim / 16);
-    if (cf.head_dim == 128) launch_pdl(attn_tc::attn_combine_kernel<128>, blocks, 256, 0, c->stream, a, l.tl);
-    else launch_pdl(attn_tc::attn_combine_kernel<64>, blocks, 256, 0, c->stream, a, l.tl);
-  }
+  return a;
+}
+template <int STREAMS, bool DIRECT>
+void launch_attention_kernel(tidar_ctx *c, int grid, const AttnMaps &m, const attn_tc::Args &a) {
+  Launch l(c, TIDAR_TC_ATTN);
+  const int threads = attn_tc::threads(STREAMS);
+  if (c->cfg.head_dim == 128)
+    launch_pdl(attn_tc::attn_tc_kernel<128, STREAMS, DIRECT>, grid, threads, attn_tc::Smem<128, STREAMS>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
+  else
+    launch_pdl(attn_tc::attn_tc_kernel<64, STREAMS, DIRECT>, grid, threads, attn_tc::Smem<64, STREAMS>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
+}
+
+template <bool DIRECT>
+void launch_attention_merge(tidar_ctx *c, int tiles, const attn_tc::Args &a) {
+  Launch l(c, TIDAR_TC_ATTN);
+  const int blocks = tiles * (c->cfg.head_dim / 16);
+  if (c->cfg.head_dim == 128) launch_pdl(attn_tc::attn_combine_kernel<128, DIRECT>, blocks, 256, 0, c->stream, a, l.tl);
+  else launch_pdl(attn_tc::attn_combine_kernel<64, DIRECT>, blocks, 256, 0, c->stream, a, l.tl);
+}
+
+// Attention of the pass that plan p was made for (the plan itself is in device memory by then).  early: see attn_tc::Args.
+void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMaps &m, const KvGeom &g, bf16 *O, bool early) {
+  attn_tc::Args a = attention_args(c, m, g, O);
+  a.items = p.items; a.tiles = p.tiles;
+  a.early = early ? 1 : 0;
+  launch_attention_kernel<2, false>(c, p.max_items * p.Hkv, m, a);
+  if (p.max_items > p.n_units && p.max_pieces > 1) launch_attention_merge<false>(c, 2 * p.n_units * p.Hkv, a);
+}
+
+// How a stand-alone call goes without a plan, every CTA working out its own item: streams per CTA (0 = planned) and items per query tile.
+// n_pages: pages a sequence may have (its length is on the device).  The plan kernel costs 4.5 us, which a pass pays once for all
+// layers but such a call alone; cutting a key range into p items saves (1 - 1/p) of 0.56 us per page and costs about 6 + 0.3 p us
+// (partial results, merge kernel).
+//   Where every tile may have as many SMs as it can use, sqrt(0.56 n_pages / 0.3), there is nothing to distribute: uncut up to 15 pages, cut
+//     evenly beyond (one sequence, k = 8, 32/8 heads of 128: 14.4 us uncut and 15.8 cut at 15 pages, 15.5 and 15.8 at 17, 16.4 and 16.1 at
+//     19; planned 18 - 18.7).
+//   Otherwise uncut while that is faster than planned: measured equal at 24 pages for four SMs per tile, 31 for two; the line
+//     lies a little below.  (k = 16, 1 k positions, 72 tiles: 18.9 us planned, 13.6 uncut.)
+//   With one to two tiles per SM, one stream per CTA and two CTAs per SM: one wave, where the plan's CTAs, which hold an SM each, need
+//     two.  Four sequences of 1 k positions there (288 tiles): 42.1 us planned, 25.7 this way, at 9 k 175 and 148; but a plan evens
+//     out ragged lengths, which pays from about 60 pages on (lengths between 2 k and 4 k: 53.9 planned, 58.1 not).
+struct DirectPlan { int streams, pieces; };
+DirectPlan attention_direct(const tidar_ctx *c, int n_seqs, int k, int n_pages) {
+  const int spt = 128 / (c->cfg.n_q_heads / c->cfg.n_kv_heads);
+  const long long tiles = (long long)n_seqs * ((k * (k + 1) + spt - 1) / spt) * c->cfg.n_kv_heads;
+  if (tiles > c->n_sms) return {tiles <= 2 * c->n_sms && n_pages <= 40 ? 1 : 0, 1};
+  const int most = std::min<int>(attn_tc::MAX_SPLITS, c->n_sms / (int)tiles);
+  const int pieces = (int)sqrt(1.9 * n_pages);
+  if (n_pages <= (pieces <= most ? 15 : 19 + 12 / most)) return {2, 1};
+  return {pieces <= most ? 2 : 0, pieces};
 }
 
 void launch_attention(tidar_ctx *c, const bf16 *Q, const bf16 *Kp, const bf16 *Vp, const KvGeom &g, const bf16 *Kl,
@@ -718,8 +751,13 @@ int init_tensor_core_path(tidar_ctx *c) {
     CUDA_TRY(c, cudaMemsetAsync(c->kv, 0, (size_t)cf.n_layers * 2 * c->pool_stride * sizeof(bf16), c->stream));
     CUDA_TRY(c, cudaMemsetAsync(c->Kloc, 0, nloc * cf.n_kv_heads * cf.head_dim * sizeof(bf16), c->stream));
     CUDA_TRY(c, cudaMemsetAsync(c->Vloc, 0, nloc * cf.n_kv_heads * cf.head_dim * sizeof(bf16), c->stream));
-    CUDA_TRY(c, cudaFuncSetAttribute(attn_tc::attn_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_tc::Smem<128>::TOTAL));
-    CUDA_TRY(c, cudaFuncSetAttribute(attn_tc::attn_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, attn_tc::Smem<64>::TOTAL));
+    auto smem = [](const void *f, int bytes) { return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 2, false>, attn_tc::Smem<128, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 2, false>, attn_tc::Smem<64, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 2, true>, attn_tc::Smem<128, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 2, true>, attn_tc::Smem<64, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 1, true>, attn_tc::Smem<128, 1>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 1, true>, attn_tc::Smem<64, 1>::TOTAL));
   }
   {
     auto max_smem_split = [&](const void *f) { return cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared); };
@@ -734,9 +772,12 @@ int init_tensor_core_path(tidar_ctx *c) {
                              (const void *)rmsnorm_reduce_kernel<512, 6, MAX_SLABS, float>, (const void *)rmsnorm_reduce_kernel<512, 6, MAX_SLABS, bf16>,
                              (const void *)rope_kv_kernel<1, float>, (const void *)rope_kv_kernel<MAX_SLABS, float>, (const void *)rope_kv_kernel<MAX_SLABS, bf16>,
                              (const void *)swiglu_slab_kernel<float>, (const void *)swiglu_slab_kernel<bf16>,
-                             (const void *)attn_tc::attn_combine_kernel<128>, (const void *)attn_tc::attn_combine_kernel<64>,
+                             (const void *)attn_tc::attn_combine_kernel<128, false>, (const void *)attn_tc::attn_combine_kernel<64, false>,
+                             (const void *)attn_tc::attn_combine_kernel<128, true>, (const void *)attn_tc::attn_combine_kernel<64, true>,
                              (const void *)mix_rows_kernel, (const void *)argmax_merge_kernel, (const void *)verify_select_kernel, (const void *)stage_step_kernel};
     for (const void *f : kernels) CUDA_TRY(c, max_smem_split(f));
+    CUDA_TRY(c, max_smem_split((const void *)attn_tc::attn_tc_kernel<128, 1, true>));
+    CUDA_TRY(c, max_smem_split((const void *)attn_tc::attn_tc_kernel<64, 1, true>));
     for (int i = 3; i < 19; ++i) CUDA_TRY(c, cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, NORM_SMEM));
   }
   const int max_smem = gemm_tc::SMEM_BUDGET + 1024;
@@ -1563,22 +1604,36 @@ int tidar_attention(tidar_ctx *c, const void *q, const void *k_pages, const void
       ((uintptr_t)page_table | (uintptr_t)seq_len) % 4)
     return fail(c, TIDAR_EINVAL, "tensors must be 16-byte aligned (page_table and seq_len 4-byte)");
   const int R = n_seqs * k * (k + 1), n_max = pages_per_seq * c->cfg.page_size - k;
-  c->split_keys = may_split(pages_per_seq * c->cfg.page_size);       // the lengths themselves are on the device
-  const attn_tc::PlanArgs plan = c->cfg.impl == 0 ? attention_plan(c, R, k * (k + 1)) : attn_tc::PlanArgs{};
-  {
-    Launch l(c, TIDAR_TC_EMBED);
-    if (c->cfg.impl == 0) launch_pdl(attn_meta_plan_kernel, 1 + (R + 511) / 512, 512, 0, c->stream, c->meta, seq_len, k, R, n_max, plan);
-    else attn_meta_kernel<<<(R + 127) / 128, 128, 0, c->stream>>>(c->meta, seq_len, k, R, n_max);
-  }
-  KvGeom g{c->cfg.n_kv_heads, c->cfg.head_dim, c->cfg.page_size, pages_per_seq, page_table, n_pages};
+  const KvGeom g{c->cfg.n_kv_heads, c->cfg.head_dim, c->cfg.page_size, pages_per_seq, page_table, n_pages};
   if (c->cfg.impl == 0) {
+    const DirectPlan d = attention_direct(c, n_seqs, k, pages_per_seq);
+    attn_tc::PlanArgs plan{};
+    if (!d.streams) {                              // (launched ahead of the host's work on the tensor maps)
+      c->split_keys = may_split(pages_per_seq * c->cfg.page_size);       // the lengths themselves are on the device
+      plan = attention_plan(c, R, k * (k + 1));
+      Launch l(c, TIDAR_TC_EMBED);
+      launch_pdl(attn_meta_plan_kernel, 1 + (R + 511) / 512, 512, 0, c->stream, c->meta, seq_len, k, R, n_max, plan);
+    }
     CUtensorMap tq, tk, tv, tkl, tvl;
     if (!encode_q_map(c, &tq, q, R) || !encode_pages_map(c, &tk, k_pages, n_pages) || !encode_pages_map(c, &tv, v_pages, n_pages) ||
         !encode_local_map(c, &tkl, k_local, (long long)n_seqs * k * k) || !encode_local_map(c, &tvl, v_local, (long long)n_seqs * k * k))
       return fail(c, TIDAR_ECUDA, "cuTensorMapEncodeTiled failed for an attention operand");
-    AttnMaps am{&tq, &tk, &tv, &tkl, &tvl, 0, 0};
-    launch_attention_tc(c, plan, am, g, (bf16 *)out, false);   // behind the kernel that makes the plan
+    const AttnMaps am{&tq, &tk, &tv, &tkl, &tvl, 0, 0};
+    if (d.streams) {
+      attn_tc::Args a = attention_args(c, am, g, (bf16 *)out);
+      a.direct.seq_len = seq_len; a.direct.k = k; a.direct.n_max = n_max; a.direct.pieces = d.pieces;
+      a.direct.per_group = (k * (k + 1) + a.spt - 1) / a.spt;
+      const int tiles = n_seqs * a.direct.per_group * a.Hkv;
+      if (d.streams == 2) launch_attention_kernel<2, true>(c, tiles * d.pieces, am, a); else launch_attention_kernel<1, true>(c, tiles, am, a);
+      if (d.pieces > 1) launch_attention_merge<true>(c, tiles, a);
+    } else {
+      launch_attention_tc(c, plan, am, g, (bf16 *)out, false);   // behind the kernel that makes the plan
+    }
   } else {
+    {
+      Launch l(c, TIDAR_TC_EMBED);
+      attn_meta_kernel<<<(R + 127) / 128, 128, 0, c->stream>>>(c->meta, seq_len, k, R, n_max);
+    }
     launch_attention(c, (const bf16 *)q, (const bf16 *)k_pages, (const bf16 *)v_pages, g, (const bf16 *)k_local, (const bf16 *)v_local,
                      (bf16 *)out, R);
   }

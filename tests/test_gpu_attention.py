@@ -128,6 +128,58 @@ def test_attention_work_plan(ns, k):
     t.close()
 
 
+@pytest.mark.parametrize("hd,Hq,Hkv,k,ns,launches", [
+    # one kernel, two streams per tile; from 16 pages on key ranges are cut and a merge kernel follows, the same number of items for every
+    # tile; with too few SMs for that the call is planned
+    (128, 8, 2, 1, [15 * 64 - 1], 1), (128, 8, 2, 1, [15 * 64], 2), (64, 4, 2, 12, [5000], 2),
+    (64, 4, 2, 3, [2500, 100, 700, 0, 400], 2),                    # eight items for the first, one or a few for the others
+    (128, 32, 8, 16, [1300], 1), (128, 32, 8, 16, [1700], 3),
+    (64, 4, 2, 8, [0, 1, 63, 64, 65, 700, 1], 1),
+    (128, 12, 2, 5, [300, 62, 63], 1),                             # 21 slots per tile: two unused rows
+    # one stream per tile, two CTAs per SM: between one and two tiles per SM
+    (128, 32, 8, 16, [0, 63, 64, 700], 1),                         # 288 tiles, the last of a sequence half empty
+    (64, 4, 2, 8, [(37 * i) % 300 for i in range(49)] + [2000], 1),
+    (64, 4, 2, 8, [5] * 49 + [2600], 3),                           # 41 pages: planned
+    (128, 12, 2, 5, [(11 * i) % 130 for i in range(40)], 1),
+    (128, 8, 8, 2, [1, 70] * 15, 1),                               # one head per KV head: a tile holds whole sequences' slots
+])
+def test_attention_without_a_plan(hd, Hq, Hkv, k, ns, launches):
+    t = _ctx(hd, Hq, Hkv, k, len(ns), 0)
+    before = t.launch_count()
+    _case(t, hd, Hq, Hkv, k, ns, 51)
+    assert t.launch_count() - before == launches
+    t.close()
+
+
+def test_attention_clamps_lengths_and_page_indices_without_a_plan():
+    """Lengths below 0 and beyond the table's positions are clamped on every route, and a page outside the pool reads as zeros: both the
+    two-stream and the one-stream instance against the same call with legal values."""
+    hd, Hq, Hkv, k, dev = 64, 4, 2, 8, "cuda:0"
+    for b in (2, 50):
+        t = _ctx(hd, Hq, Hkv, k, b, 0)
+        gen = torch.Generator(device=dev)
+        gen.manual_seed(b)
+
+        def rnd(*shape):
+            return torch.randn(*shape, device=dev, dtype=torch.bfloat16, generator=gen)
+        q, kp, vp, kl, vl = rnd(b * 72, Hq, hd), rnd(2 * b + 1, Hkv, 64, hd), rnd(2 * b + 1, Hkv, 64, hd), rnd(b * 64, Hkv, hd), rnd(b * 64, Hkv, hd)
+        kp[2 * b], vp[2 * b] = 0, 0
+        legal = torch.arange(2 * b, dtype=torch.int32, device=dev).view(b, 2)
+        legal[1, 0] = 2 * b
+        wild = legal.clone()
+        wild[1, 0] = 1 << 20
+        outs = []
+        for table, lens in ((legal, [0, 120] * (b // 2)), (wild, [-5, 100000] * (b // 2))):
+            out = torch.full((b * 72, Hq * hd), float("nan"), dtype=torch.bfloat16, device=dev)
+            before = t.launch_count()
+            t.attention(q, kp, vp, table, torch.tensor(lens, dtype=torch.int32, device=dev), kl, vl, out, b, k)
+            t.sync()
+            assert t.launch_count() - before == 1
+            outs.append(out)
+        assert torch.isfinite(outs[0]).all() and torch.equal(outs[0], outs[1])
+        t.close()
+
+
 def test_attention_beyond_32767_pages():
     """One sequence of 32770 pages.  Scores are small (weights within e^+-0.4 of each other) and V rises with the position, so that the output
     says which part of the cache was attended to: 0.5 for all of it.  Bound: bf16 rounding of the output, 2^-9 x 0.5, of V (the same,
