@@ -9,8 +9,8 @@ rows would not fit a test); for the 8B-class model its weights are handed to it 
 at a time, generated on demand, so that the host holds one layer in float64 and not 36.
 
 Every comparison is per row (3e-2 x max(1, max |reference row|)) and in rms (2.5 % of the
-reference's rms); the measured errors are printed and written to
-gpurun_out/fullsize_errors.json when that folder exists.
+reference's rms); the measured errors are printed and, when the environment variable
+TIDAR_ERROR_TABLE names a file, written there as JSON.
 """
 import json
 import os
@@ -60,9 +60,8 @@ def _run(sh, n_prompt=None, n_sample=12, lazy=False, tag=""):
         for what, v in report.items():
             print(f"{what}: max |err| {v['max_abs']:.4f} (reference max {v['max_ref']:.2f}), rms err / rms ref {v['rms_rel']:.4f}, "
                   f"worst row at {v['worst_row_err_over_tol']:.2f} of its bound")
-        out_dir = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "gpurun_out")
-        if os.path.isdir(out_dir):
-            path = os.path.join(out_dir, "fullsize_errors.json")
+        path = os.environ.get("TIDAR_ERROR_TABLE")
+        if path:
             prev = json.load(open(path)) if os.path.exists(path) else {}
             prev.update(report)
             json.dump(prev, open(path, "w"), indent=1)
