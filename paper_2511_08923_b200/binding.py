@@ -299,9 +299,9 @@ class Tidar:
         self._check(self.lib.tidar_debug_set_block(self.ctx, seq, _ip(b)))
 
     def get_block(self, seq: int, k: int) -> List[int]:
-        b = np.empty(k, dtype=np.int32)
+        b = np.zeros(max(k, self.k_max), dtype=np.int32)         # the library writes as many as the block holds
         self._check(self.lib.tidar_debug_get_block(self.ctx, seq, _ip(b)))
-        return b.tolist()
+        return b[:k].tolist()
 
     def last_rows(self):
         n, p = C.c_int32(0), C.c_int32(0)
