@@ -229,7 +229,8 @@ int tidar_ar_step(tidar_ctx *ctx, const int32_t *seqs /*host,[n_seqs]*/, int32_t
  * distribution; Section 4.2, likelihood tasks): one causal pass over ids[0..n) and
  * logprobs[i] = log softmax(logits at position i)[ids[i+1]] for i in [0, n-1).
  * Uses sequence slot `seq` as scratch: whatever it held is dropped and the slot is left
- * empty.  The log-sum-exp runs over vocabulary chunks; full logits are never kept.
+ * empty.  Full logits are never kept: the log-sum-exp is put together from pieces of 32 ids
+ * inside the LM head's projection (impl 1: from vocabulary chunks).
  * Needs 2 <= n <= max_seq_len.  Synchronises the stream.                                  */
 int tidar_score(tidar_ctx *ctx, int32_t seq, const int32_t *ids /*host,[n]*/, int32_t n, float *logprobs /*host,[n-1]*/);
 
@@ -365,8 +366,8 @@ int tidar_sync(tidar_ctx *ctx);
  *   - It always runs the plain CUDA-core kernel (one warp per row and query head, fp32
  *     accumulation, K/V re-read once per query head, no tile skipping), not the
  *     tensor-core kernel: correct and allocation-free, not fast (measured at 32 / 8 heads,
- *     k = 16: 1.1 ms against 28 us for tidar_attention with impl 0 at a thousand cached
- *     positions, 4.2 ms against 45 us at four thousand).
+ *     k = 16: 1.1 ms against 16 us for tidar_attention with impl 0 at a thousand cached
+ *     positions, 4.2 ms against 34 us at four thousand).
  *   - Limit: n_seqs * k * (k+1) <= 4352 rows (16 sequences at k = 16); beyond that the
  *     call returns TIDAR_ECAPACITY and launches nothing.  page_size is 64.
  *   - Each GPU that loads the library holds the table (85 KiB) until the process exits.

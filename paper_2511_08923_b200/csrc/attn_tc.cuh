@@ -20,9 +20,9 @@
 // for the other's latency.
 // What bounds it: shared memory.  A step's operands are 64 KB read (Q 32, K 16, V 16) and up to 32 KB written by
 // the loads, 500 - 750 cycles at 128 B per cycle against 512 cycles of MMAs (a product with N = 64 takes 48 cycles, not
-// 32, for the 6 KB it reads); a step takes 0.53 - 0.56 us, 0.93 - 0.98 kcycles, on an SM.  Whole calls, 32/8
-// heads of 128, 272 rows, 1 k / 4 k / 16 k / 32 k cached positions: 22.0 / 32.7 / 82 / 148 us; the kernel before this one
-// (two CTAs per SM, one tile and one stream each, the same split for every sequence) took 26.4 / 40 / 97 / 197 us.
+// 32, for the 6 KB it reads); a step takes 0.53 - 0.56 us, 0.93 - 0.98 kcycles, on an SM.  Whole calls with warm caches, 32/8
+// heads of 128, 272 rows, 1 k / 4 k / 16 k / 32 k cached positions: 16.5 / 33 / 84 / 153 us; the kernel before this one
+// (two CTAs per SM, one tile and one stream each, the same split for every sequence) took 26.2 / 40 / 97 / 173 us.
 //   PAIR of tiles: A and B are two query tiles, each K/V page serves both: half the loads, and 80
 //     instead of 96 KB through shared memory per step.
 //   SINGLE tile: A and B are the same query tile and take the pages in turn; their two results are merged through
@@ -44,6 +44,8 @@
 // tiles are paired, cuts key ranges into items of about equal time, whatever the sequences' lengths
 // are, and lists long items first (a causal first pass would otherwise end on its longest rows).
 // Partial (max, sum, O) results of a tile with several items are merged by attn_combine_kernel.
+// A stand-alone call pays for its plan alone (4.5 us).  Where there is little to distribute it does without: every CTA
+// works out its own item (direct_item), with an instance of one stream per CTA where that saves a wave.
 #pragma once
 #include "common.cuh"
 #include "sm100_ptx.cuh"
@@ -134,7 +136,8 @@ static_assert(sizeof(Ctl) <= 512, "control block must fit its slot");
 // SM run in later waves, of which on average half a CTA's time is lost at the end.
 // Everything is kept in shared memory until the plan is made: a trip to global memory and back costs as much as all
 // of the arithmetic.
-// (Measured inside the kernel, head_dim 128, all SMs busy: 1.05 us per page of a pair, 0.56 of a single tile.)
+// (Measured inside the kernel, head_dim 128, all SMs busy: 1.05 us per page of a pair, 0.56 of a single tile.  head_dim 64 and nearly empty
+// grids take the same figures, although a page costs them less: they were not fitted, and cuts come out somewhat finer than best.)
 constexpr float OVERHEAD = 5.f, PAIR_PAGE = 1.05f, SINGLE_PAGE = 0.56f, PAIR_STORE = 2.5f, SINGLE_STORE = 1.5f, MERGE = 3.f;
 constexpr int PLAN_UNITS = 256;                        // up to this many units are planned; beyond, every unit is one item
 constexpr int CAND = 32;                               // limits tried per pairing: longest / (1 + i / 2)

@@ -55,7 +55,8 @@ constexpr int MAX_STAGES = 12;     // of the ring (hardware barriers 1 .. 12)
 // * Per stage: each costs its producers, the watcher and the MMA warp some 600 cycles of barrier tests and issue,
 //   three times what the MMAs of a 64-wide K block take with few rows.  A stage holds two K blocks there.
 // 1.5B-class autoregressive step of 8 rows 1.90 -> 1.75 ms, 8B-class step of 20 rows 4.2 -> 4.0 ms (the gate/up projection
-// of the former 11.4 -> 10.3 us, QKV 5.3 -> 3.4 us).  Measured and not kept: fetching weights into L2 ahead of the ring, this
+// of the former 11.4 -> 10.3 us, QKV 5.3 -> 3.4 us).  80 registers are not enough for the SwiGLU epilogue, which spills 27 words per thread
+// once per item.  Measured and not kept: fetching weights into L2 ahead of the ring, this
 // launch's or the next projection's (2 - 8 % slower, the more the further ahead).
 constexpr int SMALL_ROWS = 96;
 constexpr int SMALL_TMEM_COLS = 128;

@@ -335,7 +335,8 @@ int lm_head_ctas(const tidar_ctx *c, int R, int vocab) {
 // matrix is small: such a launch is all start-up and slab store, both of which a SMALL CTA, which sits beside the kernels in
 // front of it, hides better, and re-reading a few MB of weights per block from L2 costs less.  (1.5B-class step at 272 rows, its
 // projections of 2.4 - 13.8 M weights: 2.18 -> 1.96 ms; 8B-class, from 16.8 M weights on: 1 % slower that way; the fused
-// gate/up projection of 27.5 M weights: 12 % of the step slower.)
+// gate/up projection of 27.5 M weights: 12 % of the step slower.  15 M is simply a line between the two models measured: a matrix
+// between 13.8 M and 16.8 M weights may do a per cent better on the other side.)
 bool small_gemm(int mode, int R, int N, int K) {
   if (mode != gemm_tc::MODE_SLAB && mode != gemm_tc::MODE_SWIGLU) return false;
   return R <= gemm_tc::SMALL_ROWS || (mode == gemm_tc::MODE_SLAB && R <= gemm_tc::MAX_ROWS && (long long)N * K <= 15000000);
