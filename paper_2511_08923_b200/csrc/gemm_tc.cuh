@@ -97,7 +97,7 @@ struct Args {
   float inv_temp; const uint32_t *skey;
   // MODE_LSE: (max, sum) of lse_parts(N) groups of 32 ids, [group][R]; the target id of each row, and its logit
   float2 *lse; const int32_t *target; float *tgt_logit;
-  int warm_epilogue;        // MODE_SWIGLU: walk through the epilogue once before the first accumulator is ready (see the kernel)
+  int warm_epilogue;        // walk through the epilogue once before the first accumulator is ready (see the kernel)
   int *status;              // device word set to 1 when a bounded wait gave up
   __host__ __device__ int tile_b0_or_all() const { return n_tiles_b ? tile_b0 : n_tiles; }   // tiles per row block in the fused region
   __host__ __device__ int total_items() const { return fused_items + n_rb * n_tiles_b * S; }
@@ -408,32 +408,75 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // warps have nothing to do while the first item's MMAs run, so they first walk through the
     // epilogue once with every store and barrier operation switched off (dry), which
     // brings the code in; g.warm_epilogue is a run-time value so that both walks share one copy.
+    // Slabs and additions to the residual stream of the pair instances are walked through as well: 272 rows x 128 features leave a CTA in 3.6 - 3.9 us
+    // then (4.6 - 6.4 before; 3.4 in a kernel that does nothing else, 28 B per cycle: the SM's port, whatever the instruction).  That walk
+    // starts a little later, for the role warps' first rounds fetch code too (started at once, the first stage landed 0.3 us later).  Turning them
+    // into a short loop over tensor memory instead was slower (8.3 us): a store holds its register until the port takes it.
+    // The SMALL instances' slabs are too short for a walk (it cost as much as it gave).
     // A fused item that is its CTA's last one takes a third route: nobody waits for the accumulator, so it
     // stays in tensor memory and a loop of a few hundred instructions takes 32 columns per round (the
     // 1.5B-class gate/up projection, one item per CTA, ends 4 us earlier than with the long code).  With few rows
-    // every fused item goes that way: it is one or two rounds.
-    bool dry = (MODE == MODE_SWIGLU) && !SMALL && g.warm_epilogue != 0 && worker + n_workers < n_items;
+    // every fused item goes that way: it is one or two rounds.  So does a split item of a SwiGLU launch, 16 columns per round.  Their first round
+    // is a dry one, on whatever tensor memory holds, before the wait for the accumulator (8B-class gate/up at 20 rows 33.3 -> 30.3 us, at 272 rows
+    // 47.9 -> 46).
+    const bool may_walk = !SMALL && g.warm_epilogue != 0;
+    bool walk = may_walk && (MODE == MODE_SLAB || (MODE == MODE_SWIGLU && worker + n_workers < n_items));
     for (int item = worker; item < n_items && ok;) {
       const Item w = decode_item<MODE>(g, item);
       const int split = w.split, rb = w.rb, row_block = rb * g.rb_rows;
       const int n0 = (PAIR ? w.tile * 2 + rank : w.tile) * TILE_N;      // first weight row of this CTA's tile
       if (MODE == MODE_SWIGLU && w.fused && (SMALL || item + n_workers >= n_items)) {
-        if (!sm100::mbar_wait(sm100::smem_u32(&tmem_full_bar), it & 1u, abortp)) { ok = false; break; }
-        sm100::tc_fence_after();
         const uint32_t t0 = tmem_acc + ((uint32_t)(q * 32) << 16) + (uint32_t)c_begin;
+        bool live = false;
 #pragma unroll 1
-        for (int cc = 0; cc < ncols; cc += 32) {
+        for (int cc = 0; !live || cc < ncols;) {       // (a warp without columns waits for the accumulator too, or it would run ahead of the others)
           uint32_t c0[16], c1[16];
           const bool second = cc + 16 < ncols;
           sm100::tmem_ld16(t0 + cc, c0);
           if (second) sm100::tmem_ld16(t0 + cc + 16, c1);
           sm100::tmem_wait_ld();
-          swiglu_pass(c0, c1, second, c_begin + cc, row_block, g.R, n0);
+          swiglu_pass(c0, c1, second, c_begin + cc, row_block, live ? g.R : 0, n0);
+          if (live) { cc += 32; continue; }
+          if (!sm100::mbar_wait(sm100::smem_u32(&tmem_full_bar), it & 1u, abortp)) { ok = false; break; }
+          sm100::tc_fence_after();
+          live = true;
         }
+        if (!ok) break;
         drained();
         item += n_workers; ++it;
         continue;
       }
+      if (MODE == MODE_SWIGLU && !w.fused && !g.slab_bf16) {
+        // Partial sums of a split tile (always its CTA's last item).
+        const int n = n0 + q * 32 + lane, n_rows = n < g.N ? g.R : 0;
+        float *out = reinterpret_cast<float *>(g.out) + (long long)split * g.slab_stride + (n - g.tile_b0 * tile_rows(SMALL));
+        const uint32_t t0 = tmem_acc + ((uint32_t)(q * 32) << 16) + (uint32_t)c_begin;
+        bool live = false;
+#pragma unroll 1
+        for (int cc = 0; !live || cc < ncols;) {
+          uint32_t c0[16];
+          sm100::tmem_ld16(t0 + cc, c0);
+          sm100::tmem_wait_ld();
+#pragma unroll
+          for (int h = 0; h < 16; h += 8) {
+            const int r0 = row_block + col_row(c_begin + cc + h);
+            float *p = out + (long long)r0 * g.ldo;
+            const int rows_left = live ? n_rows - r0 : 0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { if (j < rows_left) *p = __uint_as_float(c0[h + j]); p += g.ldo; }
+          }
+          if (live) { cc += 16; continue; }
+          if (!sm100::mbar_wait(sm100::smem_u32(&tmem_full_bar), it & 1u, abortp)) { ok = false; break; }
+          sm100::tc_fence_after();
+          live = true;
+        }
+        if (!ok) break;
+        drained();
+        item += n_workers; ++it;
+        continue;
+      }
+      const bool dry = walk;
+      if (MODE == MODE_SLAB && dry) __nanosleep(1500);
       uint32_t v[NCH][16];
       if (!dry) {
         if (!sm100::mbar_wait(sm100::smem_u32(&tmem_full_bar), it & 1u, abortp)) { ok = false; break; }
@@ -452,7 +495,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         // split-K partial sums; columns are counted from the first tile of the split region
         const int nc = n - g.tile_b0 * tile_rows(SMALL);
         const bool n_ok = n < g.N;
-        if (g.accumulate) {
+        if (MODE == MODE_SLAB && g.accumulate) {
           constexpr int RUN = SMALL ? 16 : 8;            // columns that are consecutive rows
           float *out = reinterpret_cast<float *>(g.out) + nc;
 #pragma unroll
@@ -471,7 +514,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
               }
             }
           }
-        } else if (!g.slab_bf16) {
+        } else if (MODE == MODE_SLAB && !g.slab_bf16) {
           // One running pointer and a bound counted from the first row of eight: with the address
           // and the row test recomputed per store (r * ldo, r < R) the same 144 stores take 1.65 times
           // as long (19.5 instead of 32 bytes per cycle and SM, the rate the L2 takes stores at).
@@ -624,7 +667,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           }
         }
       }
-      if (dry) dry = false;                              // the same item again, for real
+      if (walk) walk = false;                            // the same item again, for real
       else { item += n_workers; ++it; }
     }
     if (MODE == MODE_ARGMAX || MODE == MODE_SAMPLE) flush_best();

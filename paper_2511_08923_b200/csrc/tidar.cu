@@ -408,7 +408,7 @@ int gemm_tc_launch(tidar_ctx *c, int mode, const bf16 *A, int a_rows, const tida
     a.inv_temp = c->cfg.temperature > 0.f ? 1.0f / c->cfg.temperature : 0.f; a.skey = c->meta.skey + c->head_row0;
   }
   a.status = c->d_status;
-  a.warm_epilogue = mode == gemm_tc::MODE_SWIGLU ? 1 : 0;
+  a.warm_epilogue = 1;
   const int box = small ? a.rb_rows : a.rb_rows / 2;
   const CUtensorMap *tmA = act_map(c, A, a_rows, K, box, small);
   if (!tmA) return fail(c, TIDAR_ECUDA, "cuTensorMapEncodeTiled failed for an activation matrix (%d x %d, box %d)", a_rows, K, box);

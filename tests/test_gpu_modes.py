@@ -113,6 +113,28 @@ def test_scoring_without_logits_matches_the_replay_kernels(n, vocab):
     assert np.abs(got[0] - got[1]).max() <= TOL_LOGITS
 
 
+@pytest.mark.parametrize("rows", [3, 16, 17, 96, 97, 256, 272, 288, 300])
+def test_gate_up_tiles_beyond_one_wave(rows):
+    """A gate/up matrix with more tiles than a wave holds: whole tiles followed by split ones on the same CTA, for row blocks of which half the
+    epilogue warps have no columns (16 rows), both instances, one and two instructions, two row blocks.  Hidden states after two layers and the
+    cached K/V of the second against the fp32 CUDA-core kernels."""
+    from dataclasses import replace as _r
+    from paper_2511_08923_b200 import Tidar, pack_weights
+    from paper_2511_08923_b200.binding import bf16_bits_to_f32
+    from tidar_synth import CONFIGS as CONFIGS_, gen_model_weights as gen_model_weights_
+    sh = _r(CONFIGS_["tiny"], d_model=512, d_ffn=12288, vocab=300)
+    packed = pack_weights(gen_model_weights_(sh), "cuda:0")
+    ids = prompt_ids(sh, n=rows - 2, seed=rows)
+    got = []
+    for impl in IMPLS:
+        t = Tidar(sh, packed, k_max=2, max_batch=1, max_seq_len=512, debug=1, impl=impl, guard_bytes=64 * 1024, prefill_rows=304)
+        t.prefill(0, ids, 2)
+        got.append((t.hidden(2, 0, t.last_rows()[0]), np.stack([bf16_bits_to_f32(x) for x in t.kv(0, 1, 0, len(ids))])))
+        _close(t)
+    for a, b in zip(*got):
+        assert np.isfinite(a).all() and np.abs(a - b).max() <= TOL_LOGITS * max(1.0, float(np.abs(b).max())), np.abs(a - b).max()
+
+
 def test_autoregressive_mode_at_the_benchmark_widths():
     """The one-slot step and the scoring pass at the 8B-class widths (two layers, 8192-entry vocabulary so
     that the oracle stays fast): one-row projections (a 16-row MMA block), 4096-wide rows, 32 / 8 heads.
