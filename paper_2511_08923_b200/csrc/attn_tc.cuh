@@ -92,8 +92,8 @@ struct Args {
   bf16 *O;                                   // [R][Hq*hd]
   float *part_O;                             // [CTA][tile of the pair][hd / 4][128 rows][4]: a warp's stores are contiguous
   float2 *part_ml;                           // [CTA][tile of the pair][128 rows] (reference max, sum)
-  // early: plan, row metadata and page table were written before the kernel in front of this one started, and that one lets its
-  // successor in only once its own predecessors are complete, so they are read ahead of pdl_wait()
+  // early: plan, row metadata and page table, which were written before the pass's first RoPE kernel, are read ahead of pdl_wait(): that kernel
+  // lets its successor in only once its own predecessors are complete, and every later kernel of the pass starts after that
   int early;
   // Stand-alone calls without a plan (items = null; DIRECT instances): what a CTA works out its item and its rows' keys from.
   struct { const int32_t *seq_len; int k, n_max; int per_group, pieces; } direct;    // query tiles per sequence, items per tile at most
@@ -330,7 +330,14 @@ __device__ __forceinline__ Item direct_item(const Args &a, int e) {
 
 // STREAMS = 1: one tile and one stream per CTA and two CTAs per SM, which fill each other's latencies as two streams do.  It serves calls that are
 // one wave that way and two otherwise (see attention_direct for both sides' figures).  DIRECT: no plan, see direct_item.
-template <int HD, int STREAMS, bool DIRECT>
+// AHEAD (decode steps of few rows, whose CTAs become resident well before the RoPE kernel ends): what does not depend on that kernel is done ahead of
+// the wait.  The rows of a step see at most 64 positions more than their sequence had cached before it, so of n cached pages a query tile
+// needs, no kernel of the step writes the first n - 2, and those go into the rings at once; they come from HBM, the weights of a step having passed
+// through the L2 since the last one.  And the softmax warps walk through one step with nothing stored, on whatever tensor memory holds, which
+// fetches the loop's code.  (8B-class step of 20 rows: 10.1 us behind a gap of 0.77 -> 8.9 behind 0.70; 1.5B-class autoregressive step of 8 rows 6.05 -> 4.75.
+// At 272 rows the CTAs wait for the SMs of the projection in front of the RoPE kernel and only lose by it; walking through the output code too was slower
+// everywhere, by 0.8 - 2 us.)
+template <int HD, int STREAMS, bool DIRECT, bool AHEAD>
 __global__ void __launch_bounds__(threads(STREAMS), 3 - STREAMS)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                const __grid_constant__ CUtensorMap tmKloc, const __grid_constant__ CUtensorMap tmVloc, const Args a, const TlSlot tl) {
@@ -393,21 +400,27 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       const int32_t *table = a.page_table + (size_t)item.seq * a.pages_per_seq;
       const int n_table = min(item.n_cache_pages, item.p_end) - p_begin;         // pages of this item that the table backs
       int cur = lane < n_table ? table[p_begin + lane] : 0, next = 0;
-      pdl_wait();                                      // Q, K and V are the previous kernel's output
-      if (threadIdx.x == 0) tl_go(tl);
-      if (!is_k && sm100::elect_one()) {
-        const uint32_t qb = sm100::smem_u32(&ctl.q_full);
-        sm100::mbar_expect_tx(qb, (uint32_t)(NH * rows_used * 128 * (pair ? 2 : 1)));
-        for (int t = 0; t < (pair ? 2 : 1); ++t)
-          for (int h = 0; h < NH; ++h)
-            sm100::tma_load_3d(smem0 + L::Q_OFF + t * L::Q_BYTES + h * (128 * 128), &tmQ, qb, h * 64, kvh * a.G, row0 + t * a.spt, pol);
-      }
       const CUtensorMap *tm = is_k ? &tmK : &tmV, *tm_loc = is_k ? &tmKloc : &tmVloc;
       const int base = is_k ? a.page_base_k : a.page_base_v;
+      const int stages = is_k ? L::K_STAGES : L::V_STAGES;
       const uint32_t full0 = sm100::smem_u32(is_k ? ctl.k_full : ctl.v_full), empty0 = sm100::smem_u32(is_k ? ctl.k_empty : ctl.v_empty);
       const uint32_t dst0 = smem0 + (is_k ? L::K_OFF : L::V_OFF);
+      const int n_ahead = AHEAD ? max(min(min(item.n_cache_pages - 2 - p_begin, np), stages), 0) : 0;
       int s = 0; uint32_t ph = 1u;
-      for (int p = 0; p < np; ++p) {
+      for (int p = 0;; ++p) {
+        if (p == n_ahead) {
+          pdl_wait();                                  // Q and all other pages are the previous kernel's output
+          if (threadIdx.x == 0) tl_go(tl);
+          if (!is_k && sm100::elect_one()) {
+            const uint32_t qb = sm100::smem_u32(&ctl.q_full);
+            sm100::mbar_expect_tx(qb, (uint32_t)(NH * rows_used * 128 * (pair ? 2 : 1)));
+            for (int t = 0; t < (pair ? 2 : 1); ++t)
+              for (int h = 0; h < NH; ++h)
+                sm100::tma_load_3d(smem0 + L::Q_OFF + t * L::Q_BYTES + h * (128 * 128), &tmQ, qb, h * 64, kvh * a.G, row0 + t * a.spt, pol);
+          }
+          __syncwarp();
+        }
+        if (p == np) break;
         if ((p & 31) == 0) {
           if (p) cur = next;
           next = p + 32 + lane < n_table ? table[p_begin + p + 32 + lane] : 0;
@@ -421,7 +434,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
           else sm100::tma_load_4d(dst, tm_loc, fb, 0, item.loc_lo + (p_begin + p - item.n_cache_pages) * PAGE, 0, kvh, pol);
         }
         __syncwarp();
-        if (++s == (is_k ? L::K_STAGES : L::V_STAGES)) { s = 0; ph ^= 1u; }
+        if (++s == stages) { s = 0; ph ^= 1u; }
       }
     }
   } else if (warp == 1) {
@@ -535,9 +548,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     auto wait_s = [&](int j) { return __all_sync(0xffffffffu, sm100::mbar_wait(s_bar0 + (uint32_t)(j & 1) * 8u, (uint32_t)(j >> 1) & 1u, abortp)) != 0; };
     float m_ref = -INFINITY, l_run = 0.f;
     bool ok = true;
-    for (int j = 0; j < nj; ++j) {
-      if (!(ok = wait_s(j))) break;
-      sm100::tc_fence_after();
+#pragma unroll 1
+    for (int j = AHEAD ? -1 : 0; j < nj; ++j) {          // (step -1: the walk)
+      const bool live = !AHEAD || j >= 0;
+      if (live) {
+        if (!(ok = wait_s(j))) break;
+        sm100::tc_fence_after();
+      }
       const uint32_t s_addr = s_addr0 + (uint32_t)((j & 1) * PAGE);
       uint32_t sv[2][32];
       sm100::tmem_ld32(s_addr, sv[0]);
@@ -548,7 +565,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       {
         const int p = p_begin + (shared ? j : 2 * j + t);
         int lo = 0, hi = 0;
-        if (p < item.n_cache_pages) hi = my_nvis - p * PAGE;
+        if (!live) { }
+        else if (p < item.n_cache_pages) hi = my_nvis - p * PAGE;
         else if (my_nloc > 0) { lo = my_loc0 - (item.loc_lo + (p - item.n_cache_pages) * PAGE); hi = lo + my_nloc; }
         if (lo > 0 || hi < PAGE) {
 #pragma unroll
@@ -567,7 +585,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       const float m_new = (mx > m_ref + RAISE_THRESHOLD) ? mx : m_ref;
       const float alpha = (m_new == m_ref) ? 1.f : exp2f(m_ref - m_new);      // m_ref = -inf gives 0
       const float neg_m = (m_new == -INFINITY) ? 0.f : -m_new;
-      m_ref = m_new;
+      m_ref = live ? m_new : m_ref;
       if (j > 0 && __any_sync(0xffffffffu, alpha != 1.f)) {
         // O is rescaled in place: P V of step j - 1 must be done; that of step j waits for P
         if (!(ok = wait_s(j + 1))) break;
@@ -594,14 +612,16 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
         pk[c >> 1] = *reinterpret_cast<uint32_t *>(&h);
       }
-      sm100::tmem_st32(s_addr, pk);
-      sm100::tmem_wait_st();
-      sm100::tc_fence_before();
-      __syncwarp();
-      if (lane == 0) sm100::mbar_arrive(p_bar0 + (uint32_t)(j & 1) * 8u);
+      if (live) {
+        sm100::tmem_st32(s_addr, pk);
+        sm100::tmem_wait_st();
+        sm100::tc_fence_before();
+        __syncwarp();
+        if (lane == 0) sm100::mbar_arrive(p_bar0 + (uint32_t)(j & 1) * 8u);
+      }
       float sa, sb;
       sm100::unpack2(sm100::add2(sum2[0], sum2[1]), sa, sb);
-      l_run = l_run * alpha + (sa + sb);
+      l_run = live ? l_run * alpha + (sa + sb) : 0.f;
     }
     // ---- output: O is complete once the last P V has finished ----
     pdl_wait();                                          // (long over; the stores below must not overtake it formally either)

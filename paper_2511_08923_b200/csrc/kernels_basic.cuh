@@ -213,10 +213,14 @@ __global__ void __launch_bounds__(256) pass_setup_kernel(RowMeta m, int R, int h
 // groups of four columns in registers (NV * 4 * THREADS >= d).
 // ---------------------------------------------------------------------------
 // SLABS: the most partial results there can be (1 or MAX_SLABS: with one, four blocks of a many-row pass fit on an SM).
-template <int THREADS, int NV, int SLABS, typename SLAB>
-__global__ void __launch_bounds__(THREADS, SLABS == 1 && NV <= 2 ? 4 : 1)
+// WALK (passes of few rows, whose blocks are resident long before their input is ready): the block goes through everything twice, the first time
+// ahead of the wait, with the loads from its output buffer, which it reads nowhere else, and nothing stored.  That brings the code into the
+// instruction cache, from which a layer's other kernels push it between two launches.  (8 rows of 1536: 1.5 - 1.8 us behind a gap of 1.35 -> 1.3 - 1.4
+// behind 0.8; 20 rows of 4096: gap 1.35 -> 0.85.  With many rows the blocks start late and the walk is in their way: 272 rows of 1536 1.8 -> 3.0 us.)
+template <int THREADS, int NV, int SLABS, bool WALK, typename SLAB>
+__global__ void __launch_bounds__(THREADS, SLABS == 1 && NV <= 2 && !WALK ? 4 : 1)
 rmsnorm_reduce_kernel(float *__restrict__ X, const SLAB *__restrict__ partials, int S, size_t partial_stride,
-                      const bf16 *__restrict__ gain, float eps, int d, bf16 *__restrict__ A, TlSlot tl) {
+                      const bf16 *__restrict__ gain, float eps, int d, bf16 *A, TlSlot tl) {
   pdl_trigger();
   __shared__ float red[THREADS / 32];
   const int r = blockIdx.x;
@@ -226,38 +230,48 @@ rmsnorm_reduce_kernel(float *__restrict__ X, const SLAB *__restrict__ partials, 
     const int c = (i * THREADS + threadIdx.x) * 4;
     gb[i] = c < d ? *reinterpret_cast<const uint2 *>(gain + c) : make_uint2(0u, 0u);
   }
-  pdl_wait();
-  if (threadIdx.x == 0) tl_go(tl);
   float *xr = X + (size_t)r * d;
-  float4 v[NV];
-  float ss = 0.f;
-#pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    const int c = (i * THREADS + threadIdx.x) * 4;
-    v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (c < d) {
-      v[i] = *reinterpret_cast<const float4 *>(xr + c);
-      add_slabs<SLABS, SLABS>(v[i], partials + (size_t)r * d + c, S, partial_stride);
+#pragma unroll 1
+  for (int walk = WALK ? 0 : 1; walk < 2; ++walk) {
+    const bool live = !WALK || walk != 0;
+    if (live) {
+      pdl_wait();
+      if (threadIdx.x == 0) tl_go(tl);
     }
-    ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
-  }
-  ss = warp_sum(ss);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
-  __syncthreads();
-  float tot = 0.f;
+    const float *x = live ? xr : reinterpret_cast<const float *>(A);
+    const SLAB *p = live ? partials + (size_t)r * d : reinterpret_cast<const SLAB *>(A);
+    const size_t stride = live ? partial_stride : 0;
+    float4 v[NV];
+    float ss = 0.f;
 #pragma unroll
-  for (int i = 0; i < THREADS / 32; ++i) tot += red[i];
-  const float inv = rsqrtf(tot / (float)d + eps);
-#pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    const int c = (i * THREADS + threadIdx.x) * 4;
-    if (c < d) {
-      if (S > 0) *reinterpret_cast<float4 *>(xr + c) = v[i];
-      const float2 g0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gb[i].x)), g1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gb[i].y));
-      __nv_bfloat162 o0 = __floats2bfloat162_rn(v[i].x * inv * g0.x, v[i].y * inv * g0.y), o1 = __floats2bfloat162_rn(v[i].z * inv * g1.x, v[i].w * inv * g1.y);
-      uint2 ob; ob.x = *reinterpret_cast<uint32_t *>(&o0); ob.y = *reinterpret_cast<uint32_t *>(&o1);
-      *reinterpret_cast<uint2 *>(A + (size_t)r * d + c) = ob;
+    for (int i = 0; i < NV; ++i) {
+      const int c = (i * THREADS + threadIdx.x) * 4, at = live ? c : 0;
+      v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c < d) {
+        v[i] = *reinterpret_cast<const float4 *>(x + at);
+        add_slabs<SLABS, SLABS>(v[i], p + at, S, stride);
+      }
+      ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
     }
+    ss = warp_sum(ss);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+    __syncthreads();
+    float tot = 0.f;
+#pragma unroll
+    for (int i = 0; i < THREADS / 32; ++i) tot += red[i];
+    const float inv = rsqrtf(tot / (float)d + eps);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int c = (i * THREADS + threadIdx.x) * 4;
+      if (c < d) {
+        if (live && S > 0) *reinterpret_cast<float4 *>(xr + c) = v[i];
+        const float2 g0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gb[i].x)), g1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gb[i].y));
+        __nv_bfloat162 o0 = __floats2bfloat162_rn(v[i].x * inv * g0.x, v[i].y * inv * g0.y), o1 = __floats2bfloat162_rn(v[i].z * inv * g1.x, v[i].w * inv * g1.y);
+        uint2 ob; ob.x = *reinterpret_cast<uint32_t *>(&o0); ob.y = *reinterpret_cast<uint32_t *>(&o1);
+        if (live) *reinterpret_cast<uint2 *>(A + (size_t)r * d + c) = ob;
+      }
+    }
+    if (WALK && !live) __syncthreads();            // red is written again
   }
   if (threadIdx.x == 0) tl_end(tl);
 }
@@ -274,25 +288,56 @@ rmsnorm_reduce_kernel(float *__restrict__ X, const SLAB *__restrict__ partials, 
 // ---------------------------------------------------------------------------
 // SLABS: the most partial results there can be (1 or MAX_SLABS: with one, and few registers, a pass of many rows keeps
 // three times as many loads in flight).
-template <int SLABS, typename SLAB>
+// WALK (few rows, not in the first layer): everything the layers before this one have used too, row metadata, page table, cos/sin, and the weights,
+// is read ahead of the wait, and the code behind the wait is walked through once there, as in the norm, with the partial results' loads from
+// the cos/sin table and nothing stored.
+template <int SLABS, bool WALK, typename SLAB>
 __global__ void __launch_bounds__(256, SLABS == 1 ? 6 : 3)
 rope_kv_kernel(const SLAB *__restrict__ partials, int S, size_t partial_stride, int Hq, int Hkv, int hd,
                RowMeta m, const float *__restrict__ cs, const float *__restrict__ sn, KvGeom g,
                bf16 *__restrict__ Q, bf16 *__restrict__ Kpool, bf16 *__restrict__ Vpool,
                bf16 *__restrict__ Kloc, bf16 *__restrict__ Vloc,
-               const bf16 *__restrict__ bias, const bf16 *__restrict__ qn, const bf16 *__restrict__ kn, float eps, TlSlot tl) {
-  pdl_wait();
-  pdl_trigger();             // in this order: the attention kernel relies on it (see attn_tc::Args::early)
-  if (threadIdx.x == 0) tl_go(tl);
+               const bf16 *__restrict__ bias, const bf16 *__restrict__ qn, const bf16 *__restrict__ kn, float eps, int let_in, TlSlot tl) {
+  // let_in (not in a pass's first layer): the attention kernel may start at once.  Otherwise it is let in behind the wait, as the first layer's must
+  // be: it and everything after it then know that what was prepared for the whole pass is there (see attn_tc::Args::early).
+  if (let_in) pdl_trigger();
+  if (!WALK) {
+    pdl_wait();
+    if (!let_in) pdl_trigger();
+    if (threadIdx.x == 0) tl_go(tl);
+  }
   // a work unit is 4 consecutive dims i..i+3 of the first half of one
   // head together with their rotation partners i+hd/2..
   const int r = blockIdx.x, half = hd / 2, upr = half / 4;          // units per head
   const int H = Hq + 2 * Hkv, N = H * hd;
   const int cp = m.cache_pos[r], seq = m.seq[r], li = m.local_idx[r];
   // grid (rows, ceil(units / 256)): one unit per thread, so a row's latency is one round of loads
-  for (int u = blockIdx.y * blockDim.x + threadIdx.x; u < H * upr; u += gridDim.y * blockDim.x) {
-    const int h = u / upr, i = (u % upr) * 4;
-    const size_t base = (size_t)r * N + (size_t)h * hd + i;
+  const int u = blockIdx.y * blockDim.x + threadIdx.x;
+  const bool mine = u < H * upr;
+  const int h = mine ? u / upr : 0, i = (u % upr) * 4;
+  const bf16 *hn = h < Hq ? qn : (h < Hq + Hkv ? kn : nullptr);
+  bf16 *dst = nullptr;                           // (null: a row whose K and V go nowhere)
+  const bool rotate = h < Hq + Hkv;
+  if (h < Hq) {
+    dst = Q + ((size_t)r * Hq + h) * hd;
+  } else {
+    const bool isk = h < Hq + Hkv;
+    const int kvh = isk ? h - Hq : h - Hq - Hkv;
+    if (cp >= 0) dst = (isk ? Kpool : Vpool) + kv_row_offset(g, seq, cp, kvh);
+    else if (li >= 0) dst = (isk ? Kloc : Vloc) + ((size_t)li * Hkv + kvh) * hd;
+  }
+  float4 c = make_float4(0.f, 0.f, 0.f, 0.f), sv = c;
+  if (rotate) { c = *reinterpret_cast<const float4 *>(cs + r * half + i); sv = *reinterpret_cast<const float4 *>(sn + r * half + i); }
+#pragma unroll 1
+  for (int walk = WALK ? 0 : 1; walk < 2; ++walk) {
+    const bool live = !WALK || walk != 0;
+    if (WALK && live) {
+      pdl_wait();
+      if (threadIdx.x == 0) tl_go(tl);
+    }
+    if (!mine) continue;
+    const SLAB *p = live ? partials + (size_t)r * N + (size_t)h * hd + i : reinterpret_cast<const SLAB *>(cs);
+    const size_t stride = live ? partial_stride : 0, half_at = live ? half : 0;
     float4 x1 = make_float4(0.f, 0.f, 0.f, 0.f), x2 = x1;
     // (both halves' loads together: two chains of additions)
 #pragma unroll
@@ -302,7 +347,7 @@ rope_kv_kernel(const SLAB *__restrict__ partials, int S, size_t partial_stride, 
       float4 q1[AT_ONCE], q2[AT_ONCE];
 #pragma unroll
       for (int t = 0; t < AT_ONCE; ++t)
-        if (s0 + t < S) { q1[t] = load4<SLAB>(partials + (s0 + t) * partial_stride + base); q2[t] = load4<SLAB>(partials + (s0 + t) * partial_stride + base + half); }
+        if (s0 + t < S) { q1[t] = load4<SLAB>(p + (s0 + t) * stride); q2[t] = load4<SLAB>(p + (s0 + t) * stride + half_at); }
 #pragma unroll
       for (int t = 0; t < AT_ONCE; ++t)
         if (s0 + t < S) {
@@ -317,10 +362,9 @@ rope_kv_kernel(const SLAB *__restrict__ partials, int S, size_t partial_stride, 
       x1.x += p0.x; x1.y += p0.y; x1.z += p1.x; x1.w += p1.y;
       x2.x += q0.x; x2.y += q0.y; x2.z += q1.x; x2.w += q1.y;
     }
-    const bf16 *hn = h < Hq ? qn : (h < Hq + Hkv ? kn : nullptr);
     if (hn) {
       // the upr = hd/8 threads of this head are consecutive lanes of one warp (upr is 8 or 16 and
-      // divides the unit index), and all of them are here: the loop bound is a multiple of upr
+      // divides the unit index), and all of them are here: the number of units is a multiple of upr
       float ss = x1.x * x1.x + x1.y * x1.y + x1.z * x1.z + x1.w * x1.w + x2.x * x2.x + x2.y * x2.y + x2.z * x2.z + x2.w * x2.w;
       const int lane = threadIdx.x & 31;
       const unsigned gmask = (upr >= 32 ? 0xffffffffu : ((1u << upr) - 1u)) << (lane & ~(upr - 1));
@@ -332,21 +376,8 @@ rope_kv_kernel(const SLAB *__restrict__ partials, int S, size_t partial_stride, 
       x1.x *= inv * p0.x; x1.y *= inv * p0.y; x1.z *= inv * p1.x; x1.w *= inv * p1.y;
       x2.x *= inv * q0.x; x2.y *= inv * q0.y; x2.z *= inv * q1.x; x2.w *= inv * q1.y;
     }
-    bf16 *dst;
-    bool rotate = true;
-    if (h < Hq) {
-      dst = Q + ((size_t)r * Hq + h) * hd;
-    } else {
-      const bool isk = h < Hq + Hkv;
-      const int kvh = isk ? h - Hq : h - Hq - Hkv;
-      if (cp < 0 && li < 0) continue;
-      if (cp >= 0) dst = (isk ? Kpool : Vpool) + kv_row_offset(g, seq, cp, kvh);
-      else dst = (isk ? Kloc : Vloc) + ((size_t)li * Hkv + kvh) * hd;
-      rotate = isk;
-    }
     float4 y1 = x1, y2 = x2;
     if (rotate) {
-      const float4 c = *reinterpret_cast<const float4 *>(cs + r * half + i), sv = *reinterpret_cast<const float4 *>(sn + r * half + i);
       y1 = make_float4(x1.x * c.x - x2.x * sv.x, x1.y * c.y - x2.y * sv.y, x1.z * c.z - x2.z * sv.z, x1.w * c.w - x2.w * sv.w);
       y2 = make_float4(x2.x * c.x + x1.x * sv.x, x2.y * c.y + x1.y * sv.y, x2.z * c.z + x1.z * sv.z, x2.w * c.w + x1.w * sv.w);
     }
@@ -355,8 +386,10 @@ rope_kv_kernel(const SLAB *__restrict__ partials, int S, size_t partial_stride, 
     uint2 o1, o2;
     o1.x = *reinterpret_cast<uint32_t *>(&a0); o1.y = *reinterpret_cast<uint32_t *>(&a1);
     o2.x = *reinterpret_cast<uint32_t *>(&b0); o2.y = *reinterpret_cast<uint32_t *>(&b1);
-    *reinterpret_cast<uint2 *>(dst + i) = o1;
-    *reinterpret_cast<uint2 *>(dst + i + half) = o2;
+    if (live && dst) {
+      *reinterpret_cast<uint2 *>(dst + i) = o1;
+      *reinterpret_cast<uint2 *>(dst + i + half) = o2;
+    }
   }
   if (threadIdx.x == 0) tl_end(tl);
 }

@@ -534,14 +534,14 @@ attn_tc::Args attention_args(const tidar_ctx *c, const AttnMaps &m, const KvGeom
   a.tile_count = c->count_tiles ? c->d_tl + 2 * tidar_ctx::TL_MAX : nullptr;
   return a;
 }
-template <int STREAMS, bool DIRECT>
+template <int STREAMS, bool DIRECT, bool AHEAD = false>
 void launch_attention_kernel(tidar_ctx *c, int grid, const AttnMaps &m, const attn_tc::Args &a) {
   Launch l(c, TIDAR_TC_ATTN);
   const int threads = attn_tc::threads(STREAMS);
   if (c->cfg.head_dim == 128)
-    launch_pdl(attn_tc::attn_tc_kernel<128, STREAMS, DIRECT>, grid, threads, attn_tc::Smem<128, STREAMS>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
+    launch_pdl(attn_tc::attn_tc_kernel<128, STREAMS, DIRECT, AHEAD>, grid, threads, attn_tc::Smem<128, STREAMS>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
   else
-    launch_pdl(attn_tc::attn_tc_kernel<64, STREAMS, DIRECT>, grid, threads, attn_tc::Smem<64, STREAMS>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
+    launch_pdl(attn_tc::attn_tc_kernel<64, STREAMS, DIRECT, AHEAD>, grid, threads, attn_tc::Smem<64, STREAMS>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
 }
 
 template <bool DIRECT>
@@ -552,12 +552,12 @@ void launch_attention_merge(tidar_ctx *c, int tiles, const attn_tc::Args &a) {
   else launch_pdl(attn_tc::attn_combine_kernel<64, DIRECT>, blocks, 256, 0, c->stream, a, l.tl);
 }
 
-// Attention of the pass that plan p was made for (the plan itself is in device memory by then).  early: see attn_tc::Args.
-void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMaps &m, const KvGeom &g, bf16 *O, bool early) {
+// Attention of the pass that plan p was made for (the plan itself is in device memory by then).  early: see attn_tc::Args; ahead: see attn_tc_kernel.
+void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMaps &m, const KvGeom &g, bf16 *O, bool early, bool ahead) {
   attn_tc::Args a = attention_args(c, m, g, O);
   a.items = p.items; a.tiles = p.tiles;
   a.early = early ? 1 : 0;
-  launch_attention_kernel<2, false>(c, p.max_items * p.Hkv, m, a);
+  if (early && ahead) launch_attention_kernel<2, false, true>(c, p.max_items * p.Hkv, m, a); else launch_attention_kernel<2, false>(c, p.max_items * p.Hkv, m, a);
   if (p.max_items > p.n_units && p.max_pieces > 1) launch_attention_merge<false>(c, 2 * p.n_units * p.Hkv, a);
 }
 
@@ -606,14 +606,16 @@ void launch_norm_as(tidar_ctx *c, int R, const SLAB *partials, int S, size_t str
   const int per_sm = c->cfg.impl == 0 ? (R + c->n_sms - 1) / c->n_sms : 0;
   const size_t smem = R > gemm_tc::SMALL_ROWS && per_sm <= 4 && per_sm > 0 ? (size_t)(NORM_SMEM / per_sm) & ~(size_t)1023 : 0;
   auto go = [&](auto kernel) { launch_pdl(kernel, R, 512, smem, c->stream, c->X, partials, S, stride, gain, c->cfg.rms_eps, d, c->A, l.tl); };
-  auto by_width = [&](auto slabs) {
+  auto by_width = [&](auto slabs, auto walk) {
     constexpr int SL = decltype(slabs)::value;
-    if (nv <= 1) go(rmsnorm_reduce_kernel<512, 1, SL, SLAB>);
-    else if (nv <= 2) go(rmsnorm_reduce_kernel<512, 2, SL, SLAB>);
-    else if (nv <= 3) go(rmsnorm_reduce_kernel<512, 3, SL, SLAB>);
-    else go(rmsnorm_reduce_kernel<512, 6, SL, SLAB>);
+    constexpr bool WK = decltype(walk)::value;
+    if (nv <= 1) go(rmsnorm_reduce_kernel<512, 1, SL, WK, SLAB>);
+    else if (nv <= 2) go(rmsnorm_reduce_kernel<512, 2, SL, WK, SLAB>);
+    else if (nv <= 3) go(rmsnorm_reduce_kernel<512, 3, SL, WK, SLAB>);
+    else go(rmsnorm_reduce_kernel<512, 6, SL, WK, SLAB>);
   };
-  if (S <= 1) by_width(std::integral_constant<int, 1>()); else by_width(std::integral_constant<int, MAX_SLABS>());
+  auto by_rows = [&](auto slabs) { if (R <= gemm_tc::SMALL_ROWS) by_width(slabs, std::true_type()); else by_width(slabs, std::false_type()); };
+  if (S <= 1) by_rows(std::integral_constant<int, 1>()); else by_rows(std::integral_constant<int, MAX_SLABS>());
 }
 void launch_norm(tidar_ctx *c, int R, const float *partials, int S, size_t stride, const bf16 *gain) {
   if (c->cfg.impl == 0 && c->slab_bf16) launch_norm_as<bf16>(c, R, (const bf16 *)partials, S, stride, gain);
@@ -627,7 +629,8 @@ struct MixRows { int n = 0, k = 1, a0 = 0, a_seq = 0, a_j = 0, b0 = 0, b_seq = 0
 
 // head_row0: the LM head (with_head) runs on rows [head_row0, R) only, followed by the mixed rows; the
 // argmax ids and the logits dump are indexed from head_row0.
-int forward_rows(tidar_ctx *c, int R, bool with_head, int rows_per_group, const MixRows &mix = MixRows(), int head_row0 = 0) {
+// step: a decode step (its rows see at most k_max positions more than are cached).
+int forward_rows(tidar_ctx *c, int R, bool with_head, int rows_per_group, const MixRows &mix = MixRows(), int head_row0 = 0, bool step = false) {
   const tidar_config &cf = c->cfg;
   const int d = cf.d_model, hd = cf.head_dim, Hq = cf.n_q_heads, Hkv = cf.n_kv_heads;
   const KvGeom g = geom(c);
@@ -639,7 +642,7 @@ int forward_rows(tidar_ctx *c, int R, bool with_head, int rows_per_group, const 
                  c->rope_sin, plan, l.tl);
   }
   int S = 0; size_t stride = 0;          // pending partials of the previous down projection
-  const bool tc = cf.impl == 0;
+  const bool tc = cf.impl == 0, few = R <= gemm_tc::SMALL_ROWS;
   const int RA = c->R_cap;               // allocated rows of the activation buffers
   int rc;
   for (int l = 0; l < cf.n_layers; ++l) {
@@ -656,15 +659,16 @@ int forward_rows(tidar_ctx *c, int R, bool with_head, int rows_per_group, const 
                  *kn_l = c->k_norm.empty() ? nullptr : c->k_norm[l];
       auto rope = [&](auto kernel, auto *partials) {
         launch_pdl(kernel, dim3(R, rope_chunks), 256, 0, c->stream, partials, S, stride, Hq, Hkv, hd, c->meta, c->rope_cos, c->rope_sin, g, c->Q, Kp, Vp,
-                   c->Kloc, c->Vloc, bias_l, qn_l, kn_l, cf.rms_eps, ll.tl);
+                   c->Kloc, c->Vloc, bias_l, qn_l, kn_l, cf.rms_eps, l > 0 && few ? 1 : 0, ll.tl);
       };
-      if (tc && c->slab_bf16) rope(rope_kv_kernel<MAX_SLABS, bf16>, (const bf16 *)c->partials);
-      else if (S <= 1) rope(rope_kv_kernel<1, float>, (const float *)c->partials);
-      else rope(rope_kv_kernel<MAX_SLABS, float>, (const float *)c->partials);
+      const bool walk = tc && l > 0 && few;                  // (the first layer's attention lies between the metadata's writer and this kernel)
+      if (tc && c->slab_bf16) rope(rope_kv_kernel<MAX_SLABS, false, bf16>, (const bf16 *)c->partials);
+      else if (S <= 1) walk ? rope(rope_kv_kernel<1, true, float>, (const float *)c->partials) : rope(rope_kv_kernel<1, false, float>, (const float *)c->partials);
+      else walk ? rope(rope_kv_kernel<MAX_SLABS, true, float>, (const float *)c->partials) : rope(rope_kv_kernel<MAX_SLABS, false, float>, (const float *)c->partials);
     }
     if (tc) {
       AttnMaps am{&c->tm_q, &c->tm_kv, &c->tm_kv, &c->tm_kloc, &c->tm_vloc, (2 * l) * c->n_pages, (2 * l + 1) * c->n_pages};
-      launch_attention_tc(c, plan, am, g, c->O, true);          // behind the RoPE kernel
+      launch_attention_tc(c, plan, am, g, c->O, true, step && few);     // behind the RoPE kernel
     } else {
       launch_attention(c, c->Q, Kp, Vp, g, c->Kloc, c->Vloc, c->O, R);
     }
@@ -753,33 +757,42 @@ int init_tensor_core_path(tidar_ctx *c) {
     CUDA_TRY(c, cudaMemsetAsync(c->Kloc, 0, nloc * cf.n_kv_heads * cf.head_dim * sizeof(bf16), c->stream));
     CUDA_TRY(c, cudaMemsetAsync(c->Vloc, 0, nloc * cf.n_kv_heads * cf.head_dim * sizeof(bf16), c->stream));
     auto smem = [](const void *f, int bytes) { return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 2, false>, attn_tc::Smem<128, 2>::TOTAL));
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 2, false>, attn_tc::Smem<64, 2>::TOTAL));
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 2, true>, attn_tc::Smem<128, 2>::TOTAL));
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 2, true>, attn_tc::Smem<64, 2>::TOTAL));
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 1, true>, attn_tc::Smem<128, 1>::TOTAL));
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 1, true>, attn_tc::Smem<64, 1>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 2, false, false>, attn_tc::Smem<128, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 2, false, true>, attn_tc::Smem<128, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 2, false, false>, attn_tc::Smem<64, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 2, false, true>, attn_tc::Smem<64, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 2, true, false>, attn_tc::Smem<128, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 2, true, false>, attn_tc::Smem<64, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 1, true, false>, attn_tc::Smem<128, 1>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 1, true, false>, attn_tc::Smem<64, 1>::TOTAL));
   }
   {
     auto max_smem_split = [&](const void *f) { return cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared); };
     const void *kernels[] = {(const void *)assemble_step_kernel, (const void *)pass_setup_kernel, (const void *)attn_meta_plan_kernel,
-                             (const void *)rmsnorm_reduce_kernel<512, 1, 1, float>, (const void *)rmsnorm_reduce_kernel<512, 1, 1, bf16>,
-                             (const void *)rmsnorm_reduce_kernel<512, 2, 1, float>, (const void *)rmsnorm_reduce_kernel<512, 2, 1, bf16>,
-                             (const void *)rmsnorm_reduce_kernel<512, 3, 1, float>, (const void *)rmsnorm_reduce_kernel<512, 3, 1, bf16>,
-                             (const void *)rmsnorm_reduce_kernel<512, 6, 1, float>, (const void *)rmsnorm_reduce_kernel<512, 6, 1, bf16>,
-                             (const void *)rmsnorm_reduce_kernel<512, 1, MAX_SLABS, float>, (const void *)rmsnorm_reduce_kernel<512, 1, MAX_SLABS, bf16>,
-                             (const void *)rmsnorm_reduce_kernel<512, 2, MAX_SLABS, float>, (const void *)rmsnorm_reduce_kernel<512, 2, MAX_SLABS, bf16>,
-                             (const void *)rmsnorm_reduce_kernel<512, 3, MAX_SLABS, float>, (const void *)rmsnorm_reduce_kernel<512, 3, MAX_SLABS, bf16>,
-                             (const void *)rmsnorm_reduce_kernel<512, 6, MAX_SLABS, float>, (const void *)rmsnorm_reduce_kernel<512, 6, MAX_SLABS, bf16>,
-                             (const void *)rope_kv_kernel<1, float>, (const void *)rope_kv_kernel<MAX_SLABS, float>, (const void *)rope_kv_kernel<MAX_SLABS, bf16>,
+                             (const void *)rope_kv_kernel<1, false, float>, (const void *)rope_kv_kernel<MAX_SLABS, false, float>, (const void *)rope_kv_kernel<MAX_SLABS, false, bf16>,
+                             (const void *)rope_kv_kernel<1, true, float>, (const void *)rope_kv_kernel<MAX_SLABS, true, float>,
                              (const void *)swiglu_slab_kernel<float>, (const void *)swiglu_slab_kernel<bf16>,
                              (const void *)attn_tc::attn_combine_kernel<128, false>, (const void *)attn_tc::attn_combine_kernel<64, false>,
                              (const void *)attn_tc::attn_combine_kernel<128, true>, (const void *)attn_tc::attn_combine_kernel<64, true>,
                              (const void *)mix_rows_kernel, (const void *)argmax_merge_kernel, (const void *)verify_select_kernel, (const void *)stage_step_kernel};
     for (const void *f : kernels) CUDA_TRY(c, max_smem_split(f));
-    CUDA_TRY(c, max_smem_split((const void *)attn_tc::attn_tc_kernel<128, 1, true>));
-    CUDA_TRY(c, max_smem_split((const void *)attn_tc::attn_tc_kernel<64, 1, true>));
-    for (int i = 3; i < 19; ++i) CUDA_TRY(c, cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, NORM_SMEM));
+    std::vector<const void *> norms;
+    auto add_norms = [&](auto slabs, auto slab) {
+      constexpr int SL = decltype(slabs)::value;
+      using T = decltype(slab);
+      for (const void *f : {(const void *)rmsnorm_reduce_kernel<512, 1, SL, false, T>, (const void *)rmsnorm_reduce_kernel<512, 1, SL, true, T>,
+                            (const void *)rmsnorm_reduce_kernel<512, 2, SL, false, T>, (const void *)rmsnorm_reduce_kernel<512, 2, SL, true, T>,
+                            (const void *)rmsnorm_reduce_kernel<512, 3, SL, false, T>, (const void *)rmsnorm_reduce_kernel<512, 3, SL, true, T>,
+                            (const void *)rmsnorm_reduce_kernel<512, 6, SL, false, T>, (const void *)rmsnorm_reduce_kernel<512, 6, SL, true, T>}) norms.push_back(f);
+    };
+    add_norms(std::integral_constant<int, 1>(), float()); add_norms(std::integral_constant<int, 1>(), bf16());
+    add_norms(std::integral_constant<int, MAX_SLABS>(), float()); add_norms(std::integral_constant<int, MAX_SLABS>(), bf16());
+    for (const void *f : norms) {
+      CUDA_TRY(c, max_smem_split(f));
+      CUDA_TRY(c, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, NORM_SMEM));
+    }
+    CUDA_TRY(c, max_smem_split((const void *)attn_tc::attn_tc_kernel<128, 1, true, false>));
+    CUDA_TRY(c, max_smem_split((const void *)attn_tc::attn_tc_kernel<64, 1, true, false>));
   }
   const int max_smem = gemm_tc::SMEM_BUDGET + 1024;
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
@@ -879,7 +892,7 @@ int record_step(tidar_ctx *c, const tidar_ctx::StepKey &key) {
     if (key.mixed_R > 0) { mix.n = key.mixed_K; mix.lay = lay; }
     else { mix.n = n_seqs * k; mix.k = k; mix.a0 = 0; mix.a_seq = T; mix.a_j = 1; mix.b0 = k; mix.b_seq = T; mix.b_j = k; }
   }
-  if (int rc = forward_rows(c, R, true, key.mixed_R > 0 ? 0 : T, mix)) return rc;
+  if (int rc = forward_rows(c, R, true, key.mixed_R > 0 ? 0 : T, mix, 0, true)) return rc;
   {
     Launch l(c, TIDAR_TC_VERIFY);
     launch_pdl(verify_select_kernel, n_seqs, 32, 0, c->stream, c->d_arg_idx, mix.n ? c->d_arg_idx + R : (const int32_t *)nullptr, c->d_step_seqs,
@@ -1628,7 +1641,7 @@ int tidar_attention(tidar_ctx *c, const void *q, const void *k_pages, const void
       if (d.streams == 2) launch_attention_kernel<2, true>(c, tiles * d.pieces, am, a); else launch_attention_kernel<1, true>(c, tiles, am, a);
       if (d.pieces > 1) launch_attention_merge<true>(c, tiles, a);
     } else {
-      launch_attention_tc(c, plan, am, g, (bf16 *)out, false);   // behind the kernel that makes the plan
+      launch_attention_tc(c, plan, am, g, (bf16 *)out, false, false);   // behind the kernel that makes the plan
     }
   } else {
     {
