@@ -522,6 +522,60 @@ attn_tc::PlanArgs attention_plan(const tidar_ctx *c, int R, int rows_per_group) 
 // kernel, about 5 us, and saves half of 0.56 us per page at best.
 bool may_split(int n_keys) { return n_keys > 12 * attn_tc::PAGE; }
 
+// The same for a decode step, whose sequences' lengths n[] and block lengths ks[] the host knows: whether the work plan (attn_tc::plan_block, whose
+// estimate this repeats) would cut any key range.  Where it would not, the step goes without the merge kernel, which would find nothing to do
+// (8B-class step of 272 rows, 1.1 k positions: 2.4 us per layer).  A step planned as uncut on the host is not cut on the device.
+bool step_would_split(const tidar_ctx *c, const int *n, const int *ks, int n_seqs, bool ar) {
+  using namespace attn_tc;
+  const int spt = 128 / (c->cfg.n_q_heads / c->cfg.n_kv_heads), Hkv = c->cfg.n_kv_heads;
+  std::vector<float> ent[2];                           // us of the units, of the tiles
+  std::vector<char> two;                               // units of two tiles
+  int longest = 0;
+  for (int s = 0; s < n_seqs; ++s) {
+    longest = std::max(longest, n[s]);
+    const int k = ks[s], T = ar ? 1 : k * (k + 1);
+    auto pages = [&](int first, int last) {            // pages that slots first .. last need
+      int nvis = first < k ? std::min(last, k - 1) + 1 : 0, loc = 0;
+      if (last >= k) { nvis = std::max(nvis, (last - k) / k + 1); loc = ((last - k) / k - (std::max(first, k) - k) / k + 1) * k; }
+      return (n[s] + nvis + PAGE - 1) / PAGE + (loc + PAGE - 1) / PAGE;
+    };
+    for (int r = 0; r < T; r += 2 * spt) {
+      const bool dbl = r + spt < T;
+      two.push_back(dbl);
+      ent[0].push_back(pages(r, std::min(r + 2 * spt, T) - 1) * (dbl ? PAIR_PAGE : SINGLE_PAGE));
+      ent[1].push_back(pages(r, std::min(r + spt, T) - 1) * SINGLE_PAGE);
+      ent[1].push_back(dbl ? pages(r + spt, std::min(r + 2 * spt, T) - 1) * SINGLE_PAGE : 0.f);
+    }
+  }
+  if (!may_split(longest)) return false;
+  const int n_units = (int)two.size(), units = n_units * Hkv;
+  const int most_items = units <= c->n_sms ? c->n_sms / Hkv : 2 * units < 3 * c->n_sms ? SLOTS_PER_SM * c->n_sms / Hkv : n_units;     // as in attention_plan
+  if (n_units > PLAN_UNITS || most_items <= n_units) return true;      // nothing is cut and no merge launched whatever is said here
+  float best = 1e30f;
+  bool split = true;
+  for (int cnd = 0; cnd < 2 * CAND; ++cnd) {
+    const bool pr = cnd < CAND;
+    const std::vector<float> &us = ent[pr ? 0 : 1];
+    const float lim = std::max(*std::max_element(us.begin(), us.end()) / (1.f + 0.5f * (cnd % CAND)), 0.1f) * 1.0001f;
+    int items = 0, live = 0, most = 0; float sum = 0.f, mx = 0.f;
+    for (size_t e = 0; e < us.size(); ++e) {
+      if (us[e] <= 0.f) continue;
+      const bool dbl = pr && two[e];
+      const int p = (int)std::min(std::ceil(us[e] / lim), us[e] * (dbl ? 1.0001f / PAIR_PAGE : 1.0001f / SINGLE_PAGE));
+      const float store = p > 1 ? (dbl ? PAIR_STORE : SINGLE_STORE) : 0.f;
+      items += p; ++live; most = std::max(most, p);
+      sum += us[e] + p * (OVERHEAD + store);
+      mx = std::max(mx, us[e] / p + (p > 1 ? 0.5f * SINGLE_PAGE : 0.f) + store + OVERHEAD);
+    }
+    if (items > most_items || most > MAX_SPLITS) continue;
+    float t = mx;
+    if (items * Hkv > c->n_sms) t = std::max(t, Hkv * sum / c->n_sms + 0.5f * mx);
+    if (items > live) t += MERGE + 0.3f * items / live;
+    if (t < best) { best = t; split = items > live || (!pr && 2 * units > c->n_sms); }       // (single tiles beyond one wave need the larger grid)
+  }
+  return split;
+}
+
 attn_tc::Args attention_args(const tidar_ctx *c, const AttnMaps &m, const KvGeom &g, bf16 *O) {
   const tidar_config &cf = c->cfg;
   attn_tc::Args a{};
@@ -1022,14 +1076,15 @@ int enqueue_step(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int32_t *f
   }
   const int T = ar ? 1 : k * (k + 1), R = n_seqs * T;
   const int slot = c->turn & 1;
-  int max_n = 0;
+  std::vector<int> lens(n_seqs), lengths(n_seqs, k);
   for (int i = 0; i < n_seqs; ++i) {
     c->h_stage2[slot][i] = seqs[i]; c->h_stage2[slot][cf.max_batch + i] = forced ? forced[i] : 0;
-    max_n = std::max(max_n, c->seqs[seqs[i]].n);
+    lens[i] = c->seqs[seqs[i]].n;
   }
   const int spt = 2 * (128 / (cf.n_q_heads / cf.n_kv_heads));      // slots per attention unit (two query tiles)
   tidar_ctx::StepKey key;
-  key.k = k; key.n_seqs = n_seqs; key.ar = ar; key.units = n_seqs * ((T + spt - 1) / spt); key.split = may_split(max_n);
+  key.k = k; key.n_seqs = n_seqs; key.ar = ar; key.units = n_seqs * ((T + spt - 1) / spt);
+  key.split = step_would_split(c, lens.data(), lengths.data(), n_seqs, ar);
   if (int rc = launch_step(c, key)) return rc;
   CUDA_TRY(c, cudaEventRecord(c->flight_done[slot], c->stream));
   push_flight(c, seqs, n_seqs, forced, k, nullptr);
@@ -1068,19 +1123,21 @@ int enqueue_step_mixed(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int3
   const int mb = cf.max_batch, spt = 2 * (128 / (cf.n_q_heads / cf.n_kv_heads));
   int32_t *hk = c->h_lay, *hoff = hk + (mb + 1), *hloc = hoff + (mb + 1), *ht0 = hloc + (mb + 1), *hte = ht0 + (c->R_head + mb);
   const int slot = c->turn & 1;
-  int max_n = 0, R = 0, loc = 0, tiles = 0, sum_k = 0;
+  int R = 0, loc = 0, tiles = 0, sum_k = 0;
+  std::vector<int> lens(n_seqs);
   for (int i = 0; i < n_seqs; ++i) {
     const int k = ks[i], T = k * (k + 1);
     hk[i] = k; hoff[i] = R; hloc[i] = loc; sum_k += k;
     for (int r0 = R; r0 < R + T; r0 += spt) { ht0[tiles] = r0; hte[tiles] = R + T; ++tiles; }
     R += T; loc += k * k;
     c->h_stage2[slot][i] = seqs[i]; c->h_stage2[slot][mb + i] = forced ? forced[i] : 0;
-    max_n = std::max(max_n, c->seqs[seqs[i]].n);
+    lens[i] = c->seqs[seqs[i]].n;
   }
   hk[n_seqs] = 0; hoff[n_seqs] = R; hloc[n_seqs] = loc;
   // a mixed step's kernels take every per-sequence length from the staged layout: the nominal k is unused
   tidar_ctx::StepKey key;
-  key.n_seqs = n_seqs; key.mixed_R = R; key.units = tiles; key.split = may_split(max_n);
+  key.n_seqs = n_seqs; key.mixed_R = R; key.units = tiles;
+  key.split = step_would_split(c, lens.data(), ks, n_seqs, false);
   const int mixed_rows = cf.beta < 1.0f ? sum_k : 0;         // one mixed LM-head input row per verified position
   key.mixed_K = mixed_rows;
   // Steps of nearly the same size share one captured graph: rows are filled up to a multiple of 16 (the projections' row
