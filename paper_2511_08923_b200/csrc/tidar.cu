@@ -107,6 +107,11 @@ struct tidar_ctx {
   std::deque<StepGraph> graphs;      // most recently used first
   bool split_keys = true;            // attention key ranges of the current pass may be cut (see attention_plan)
   bool graphs_ok = true;             // steps can be captured on this stream (the legacy default stream refuses it)
+  // On the legacy default stream a step is captured on a stream of the context's own, once its shape has been run GRAPH_AFTER times, and replayed
+  // on the default stream from then on (see launch_step).
+  bool side_capture = false;
+  cudaStream_t capture_stream = nullptr;
+  std::deque<std::pair<StepKey, int>> seen;      // shapes without a graph and how often they were run, most recent first
   int64_t graphs_captured = 0, graphs_launched = 0;
   bool slab_bf16 = false;          // split-K partial sums of the step in bf16 instead of fp32 (config debug bit 2)
   int32_t *d_status = nullptr, *cand_idx = nullptr;
@@ -961,7 +966,7 @@ int record_step(tidar_ctx *c, const tidar_ctx::StepKey &key) {
   return TIDAR_OK;
 }
 
-bool use_graphs(const tidar_ctx *c) { return c->cfg.impl == 0 && c->graphs_ok && !c->timing && !(c->cfg.debug & (1 | 8)); }
+bool use_graphs(const tidar_ctx *c) { return c->cfg.impl == 0 && (c->graphs_ok || c->side_capture) && !c->timing && !(c->cfg.debug & (1 | 8)); }
 
 void drop_graphs(tidar_ctx *c, size_t keep) {
   while (c->graphs.size() > keep) {
@@ -971,53 +976,85 @@ void drop_graphs(tidar_ctx *c, size_t keep) {
   }
 }
 
+// Captures the step of `key` on stream st and keeps it as the most recently used graph.
+bool capture_step(tidar_ctx *c, const tidar_ctx::StepKey &key, cudaStream_t st) {
+  drop_graphs(c, tidar_ctx::MAX_GRAPHS - 1);
+  tidar_ctx::StepGraph sg;
+  sg.key = key;
+  const int64_t l0 = c->launches;
+  const cudaStream_t own = c->stream;
+  cudaGraph_t graph = nullptr;
+  int rc = TIDAR_OK;
+  c->stream = st;
+  cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
+  if (e == cudaSuccess) {
+    rc = record_step(c, key);
+    e = cudaStreamEndCapture(st, &graph);
+  }
+  c->stream = own;
+  if (e == cudaSuccess && rc == TIDAR_OK && graph) e = cudaGraphInstantiate(&sg.exec, graph, 0);
+  if (graph) cudaGraphDestroy(graph);
+  if (key.timeline) sg.tl_cls = c->tl_cls;
+  sg.launches = c->launches - l0;
+  c->launches = l0;
+  if (e != cudaSuccess || rc != TIDAR_OK || !sg.exec) {
+    cudaGetLastError();
+    return false;
+  }
+  c->graphs.push_front(sg);
+  c->graphs_captured++;
+  return true;
+}
+
+// Behind a step that was launched kernel by kernel on the legacy default stream, while it runs: captures its shape once it has been run often enough.
+// A capture costs the host about 4 us per launch and a replayed launch is 0.3 us faster, which a shape has to come back for.  (Tiny model, 23
+// launches: 119 -> 107 us per step; 1.5B-class autoregressive step of 8 rows, 259 launches: 1.52 -> 1.43 ms.)  Steps of mixed block lengths seldom
+// meet the same shape again and stay as they are.
+constexpr int GRAPH_AFTER = 8;
+void capture_aside(tidar_ctx *c, const tidar_ctx::StepKey &key) {
+  if (key.mixed_R > 0 || key.timeline || key.count_tiles) return;
+  auto it = std::find_if(c->seen.begin(), c->seen.end(), [&](const std::pair<tidar_ctx::StepKey, int> &s) { return s.first == key; });
+  std::pair<tidar_ctx::StepKey, int> entry(key, 0);
+  if (it != c->seen.end()) { entry = *it; c->seen.erase(it); }
+  if (++entry.second < GRAPH_AFTER) {
+    c->seen.push_front(entry);
+    if (c->seen.size() > 2 * tidar_ctx::MAX_GRAPHS) c->seen.pop_back();
+    return;
+  }
+  if (!c->capture_stream && cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); c->capture_stream = nullptr; c->side_capture = false; return; }
+  if (!capture_step(c, key, c->capture_stream)) c->side_capture = false;
+}
+
 // The step proper.  Every launch of a step has the same arguments from step to step (lengths, page tables, token
 // blocks and, for a step of mixed block lengths, the row layout live in device memory), except
-// for the grid sizes, so on a stream of the caller's the step is captured once per key and replayed.  The legacy default
-// stream, which cannot be captured, per-launch timing and the debug read-backs use plain launches of the same kernels.  key.units: attention units per KV head.
+// for the grid sizes, so on a stream of the caller's the step is captured once per key and replayed.  On the legacy default
+// stream, which cannot be captured, that begins with a shape's ninth step (capture_aside).  Per-launch timing and the debug read-backs use plain
+// launches of the same kernels.  key.units: attention units per KV head.
 int launch_step(tidar_ctx *c, tidar_ctx::StepKey key) {
   key.timeline = c->timeline; key.count_tiles = c->count_tiles;
-  if (use_graphs(c)) {
-    auto it = std::find_if(c->graphs.begin(), c->graphs.end(), [&](const tidar_ctx::StepGraph &g) { return g.key == key; });
-    if (it == c->graphs.end()) {
-      drop_graphs(c, tidar_ctx::MAX_GRAPHS - 1);
-      tidar_ctx::StepGraph sg;
-      sg.key = key;
-      const int64_t l0 = c->launches;
-      cudaGraph_t graph = nullptr;
-      int rc = TIDAR_OK;
-      cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
-      if (e == cudaSuccess) {
-        rc = record_step(c, key);
-        e = cudaStreamEndCapture(c->stream, &graph);
-      }
-      if (e == cudaSuccess && rc == TIDAR_OK && graph) e = cudaGraphInstantiate(&sg.exec, graph, 0);
-      if (graph) cudaGraphDestroy(graph);
-      if (key.timeline) sg.tl_cls = c->tl_cls;
-      sg.launches = c->launches - l0;
-      c->launches = l0;
-      if (e != cudaSuccess || rc != TIDAR_OK || !sg.exec) {
-        cudaGetLastError();                         // capture is not available here: plain launches from now on
-        c->graphs_ok = false;
-      } else {
-        c->graphs.push_front(sg);
-        c->graphs_captured++;
-      }
-    } else if (it != c->graphs.begin()) {
-      const tidar_ctx::StepGraph sg = *it;
-      c->graphs.erase(it);
-      c->graphs.push_front(sg);
-    }
-    if (c->graphs_ok) {
-      const tidar_ctx::StepGraph &sg = c->graphs.front();
-      CUDA_TRY(c, cudaGraphLaunch(sg.exec, c->stream));
-      c->launches += sg.launches;
-      c->graphs_launched++;
-      if (key.timeline) { c->tl_cls = sg.tl_cls; c->tl_n = (int)sg.tl_cls.size(); }      // (another step may have been recorded since)
+  if (!use_graphs(c)) return record_step(c, key);
+  auto it = std::find_if(c->graphs.begin(), c->graphs.end(), [&](const tidar_ctx::StepGraph &g) { return g.key == key; });
+  if (it == c->graphs.end()) {
+    if (!c->graphs_ok) {
+      if (int rc = record_step(c, key)) return rc;
+      capture_aside(c, key);
       return TIDAR_OK;
     }
+    if (!capture_step(c, key, c->stream)) {           // capture is not available here: plain launches from now on
+      c->graphs_ok = false;
+      return record_step(c, key);
+    }
+  } else if (it != c->graphs.begin()) {
+    const tidar_ctx::StepGraph sg = *it;
+    c->graphs.erase(it);
+    c->graphs.push_front(sg);
   }
-  return record_step(c, key);
+  const tidar_ctx::StepGraph &sg = c->graphs.front();
+  CUDA_TRY(c, cudaGraphLaunch(sg.exec, c->stream));
+  c->launches += sg.launches;
+  c->graphs_launched++;
+  if (key.timeline) { c->tl_cls = sg.tl_cls; c->tl_n = (int)sg.tl_cls.size(); }      // (another step may have been recorded since)
+  return TIDAR_OK;
 }
 
 // Whether one more step may be enqueued: always when none is in flight; behind a step in flight only when
@@ -1225,6 +1262,7 @@ int tidar_init(const tidar_config *cfg, const tidar_weights *w, void *arena, siz
   c->slab_bf16 = (cfg->debug & 4) != 0;
   c->stream = (cudaStream_t)cuda_stream;
   c->graphs_ok = c->stream != nullptr && c->stream != cudaStreamLegacy;
+  c->side_capture = !c->graphs_ok && cfg->impl == 0;
   size_t need = 0;
   layout(*c, arena, &need);
   if (need > arena_bytes) { delete c; return fail(nullptr, TIDAR_ENOMEM, "arena has %zu bytes, %zu needed", arena_bytes, need); }
@@ -1471,6 +1509,7 @@ int tidar_free(tidar_ctx *c) {
   cudaStreamSynchronize(c->stream);
   for (auto &t : c->timed) { cudaEventDestroy(t.a); cudaEventDestroy(t.b); }
   drop_graphs(c, 0);
+  if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
   for (cudaEvent_t ev : c->flight_done) cudaEventDestroy(ev);
   if (c->h_pinned) cudaFreeHost(c->h_pinned);
   delete c;

@@ -505,6 +505,33 @@ def test_kept_graphs_are_reused_and_replaced():
         np.testing.assert_array_equal(a[0], b[0]); np.testing.assert_array_equal(a[1], b[1])
 
 
+def test_default_stream_replays_a_shape_that_recurs():
+    """On the default stream a step is launched kernel by kernel until its shape has been run eight times, and replayed from a graph afterwards, also with
+    two steps in flight and with other shapes in between: the same tokens, and bit-identical cached K/V, as without graphs."""
+    sh, wt = make_model("tiny")
+    k = sh.k
+    runs = {}
+    for tag, debug in (("graph", 0), ("plain", 8)):
+        t = _gpu(sh, wt, 0, k_max=k, debug=debug, max_batch=2, max_seq_len=512)
+        rec = [t.prefill(q, prompt_ids(sh, 50 + 9 * q), k) for q in range(2)]
+        for i in range(13):
+            rec.append(t.step([0, 1], forced=[1 + i % k, 1 + (i + 1) % k]))
+            if i % 4 == 0:
+                rec.append(t.step([1], forced=[2]))                # four times: never often enough
+        assert t.graph_stats() == ((1, 5, 1) if tag == "graph" else (0, 0, 0))
+        if tag == "graph":
+            t.step_async([0, 1], [1, 2])
+            t.step_async([0, 1], [3, 1])
+            rec += [t.step_wait(), t.step_wait()]
+        else:
+            rec += [t.step([0, 1], forced=[1, 2]), t.step([0, 1], forced=[3, 1])]
+        runs[tag] = rec, [t.get_block(q, k) for q in range(2)], [t.kv(q, l, 0, t.seq_len(q)) for q in range(2) for l in range(sh.n_layers)], t.launch_count()
+        _close(t)
+    assert runs["graph"][0] == runs["plain"][0] and runs["graph"][1] == runs["plain"][1] and runs["graph"][3] == runs["plain"][3]
+    for a, b in zip(runs["graph"][2], runs["plain"][2]):
+        np.testing.assert_array_equal(a[0], b[0]); np.testing.assert_array_equal(a[1], b[1])
+
+
 def test_timeline_of_a_replayed_step_is_its_own():
     """Two kept graphs with different launch lists (a long context adds the merge of split key ranges in every layer): replaying the first
     after the second was recorded still attributes every launch of the first to its class."""
