@@ -56,6 +56,7 @@ constexpr int PAGE = 64;             // keys per step (= page size)
 // warp 0: K loads, 1: MMA, 2: watcher, 3: Q and V loads; warps 4..7 / 8..11: softmax of stream A / B
 __host__ __device__ constexpr int threads(int streams) { return 128 + 128 * streams; }
 constexpr int MAX_SPLITS = 32;       // items per tile
+constexpr int MAX_CLUSTER = 8;       // CTAs that may share an item
 constexpr int SLOTS_PER_SM = 2;      // partial results that fit the scratch = grid of a pass whose key ranges may be split
 constexpr float RAISE_THRESHOLD = 8.f;   // log2 units
 
@@ -78,6 +79,7 @@ struct PlanArgs {
   int Hkv;
   int n_sms, max_items;     // items a pass may have; n_units = every unit is one item
   int max_pieces;           // items a tile or pair may have (1: nothing is split, the merge kernel is not launched)
+  int singles;              // tiles are not paired (an item is shared by a cluster, see attn_tc_kernel)
   Item *items; Tile *tiles; // out: [max_items] (unused ones are zero), [2 n_units] (only where items may be split)
 };
 
@@ -103,21 +105,26 @@ struct Args {
 
 // Shared memory of one CTA; everything is dynamic so that the 1024-byte alignment the
 // swizzled tiles need costs no padding (the kernel checks the base address).
-template <int HD, int STREAMS = 2>
+template <int HD, int STREAMS = 2, bool CLUSTER = false>
 struct Smem {
-  static constexpr int K_STAGES = STREAMS == 2 ? 5 : 3, V_STAGES = STREAMS == 2 ? 5 : 2;     // pages in flight (one stream: two CTAs fit an SM)
+  static constexpr int K_STAGES = CLUSTER ? 4 : STREAMS == 2 ? 5 : 3, V_STAGES = CLUSTER ? 3 : STREAMS == 2 ? 5 : 2;     // pages in flight (one stream: two CTAs fit an SM)
   static constexpr int NH = HD / 64;                 // 64-element halves of a head
   static constexpr int Q_BYTES = 128 * HD * 2;       // one query tile
   static constexpr int KV_BYTES = PAGE * HD * 2;
   static constexpr int Q_OFF = 0;
-  static constexpr int K_OFF = Q_OFF + STREAMS * Q_BYTES;
+  static constexpr int K_OFF = Q_OFF + (CLUSTER ? 1 : STREAMS) * Q_BYTES;
   static constexpr int V_OFF = K_OFF + K_STAGES * KV_BYTES;
-  static constexpr int BAR_OFF = V_OFF + V_STAGES * KV_BYTES;    // mbarriers and a few words
+  // CLUSTER: this CTA's columns of the tile's result as every CTA of the cluster has them, [CTA][stream][columns / 4][128 rows][4] floats, and
+  // the CTAs' (reference max, sum), [CTA][128 rows].  (Written by the others at any time, hence a place of its own.)
+  static constexpr int PEER_OFF = V_OFF + V_STAGES * KV_BYTES, PEER_ML_OFF = PEER_OFF + (CLUSTER ? 128 * HD * 4 : 0);
+  static constexpr int BAR_OFF = PEER_ML_OFF + (CLUSTER ? MAX_CLUSTER * 128 * 8 : 0);    // mbarriers and a few words
   static constexpr int TOTAL = BAR_OFF + 512;
   static constexpr int XCHG_OFF = K_OFF;             // single tile: the streams' results, [stream][hd / 8][128 rows][4] floats; (max, sum) behind them
   static constexpr int XCHG_ML_OFF = XCHG_OFF + 128 * HD * 4;
   static constexpr int TMEM_COLS = 256 * STREAMS;    // per stream 2 x 64 (S) + HD (O), rounded up to a power of two
 };
+static_assert(Smem<128, 2, true>::XCHG_ML_OFF + 2 * 128 * 8 <= Smem<128, 2, true>::PEER_OFF && Smem<64, 2, true>::XCHG_ML_OFF + 2 * 128 * 8 <= Smem<64, 2, true>::PEER_OFF &&
+              Smem<128, 2, true>::TOTAL <= 227 * 1024, "exchange area fits the K/V rings of a cluster's CTA");
 static_assert(Smem<128>::XCHG_ML_OFF + 2 * 128 * 8 <= Smem<128>::BAR_OFF && Smem<64>::XCHG_ML_OFF + 2 * 128 * 8 <= Smem<64>::BAR_OFF, "exchange area fits the K/V rings");
 
 struct Ctl {                                         // lives at Smem::BAR_OFF
@@ -138,6 +145,7 @@ static_assert(sizeof(Ctl) <= 512, "control block must fit its slot");
 // of the arithmetic.
 // (Measured inside the kernel, head_dim 128, all SMs busy: 1.05 us per page of a pair, 0.56 of a single tile.  head_dim 64 and nearly empty
 // grids take the same figures, although a page costs them less: they were not fitted, and cuts come out somewhat finer than best.)
+constexpr float CLUSTER_MERGE = 2.f;                   // what sharing an item within a cluster adds
 constexpr float OVERHEAD = 5.f, PAIR_PAGE = 1.05f, SINGLE_PAGE = 0.56f, PAIR_STORE = 2.5f, SINGLE_STORE = 1.5f, MERGE = 3.f;
 constexpr int PLAN_UNITS = 256;                        // up to this many units are planned; beyond, every unit is one item
 constexpr int CAND = 32;                               // limits tried per pairing: longest / (1 + i / 2)
@@ -226,7 +234,7 @@ __device__ inline void plan_block(const PlanArgs &p, ROW row_keys) {
       us_sum += __shfl_xor_sync(0xffffffffu, us_sum, o); us_max = fmaxf(us_max, __shfl_xor_sync(0xffffffffu, us_max, o));
     }
     unsigned long long mine = ~0ull;
-    if (live_cnd && items <= p.max_items && most <= p.max_pieces) {
+    if (live_cnd && items <= p.max_items && most <= p.max_pieces && !(pr && p.singles)) {
       float us = us_max;
       if (items * p.Hkv > p.n_sms) us = fmaxf(us, p.Hkv * us_sum / p.n_sms + 0.5f * us_max);
       if (items > live) us += MERGE + 0.3f * items / live;
@@ -337,11 +345,17 @@ __device__ __forceinline__ Item direct_item(const Args &a, int e) {
 // fetches the loop's code.  (8B-class step of 20 rows: 10.1 us behind a gap of 0.77 -> 8.9 behind 0.70; 1.5B-class autoregressive step of 8 rows 6.05 -> 4.75.
 // At 272 rows the CTAs wait for the SMs of the projection in front of the RoPE kernel and only lose by it; walking through the output code too was slower
 // everywhere, by 0.8 - 2 us.)
-template <int HD, int STREAMS, bool DIRECT, bool AHEAD>
+// CLUSTER: the CTAs of a cluster share an item (a single tile, not cut): each takes an even share of its pages, and their results are merged over
+// distributed shared memory: every CTA finishes 1 / size of the head's columns, which the others store into its shared memory.  For calls and steps of few
+// tiles and contexts of some pages (see attention_direct, step_attention); bound by the latencies of first load and merge, about 2 us for the latter
+// (CLUSTER_MERGE).  Alone, 32/8 heads of 128, 272 rows, 1 k positions, clusters of two: 15.8 -> 13.2 us; 12/2 heads, four sequences of 72 rows, 1 k
+// positions, clusters of four: 16.5 -> 11.7.  1.5B-class step of 272 rows: 10.4 -> 8.1 us per layer; autoregressive step of 8 rows, where it replaces
+// a cut and the merge kernel: 5.1 + 3.4 -> 7.5 us.
+template <int HD, int STREAMS, bool DIRECT, bool AHEAD, bool CLUSTER>
 __global__ void __launch_bounds__(threads(STREAMS), 3 - STREAMS)
 attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                const __grid_constant__ CUtensorMap tmKloc, const __grid_constant__ CUtensorMap tmVloc, const Args a, const TlSlot tl) {
-  using L = Smem<HD, STREAMS>;
+  using L = Smem<HD, STREAMS, CLUSTER>;
   constexpr int NH = L::NH;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const int warp = sm100::warp_index(), lane = threadIdx.x & 31;
@@ -371,6 +385,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   sm100::tc_fence_before();
   __syncthreads();
   sm100::tc_fence_after();
+  if constexpr (CLUSTER) sm100::cluster_arrive_relaxed();     // this CTA runs (waited for before the first store to another one)
   const uint32_t tmem = ctl.tmem_base;
   const uint32_t tmem_S = tmem, tmem_O = tmem + STREAMS * 2 * PAGE;   // per stream: 2 x 64 columns of S, HD columns of O
   volatile int *abortp = &ctl.abort_flag;
@@ -378,16 +393,26 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   if (DIRECT || !a.early) pdl_wait();
 
   // ---- which work item (every thread reads it: no barrier before the first loads go out) ----
-  const int kvh = blockIdx.x % a.Hkv, item_no = blockIdx.x / a.Hkv;
-  const Item item = DIRECT ? direct_item(a, item_no) : a.items[item_no];   // all zero where the grid is larger than the plan: nothing to do
+  const int c_size = CLUSTER ? (int)sm100::cluster_size() : 1, c_rank = CLUSTER ? (int)sm100::cluster_rank() : 0;
+  const int kvh = blockIdx.x / c_size % a.Hkv, item_no = blockIdx.x / c_size / a.Hkv;
+  Item item = DIRECT ? direct_item(a, item_no) : a.items[item_no];   // all zero where the grid is larger than the plan: nothing to do
+  const int np_item = item.p_end - item.p_begin;
+  if constexpr (CLUSTER) {
+    const int b = item.p_begin;
+    item.p_begin = b + np_item * c_rank / c_size; item.p_end = b + np_item * (c_rank + 1) / c_size;
+  }
   const int row0 = item.row0, p_begin = item.p_begin, np = item.p_end - item.p_begin;
-  const bool pair = STREAMS == 2 && item.pair != 0;
+  const bool pair = STREAMS == 2 && !CLUSTER && item.pair != 0;
   const bool shared = STREAMS == 1 || pair;                            // every stream takes every page; otherwise two streams take them in turn
   const int ahead = shared ? 2 : 4;                                    // pages whose scores are computed ahead: two steps of every stream
   auto stream0 = [&](int p) { return shared ? 0 : p & 1; };            // streams [stream0(p), stream1(p)) take page p
   auto stream1 = [&](int p) { return pair ? 2 : stream0(p) + 1; };
   if (threadIdx.x == 0 && a.tile_count && np > 0) atomicAdd(a.tile_count, (unsigned long long)np * (pair ? 2 : 1));
 
+  const int t = (warp - 4) >> 2;                         // softmax warps: stream
+  const int my_row = (warp & 3) * 32 + lane;             // and this thread's MMA row = TMEM lane
+  int my_slot = -1;                                      // and its slot, -1: none
+  const int c_cols = HD / 2 / c_size, c_shift = 31 - __clz(c_cols);     // columns of a stream's half that a CTA of the cluster finishes (at least 8)
   if (warp == 0 || warp == 3) {
     // ===================== K producer / Q and V producer =====================
     // Lane i holds the i-th entry of a group of 32 entries of the page table, so that a page's load does not wait for
@@ -525,12 +550,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     }
   } else if (warp >= 4) {
     // ===================== softmax =====================
-    const int t = (warp - 4) >> 2;                       // stream
     const int tile = pair ? t : 0;
-    const int my_row = (warp & 3) * 32 + lane;           // this thread's MMA row = TMEM lane
     const int nj = shared ? np : (np + 1 - t) >> 1;      // steps of this stream
     // (a row without a slot sees everything, so that its warp does not mask page after page for it)
-    int my_slot = -1, my_nvis = 0x7fffffff, my_loc0 = item.loc_lo, my_nloc = 1 << 30;
+    int my_nvis = 0x7fffffff, my_loc0 = item.loc_lo, my_nloc = 1 << 30;
     {
       const int pr = row0 + tile * a.spt + my_row / a.G;
       if (my_row < rows_used && pr < item.row_end) {
@@ -624,6 +647,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
       l_run = live ? l_run * alpha + (sa + sb) : 0.f;
     }
     // ---- output: O is complete once the last P V has finished ----
+    if constexpr (CLUSTER) sm100::cluster_wait();        // the cluster's other CTAs run
     pdl_wait();                                          // (long over; the stores below must not overtake it formally either)
     if (ok && nj > 1) ok = wait_s(nj);                   // (P V of the last step but one; in order, so that the parity wait below is unambiguous)
     if (ok && nj > 0) ok = wait_s(nj + 1);
@@ -663,7 +687,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         for (int c = 0; c < HD; c += 32) { float v[32]; load32(c, v); write32(v, c, inv); }
         if (my_slot >= 0 && item.split) a.part_ml[part * 128 + my_row] = make_float2(m_ref, l_run);
       }
-    } else if (np > 0) {
+    } else if (CLUSTER ? np_item > 0 : np > 0) {
       // The streams' halves of the same rows: each hands the other's columns over and finishes its own.  All MMAs have
       // read the K/V rings once every warp has got here (a failed stream only has to show up).
       float4 *xo = reinterpret_cast<float4 *>(smem_raw + L::XCHG_OFF);   // [stream that reads][HD / 8][128]
@@ -702,9 +726,53 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
             const float4 x = xo[(t * (HD / 8) + (c + i) / 4) * 128 + my_row];
             v[i] = wm * v[i] + wo * x.x; v[i + 1] = wm * v[i + 1] + wo * x.y; v[i + 2] = wm * v[i + 2] + wo * x.z; v[i + 3] = wm * v[i + 3] + wo * x.w;
           }
-          write32(v, t * (HD / 2) + c, inv);
+          if constexpr (CLUSTER) {
+            if (my_slot >= 0) {
+#pragma unroll
+              for (int i = 0; i < 32; i += 4) {
+                const int owner = (c + i) >> c_shift, at = (c + i) & (c_cols - 1);
+                sm100::st_cluster_v4(sm100::cluster_addr(smem0 + L::PEER_OFF, (uint32_t)owner) + (uint32_t)((((c_rank * 2 + t) * (c_cols / 4) + at / 4) * 128 + my_row) * 16),
+                                     v[i], v[i + 1], v[i + 2], v[i + 3]);
+              }
+            }
+          } else {
+            write32(v, t * (HD / 2) + c, inv);
+          }
         }
-        if (t == 0 && my_slot >= 0 && item.split) a.part_ml[part * 128 + my_row] = make_float2(M, l);
+        if constexpr (CLUSTER) {
+          if (t == 0 && my_slot >= 0)
+            for (int r = 0; r < c_size; ++r) sm100::st_cluster_v2(sm100::cluster_addr(smem0 + L::PEER_ML_OFF, (uint32_t)r) + (uint32_t)((c_rank * 128 + my_row) * 8), M, l);
+        } else {
+          if (t == 0 && my_slot >= 0 && item.split) a.part_ml[part * 128 + my_row] = make_float2(M, l);
+        }
+      }
+    }
+  }
+  if constexpr (CLUSTER) {
+    if (warp < 4) sm100::cluster_wait();
+    sm100::cluster_sync();                               // the stores to one another have arrived
+    if (warp >= 4 && np_item > 0 && my_slot >= 0) {
+      const float2 *ml = reinterpret_cast<const float2 *>(smem_raw + L::PEER_ML_OFF) + my_row;
+      const float4 *x = reinterpret_cast<const float4 *>(smem_raw + L::PEER_OFF) + t * (c_cols / 4) * 128 + my_row;
+      float M = -INFINITY, den = 0.f;
+      for (int r = 0; r < c_size; ++r) M = fmaxf(M, ml[r * 128].x);
+      for (int r = 0; r < c_size; ++r) den += exp2f(ml[r * 128].x - M) * ml[r * 128].y;
+      const float inv = 1.f / den;
+      bf16 *o = a.O + ((size_t)my_slot * a.Hq + kvh * a.G + my_row % a.G) * HD + t * (HD / 2) + c_rank * c_cols;
+      for (int g = 0; g < c_cols / 4; g += 2) {          // eight columns
+        float acc[8] = {};
+        for (int r = 0; r < c_size; ++r) {
+          const float w = exp2f(ml[r * 128].x - M);      // (a CTA without pages: 0)
+          const float4 u = x[(r * 2 * (c_cols / 4) + g) * 128], v = x[(r * 2 * (c_cols / 4) + g + 1) * 128];
+          acc[0] = fmaf(w, u.x, acc[0]); acc[1] = fmaf(w, u.y, acc[1]); acc[2] = fmaf(w, u.z, acc[2]); acc[3] = fmaf(w, u.w, acc[3]);
+          acc[4] = fmaf(w, v.x, acc[4]); acc[5] = fmaf(w, v.y, acc[5]); acc[6] = fmaf(w, v.z, acc[6]); acc[7] = fmaf(w, v.w, acc[7]);
+        }
+        __nv_bfloat162 h0 = __floats2bfloat162_rn(acc[0] * inv, acc[1] * inv), h1 = __floats2bfloat162_rn(acc[2] * inv, acc[3] * inv),
+                       h2 = __floats2bfloat162_rn(acc[4] * inv, acc[5] * inv), h3 = __floats2bfloat162_rn(acc[6] * inv, acc[7] * inv);
+        uint4 w4;
+        w4.x = *reinterpret_cast<uint32_t *>(&h0); w4.y = *reinterpret_cast<uint32_t *>(&h1);
+        w4.z = *reinterpret_cast<uint32_t *>(&h2); w4.w = *reinterpret_cast<uint32_t *>(&h3);
+        *reinterpret_cast<uint4 *>(o + g * 4) = w4;
       }
     }
   }

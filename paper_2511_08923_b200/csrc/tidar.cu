@@ -96,16 +96,18 @@ struct tidar_ctx {
   int n_sms = 0;
   // the launches of one decode step as an executable graph, valid for one key; the most recently used ones are kept
   struct StepKey {
-    int k = 0, n_seqs = 0, mixed_R = 0, units = 0, mixed_K = 0; bool ar = false, timeline = false, count_tiles = false, split = false;
+    int k = 0, n_seqs = 0, mixed_R = 0, units = 0, mixed_K = 0; bool ar = false, timeline = false, count_tiles = false, split = false; int cluster = 1;
     bool operator==(const StepKey &o) const {
       return k == o.k && n_seqs == o.n_seqs && mixed_R == o.mixed_R && units == o.units && mixed_K == o.mixed_K && ar == o.ar && timeline == o.timeline &&
-             count_tiles == o.count_tiles && split == o.split;
+             count_tiles == o.count_tiles && split == o.split && cluster == o.cluster;
     }
   };
   struct StepGraph { StepKey key; cudaGraphExec_t exec = nullptr; int64_t launches = 0; std::vector<int> tl_cls; };   // tl_cls: of its timeline slots
   static constexpr size_t MAX_GRAPHS = 16;
   std::deque<StepGraph> graphs;      // most recently used first
   bool split_keys = true;            // attention key ranges of the current pass may be cut (see attention_plan)
+  int attn_cluster = 1;              // CTAs that share an attention item of the current pass (see step_attention)
+  int max_clusters[attn_tc::MAX_CLUSTER + 1] = {};      // clusters of 2, 4, 8 attention CTAs that are resident at once
   bool graphs_ok = true;             // steps can be captured on this stream (the legacy default stream refuses it)
   // On the legacy default stream a step is captured on a stream of the context's own, once its shape has been run GRAPH_AFTER times, and replayed
   // on the default stream from then on (see launch_step).
@@ -519,6 +521,10 @@ attn_tc::PlanArgs attention_plan(const tidar_ctx *c, int R, int rows_per_group) 
   p.max_items = units <= c->n_sms ? c->n_sms / p.Hkv : 2 * units < 3 * c->n_sms ? attn_tc::SLOTS_PER_SM * c->n_sms / p.Hkv : p.n_units;
   p.max_pieces = attn_tc::MAX_SPLITS;
   if (!c->split_keys) { p.max_pieces = 1; p.max_items = 2 * units <= c->n_sms ? 2 * p.n_units : p.n_units; }
+  if (c->attn_cluster > 1) {                           // one item per tile, shared by a cluster
+    p.max_pieces = 1; p.singles = 1;
+    p.max_items = rows_per_group > 0 ? (R + rows_per_group - 1) / rows_per_group * ((rows_per_group + p.spt - 1) / p.spt) : 2 * p.n_units;
+  }
   p.items = c->plan_items; p.tiles = c->plan_tiles;
   return p;
 }
@@ -530,8 +536,10 @@ bool may_split(int n_keys) { return n_keys > 12 * attn_tc::PAGE; }
 // The same for a decode step, whose sequences' lengths n[] and block lengths ks[] the host knows: whether the work plan (attn_tc::plan_block, whose
 // estimate this repeats) would cut any key range.  Where it would not, the step goes without the merge kernel, which would find nothing to do
 // (8B-class step of 272 rows, 1.1 k positions: 2.4 us per layer).  A step planned as uncut on the host is not cut on the device.
-bool step_would_split(const tidar_ctx *c, const int *n, const int *ks, int n_seqs, bool ar) {
+struct StepAttention { bool split; int cluster; };
+StepAttention step_attention(const tidar_ctx *c, const int *n, const int *ks, int n_seqs, bool ar, bool mixed) {
   using namespace attn_tc;
+  const StepAttention uncut{false, 1}, cut{true, 1};
   const int spt = 128 / (c->cfg.n_q_heads / c->cfg.n_kv_heads), Hkv = c->cfg.n_kv_heads;
   std::vector<float> ent[2];                           // us of the units, of the tiles
   std::vector<char> two;                               // units of two tiles
@@ -552,33 +560,46 @@ bool step_would_split(const tidar_ctx *c, const int *n, const int *ks, int n_seq
       ent[1].push_back(dbl ? pages(r + spt, std::min(r + 2 * spt, T) - 1) * SINGLE_PAGE : 0.f);
     }
   }
-  if (!may_split(longest)) return false;
   const int n_units = (int)two.size(), units = n_units * Hkv;
   const int most_items = units <= c->n_sms ? c->n_sms / Hkv : 2 * units < 3 * c->n_sms ? SLOTS_PER_SM * c->n_sms / Hkv : n_units;     // as in attention_plan
-  if (n_units > PLAN_UNITS || most_items <= n_units) return true;      // nothing is cut and no merge launched whatever is said here
+  if (n_units > PLAN_UNITS || most_items <= n_units) return cut;       // nothing is cut and no merge launched whatever is said here
   float best = 1e30f;
   bool split = true;
-  for (int cnd = 0; cnd < 2 * CAND; ++cnd) {
+  const bool may_cut = may_split(longest);
+  for (int cnd = 0; cnd < 2 * CAND; cnd += 2) {        // (every other limit: this runs ahead of each step's first launch)
     const bool pr = cnd < CAND;
     const std::vector<float> &us = ent[pr ? 0 : 1];
     const float lim = std::max(*std::max_element(us.begin(), us.end()) / (1.f + 0.5f * (cnd % CAND)), 0.1f) * 1.0001f;
+    const float inv = 1.f / lim;
     int items = 0, live = 0, most = 0; float sum = 0.f, mx = 0.f;
     for (size_t e = 0; e < us.size(); ++e) {
       if (us[e] <= 0.f) continue;
       const bool dbl = pr && two[e];
-      const int p = (int)std::min(std::ceil(us[e] / lim), us[e] * (dbl ? 1.0001f / PAIR_PAGE : 1.0001f / SINGLE_PAGE));
+      const int p = (int)std::min(us[e] * inv + 0.9999f, us[e] * (dbl ? 1.0001f / PAIR_PAGE : 1.0001f / SINGLE_PAGE));
       const float store = p > 1 ? (dbl ? PAIR_STORE : SINGLE_STORE) : 0.f;
       items += p; ++live; most = std::max(most, p);
       sum += us[e] + p * (OVERHEAD + store);
       mx = std::max(mx, us[e] / p + (p > 1 ? 0.5f * SINGLE_PAGE : 0.f) + store + OVERHEAD);
     }
-    if (items > most_items || most > MAX_SPLITS) continue;
+    if (items > most_items || most > (may_cut ? MAX_SPLITS : 1)) continue;
     float t = mx;
     if (items * Hkv > c->n_sms) t = std::max(t, Hkv * sum / c->n_sms + 0.5f * mx);
     if (items > live) t += MERGE + 0.3f * items / live;
     if (t < best) { best = t; split = items > live || (!pr && 2 * units > c->n_sms); }       // (single tiles beyond one wave need the larger grid)
   }
-  return split;
+  // A cluster per tile, its pages shared evenly; on three quarters of the SMs at most, for on the others the projection behind the attention fills its
+  // rings (8B-class step of 272 rows, clusters of two on 144 SMs: attention 15.9 -> 12.7 us, the O projection 14.9 -> 18).
+  int tiles = 0;
+  for (float us : ent[1]) tiles += us > 0.f;
+  const int places = mixed ? 2 * ((n_units + 3) / 4 * 4) : tiles;      // items of the launch (see attention_plan)
+  const float longest_us = *std::max_element(ent[1].begin(), ent[1].end());
+  if (split) best += 1.5f;                               // (the boundary in front of the merge kernel)
+  StepAttention pick = split ? cut : uncut;
+  for (int size = 2; size <= MAX_CLUSTER && size * 16 <= c->cfg.head_dim; size *= 2) {
+    const float t = std::ceil(longest_us / SINGLE_PAGE / size) * SINGLE_PAGE + OVERHEAD + CLUSTER_MERGE;
+    if (places * Hkv <= c->max_clusters[size] && 4 * places * Hkv * size <= 3 * c->n_sms && t < best - 0.3f) { best = t; pick = {false, size}; }
+  }
+  return pick;
 }
 
 attn_tc::Args attention_args(const tidar_ctx *c, const AttnMaps &m, const KvGeom &g, bf16 *O) {
@@ -593,14 +614,26 @@ attn_tc::Args attention_args(const tidar_ctx *c, const AttnMaps &m, const KvGeom
   a.tile_count = c->count_tiles ? c->d_tl + 2 * tidar_ctx::TL_MAX : nullptr;
   return a;
 }
+// One CTA per item, or (cluster > 1) a cluster of CTAs per item.
 template <int STREAMS, bool DIRECT, bool AHEAD = false>
-void launch_attention_kernel(tidar_ctx *c, int grid, const AttnMaps &m, const attn_tc::Args &a) {
+void launch_attention_kernel(tidar_ctx *c, int grid, const AttnMaps &m, const attn_tc::Args &a, int cluster = 1) {
   Launch l(c, TIDAR_TC_ATTN);
   const int threads = attn_tc::threads(STREAMS);
+  if constexpr (STREAMS == 2) {
+    if (cluster > 1) {
+      if (c->cfg.head_dim == 128)
+        launch_pdl_cluster(cluster, attn_tc::attn_tc_kernel<128, 2, DIRECT, AHEAD, true>, grid * cluster, threads, attn_tc::Smem<128, 2, true>::TOTAL, c->stream, *m.q, *m.k,
+                           *m.v, *m.kloc, *m.vloc, a, l.tl);
+      else
+        launch_pdl_cluster(cluster, attn_tc::attn_tc_kernel<64, 2, DIRECT, AHEAD, true>, grid * cluster, threads, attn_tc::Smem<64, 2, true>::TOTAL, c->stream, *m.q, *m.k,
+                           *m.v, *m.kloc, *m.vloc, a, l.tl);
+      return;
+    }
+  }
   if (c->cfg.head_dim == 128)
-    launch_pdl(attn_tc::attn_tc_kernel<128, STREAMS, DIRECT, AHEAD>, grid, threads, attn_tc::Smem<128, STREAMS>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
+    launch_pdl(attn_tc::attn_tc_kernel<128, STREAMS, DIRECT, AHEAD, false>, grid, threads, attn_tc::Smem<128, STREAMS>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
   else
-    launch_pdl(attn_tc::attn_tc_kernel<64, STREAMS, DIRECT, AHEAD>, grid, threads, attn_tc::Smem<64, STREAMS>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
+    launch_pdl(attn_tc::attn_tc_kernel<64, STREAMS, DIRECT, AHEAD, false>, grid, threads, attn_tc::Smem<64, STREAMS>::TOTAL, c->stream, *m.q, *m.k, *m.v, *m.kloc, *m.vloc, a, l.tl);
 }
 
 template <bool DIRECT>
@@ -616,7 +649,8 @@ void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMap
   attn_tc::Args a = attention_args(c, m, g, O);
   a.items = p.items; a.tiles = p.tiles;
   a.early = early ? 1 : 0;
-  if (early && ahead) launch_attention_kernel<2, false, true>(c, p.max_items * p.Hkv, m, a); else launch_attention_kernel<2, false>(c, p.max_items * p.Hkv, m, a);
+  const int cluster = p.singles ? c->attn_cluster : 1;
+  if (early && ahead) launch_attention_kernel<2, false, true>(c, p.max_items * p.Hkv, m, a, cluster); else launch_attention_kernel<2, false>(c, p.max_items * p.Hkv, m, a, cluster);
   if (p.max_items > p.n_units && p.max_pieces > 1) launch_attention_merge<false>(c, 2 * p.n_units * p.Hkv, a);
 }
 
@@ -632,15 +666,23 @@ void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMap
 //   With one to two tiles per SM, one stream per CTA and two CTAs per SM: one wave, where the plan's CTAs, which hold an SM each, need
 //     two.  Four sequences of 1 k positions there (288 tiles): 42.1 us planned, 25.7 this way, at 9 k 175 and 148; but a plan evens
 //     out ragged lengths, which pays from about 60 pages on (lengths between 2 k and 4 k: 53.9 planned, 58.1 not).
-struct DirectPlan { int streams, pieces; };
+struct DirectPlan { int streams, pieces, cluster; };
 DirectPlan attention_direct(const tidar_ctx *c, int n_seqs, int k, int n_pages) {
   const int spt = 128 / (c->cfg.n_q_heads / c->cfg.n_kv_heads);
   const long long tiles = (long long)n_seqs * ((k * (k + 1) + spt - 1) / spt) * c->cfg.n_kv_heads;
-  if (tiles > c->n_sms) return {tiles <= 2 * c->n_sms && n_pages <= 40 ? 1 : 0, 1};
+  if (tiles > c->n_sms) return {tiles <= 2 * c->n_sms && n_pages <= 40 ? 1 : 0, 1, 1};
   const int most = std::min<int>(attn_tc::MAX_SPLITS, c->n_sms / (int)tiles);
   const int pieces = (int)sqrt(1.9 * n_pages);
-  if (n_pages <= (pieces <= most ? 15 : 19 + 12 / most)) return {2, 1};
-  return {pieces <= most ? 2 : 0, pieces};
+  if (n_pages <= (pieces <= most ? 15 : 19 + 12 / most)) {
+    DirectPlan pick{2, 1, 1};
+    float best = n_pages * attn_tc::SINGLE_PAGE - 0.3f;
+    for (int size = 2; size <= attn_tc::MAX_CLUSTER && size * 16 <= c->cfg.head_dim; size *= 2) {
+      const float t = (n_pages + size - 1) / size * attn_tc::SINGLE_PAGE + attn_tc::CLUSTER_MERGE;
+      if (tiles <= c->max_clusters[size] && t < best) { best = t; pick.cluster = size; }
+    }
+    return pick;
+  }
+  return {pieces <= most ? 2 : 0, pieces, 1};
 }
 
 void launch_attention(tidar_ctx *c, const bf16 *Q, const bf16 *Kp, const bf16 *Vp, const KvGeom &g, const bf16 *Kl,
@@ -816,14 +858,33 @@ int init_tensor_core_path(tidar_ctx *c) {
     CUDA_TRY(c, cudaMemsetAsync(c->Kloc, 0, nloc * cf.n_kv_heads * cf.head_dim * sizeof(bf16), c->stream));
     CUDA_TRY(c, cudaMemsetAsync(c->Vloc, 0, nloc * cf.n_kv_heads * cf.head_dim * sizeof(bf16), c->stream));
     auto smem = [](const void *f, int bytes) { return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 2, false, false>, attn_tc::Smem<128, 2>::TOTAL));
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 2, false, true>, attn_tc::Smem<128, 2>::TOTAL));
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 2, false, false>, attn_tc::Smem<64, 2>::TOTAL));
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 2, false, true>, attn_tc::Smem<64, 2>::TOTAL));
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 2, true, false>, attn_tc::Smem<128, 2>::TOTAL));
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 2, true, false>, attn_tc::Smem<64, 2>::TOTAL));
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 1, true, false>, attn_tc::Smem<128, 1>::TOTAL));
-    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 1, true, false>, attn_tc::Smem<64, 1>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 2, false, false, false>, attn_tc::Smem<128, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 2, false, true, false>, attn_tc::Smem<128, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 2, false, false, false>, attn_tc::Smem<64, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 2, false, true, false>, attn_tc::Smem<64, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 2, true, false, false>, attn_tc::Smem<128, 2>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 2, true, false, false>, attn_tc::Smem<64, 2>::TOTAL));
+    auto clusters = [&](auto kernel_128, auto kernel_64) {
+      const void *f = cf.head_dim == 128 ? (const void *)kernel_128 : (const void *)kernel_64;
+      const int bytes = cf.head_dim == 128 ? attn_tc::Smem<128, 2, true>::TOTAL : attn_tc::Smem<64, 2, true>::TOTAL;
+      return smem(f, bytes);
+    };
+    CUDA_TRY(c, clusters(attn_tc::attn_tc_kernel<128, 2, false, false, true>, attn_tc::attn_tc_kernel<64, 2, false, false, true>));
+    CUDA_TRY(c, clusters(attn_tc::attn_tc_kernel<128, 2, false, true, true>, attn_tc::attn_tc_kernel<64, 2, false, true, true>));
+    CUDA_TRY(c, clusters(attn_tc::attn_tc_kernel<128, 2, true, false, true>, attn_tc::attn_tc_kernel<64, 2, true, false, true>));
+    for (int size = 2; size <= attn_tc::MAX_CLUSTER && size * 16 <= cf.head_dim; size *= 2) {
+      cudaLaunchConfig_t lc{};
+      lc.gridDim = dim3(size); lc.blockDim = dim3(attn_tc::threads(2));
+      lc.dynamicSmemBytes = cf.head_dim == 128 ? attn_tc::Smem<128, 2, true>::TOTAL : attn_tc::Smem<64, 2, true>::TOTAL;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = size; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+      lc.attrs = at; lc.numAttrs = 1;
+      CUDA_TRY(c, cudaOccupancyMaxActiveClusters(&c->max_clusters[size], cf.head_dim == 128 ? (const void *)attn_tc::attn_tc_kernel<128, 2, false, false, true>
+                                                                                            : (const void *)attn_tc::attn_tc_kernel<64, 2, false, false, true>, &lc));
+    }
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<128, 1, true, false, false>, attn_tc::Smem<128, 1>::TOTAL));
+    CUDA_TRY(c, smem((const void *)attn_tc::attn_tc_kernel<64, 1, true, false, false>, attn_tc::Smem<64, 1>::TOTAL));
   }
   {
     auto max_smem_split = [&](const void *f) { return cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared); };
@@ -850,8 +911,8 @@ int init_tensor_core_path(tidar_ctx *c) {
       CUDA_TRY(c, max_smem_split(f));
       CUDA_TRY(c, cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, NORM_SMEM));
     }
-    CUDA_TRY(c, max_smem_split((const void *)attn_tc::attn_tc_kernel<128, 1, true, false>));
-    CUDA_TRY(c, max_smem_split((const void *)attn_tc::attn_tc_kernel<64, 1, true, false>));
+    CUDA_TRY(c, max_smem_split((const void *)attn_tc::attn_tc_kernel<128, 1, true, false, false>));
+    CUDA_TRY(c, max_smem_split((const void *)attn_tc::attn_tc_kernel<64, 1, true, false, false>));
   }
   const int max_smem = gemm_tc::SMEM_BUDGET + 1024;
   CUDA_TRY(c, cudaFuncSetAttribute(gemm_tc::gemm_tc_kernel<gemm_tc::MODE_SLAB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
@@ -928,7 +989,7 @@ int record_step(tidar_ctx *c, const tidar_ctx::StepKey &key) {
   const int T = k * (n_blocks + 1), R = key.mixed_R > 0 ? key.mixed_R : n_seqs * T;
   StepLayout lay{nullptr, nullptr, nullptr, n_seqs};
   if (key.mixed_R > 0) { lay.k = c->d_step_k; lay.off = c->d_step_off; lay.loc = c->d_step_loc; }
-  c->split_keys = key.split;
+  c->split_keys = key.split; c->attn_cluster = key.cluster;
   c->mixed_units = key.units;
   if (c->timeline) {
     c->tl_n = 0; c->tl_cls.clear();
@@ -1121,7 +1182,8 @@ int enqueue_step(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int32_t *f
   const int spt = 2 * (128 / (cf.n_q_heads / cf.n_kv_heads));      // slots per attention unit (two query tiles)
   tidar_ctx::StepKey key;
   key.k = k; key.n_seqs = n_seqs; key.ar = ar; key.units = n_seqs * ((T + spt - 1) / spt);
-  key.split = step_would_split(c, lens.data(), lengths.data(), n_seqs, ar);
+  const StepAttention att = step_attention(c, lens.data(), lengths.data(), n_seqs, ar, false);
+  key.split = att.split; key.cluster = att.cluster;
   if (int rc = launch_step(c, key)) return rc;
   CUDA_TRY(c, cudaEventRecord(c->flight_done[slot], c->stream));
   push_flight(c, seqs, n_seqs, forced, k, nullptr);
@@ -1174,7 +1236,8 @@ int enqueue_step_mixed(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int3
   // a mixed step's kernels take every per-sequence length from the staged layout: the nominal k is unused
   tidar_ctx::StepKey key;
   key.n_seqs = n_seqs; key.mixed_R = R; key.units = tiles;
-  key.split = step_would_split(c, lens.data(), ks, n_seqs, false);
+  const StepAttention att = step_attention(c, lens.data(), ks, n_seqs, false, true);
+  key.split = att.split; key.cluster = att.cluster;
   const int mixed_rows = cf.beta < 1.0f ? sum_k : 0;         // one mixed LM-head input row per verified position
   key.mixed_K = mixed_rows;
   // Steps of nearly the same size share one captured graph: rows are filled up to a multiple of 16 (the projections' row
@@ -1354,7 +1417,7 @@ int tidar_prefill(tidar_ctx *c, int32_t seq, const int32_t *prompt, int32_t n_pr
     if (last && cf.beta < 1.0f) { mix.n = 1; mix.k = 1; mix.a0 = rlp; mix.b0 = rlp + 1; }
     // logits are needed for the last prompt row and the k mask rows only; the LM head runs on the
     // trailing rows of the last chunk, as many as a decode step has (all of them for a short prompt)
-    c->split_keys = may_split(row0 + rows);
+    c->split_keys = may_split(row0 + rows); c->attn_cluster = 1;
     const int head_row0 = last ? std::max(0, rows + mix.n - c->R_head) : 0;
     if (int rc = forward_rows(c, rows, last, rows, mix, head_row0)) return rc;
     if (last) {
@@ -1475,7 +1538,7 @@ int tidar_score(tidar_ctx *c, int32_t seq, const int32_t *ids, int32_t n, float 
       Launch l(c, TIDAR_TC_EMBED);
       assemble_prefill_kernel<<<rows, 256, 0, c->stream>>>(c->meta, seq, row0, n, 0, cf.mask_token_id, c->d_prompt, c->embed, d, c->X, 0, 0ull);
     }
-    c->split_keys = may_split(row0 + rows);
+    c->split_keys = may_split(row0 + rows); c->attn_cluster = 1;
     if (int rc = forward_rows(c, rows, false, rows)) return rc;      // ends with the final norm in c->A
     const int32_t *target = c->d_prompt + row0 + 1;
     if (cf.impl == 0) {
@@ -1719,7 +1782,7 @@ int tidar_attention(tidar_ctx *c, const void *q, const void *k_pages, const void
     const DirectPlan d = attention_direct(c, n_seqs, k, pages_per_seq);
     attn_tc::PlanArgs plan{};
     if (!d.streams) {                              // (launched ahead of the host's work on the tensor maps)
-      c->split_keys = may_split(pages_per_seq * c->cfg.page_size);       // the lengths themselves are on the device
+      c->split_keys = may_split(pages_per_seq * c->cfg.page_size); c->attn_cluster = 1;       // the lengths themselves are on the device
       plan = attention_plan(c, R, k * (k + 1));
       Launch l(c, TIDAR_TC_EMBED);
       launch_pdl(attn_meta_plan_kernel, 1 + (R + 511) / 512, 512, 0, c->stream, c->meta, seq_len, k, R, n_max, plan);
@@ -1734,7 +1797,7 @@ int tidar_attention(tidar_ctx *c, const void *q, const void *k_pages, const void
       a.direct.seq_len = seq_len; a.direct.k = k; a.direct.n_max = n_max; a.direct.pieces = d.pieces;
       a.direct.per_group = (k * (k + 1) + a.spt - 1) / a.spt;
       const int tiles = n_seqs * a.direct.per_group * a.Hkv;
-      if (d.streams == 2) launch_attention_kernel<2, true>(c, tiles * d.pieces, am, a); else launch_attention_kernel<1, true>(c, tiles, am, a);
+      if (d.streams == 2) launch_attention_kernel<2, true>(c, tiles * d.pieces, am, a, d.cluster); else launch_attention_kernel<1, true>(c, tiles, am, a);
       if (d.pieces > 1) launch_attention_merge<true>(c, tiles, a);
     } else {
       launch_attention_tc(c, plan, am, g, (bf16 *)out, false, false);   // behind the kernel that makes the plan

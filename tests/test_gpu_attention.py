@@ -151,6 +151,19 @@ def test_attention_without_a_plan(hd, Hq, Hkv, k, ns, launches):
     t.close()
 
 
+@pytest.mark.parametrize("hd,Hq,Hkv,k,ns", [
+    (128, 8, 2, 1, [600]), (128, 8, 2, 4, [900, 0, 70]),           # clusters of eight, some of whose CTAs have no pages
+    (128, 12, 2, 16, [640]), (64, 4, 2, 8, [700, 1, 350, 64]),     # clusters of four, two unused rows per tile; head_dim 64
+    (128, 32, 8, 16, [1000]), (64, 8, 8, 16, [900]),               # clusters of two; one head per KV head
+])
+def test_attention_shared_by_clusters(hd, Hq, Hkv, k, ns):
+    t = _ctx(hd, Hq, Hkv, k, len(ns), 0)
+    before = t.launch_count()
+    _case(t, hd, Hq, Hkv, k, ns, 61)
+    assert t.launch_count() - before == 1
+    t.close()
+
+
 def test_attention_clamps_lengths_and_page_indices_without_a_plan():
     """Lengths below 0 and beyond the table's positions are clamped on every route, and a page outside the pool reads as zeros: both the
     two-stream and the one-stream instance against the same call with legal values."""

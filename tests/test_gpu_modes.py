@@ -135,6 +135,29 @@ def test_gate_up_tiles_beyond_one_wave(rows):
         assert np.isfinite(a).all() and np.abs(a - b).max() <= TOL_LOGITS * max(1.0, float(np.abs(b).max())), np.abs(a - b).max()
 
 
+@pytest.mark.parametrize("lens,ks", [([900], [4]), ([760, 20, 410], [4, 4, 4]), ([760, 20, 410], [4, 2, 3]), ([430], [12]), ([1000, 3], [1, 1])])
+def test_steps_over_long_contexts_match_the_replay_kernels(lens, ks):
+    """Steps whose attention is cut, or shared by clusters of CTAs (some without pages), or loads old pages ahead of its wait: hidden states of three
+    teacher-forced steps, equal and mixed block lengths, against the fp32 CUDA-core kernels."""
+    from paper_2511_08923_b200 import Tidar, pack_weights
+    sh, wt = make_model("tiny")
+    runs = []
+    for impl in IMPLS:
+        t = Tidar(sh, pack_weights(wt, "cuda:0"), k_max=12, max_batch=len(lens), max_seq_len=1088, debug=1, impl=impl, guard_bytes=64 * 1024, prefill_rows=512)
+        for q, n in enumerate(lens):
+            t.prefill(q, prompt_ids(sh, n, seed=n), max(ks))
+        out = []
+        for i in range(3):
+            for q in range(len(lens)):
+                t.set_block(q, prompt_ids(sh, 12, seed=50 + i))
+            t.step_ks(list(range(len(lens))), ks, [1 + i % k for k in ks])
+            out.append(t.hidden(2, 0, sum(k * (k + 1) for k in ks)))
+        runs.append(out)
+        _close(t)
+    for a, b in zip(*runs):
+        assert np.isfinite(a).all() and np.abs(a - b).max() <= TOL_LOGITS, np.abs(a - b).max()
+
+
 def test_autoregressive_mode_at_the_benchmark_widths():
     """The one-slot step and the scoring pass at the 8B-class widths (two layers, 8192-entry vocabulary so
     that the oracle stays fast): one-row projections (a 16-row MMA block), 4096-wide rows, 32 / 8 heads.
