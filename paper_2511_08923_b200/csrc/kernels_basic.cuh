@@ -276,6 +276,89 @@ rmsnorm_reduce_kernel(float *__restrict__ X, const SLAB *__restrict__ partials, 
   if (threadIdx.x == 0) tl_end(tl);
 }
 
+// The same with the row and its fp32 partial results brought to shared memory by bulk copies, one per source, and added in the same order.  For rows of
+// many bytes on every SM (see launch_norm_as), where the loads into registers are bound by how many of them an SM keeps in flight: 272
+// rows of 4096 with four slabs, 82 KB each, two per SM, 5.2 - 5.4 us -> 3.8.  Dynamic shared memory: (S + 1) * d floats at least.
+template <int THREADS, int NV>
+__global__ void __launch_bounds__(THREADS, NV <= 2 ? 2048 / THREADS : 1)
+rmsnorm_bulk_kernel(float *__restrict__ X, const float *__restrict__ partials, int S, size_t partial_stride,
+                    const bf16 *__restrict__ gain, float eps, int d, bf16 *__restrict__ A, int *status, TlSlot tl) {
+  pdl_trigger();
+  extern __shared__ __align__(128) uint8_t norm_smem[];
+  __shared__ __align__(8) uint64_t full[MAX_SLABS + 1];
+  __shared__ float red[THREADS / 32];
+  __shared__ int abort_flag;
+  const int r = blockIdx.x;
+  const float *buf = reinterpret_cast<const float *>(norm_smem);
+  if (threadIdx.x == 0) {
+    abort_flag = 0;
+    for (int s = 0; s <= S; ++s) sm100::mbar_init(sm100::smem_u32(&full[s]), 1);
+    sm100::fence_mbar_init();
+  }
+  uint2 gb[NV];                                  // weights: no need to wait for the previous kernel
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int c = (i * THREADS + threadIdx.x) * 4;
+    gb[i] = c < d ? *reinterpret_cast<const uint2 *>(gain + c) : make_uint2(0u, 0u);
+  }
+  __syncthreads();
+  pdl_wait();
+  float *xr = X + (size_t)r * d;
+  if (threadIdx.x == 0) {
+    tl_go(tl);
+    const uint32_t bytes = (uint32_t)d * 4u;
+    for (int s = 0; s <= S; ++s) {
+      const uint32_t bar = sm100::smem_u32(&full[s]);
+      sm100::mbar_expect_tx(bar, bytes);
+      sm100::bulk_load(sm100::smem_u32(norm_smem) + (uint32_t)s * bytes, s == 0 ? xr : partials + (size_t)(s - 1) * partial_stride + (size_t)r * d, bytes, bar);
+    }
+  }
+  float4 v[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  bool ok = true;
+#pragma unroll 1
+  for (int s = 0; s <= S && ok; ++s) {
+    ok = sm100::mbar_wait(sm100::smem_u32(&full[s]), 0u, &abort_flag);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const int c = (i * THREADS + threadIdx.x) * 4;
+      if (ok && c < d) {
+        const float4 q = *reinterpret_cast<const float4 *>(buf + (size_t)s * d + c);
+        v[i].x += q.x; v[i].y += q.y; v[i].z += q.z; v[i].w += q.w;
+      }
+    }
+  }
+  float ss = 0.f;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) ss += v[i].x * v[i].x + v[i].y * v[i].y + v[i].z * v[i].z + v[i].w * v[i].w;
+  ss = warp_sum(ss);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
+  __syncthreads();
+  float tot = 0.f;
+#pragma unroll
+  for (int i = 0; i < THREADS / 32; ++i) tot += red[i];
+  const float inv = rsqrtf(tot / (float)d + eps);
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int c = (i * THREADS + threadIdx.x) * 4;
+    if (c < d) {
+      if (S > 0) *reinterpret_cast<float4 *>(xr + c) = v[i];
+      const float2 g0 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gb[i].x)), g1 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&gb[i].y));
+      __nv_bfloat162 o0 = __floats2bfloat162_rn(v[i].x * inv * g0.x, v[i].y * inv * g0.y), o1 = __floats2bfloat162_rn(v[i].z * inv * g1.x, v[i].w * inv * g1.y);
+      uint2 ob; ob.x = *reinterpret_cast<uint32_t *>(&o0); ob.y = *reinterpret_cast<uint32_t *>(&o1);
+      *reinterpret_cast<uint2 *>(A + (size_t)r * d + c) = ob;
+    }
+  }
+  if (threadIdx.x == 0) {
+    if (abort_flag && status) atomicExch(status, 4);
+    tl_end(tl);
+  }
+  if (abort_flag) {                              // (a copy may still be on its way: the block stays until it has had time to land)
+    for (int i = 0; i < 2000; ++i) __nanosleep(1000);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // RoPE + KV placement.  Input: S split-K partials of the QKV projection, fp32
 // [S][R][(Hq+2Hkv)*hd].  Q heads are rotated and stored bf16 [R][Hq][hd]; K heads are
