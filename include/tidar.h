@@ -30,7 +30,7 @@
  *     and tidar_step synchronise that stream before they return the tokens.  On a stream
  *     that the caller created, a step is captured once per shape and replayed as one graph
  *     launch.  On the default stream (NULL), which CUDA does not let be captured, the same
- *     kernels are launched one by one; a shape of equal block lengths that has been run eight
+ *     kernels are launched one by one; a shape of equal block lengths that has been run sixteen
  *     times is then captured on a stream of the context's own and replayed on the default one.
  *   - A context is not synchronised between host threads: one thread at a time may call
  *     into it (different contexts are independent).

@@ -1084,10 +1084,11 @@ bool capture_step(tidar_ctx *c, const tidar_ctx::StepKey &key, cudaStream_t st) 
 }
 
 // Behind a step that was launched kernel by kernel on the legacy default stream, while it runs: captures its shape once it has been run often enough.
-// A capture costs the host about 4 us per launch and a replayed launch is 0.3 us faster, which a shape has to come back for.  (Tiny model, 23
-// launches: 119 -> 107 us per step; 1.5B-class autoregressive step of 8 rows, 259 launches: 1.52 -> 1.43 ms.)  Steps of mixed block lengths seldom
+// A capture and its graph cost the host about 9 us per launch, hidden behind the running step only where that is long enough, and a replayed launch is 0.3 -
+// 0.5 us faster: worth it after some 16 steps, so a shape that was run that often is expected to come back.  (Tiny model, 23
+// launches: 119 -> 107 us per step, 0.2 ms for the capture; 1.5B-class autoregressive step of 8 rows, 259 launches: 1.52 -> 1.43 ms.)  Steps of mixed block lengths seldom
 // meet the same shape again and stay as they are.
-constexpr int GRAPH_AFTER = 8;
+constexpr int GRAPH_AFTER = 16;
 void capture_aside(tidar_ctx *c, const tidar_ctx::StepKey &key) {
   if (key.mixed_R > 0 || key.timeline || key.count_tiles) return;
   auto it = std::find_if(c->seen.begin(), c->seen.end(), [&](const std::pair<tidar_ctx::StepKey, int> &s) { return s.first == key; });
@@ -1105,7 +1106,7 @@ void capture_aside(tidar_ctx *c, const tidar_ctx::StepKey &key) {
 // The step proper.  Every launch of a step has the same arguments from step to step (lengths, page tables, token
 // blocks and, for a step of mixed block lengths, the row layout live in device memory), except
 // for the grid sizes, so on a stream of the caller's the step is captured once per key and replayed.  On the legacy default
-// stream, which cannot be captured, that begins with a shape's ninth step (capture_aside).  Per-launch timing and the debug read-backs use plain
+// stream, which cannot be captured, that begins with a shape's seventeenth step (capture_aside).  Per-launch timing and the debug read-backs use plain
 // launches of the same kernels.  key.units: attention units per KV head.
 int launch_step(tidar_ctx *c, tidar_ctx::StepKey key) {
   key.timeline = c->timeline; key.count_tiles = c->count_tiles;

@@ -506,7 +506,7 @@ def test_kept_graphs_are_reused_and_replaced():
 
 
 def test_default_stream_replays_a_shape_that_recurs():
-    """On the default stream a step is launched kernel by kernel until its shape has been run eight times, and replayed from a graph afterwards, also with
+    """On the default stream a step is launched kernel by kernel until its shape has been run sixteen times, and replayed from a graph afterwards, also with
     two steps in flight and with other shapes in between: the same tokens, and bit-identical cached K/V, as without graphs."""
     sh, wt = make_model("tiny")
     k = sh.k
@@ -514,10 +514,10 @@ def test_default_stream_replays_a_shape_that_recurs():
     for tag, debug in (("graph", 0), ("plain", 8)):
         t = _gpu(sh, wt, 0, k_max=k, debug=debug, max_batch=2, max_seq_len=512)
         rec = [t.prefill(q, prompt_ids(sh, 50 + 9 * q), k) for q in range(2)]
-        for i in range(13):
+        for i in range(21):
             rec.append(t.step([0, 1], forced=[1 + i % k, 1 + (i + 1) % k]))
             if i % 4 == 0:
-                rec.append(t.step([1], forced=[2]))                # four times: never often enough
+                rec.append(t.step([1], forced=[2]))                # six times: never often enough
         assert t.graph_stats() == ((1, 5, 1) if tag == "graph" else (0, 0, 0))
         if tag == "graph":
             t.step_async([0, 1], [1, 2])
