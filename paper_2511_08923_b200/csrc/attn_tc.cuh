@@ -451,7 +451,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
           next = p + 32 + lane < n_table ? table[p_begin + p + 32 + lane] : 0;
         }
         const int page = __shfl_sync(0xffffffffu, cur, p & 31) + base;
-        if (!__all_sync(0xffffffffu, sm100::mbar_wait(empty0 + (uint32_t)s * 8u, ph, abortp))) break;
+        if (!sm100::mbar_wait_warp(empty0 + (uint32_t)s * 8u, ph, abortp)) break;
         if (sm100::elect_one()) {
           const uint32_t fb = full0 + (uint32_t)s * 8u, dst = dst0 + (uint32_t)s * L::KV_BYTES;
           sm100::mbar_expect_tx(fb, (uint32_t)L::KV_BYTES);
@@ -566,9 +566,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
     const uint32_t s_addr0 = tmem_S + (uint32_t)(t * 2 * PAGE) + lane_addr, o_addr = tmem_O + (uint32_t)(t * HD) + lane_addr;
     const uint32_t s_bar0 = sm100::smem_u32(&ctl.s_full[t][0]), p_bar0 = sm100::smem_u32(&ctl.p_full[t][0]);
     // wait until the scores of step j are there (for j >= nj: until P V of step j - 2 is done).  A parity wait means what it says
-    // because the barrier's next completion needs a P that this warp has not yet written.  A wait that gives up must
-    // take the whole warp out: the TMEM accesses are warp-collective.
-    auto wait_s = [&](int j) { return __all_sync(0xffffffffu, sm100::mbar_wait(s_bar0 + (uint32_t)(j & 1) * 8u, (uint32_t)(j >> 1) & 1u, abortp)) != 0; };
+    // because the barrier's next completion needs a P that this warp has not yet written.
+    auto wait_s = [&](int j) { return sm100::mbar_wait_warp(s_bar0 + (uint32_t)(j & 1) * 8u, (uint32_t)(j >> 1) & 1u, abortp); };
     float m_ref = -INFINITY, l_run = 0.f;
     bool ok = true;
 #pragma unroll 1

@@ -205,7 +205,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       const Item w = decode_item<MODE>(g, item);
       const int row = is_w ? (PAIR ? (w.tile * 2 + rank) * TILE_N : w.tile * TILE_N) : w.rb * g.rb_rows + rank * a_rows;
       for (int kb = w.kb0; kb < w.kb1; ++kb) {
-        if (!__all_sync(0xffffffffu, sm100::mbar_wait(sm100::smem_u32(&empty[s]), ph ^ 1u, abortp))) { ok = false; break; }
+        if (!sm100::mbar_wait_warp(sm100::smem_u32(&empty[s]), ph ^ 1u, abortp)) { ok = false; break; }
         if (sm100::elect_one()) {
           const uint32_t fb = sm100::smem_u32(&full[s]);
           const uint32_t dst = smem0 + (uint32_t)s * stage_bytes + (is_w ? 0u : (uint32_t)(KPS * W_STAGE_BYTES));
@@ -329,6 +329,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       if (lane == 0) { if constexpr (PAIR) sm100::mbar_arrive_cluster(drained_bar); else sm100::mbar_arrive(drained_bar); }
     };
     uint32_t it = 0; bool ok = true;
+    // Wait for the accumulator; the lanes leave together, but each with an answer of its own.  After a wait that gave up the item is gone through all the
+    // same, on stale values (all of a warp's lanes take part in its tensor-memory accesses, and the status word reports the failure): the
+    // lanes agree behind the item (`next`), for a vote here would stand in the way of every item (1.5B-class step: 0.1 % longer).
+    auto wait_full = [&](uint32_t n) { return sm100::mbar_wait_converged(sm100::smem_u32(&tmem_full_bar), n & 1u, abortp); };
+    auto next = [&](int item) { ok = __all_sync(0xffffffffu, ok) != 0; ++it; return item + n_workers; };
     // MODE_ARGMAX: running best of column c_begin + 32*slot + lane, and the row block it belongs to
     float best_v[5]; int best_i[5]; int cur_rb = -1;
 #pragma unroll
@@ -437,13 +442,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           sm100::tmem_wait_ld();
           swiglu_pass(c0, c1, second, c_begin + cc, row_block, live ? g.R : 0, n0);
           if (live) { cc += 32; continue; }
-          if (!sm100::mbar_wait(sm100::smem_u32(&tmem_full_bar), it & 1u, abortp)) { ok = false; break; }
+          ok = wait_full(it);
           sm100::tc_fence_after();
           live = true;
         }
-        if (!ok) break;
         drained();
-        item += n_workers; ++it;
+        item = next(item);
         continue;
       }
       if (MODE == MODE_SWIGLU && !w.fused && !g.slab_bf16) {
@@ -466,20 +470,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
             for (int j = 0; j < 8; ++j) { if (j < rows_left) *p = __uint_as_float(c0[h + j]); p += g.ldo; }
           }
           if (live) { cc += 16; continue; }
-          if (!sm100::mbar_wait(sm100::smem_u32(&tmem_full_bar), it & 1u, abortp)) { ok = false; break; }
+          ok = wait_full(it);
           sm100::tc_fence_after();
           live = true;
         }
-        if (!ok) break;
         drained();
-        item += n_workers; ++it;
+        item = next(item);
         continue;
       }
       const bool dry = walk;
       if (MODE == MODE_SLAB && dry) __nanosleep(1500);
       uint32_t v[NCH][16];
       if (!dry) {
-        if (!sm100::mbar_wait(sm100::smem_u32(&tmem_full_bar), it & 1u, abortp)) { ok = false; break; }
+        ok = wait_full(it);
         sm100::tc_fence_after();
         const uint32_t t0 = tmem_acc + ((uint32_t)(q * 32) << 16) + (uint32_t)c_begin;
 #pragma unroll
@@ -668,7 +671,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         }
       }
       if (walk) walk = false;                            // the same item again, for real
-      else { item += n_workers; ++it; }
+      else item = next(item);
     }
     if (MODE == MODE_ARGMAX || MODE == MODE_SAMPLE) flush_best();
   }

@@ -50,6 +50,17 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   return false;
 }
 
+// The same by a whole warp.  What follows a wait in the kernels is mostly warp-collective (tensor-memory accesses, elections), so lanes that leave the
+// loop apart must meet again; and since a wait that gives up may do so in some lanes only, the answers differ (converged) or are made one (warp).
+__device__ __forceinline__ bool mbar_wait_converged(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+  const bool ok = mbar_wait(bar, parity, abort_flag);
+  __syncwarp();
+  return ok;
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)) != 0;
+}
+
 // 2^x on the special-function unit, one instruction (denormal results flush to zero;
 // 2^-inf = 0, relative error about 2^-22).
 __device__ __forceinline__ float ex2_approx(float x) {

@@ -29,3 +29,16 @@ def test_aligned_cluster_barriers_are_reached_by_converged_warps():
     assert {"cluster_sync", "cluster_arrive_relaxed", "cluster_wait"} <= set(found)
     for f in os.listdir(CSRC):
         assert f == "sm100_ptx.cuh" or "barrier.cluster" not in _source(f), f
+
+
+def test_warps_leave_a_wait_together_and_branch_on_one_answer():
+    """In the tensor-core kernels a barrier is waited for through the helpers that bring the lanes together again, or by lane 0 for the others; and an
+    answer that may differ between lanes is not branched on before a vote."""
+    helpers = dict(_functions(_source("sm100_ptx.cuh")))
+    assert "__syncwarp()" in helpers["mbar_wait_converged"] and "__all_sync" in helpers["mbar_wait_warp"]
+    for f in ("gemm_tc.cuh", "attn_tc.cuh"):
+        src = _source(f)
+        for m in re.finditer(r"[^;{}]*\bmbar_wait\([^;]*;", src):
+            assert "if (lane == 0)" in m[0], (f, m[0].strip())
+        for call in ("mbar_wait_converged(", "wait_full("):
+            assert not re.search(r"if \([^;{]*" + re.escape(call), src), (f, call)
