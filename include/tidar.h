@@ -302,6 +302,9 @@ int tidar_debug_graph_stats(const tidar_ctx *ctx, int64_t *captured /*host*/, in
 /* How a projection of R rows by an [N][K] matrix would be launched on a GPU of n_sms SMs (no device needed; a test hook).  swiglu: the
  * fused gate/up projection.  out[0..4]: row blocks, rows per block, K splits, work items, whether the epilogue is walked through ahead. */
 int tidar_debug_plan_projection(const tidar_config *cfg, int32_t n_sms, int32_t swiglu, int32_t R, int32_t N, int32_t K, int32_t *out /*host,[5]*/);
+/* The same for the norm of R rows of d floats with S fp32 partial results each.  out[0]: sources are brought to shared memory by bulk copies;
+ * out[1]: dynamic shared memory of a block in bytes. */
+int tidar_debug_plan_norm(int32_t n_sms, int32_t R, int32_t d, int32_t S, int32_t *out /*host,[2]*/);
 /* Exercises the bounded wait the tensor-core kernels are built on: enqueues a one-thread kernel
  * that waits, for at most limit_polls polls (a few milliseconds at 2^14), on a barrier that
  * nothing arrives on, gives up and sets the status word.  tidar_sync then returns

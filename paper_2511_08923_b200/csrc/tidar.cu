@@ -700,23 +700,29 @@ void launch_attention(tidar_ctx *c, const bf16 *Q, const bf16 *Kp, const bf16 *V
     attn_replay_kernel<64><<<grid, 32, 0, c->stream>>>(Q, Kp, Vp, g, c->meta, Kl, Vl, O, c->cfg.n_q_heads, scale);
 }
 
+// How the norm of R rows of d floats with S fp32 partial results each is launched.
+// Behind a projection of many rows the blocks would all crowd onto the SMs that run out of work first (5.6 instead of
+// 3.6 us at 272 rows); claiming a share of the shared memory spreads them evenly.  With few rows they must leave room
+// for the next projection's CTAs.
+// Bulk copies where a row and its partial results are many bytes and every SM has one or two rows (measured: 82 KB 1.4 times as fast; 30 KB, 272 rows of
+// 1536 with four slabs, 1.8 -> 2.3 us; 16 KB, 1152 rows of 4096 without slabs, 5.5 -> 6.4; 20 rows of 82 KB no difference).
+struct NormPlan { bool bulk; size_t smem; };
+NormPlan norm_plan(int n_sms, int R, int d, int S, bool fp32_slabs) {
+  const int per_sm = (R + n_sms - 1) / n_sms;
+  if (R <= gemm_tc::SMALL_ROWS || per_sm > 4) return {false, 0};
+  const size_t share = (size_t)(NORM_SMEM / per_sm) & ~(size_t)1023, bytes = (size_t)(S + 1) * d * sizeof(float);
+  return {fp32_slabs && R <= gemm_tc::MAX_ROWS && per_sm <= 2 && bytes >= 48 * 1024 && bytes <= share, share};
+}
+
 // partials: split-K slabs of the previous projection, bf16 on the tensor-core path, fp32 on the replay path
 template <typename SLAB>
 void launch_norm_as(tidar_ctx *c, int R, const SLAB *partials, int S, size_t stride, const bf16 *gain) {
   Launch l(c, TIDAR_TC_NORM);
   const int d = c->cfg.d_model, nv = (d + 2047) / 2048;
-  // Behind a projection of many rows the blocks would all crowd onto the SMs that run out of work first (5.6 instead of
-  // 3.6 us at 272 rows); claiming a share of the shared memory spreads them evenly.  With few rows they must leave room
-  // for the next projection's CTAs.
-  const int per_sm = c->cfg.impl == 0 ? (R + c->n_sms - 1) / c->n_sms : 0;
-  // Bulk copies where a row and its partial results are many bytes and every SM has one or two rows (measured: 82 KB 1.4 times as fast; 30 KB, 272 rows of
-  // 1536 with four slabs, 1.8 -> 2.3 us; 16 KB, 1152 rows of 4096 without slabs, 5.5 -> 6.4; 20 rows of 82 KB no difference).
+  const NormPlan plan = c->cfg.impl == 0 ? norm_plan(c->n_sms, R, d, S, std::is_same_v<SLAB, float>) : NormPlan{false, 0};
   if constexpr (std::is_same_v<SLAB, float>) {
-    const size_t bytes = (size_t)(S + 1) * d * sizeof(float);
-    if (c->cfg.impl == 0 && R > gemm_tc::SMALL_ROWS && R <= gemm_tc::MAX_ROWS && bytes >= 48 * 1024 && bytes <= (size_t)NORM_SMEM / per_sm) {
-      auto bulk = [&](auto kernel) {
-        launch_pdl(kernel, R, 512, (size_t)(NORM_SMEM / per_sm) & ~(size_t)1023, c->stream, c->X, partials, S, stride, gain, c->cfg.rms_eps, d, c->A, c->d_status, l.tl);
-      };
+    if (plan.bulk) {
+      auto bulk = [&](auto kernel) { launch_pdl(kernel, R, 512, plan.smem, c->stream, c->X, partials, S, stride, gain, c->cfg.rms_eps, d, c->A, c->d_status, l.tl); };
       if (nv <= 1) bulk(rmsnorm_bulk_kernel<512, 1>);
       else if (nv <= 2) bulk(rmsnorm_bulk_kernel<512, 2>);
       else if (nv <= 3) bulk(rmsnorm_bulk_kernel<512, 3>);
@@ -724,8 +730,7 @@ void launch_norm_as(tidar_ctx *c, int R, const SLAB *partials, int S, size_t str
       return;
     }
   }
-  const size_t smem = R > gemm_tc::SMALL_ROWS && per_sm <= 4 && per_sm > 0 ? (size_t)(NORM_SMEM / per_sm) & ~(size_t)1023 : 0;
-  auto go = [&](auto kernel) { launch_pdl(kernel, R, 512, smem, c->stream, c->X, partials, S, stride, gain, c->cfg.rms_eps, d, c->A, l.tl); };
+  auto go = [&](auto kernel) { launch_pdl(kernel, R, 512, plan.smem, c->stream, c->X, partials, S, stride, gain, c->cfg.rms_eps, d, c->A, l.tl); };
   auto by_width = [&](auto slabs, auto walk) {
     constexpr int SL = decltype(slabs)::value;
     constexpr bool WK = decltype(walk)::value;
@@ -1751,6 +1756,13 @@ int tidar_debug_plan_projection(const tidar_config *cfg, int32_t n_sms, int32_t 
   layout(c, nullptr, &need);
   const gemm_tc::Args a = plan_gemm(&c, swiglu ? gemm_tc::MODE_SWIGLU : gemm_tc::MODE_SLAB, R, N, K);
   out[0] = a.n_rb; out[1] = a.rb_rows; out[2] = a.S; out[3] = a.total_items(); out[4] = a.warm_epilogue;
+  return TIDAR_OK;
+}
+
+int tidar_debug_plan_norm(int32_t n_sms, int32_t R, int32_t d, int32_t S, int32_t *out) {
+  if (!out || n_sms < 1 || R < 1 || d < 1 || S < 0 || S > MAX_SLABS) return fail(nullptr, TIDAR_EINVAL, "argument out of range");
+  const NormPlan p = norm_plan(n_sms, R, d, S, true);
+  out[0] = p.bulk ? 1 : 0; out[1] = (int32_t)p.smem;
   return TIDAR_OK;
 }
 

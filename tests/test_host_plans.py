@@ -41,3 +41,22 @@ def test_epilogues_are_walked_through_only_ahead_of_a_workers_single_item(model)
     assert seen == {0, 1} or model == "tiny"
     assert lib.tidar_debug_plan_projection(None, N_SMS, 0, 1, 64, 64, binding._ip(out)) == -1
     assert lib.tidar_debug_plan_projection(C.byref(_cfg(model)), 0, 0, 1, 64, 64, binding._ip(out)) == -1
+
+
+@pytest.mark.parametrize("n_sms", [148, 144, 143, 132, 100, 96, 74])
+def test_bulk_norm_fits_the_shared_memory_it_is_given(n_sms):
+    """Every row count and width: the row and its partial results fit the block's shared memory, the blocks of an SM fit beside one another, and on the
+    full chip wide rows behind a split projection do go this way."""
+    lib, out = binding.load(), np.zeros(2, dtype=np.int32)
+    taken = 0
+    for R in range(90, 300):
+        for d in range(64, 12289, 64):
+            for S in (0, 1, 2, 4, 8) if d % 128 == 0 else (3, 4, 5, 6, 7):
+                assert lib.tidar_debug_plan_norm(n_sms, R, d, S, binding._ip(out)) == 0
+                if out[0]:
+                    assert 96 < R <= 288 and 48 * 1024 <= (S + 1) * d * 4 <= out[1], (R, d, S, out)
+                    assert -(-R // n_sms) * out[1] <= 200 * 1024
+                    taken += 1
+    assert taken > 0
+    assert lib.tidar_debug_plan_norm(148, 272, 4096, 4, binding._ip(out)) == 0 and out.tolist() == [1, 100 * 1024]
+    assert lib.tidar_debug_plan_norm(148, 272, 4096, 9, binding._ip(out)) == -1
