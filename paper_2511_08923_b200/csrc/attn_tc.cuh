@@ -146,6 +146,12 @@ static_assert(sizeof(Ctl) <= 512, "control block must fit its slot");
 // (Measured inside the kernel, head_dim 128, all SMs busy: 1.05 us per page of a pair, 0.56 of a single tile.  head_dim 64 and nearly empty
 // grids take the same figures, although a page costs them less: they were not fitted, and cuts come out somewhat finer than best.)
 constexpr float CLUSTER_MERGE = 2.f;                   // what sharing an item within a cluster adds
+// A stand-alone call is launched in clusters for the width of its page table, which is all the host knows; a tile whose own pages (known on the device) are
+// few is its cluster's first CTA's alone.  Shared where that takes at least CLUSTER_SAVES pages off the longest CTA (five SINGLE_PAGE: just above what
+// sharing costs).  Alone / shared, tables of 8 to 16 pages: 32/8 heads of 128, k = 4, clusters of eight, 2 pages per tile 6.9 / 8.1 us, 5 pages 7.9 / 8.3, 6 pages
+// 8.9 / 8.5; 12/2 heads, k = 16, clusters of four, 2 pages 7.9 / 9.8, 6 pages 10.4 / 10.3, 10 pages 12.3 / 10.8.  (A step's sizes are known on the host.)
+constexpr int CLUSTER_SAVES = 5;
+__host__ __device__ constexpr bool cluster_shares(int n_pages, int log_size) { return n_pages - ((n_pages + (1 << log_size) - 1) >> log_size) >= CLUSTER_SAVES; }
 constexpr float OVERHEAD = 5.f, PAIR_PAGE = 1.05f, SINGLE_PAGE = 0.56f, PAIR_STORE = 2.5f, SINGLE_STORE = 1.5f, MERGE = 3.f;
 constexpr int PLAN_UNITS = 256;                        // up to this many units are planned; beyond, every unit is one item
 constexpr int CAND = 32;                               // limits tried per pairing: longest / (1 + i / 2)
@@ -345,7 +351,8 @@ __device__ __forceinline__ Item direct_item(const Args &a, int e) {
 // fetches the loop's code.  (8B-class step of 20 rows: 10.1 us behind a gap of 0.77 -> 8.9 behind 0.70; 1.5B-class autoregressive step of 8 rows 6.05 -> 4.75.
 // At 272 rows the CTAs wait for the SMs of the projection in front of the RoPE kernel and only lose by it; walking through the output code too was slower
 // everywhere, by 0.8 - 2 us.)
-// CLUSTER: the CTAs of a cluster share an item (a single tile, not cut): each takes an even share of its pages, and their results are merged over
+// CLUSTER: the CTAs of a cluster share an item (a single tile, not cut; of a stand-alone call only one of enough pages, see cluster_shares): each takes an
+// even share of its pages, and their results are merged over
 // distributed shared memory: every CTA finishes 1 / size of the head's columns, which the others store into its shared memory.  For calls and steps of few
 // tiles and contexts of some pages (see attention_direct, step_attention); bound by the latencies of first load and merge, about 2 us for the latter
 // (CLUSTER_MERGE).  Alone, 32/8 heads of 128, 272 rows, 1 k positions, clusters of two: 15.8 -> 13.2 us; 12/2 heads, four sequences of 72 rows, 1 k
@@ -394,12 +401,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
 
   // ---- which work item (every thread reads it: no barrier before the first loads go out) ----
   const int c_size = CLUSTER ? (int)sm100::cluster_size() : 1, c_rank = CLUSTER ? (int)sm100::cluster_rank() : 0;
-  const int kvh = blockIdx.x / c_size % a.Hkv, item_no = blockIdx.x / c_size / a.Hkv;
+  const int c_log = 31 - __clz(c_size);                // (a power of two: shifts instead of divisions ahead of the first loads, 0.1 us)
+  const int kvh = (blockIdx.x >> c_log) % a.Hkv, item_no = (blockIdx.x >> c_log) / a.Hkv;
   Item item = DIRECT ? direct_item(a, item_no) : a.items[item_no];   // all zero where the grid is larger than the plan: nothing to do
   const int np_item = item.p_end - item.p_begin;
+  const bool sharing = CLUSTER && (!DIRECT || cluster_shares(np_item, c_log));     // (the same in all CTAs of a cluster)
   if constexpr (CLUSTER) {
     const int b = item.p_begin;
-    item.p_begin = b + np_item * c_rank / c_size; item.p_end = b + np_item * (c_rank + 1) / c_size;
+    if (sharing) { item.p_begin = b + (np_item * c_rank >> c_log); item.p_end = b + (np_item * (c_rank + 1) >> c_log); }
+    else if (c_rank > 0) item.p_end = b;
   }
   const int row0 = item.row0, p_begin = item.p_begin, np = item.p_end - item.p_begin;
   const bool pair = STREAMS == 2 && !CLUSTER && item.pair != 0;
@@ -412,7 +422,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   const int t = (warp - 4) >> 2;                         // softmax warps: stream
   const int my_row = (warp & 3) * 32 + lane;             // and this thread's MMA row = TMEM lane
   int my_slot = -1;                                      // and its slot, -1: none
-  const int c_cols = HD / 2 / c_size, c_shift = 31 - __clz(c_cols);     // columns of a stream's half that a CTA of the cluster finishes (at least 8)
+  const int c_cols = HD / 2 >> c_log, c_shift = 31 - __clz(c_cols);     // columns of a stream's half that a CTA of the cluster finishes (at least 8)
   if (warp == 0 || warp == 3) {
     // ===================== K producer / Q and V producer =====================
     // Lane i holds the i-th entry of a group of 32 entries of the page table, so that a page's load does not wait for
@@ -686,7 +696,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         for (int c = 0; c < HD; c += 32) { float v[32]; load32(c, v); write32(v, c, inv); }
         if (my_slot >= 0 && item.split) a.part_ml[part * 128 + my_row] = make_float2(m_ref, l_run);
       }
-    } else if (CLUSTER ? np_item > 0 : np > 0) {
+    } else if (CLUSTER && sharing ? np_item > 0 : np > 0) {
       // The streams' halves of the same rows: each hands the other's columns over and finishes its own.  All MMAs have
       // read the K/V rings once every warp has got here (a failed stream only has to show up).
       float4 *xo = reinterpret_cast<float4 *>(smem_raw + L::XCHG_OFF);   // [stream that reads][HD / 8][128]
@@ -711,7 +721,24 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         const float2 other = xml[(1 - t) * 128 + my_row];
         const float M = fmaxf(m_ref, other.x);
         const float wm = m_ref == -INFINITY ? 0.f : exp2f(m_ref - M), wo = other.x == -INFINITY ? 0.f : exp2f(other.x - M);
-        const float l = wm * l_run + wo * other.y, inv = item.split ? 1.f : 1.f / l;
+        const float l = wm * l_run + wo * other.y, inv = (CLUSTER && sharing) || item.split ? 1.f : 1.f / l;
+        if (CLUSTER && DIRECT && __builtin_expect(!sharing, 0)) {       // (a short loop of its own, out of the way: as branches in the one below it cost shared tiles 0.3 us)
+#pragma unroll 1
+          for (int c = 0; c < HD / 2; c += 32) {
+            float v[32];
+            if (nj > 0) load32(t * (HD / 2) + c, v);
+            else {
+#pragma unroll
+              for (int i = 0; i < 32; ++i) v[i] = 0.f;
+            }
+#pragma unroll
+            for (int i = 0; i < 32; i += 4) {
+              const float4 x = xo[(t * (HD / 8) + (c + i) / 4) * 128 + my_row];
+              v[i] = wm * v[i] + wo * x.x; v[i + 1] = wm * v[i + 1] + wo * x.y; v[i + 2] = wm * v[i + 2] + wo * x.z; v[i + 3] = wm * v[i + 3] + wo * x.w;
+            }
+            write32(v, t * (HD / 2) + c, inv);
+          }
+        } else {
 #pragma unroll
         for (int c = 0; c < HD / 2; c += 32) {
           float v[32];
@@ -744,13 +771,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         } else {
           if (t == 0 && my_slot >= 0 && item.split) a.part_ml[part * 128 + my_row] = make_float2(M, l);
         }
+        }
       }
     }
   }
   if constexpr (CLUSTER) {
     if (warp < 4) sm100::cluster_wait();
-    sm100::cluster_sync();                               // the stores to one another have arrived
-    if (warp >= 4 && np_item > 0 && my_slot >= 0) {
+    if (sharing) sm100::cluster_sync();                  // the stores to one another have arrived
+    if (sharing && warp >= 4 && np_item > 0 && my_slot >= 0) {
       const float2 *ml = reinterpret_cast<const float2 *>(smem_raw + L::PEER_ML_OFF) + my_row;
       const float4 *x = reinterpret_cast<const float4 *>(smem_raw + L::PEER_OFF) + t * (c_cols / 4) * 128 + my_row;
       float M = -INFINITY, den = 0.f;

@@ -164,6 +164,32 @@ def test_attention_shared_by_clusters(hd, Hq, Hkv, k, ns):
     t.close()
 
 
+@pytest.mark.parametrize("hd,Hq,Hkv,k,lens", [
+    (128, 32, 8, 4, [200]), (128, 32, 8, 16, [100]), (128, 12, 2, 16, [200]), (64, 4, 2, 8, [0, 50, 100, 200]),     # clusters of eight, two, four, eight
+])
+def test_a_page_table_wider_than_the_lengths_changes_nothing(hd, Hq, Hkv, k, lens):
+    """Short sequences under a table wide enough for a call to be launched in clusters: bit for bit what the narrow table gives, for a tile of few pages
+    is not shared."""
+    dev, b = "cuda:0", len(lens)
+    t = _ctx(hd, Hq, Hkv, k, b, 0)
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(k)
+
+    def rnd(*shape):
+        return torch.randn(*shape, device=dev, dtype=torch.bfloat16, generator=gen)
+    T, W = k * (k + 1), 12
+    q, kp, vp, kl, vl = rnd(b * T, Hq, hd), rnd(b * W, Hkv, 64, hd), rnd(b * W, Hkv, 64, hd), rnd(b * k * k, Hkv, hd), rnd(b * k * k, Hkv, hd)
+    table = torch.randperm(b * W, device=dev, generator=gen).to(torch.int32).view(b, W)
+    outs = []
+    for width in (4, W):
+        out = torch.full((b * T, Hq * hd), float("nan"), dtype=torch.bfloat16, device=dev)
+        t.attention(q, kp, vp, table[:, :width].contiguous(), torch.tensor(lens, dtype=torch.int32, device=dev), kl, vl, out, b, k)
+        t.sync()
+        outs.append(out)
+    assert torch.isfinite(outs[0]).all() and torch.equal(outs[0], outs[1])
+    t.close()
+
+
 def test_attention_clamps_lengths_and_page_indices_without_a_plan():
     """Lengths below 0 and beyond the table's positions are clamped on every route, and a page outside the pool reads as zeros: both the
     two-stream and the one-stream instance against the same call with legal values."""
