@@ -305,6 +305,11 @@ int tidar_debug_plan_projection(const tidar_config *cfg, int32_t n_sms, int32_t 
 /* The same for the norm of R rows of d floats with S fp32 partial results each.  out[0]: sources are brought to shared memory by bulk copies;
  * out[1]: dynamic shared memory of a block in bytes. */
 int tidar_debug_plan_norm(int32_t n_sms, int32_t R, int32_t d, int32_t S, int32_t *out /*host,[2]*/);
+/* The same for the attention of a decode step of n_seqs sequences with n[i] cached positions and block lengths ks[i] (ar: an autoregressive step, ks all 1).
+ * max_clusters[0..2]: clusters of 2, 4 and 8 attention CTAs that the GPU holds at once.  out[0]: CTAs that share an item (1: none do); out[1]:
+ * whether key ranges may be cut, with a merge kernel behind. */
+int tidar_debug_plan_step(const tidar_config *cfg, int32_t n_sms, const int32_t *max_clusters /*host,[3]*/, const int32_t *n /*host,[n_seqs]*/,
+                          const int32_t *ks /*host,[n_seqs]*/, int32_t n_seqs, int32_t ar, int32_t *out /*host,[2]*/);
 /* Exercises the bounded wait the tensor-core kernels are built on: enqueues a one-thread kernel
  * that waits, for at most limit_polls polls (a few milliseconds at 2^14), on a barrier that
  * nothing arrives on, gives up and sets the status word.  tidar_sync then returns

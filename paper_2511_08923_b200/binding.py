@@ -96,6 +96,7 @@ def load(rebuild: bool = False) -> C.CDLL:
         "tidar_debug_graph_stats": (C.c_int, [ctxp, P(C.c_int64), P(C.c_int64), P(I32)]),
         "tidar_debug_plan_projection": (C.c_int, [P(tidar_config), I32, I32, I32, I32, I32, P(I32)]),
         "tidar_debug_plan_norm": (C.c_int, [I32, I32, I32, I32, P(I32)]),
+        "tidar_debug_plan_step": (C.c_int, [P(tidar_config), I32, P(I32), P(I32), P(I32), I32, I32, P(I32)]),
         "tidar_debug_get_timeline": (C.c_int, [ctxp, P(C.c_float), P(C.c_float), P(C.c_float)]),
     }
     for name, (res, args) in sig.items():

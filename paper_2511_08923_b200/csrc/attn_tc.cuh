@@ -156,6 +156,34 @@ constexpr float OVERHEAD = 5.f, PAIR_PAGE = 1.05f, SINGLE_PAGE = 0.56f, PAIR_STO
 constexpr int PLAN_UNITS = 256;                        // up to this many units are planned; beyond, every unit is one item
 constexpr int CAND = 32;                               // limits tried per pairing: longest / (1 + i / 2)
 
+// The estimate, for the plan kernel and for the host, which decides with it whether a step's merge kernel is needed at all (step_attention): limit number i
+// of the units or tiles the longest of which takes `longest` us; pieces of an entity of `us` us, at most one per page; what all entities come to.
+struct PlanCost { int items, live, most; float sum, longest; };
+__host__ __device__ inline float plan_limit(float longest, int i) { return fmaxf(longest / (1.f + 0.5f * i), 0.1f) * 1.0001f; }
+__host__ __device__ inline int plan_pieces(float us, float limit, bool dbl) {
+  const float n = us / limit, pages = us * (dbl ? 1.0001f / PAIR_PAGE : 1.0001f / SINGLE_PAGE);
+  const int up = (int)n + ((float)(int)n < n ? 1 : 0);
+  return up < (int)pages ? up : (int)pages;
+}
+__host__ __device__ inline void plan_add(PlanCost &c, float us, float limit, bool dbl, int times = 1) {
+  const int k = plan_pieces(us, limit, dbl);
+  const float store = k > 1 ? (dbl ? PAIR_STORE : SINGLE_STORE) : 0.f;
+#ifdef __CUDA_ARCH__
+  const float piece = __fdividef(us, (float)k);
+#else
+  const float piece = us / (float)k;
+#endif
+  c.items += times * k; c.live += times; c.most = k > c.most ? k : c.most;
+  c.sum += times * (us + k * (OVERHEAD + store));
+  c.longest = fmaxf(c.longest, piece + (k > 1 ? 0.5f * SINGLE_PAGE : 0.f) + store + OVERHEAD);
+}
+__host__ __device__ inline float plan_time(const PlanCost &c, int Hkv, int n_sms) {
+  float us = c.longest;
+  if (c.items * Hkv > n_sms) us = fmaxf(us, Hkv * c.sum / n_sms + 0.5f * c.longest);
+  if (c.items > c.live) us += MERGE + 0.3f * c.items / c.live;
+  return us;
+}
+
 // What a row sees: cached positions [0, nvis), local rows [loc0, loc0 + nloc).
 struct RowKeys { int nvis, loc0, nloc, seq; };
 
@@ -215,37 +243,26 @@ __device__ inline void plan_block(const PlanArgs &p, ROW row_keys) {
   __syncthreads();
   bool paired = true;
   float limit = 1e30f;
-  auto limit_of = [&](int cnd) { return fmaxf(__int_as_float(longest_us[cnd / CAND]) / (1.f + 0.5f * (cnd % CAND)), 0.1f) * 1.0001f; };
-  // pieces of an entity of cost us under a limit, at most one per page
-  auto pieces = [&](float us, float lim, bool dbl) { return (int)fminf(ceilf(us / lim), us * (dbl ? 1.0001f / PAIR_PAGE : 1.0001f / SINGLE_PAGE)); };
+  auto limit_of = [&](int cnd) { return plan_limit(__int_as_float(longest_us[cnd / CAND]), cnd % CAND); };
   if (splits) {
     const int per = blockDim.x / (2 * CAND) >= 16 ? 16 : blockDim.x / (2 * CAND) >= 4 ? 4 : 2;       // threads per candidate
     const int cnd = threadIdx.x / per, sub = threadIdx.x % per;
     const bool live_cnd = cnd < 2 * CAND, pr = cnd < CAND;
     const float lim = limit_of(live_cnd ? cnd : 0);
     const int n_ent = live_cnd ? (pr ? p.n_units : 2 * p.n_units) : 0, e0 = pr ? 0 : p.n_units;
-    int items = 0, live = 0, most = 0; float us_sum = 0.f, us_max = 0.f;
+    PlanCost cost{0, 0, 0, 0.f, 0.f};
     for (int e = sub; e < n_ent; e += per) {
       const float us = ent_us[e0 + e];
-      if (us <= 0.f) continue;
-      const bool dbl = pr && unit_row0[e] + p.spt < unit_rend[e];
-      const int k = pieces(us, lim, dbl);
-      const float store = k > 1 ? (dbl ? PAIR_STORE : SINGLE_STORE) : 0.f;
-      items += k; ++live; most = max(most, k);
-      us_sum += us + k * (OVERHEAD + store);
-      us_max = fmaxf(us_max, __fdividef(us, (float)k) + (k > 1 ? 0.5f * SINGLE_PAGE : 0.f) + store + OVERHEAD);
+      if (us > 0.f) plan_add(cost, us, lim, pr && unit_row0[e] + p.spt < unit_rend[e]);
     }
     for (int o = per >> 1; o > 0; o >>= 1) {
-      items += __shfl_xor_sync(0xffffffffu, items, o); live += __shfl_xor_sync(0xffffffffu, live, o); most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
-      us_sum += __shfl_xor_sync(0xffffffffu, us_sum, o); us_max = fmaxf(us_max, __shfl_xor_sync(0xffffffffu, us_max, o));
+      cost.items += __shfl_xor_sync(0xffffffffu, cost.items, o); cost.live += __shfl_xor_sync(0xffffffffu, cost.live, o);
+      cost.most = max(cost.most, __shfl_xor_sync(0xffffffffu, cost.most, o));
+      cost.sum += __shfl_xor_sync(0xffffffffu, cost.sum, o); cost.longest = fmaxf(cost.longest, __shfl_xor_sync(0xffffffffu, cost.longest, o));
     }
     unsigned long long mine = ~0ull;
-    if (live_cnd && items <= p.max_items && most <= p.max_pieces && !(pr && p.singles)) {
-      float us = us_max;
-      if (items * p.Hkv > p.n_sms) us = fmaxf(us, p.Hkv * us_sum / p.n_sms + 0.5f * us_max);
-      if (items > live) us += MERGE + 0.3f * items / live;
-      mine = ((unsigned long long)__float_as_uint(us) << 32) | (unsigned)cnd;                // us > 0: its bits order like its value
-    }
+    if (live_cnd && cost.items <= p.max_items && cost.most <= p.max_pieces && !(pr && p.singles))
+      mine = ((unsigned long long)__float_as_uint(plan_time(cost, p.Hkv, p.n_sms)) << 32) | (unsigned)cnd;      // (positive: its bits order like its value)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mine = min(mine, __shfl_xor_sync(0xffffffffu, mine, o));
     if (lane == 0) best[warp] = mine;
@@ -258,7 +275,7 @@ __device__ inline void plan_block(const PlanArgs &p, ROW row_keys) {
   const int n_ent = paired ? p.n_units : 2 * p.n_units, e0 = paired ? 0 : p.n_units;
   for (int e = threadIdx.x; e < n_ent; e += blockDim.x) {
     const float us = ent_us[e0 + e];
-    const int k = us <= 0.f ? 0 : splits ? max(1, pieces(us, limit, paired && unit_row0[e] + p.spt < unit_rend[e])) : 1;
+    const int k = us <= 0.f ? 0 : splits ? max(1, plan_pieces(us, limit, paired && unit_row0[e] + p.spt < unit_rend[e])) : 1;
     ent_n[e] = (short)k; ent_us[e0 + e] = k ? us / k : -1.f;
   }
   __syncthreads();

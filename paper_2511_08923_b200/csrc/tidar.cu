@@ -69,6 +69,7 @@ struct tidar_ctx {
   bf16 *A = nullptr, *Q = nullptr, *Kloc = nullptr, *Vloc = nullptr, *O = nullptr, *H = nullptr, *dbg_kv = nullptr;
   // host state
   std::vector<SeqState> seqs;
+  std::vector<int> step_n;         // lengths of the sequences of the step being enqueued
   std::vector<int> free_pages;
   int32_t *h_pinned = nullptr;     // [max_batch*(k_max+1)] results + staging
   std::string err;
@@ -537,70 +538,82 @@ attn_tc::PlanArgs attention_plan(const tidar_ctx *c, int R, int rows_per_group) 
 // kernel, about 5 us, and saves half of 0.56 us per page at best.
 bool may_split(int n_keys) { return n_keys > 12 * attn_tc::PAGE; }
 
-// The same for a decode step, whose sequences' lengths n[] and block lengths ks[] the host knows: whether the work plan (attn_tc::plan_block, whose
-// estimate this repeats) would cut any key range.  Where it would not, the step goes without the merge kernel, which would find nothing to do
-// (8B-class step of 272 rows, 1.1 k positions: 2.4 us per layer).  A step planned as uncut on the host is not cut on the device.
+// The same for a decode step, whose sequences' lengths n[] and block lengths (ks[], or k for all) the host knows: whether the work plan
+// (attn_tc::plan_block, from the same estimate) would cut any key range.  Where it would not, the step goes without the merge kernel, which would find nothing
+// to do (8B-class step of 272 rows, 1.1 k positions: 2.4 us per layer).  A step planned as uncut on the host is not cut on the device.
+// This runs ahead of every step's first launch, so equal units are counted and not listed, nothing is allocated, and a block length's tiles are worked
+// out once for all sequences next to one another that have it (12/2 heads, 60 sequences of one row: 11.3 -> 2.8 us; 14 of 272 rows: 22.5 -> 5.1).
 struct StepAttention { bool split; int cluster; };
-StepAttention step_attention(const tidar_ctx *c, const int *n, const int *ks, int n_seqs, bool ar, bool mixed) {
+StepAttention step_attention(const tidar_ctx *c, const int *n, const int *ks, int k_all, int n_seqs, bool ar, bool mixed) {
   using namespace attn_tc;
   const StepAttention uncut{false, 1}, cut{true, 1};
   const int spt = 128 / (c->cfg.n_q_heads / c->cfg.n_kv_heads), Hkv = c->cfg.n_kv_heads;
-  std::vector<float> ent[2];                           // us of the units, of the tiles
-  std::vector<char> two;                               // units of two tiles
-  int longest = 0;
-  for (int s = 0; s < n_seqs; ++s) {
-    longest = std::max(longest, n[s]);
-    const int k = ks[s], T = ar ? 1 : k * (k + 1);
-    auto pages = [&](int first, int last) {            // pages that slots first .. last need
-      int nvis = first < k ? std::min(last, k - 1) + 1 : 0, loc = 0;
-      if (last >= k) { nvis = std::max(nvis, (last - k) / k + 1); loc = ((last - k) / k - (std::max(first, k) - k) / k + 1) * k; }
-      return (n[s] + nvis + PAGE - 1) / PAGE + (loc + PAGE - 1) / PAGE;
-    };
-    for (int r = 0; r < T; r += 2 * spt) {
-      const bool dbl = r + spt < T;
-      two.push_back(dbl);
-      ent[0].push_back(pages(r, std::min(r + 2 * spt, T) - 1) * (dbl ? PAIR_PAGE : SINGLE_PAGE));
-      ent[1].push_back(pages(r, std::min(r + spt, T) - 1) * SINGLE_PAGE);
-      ent[1].push_back(dbl ? pages(r + spt, std::min(r + 2 * spt, T) - 1) * SINGLE_PAGE : 0.f);
-    }
-  }
-  const int n_units = (int)two.size(), units = n_units * Hkv;
+  auto rows = [&](int s) { const int k = ks ? ks[s] : k_all; return ar ? 1 : k * (k + 1); };
+  int n_units = 0, longest = 0;
+  for (int s = 0; s < n_seqs; ++s) { n_units += (rows(s) + 2 * spt - 1) / (2 * spt); longest = std::max(longest, n[s]); }
+  const int units = n_units * Hkv;
   const int most_items = units <= c->n_sms ? c->n_sms / Hkv : 2 * units < 3 * c->n_sms ? SLOTS_PER_SM * c->n_sms / Hkv : n_units;     // as in attention_plan
   if (n_units > PLAN_UNITS || most_items <= n_units) return cut;       // nothing is cut and no merge launched whatever is said here
+  // entities (units, tiles) by their number of pages
+  struct Entity { float us; int times, pages; bool dbl; } ent[2][2 * PLAN_UNITS];
+  short slot_of[2][4 * PLAN_UNITS];                    // open addressing; at most half full
+  int n_ent[2] = {0, 0};
+  float most_us[2] = {0.f, 0.f};
+  memset(slot_of, 0xff, sizeof slot_of);
+  auto add = [&](int list, int pages, bool dbl) {
+    unsigned h = (unsigned)(pages * 2 + dbl) % (4 * PLAN_UNITS);
+    while (slot_of[list][h] >= 0 && (ent[list][slot_of[list][h]].pages != pages || ent[list][slot_of[list][h]].dbl != dbl)) h = (h + 1) % (4 * PLAN_UNITS);
+    if (slot_of[list][h] >= 0) { ++ent[list][slot_of[list][h]].times; return; }
+    const float us = pages * (dbl ? PAIR_PAGE : SINGLE_PAGE);
+    slot_of[list][h] = (short)n_ent[list];
+    ent[list][n_ent[list]++] = Entity{us, 1, pages, dbl};
+    most_us[list] = std::max(most_us[list], us);
+  };
+  struct Span { int nvis, loc; } span[3][PLAN_UNITS];  // of a block length's units, first tiles, second tiles: positions beyond n, local pages
+  int spans = 0, spans_T = -1, tiles = 0;
+  for (int s = 0; s < n_seqs; ++s) {
+    const int k = ks ? ks[s] : k_all, T = rows(s);
+    if (T != spans_T) {
+      spans = 0; spans_T = T;
+      auto seen = [&](int first, int last) {           // by slots first .. last
+        int nvis = first < k ? std::min(last, k - 1) + 1 : 0, loc = 0;
+        if (last >= k) { nvis = std::max(nvis, (last - k) / k + 1); loc = ((last - k) / k - (std::max(first, k) - k) / k + 1) * k; }
+        return Span{nvis, (loc + PAGE - 1) / PAGE};
+      };
+      for (int r = 0; r < T; r += 2 * spt, ++spans) {
+        span[0][spans] = seen(r, std::min(r + 2 * spt, T) - 1);
+        span[1][spans] = seen(r, std::min(r + spt, T) - 1);
+        span[2][spans] = r + spt < T ? seen(r + spt, std::min(r + 2 * spt, T) - 1) : Span{0, -1};
+      }
+    }
+    for (int u = 0; u < spans; ++u) {
+      const bool two = span[2][u].loc >= 0;
+      auto pages = [&](const Span &x) { return (n[s] + x.nvis + PAGE - 1) / PAGE + x.loc; };
+      add(0, pages(span[0][u]), two);
+      add(1, pages(span[1][u]), false);
+      if (two) add(1, pages(span[2][u]), false);
+      tiles += two ? 2 : 1;
+    }
+  }
   float best = 1e30f;
   bool split = true;
   const bool may_cut = may_split(longest);
-  for (int cnd = 0; cnd < 2 * CAND; cnd += 2) {        // (every other limit: this runs ahead of each step's first launch)
-    const bool pr = cnd < CAND;
-    const std::vector<float> &us = ent[pr ? 0 : 1];
-    const float lim = std::max(*std::max_element(us.begin(), us.end()) / (1.f + 0.5f * (cnd % CAND)), 0.1f) * 1.0001f;
-    const float inv = 1.f / lim;
-    int items = 0, live = 0, most = 0; float sum = 0.f, mx = 0.f;
-    for (size_t e = 0; e < us.size(); ++e) {
-      if (us[e] <= 0.f) continue;
-      const bool dbl = pr && two[e];
-      const int p = (int)std::min(us[e] * inv + 0.9999f, us[e] * (dbl ? 1.0001f / PAIR_PAGE : 1.0001f / SINGLE_PAGE));
-      const float store = p > 1 ? (dbl ? PAIR_STORE : SINGLE_STORE) : 0.f;
-      items += p; ++live; most = std::max(most, p);
-      sum += us[e] + p * (OVERHEAD + store);
-      mx = std::max(mx, us[e] / p + (p > 1 ? 0.5f * SINGLE_PAGE : 0.f) + store + OVERHEAD);
-    }
-    if (items > most_items || most > (may_cut ? MAX_SPLITS : 1)) continue;
-    float t = mx;
-    if (items * Hkv > c->n_sms) t = std::max(t, Hkv * sum / c->n_sms + 0.5f * mx);
-    if (items > live) t += MERGE + 0.3f * items / live;
-    if (t < best) { best = t; split = items > live || (!pr && 2 * units > c->n_sms); }       // (single tiles beyond one wave need the larger grid)
+  for (int cnd = 0; cnd < 2 * CAND; cnd += 2) {        // (every other limit)
+    const int list = cnd / CAND;
+    const float lim = plan_limit(most_us[list], cnd % CAND);
+    PlanCost cost{0, 0, 0, 0.f, 0.f};
+    for (int e = 0; e < n_ent[list]; ++e) plan_add(cost, ent[list][e].us, lim, ent[list][e].dbl, ent[list][e].times);
+    if (cost.items > most_items || cost.most > (may_cut ? MAX_SPLITS : 1)) continue;
+    const float t = plan_time(cost, Hkv, c->n_sms);
+    if (t < best) { best = t; split = cost.items > cost.live || (list == 1 && 2 * units > c->n_sms); }       // (single tiles beyond one wave need the larger grid)
   }
   // A cluster per tile, its pages shared evenly; on three quarters of the SMs at most, for on the others the projection behind the attention fills its
   // rings (8B-class step of 272 rows, clusters of two on 144 SMs: attention 15.9 -> 12.7 us, the O projection 14.9 -> 18).
-  int tiles = 0;
-  for (float us : ent[1]) tiles += us > 0.f;
   const int places = mixed ? 2 * ((n_units + 3) / 4 * 4) : tiles;      // items of the launch (see attention_plan)
-  const float longest_us = *std::max_element(ent[1].begin(), ent[1].end());
   if (split) best += 1.5f;                               // (the boundary in front of the merge kernel)
   StepAttention pick = split ? cut : uncut;
   for (int size = 2; size <= MAX_CLUSTER && size * 16 <= c->cfg.head_dim; size *= 2) {
-    const float t = std::ceil(longest_us / SINGLE_PAGE / size) * SINGLE_PAGE + OVERHEAD + CLUSTER_MERGE;
+    const float t = std::ceil(most_us[1] / SINGLE_PAGE / size) * SINGLE_PAGE + OVERHEAD + CLUSTER_MERGE;
     if (places * Hkv <= c->max_clusters[size] && 4 * places * Hkv * size <= 3 * c->n_sms && t < best - 0.3f) { best = t; pick = {false, size}; }
   }
   return pick;
@@ -1203,15 +1216,14 @@ int enqueue_step(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int32_t *f
   }
   const int T = ar ? 1 : k * (k + 1), R = n_seqs * T;
   const int slot = c->turn & 1;
-  std::vector<int> lens(n_seqs), lengths(n_seqs, k);
   for (int i = 0; i < n_seqs; ++i) {
     c->h_stage2[slot][i] = seqs[i]; c->h_stage2[slot][cf.max_batch + i] = forced ? forced[i] : 0;
-    lens[i] = c->seqs[seqs[i]].n;
+    c->step_n[i] = c->seqs[seqs[i]].n;
   }
   const int spt = 2 * (128 / (cf.n_q_heads / cf.n_kv_heads));      // slots per attention unit (two query tiles)
   tidar_ctx::StepKey key;
   key.k = k; key.n_seqs = n_seqs; key.ar = ar; key.units = n_seqs * ((T + spt - 1) / spt);
-  const StepAttention att = step_attention(c, lens.data(), lengths.data(), n_seqs, ar, false);
+  const StepAttention att = step_attention(c, c->step_n.data(), nullptr, k, n_seqs, ar, false);
   key.split = att.split; key.cluster = att.cluster;
   if (int rc = launch_step(c, key)) return rc;
   CUDA_TRY(c, cudaEventRecord(c->flight_done[slot], c->stream));
@@ -1252,20 +1264,19 @@ int enqueue_step_mixed(tidar_ctx *c, const int32_t *seqs, int n_seqs, const int3
   int32_t *hk = c->h_lay, *hoff = hk + (mb + 1), *hloc = hoff + (mb + 1), *ht0 = hloc + (mb + 1), *hte = ht0 + (c->R_head + mb);
   const int slot = c->turn & 1;
   int R = 0, loc = 0, tiles = 0, sum_k = 0;
-  std::vector<int> lens(n_seqs);
   for (int i = 0; i < n_seqs; ++i) {
     const int k = ks[i], T = k * (k + 1);
     hk[i] = k; hoff[i] = R; hloc[i] = loc; sum_k += k;
     for (int r0 = R; r0 < R + T; r0 += spt) { ht0[tiles] = r0; hte[tiles] = R + T; ++tiles; }
     R += T; loc += k * k;
     c->h_stage2[slot][i] = seqs[i]; c->h_stage2[slot][mb + i] = forced ? forced[i] : 0;
-    lens[i] = c->seqs[seqs[i]].n;
+    c->step_n[i] = c->seqs[seqs[i]].n;
   }
   hk[n_seqs] = 0; hoff[n_seqs] = R; hloc[n_seqs] = loc;
   // a mixed step's kernels take every per-sequence length from the staged layout: the nominal k is unused
   tidar_ctx::StepKey key;
   key.n_seqs = n_seqs; key.mixed_R = R; key.units = tiles;
-  const StepAttention att = step_attention(c, lens.data(), ks, n_seqs, false, true);
+  const StepAttention att = step_attention(c, c->step_n.data(), ks, 0, n_seqs, false, true);
   key.split = att.split; key.cluster = att.cluster;
   const int mixed_rows = cf.beta < 1.0f ? sum_k : 0;         // one mixed LM-head input row per verified position
   key.mixed_K = mixed_rows;
@@ -1379,6 +1390,7 @@ int tidar_init(const tidar_config *cfg, const tidar_weights *w, void *arena, siz
     if (int rc = init_tensor_core_path(c)) { std::string m = c->err; delete c; return fail(nullptr, rc, "%s", m.c_str()); }
   }
   c->seqs.resize(cfg->max_batch);
+  c->step_n.resize(cfg->max_batch);
   // free list in a scrambled order so that page tables are never contiguous
   c->free_pages.resize(c->n_pages);
   for (int i = 0; i < c->n_pages; ++i) c->free_pages[i] = i;
@@ -1766,6 +1778,21 @@ int tidar_debug_plan_norm(int32_t n_sms, int32_t R, int32_t d, int32_t S, int32_
   if (!out || n_sms < 1 || R < 1 || d < 1 || S < 0 || S > MAX_SLABS) return fail(nullptr, TIDAR_EINVAL, "argument out of range");
   const NormPlan p = norm_plan(n_sms, R, d, S, true);
   out[0] = p.bulk ? 1 : 0; out[1] = (int32_t)p.smem;
+  return TIDAR_OK;
+}
+
+int tidar_debug_plan_step(const tidar_config *cfg, int32_t n_sms, const int32_t *max_clusters, const int32_t *n, const int32_t *ks, int32_t n_seqs, int32_t ar, int32_t *out) {
+  std::string why;
+  if (!cfg || !max_clusters || !n || !ks || !out) return fail(nullptr, TIDAR_EINVAL, "null argument");
+  if (validate(*cfg, why) != TIDAR_OK) return fail(nullptr, TIDAR_EINVAL, "%s", why.c_str());
+  if (n_sms < 1 || n_sms > MAX_SMS || n_seqs < 1) return fail(nullptr, TIDAR_EINVAL, "n_sms or n_seqs out of range");
+  for (int i = 0; i < n_seqs; ++i) if (n[i] < 0 || ks[i] < 1 || ks[i] > cfg->k_max) return fail(nullptr, TIDAR_EINVAL, "length or block length %d out of range", i);
+  tidar_ctx c;
+  c.cfg = *cfg; c.n_sms = n_sms;
+  for (int i = 0; i < 3; ++i) c.max_clusters[2 << i] = max_clusters[i];
+  const bool mixed = std::any_of(ks, ks + n_seqs, [&](int k) { return k != ks[0]; });
+  const StepAttention a = step_attention(&c, n, mixed ? ks : nullptr, ks[0], n_seqs, ar != 0, mixed);
+  out[0] = a.cluster; out[1] = a.split ? 1 : 0;
   return TIDAR_OK;
 }
 

@@ -60,3 +60,73 @@ def test_bulk_norm_fits_the_shared_memory_it_is_given(n_sms):
     assert taken > 0
     assert lib.tidar_debug_plan_norm(148, 272, 4096, 4, binding._ip(out)) == 0 and out.tolist() == [1, 100 * 1024]
     assert lib.tidar_debug_plan_norm(148, 272, 4096, 9, binding._ip(out)) == -1
+
+
+def _step_route(model, n, ks, ar, max_clusters):
+    """(route, lead of the best time over the best of another route): every page counted slot by slot, every limit in 64 bits."""
+    d, hq, hkv, hd, f = SHAPES[model]
+    spt = 128 // (hq // hkv)
+    units, tiles = [], []                                # (pages, two tiles)
+    for m, k in zip(n, ks):
+        slots = [(m + 1, None)] if ar else [(m + j + 1, None) for j in range(k)] + [(m + b + 1, b) for b in range(k) for _ in range(k)]
+
+        def pages(part):
+            blocks = [b for _, b in part if b is not None]
+            return -(-max(v for v, _ in part) // 64) + (-(-(max(blocks) - min(blocks) + 1) * k // 64) if blocks else 0)
+        for r in range(0, len(slots), 2 * spt):
+            a, b = slots[r:r + spt], slots[r + spt:r + 2 * spt]
+            units.append((pages(a + b), bool(b)))
+            tiles += [(pages(x), False) for x in (a, b) if x]
+    most_items = N_SMS // hkv if len(units) * hkv <= N_SMS else 2 * N_SMS // hkv if 2 * len(units) * hkv < 3 * N_SMS else len(units)
+    if len(units) > 256 or most_items <= len(units):
+        return (1, 1), 1.0
+    times = {}
+    for paired, ents in ((True, units), (False, tiles)):
+        us = [p * (1.05 if two else 0.56) for p, two in ents]
+        for i in range(0, 32, 2):
+            limit = max(max(us) / (1 + 0.5 * i), 0.1) * 1.0001
+            cut = [min(int(np.ceil(u / limit)), p) for u, (p, _) in zip(us, ents)]
+            if sum(cut) > most_items or max(cut) > (32 if max(n) > 768 else 1):
+                continue
+            store = [(2.5 if two else 1.5) if c > 1 else 0.0 for c, (_, two) in zip(cut, ents)]
+            longest = max(u / c + (0.28 if c > 1 else 0.0) + s + 5 for u, c, s in zip(us, cut, store))
+            t = longest
+            if sum(cut) * hkv > N_SMS:
+                t = max(t, hkv * sum(u + c * (5 + s) for u, c, s in zip(us, cut, store)) / N_SMS + 0.5 * longest)
+            if sum(cut) > len(cut):
+                t += 3 + 0.3 * sum(cut) / len(cut)
+            split = int(sum(cut) > len(cut) or (not paired and 2 * len(units) * hkv > N_SMS))
+            times.setdefault((1, split), []).append(t)
+    best = {r: min(t) for r, t in times.items()}
+    ranked = sorted(best.items(), key=lambda x: x[1])
+    lead = ranked[1][1] - ranked[0][1] if len(ranked) > 1 else 1.0
+    route, t = ranked[0] if ranked else ((1, 1), 1e30)
+    t += 1.5 * route[1]
+    places = 2 * (-(-len(units) // 4) * 4) if len(set(ks)) > 1 else len(tiles)
+    for size, room in zip((2, 4, 8), max_clusters):
+        if size * 16 <= hd:
+            tc = -(-max(p for p, _ in tiles) // size) * 0.56 + 7
+            if places * hkv <= room and 4 * places * hkv * size <= 3 * N_SMS:
+                lead = min(lead, abs(tc - (t - 0.3)))
+                if tc < t - 0.3:
+                    t, route = tc, (size, 0)
+    return route, lead
+
+
+@pytest.mark.parametrize("model", list(SHAPES))
+def test_step_attention_follows_the_plan_kernels_estimate(model):
+    """Cut, uncut or shared by clusters: random batches, one row and k (k + 1) rows per sequence, equal and mixed block lengths, lengths up to 30 k.
+    (Where two routes are within a thousandth of a microsecond, 32-bit sums may choose either.)"""
+    lib, out, rng, seen = binding.load(), np.zeros(2, dtype=np.int32), np.random.default_rng(5), {}
+    room = np.array([74, 36, 16], dtype=np.int32)
+    for i in range(250):
+        ar, mixed = i % 4 == 0, i % 4 == 1
+        n_seqs = int(rng.integers(1, 41 if ar else 5))
+        n = rng.integers(0, int(np.exp(rng.uniform(np.log(20), np.log(30000)))), n_seqs).astype(np.int32)
+        k = 1 if ar else int(rng.integers(1, 17))
+        ks = (rng.integers(1, k + 1, n_seqs) if mixed else np.full(n_seqs, k)).astype(np.int32)
+        assert lib.tidar_debug_plan_step(C.byref(_cfg(model)), N_SMS, binding._ip(room), binding._ip(n), binding._ip(ks), n_seqs, int(ar), binding._ip(out)) == 0
+        route, lead = _step_route(model, n.tolist(), ks.tolist(), ar, room.tolist())
+        assert lead < 1e-3 or tuple(out.tolist()) == route, (n, ks, ar, out, route)
+        seen[route] = seen.get(route, 0) + 1
+    assert len(seen) >= 4 and (1, 0) in seen and (1, 1) in seen, seen
