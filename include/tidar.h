@@ -299,6 +299,10 @@ int tidar_debug_get_timeline(tidar_ctx *ctx, float *class_ms /*host,[TIDAR_TC_CO
  * captured ones included; all others ran as plain launches), and graphs kept at the moment (the most
  * recently used shapes, 16 at most).  Any pointer may be NULL.                            */
 int tidar_debug_graph_stats(const tidar_ctx *ctx, int64_t *captured /*host*/, int64_t *launched /*host*/, int32_t *kept /*host*/);
+/* Which way the attention of the last step or tidar_attention call went.  out[0]: CTAs that shared an item (1: none did); out[1]: whether a merge kernel for
+ * cut key ranges was launched; out[2]: query tiles whose key range the device's work plan did cut, or -1 without such a plan.  Synchronises the stream;
+ * impl 0 only. */
+int tidar_debug_attention_route(tidar_ctx *ctx, int32_t *out /*host,[3]*/);
 /* How a projection of R rows by an [N][K] matrix would be launched on a GPU of n_sms SMs (no device needed; a test hook).  swiglu: the
  * fused gate/up projection.  out[0..4]: row blocks, rows per block, K splits, work items, whether the epilogue is walked through ahead. */
 int tidar_debug_plan_projection(const tidar_config *cfg, int32_t n_sms, int32_t swiglu, int32_t R, int32_t N, int32_t K, int32_t *out /*host,[5]*/);

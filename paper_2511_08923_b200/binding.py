@@ -97,6 +97,7 @@ def load(rebuild: bool = False) -> C.CDLL:
         "tidar_debug_plan_projection": (C.c_int, [P(tidar_config), I32, I32, I32, I32, I32, P(I32)]),
         "tidar_debug_plan_norm": (C.c_int, [I32, I32, I32, I32, P(I32)]),
         "tidar_debug_plan_step": (C.c_int, [P(tidar_config), I32, P(I32), P(I32), P(I32), I32, I32, P(I32)]),
+        "tidar_debug_attention_route": (C.c_int, [ctxp, P(I32)]),
         "tidar_debug_get_timeline": (C.c_int, [ctxp, P(C.c_float), P(C.c_float), P(C.c_float)]),
     }
     for name, (res, args) in sig.items():
@@ -347,6 +348,12 @@ class Tidar:
         v = C.c_uint64(0)
         self._check(self.lib.tidar_debug_count_attention_tiles(self.ctx, int(on), C.byref(v)))
         return int(v.value)
+
+    def attention_route(self):
+        """(CTAs per item, merge kernel launched, tiles cut by the device's plan or -1): see tidar_debug_attention_route."""
+        out = np.empty(3, dtype=np.int32)
+        self._check(self.lib.tidar_debug_attention_route(self.ctx, _ip(out)))
+        return int(out[0]), bool(out[1]), int(out[2])
 
     def graph_stats(self):
         """(steps captured into a graph, steps launched as a graph, graphs kept): see tidar_debug_graph_stats."""

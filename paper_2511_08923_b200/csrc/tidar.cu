@@ -108,6 +108,7 @@ struct tidar_ctx {
   std::deque<StepGraph> graphs;      // most recently used first
   bool split_keys = true;            // attention key ranges of the current pass may be cut (see attention_plan)
   int attn_cluster = 1;              // CTAs that share an attention item of the current pass (see step_attention)
+  struct { int cluster = 1; bool merge = false; int plan_units = 0; } route;     // of the last step or stand-alone attention (tidar_debug_attention_route)
   int max_clusters[attn_tc::MAX_CLUSTER + 1] = {};      // clusters of 2, 4, 8 attention CTAs that are resident at once
   bool graphs_ok = true;             // steps can be captured on this stream (the legacy default stream refuses it)
   // On the legacy default stream a step is captured on a stream of the context's own, once its shape has been run GRAPH_AFTER times, and replayed
@@ -661,6 +662,9 @@ void launch_attention_merge(tidar_ctx *c, int tiles, const attn_tc::Args &a) {
   else launch_pdl(attn_tc::attn_combine_kernel<64, DIRECT>, blocks, 256, 0, c->stream, a, l.tl);
 }
 
+bool merges(const attn_tc::PlanArgs &p) { return p.max_items > p.n_units && p.max_pieces > 1; }
+void note_route(tidar_ctx *c, const attn_tc::PlanArgs &p) { c->route = {p.singles ? c->attn_cluster : 1, merges(p), p.n_units <= attn_tc::PLAN_UNITS ? p.n_units : 0}; }
+
 // Attention of the pass that plan p was made for (the plan itself is in device memory by then).  early: see attn_tc::Args; ahead: see attn_tc_kernel.
 void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMaps &m, const KvGeom &g, bf16 *O, bool early, bool ahead) {
   attn_tc::Args a = attention_args(c, m, g, O);
@@ -668,7 +672,7 @@ void launch_attention_tc(tidar_ctx *c, const attn_tc::PlanArgs &p, const AttnMap
   a.early = early ? 1 : 0;
   const int cluster = p.singles ? c->attn_cluster : 1;
   if (early && ahead) launch_attention_kernel<2, false, true>(c, p.max_items * p.Hkv, m, a, cluster); else launch_attention_kernel<2, false>(c, p.max_items * p.Hkv, m, a, cluster);
-  if (p.max_items > p.n_units && p.max_pieces > 1) launch_attention_merge<false>(c, 2 * p.n_units * p.Hkv, a);
+  if (merges(p)) launch_attention_merge<false>(c, 2 * p.n_units * p.Hkv, a);
 }
 
 // How a stand-alone call goes without a plan, every CTA working out its own item: streams per CTA (0 = planned) and items per query tile.
@@ -1135,6 +1139,11 @@ void capture_aside(tidar_ctx *c, const tidar_ctx::StepKey &key) {
 // launches of the same kernels.  key.units: attention units per KV head.
 int launch_step(tidar_ctx *c, tidar_ctx::StepKey key) {
   key.timeline = c->timeline; key.count_tiles = c->count_tiles;
+  if (c->cfg.impl == 0) {
+    c->split_keys = key.split; c->attn_cluster = key.cluster; c->mixed_units = key.units;
+    const int T = key.ar ? 1 : key.k * (key.k + 1);
+    note_route(c, attention_plan(c, key.mixed_R > 0 ? key.mixed_R : key.n_seqs * T, key.mixed_R > 0 ? 0 : T));
+  }
   if (!use_graphs(c)) return record_step(c, key);
   auto it = std::find_if(c->graphs.begin(), c->graphs.end(), [&](const tidar_ctx::StepGraph &g) { return g.key == key; });
   if (it == c->graphs.end()) {
@@ -1760,6 +1769,20 @@ int tidar_debug_graph_stats(const tidar_ctx *c, int64_t *captured, int64_t *laun
   return TIDAR_OK;
 }
 
+int tidar_debug_attention_route(tidar_ctx *c, int32_t *out) {
+  if (!c || !out) return TIDAR_EINVAL;
+  if (c->cfg.impl != 0) return fail(c, TIDAR_EINVAL, "tensor-core path only");
+  if (!c->inflight.empty()) return fail(c, TIDAR_EINVAL, "a step is in flight");
+  out[0] = c->route.cluster; out[1] = c->route.merge ? 1 : 0; out[2] = -1;
+  if (c->route.plan_units > 0) {
+    std::vector<attn_tc::Tile> tiles(2 * (size_t)c->route.plan_units);
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    CUDA_TRY(c, cudaMemcpy(tiles.data(), c->plan_tiles, tiles.size() * sizeof(tiles[0]), cudaMemcpyDeviceToHost));
+    out[2] = (int32_t)std::count_if(tiles.begin(), tiles.end(), [](const attn_tc::Tile &t) { return t.n_items > 1; });
+  }
+  return TIDAR_OK;
+}
+
 int tidar_debug_plan_projection(const tidar_config *cfg, int32_t n_sms, int32_t swiglu, int32_t R, int32_t N, int32_t K, int32_t *out) {
   std::string why;
   if (!cfg || !out) return fail(nullptr, TIDAR_EINVAL, "null argument");
@@ -1861,6 +1884,7 @@ int tidar_attention(tidar_ctx *c, const void *q, const void *k_pages, const void
     if (!d.streams) {                              // (launched ahead of the host's work on the tensor maps)
       c->split_keys = may_split(pages_per_seq * c->cfg.page_size); c->attn_cluster = 1;       // the lengths themselves are on the device
       plan = attention_plan(c, R, k * (k + 1));
+      note_route(c, plan);
       Launch l(c, TIDAR_TC_EMBED);
       launch_pdl(attn_meta_plan_kernel, 1 + (R + 511) / 512, 512, 0, c->stream, c->meta, seq_len, k, R, n_max, plan);
     }
@@ -1870,6 +1894,7 @@ int tidar_attention(tidar_ctx *c, const void *q, const void *k_pages, const void
       return fail(c, TIDAR_ECUDA, "cuTensorMapEncodeTiled failed for an attention operand");
     const AttnMaps am{&tq, &tk, &tv, &tkl, &tvl, 0, 0};
     if (d.streams) {
+      c->route = {d.cluster, d.pieces > 1, 0};
       attn_tc::Args a = attention_args(c, am, g, (bf16 *)out);
       a.direct.seq_len = seq_len; a.direct.k = k; a.direct.n_max = n_max; a.direct.pieces = d.pieces;
       a.direct.per_group = (k * (k + 1) + a.spt - 1) / a.spt;

@@ -125,6 +125,8 @@ def test_attention_microbench_sizes_sampled_rows(n):
 def test_attention_work_plan(ns, k):
     t = _ctx(64, 4, 2, 8, 32, 0)
     _case(t, 64, 4, 2, k, ns, 31)
+    cluster, merge, cut = t.attention_route()
+    assert cluster == 1 and (not merge or cut != 0)              # (a merge kernel comes with key ranges that were cut)
     t.close()
 
 
@@ -151,16 +153,18 @@ def test_attention_without_a_plan(hd, Hq, Hkv, k, ns, launches):
     t.close()
 
 
-@pytest.mark.parametrize("hd,Hq,Hkv,k,ns", [
-    (128, 8, 2, 1, [600]), (128, 8, 2, 4, [900, 0, 70]),           # clusters of eight, some of whose CTAs have no pages
-    (128, 12, 2, 16, [640]), (64, 4, 2, 8, [700, 1, 350, 64]),     # clusters of four, two unused rows per tile; head_dim 64
-    (128, 32, 8, 16, [1000]), (64, 8, 8, 16, [900]),               # clusters of two; one head per KV head
+@pytest.mark.parametrize("hd,Hq,Hkv,k,ns,size", [
+    (128, 8, 2, 1, [600], 8), (128, 8, 2, 4, [900, 0, 70, 320], 8),       # some tiles are not shared; six pages: CTAs of a sharing cluster without any
+    (128, 12, 2, 16, [640], 4), (64, 4, 2, 8, [700, 1, 350, 64], 4),      # two unused rows per tile; head_dim 64
+    (128, 32, 8, 16, [1000], 2), (64, 8, 8, 16, [900], 4),                # one head per KV head
+    (128, 32, 8, 16, [700], 1), (128, 8, 2, 4, [200], 1),                 # clusters would crowd the chip for little; too few pages
 ])
-def test_attention_shared_by_clusters(hd, Hq, Hkv, k, ns):
+def test_attention_shared_by_clusters(hd, Hq, Hkv, k, ns, size):
     t = _ctx(hd, Hq, Hkv, k, len(ns), 0)
     before = t.launch_count()
     _case(t, hd, Hq, Hkv, k, ns, 61)
     assert t.launch_count() - before == 1
+    assert t.attention_route() == (size, False, -1)
     t.close()
 
 

@@ -533,18 +533,25 @@ def test_default_stream_replays_a_shape_that_recurs():
 
 
 def test_timeline_of_a_replayed_step_is_its_own():
-    """Two kept graphs with different launch lists (a long context adds the merge of split key ranges in every layer): replaying the first
-    after the second was recorded still attributes every launch of the first to its class."""
+    """Two kept graphs with different launch lists (a long context among thirty sequences, too many for clusters, adds the merge of cut key ranges in every
+    layer): replaying the first after the second was recorded still attributes every launch of the first to its class."""
     sh, wt = make_model("tiny")
-    t = _gpu(sh, wt, 0, debug=0, max_batch=2, max_seq_len=1024, stream=torch.cuda.Stream())
-    t.prefill(0, prompt_ids(sh, 64), sh.k)
-    t.prefill(1, prompt_ids(sh, 900), sh.k)
+    n_seqs = 30
+    t = _gpu(sh, wt, 0, debug=0, max_batch=n_seqs, max_seq_len=1088, stream=torch.cuda.Stream())
+    for q in range(n_seqs):
+        t.prefill(q, prompt_ids(sh, 1000 if q == n_seqs - 1 else 20 + q), sh.k)
     t.set_timeline(True)
-    for seq in (0, 1, 0, 1, 0):
-        t.step([seq])
+    launches = {}
+    for seqs in ([0], list(range(n_seqs)), [0], list(range(n_seqs)), [0]):
+        before = t.launch_count()
+        t.step(seqs)
+        launches.setdefault(len(seqs), set()).add(t.launch_count() - before)
+        cluster, merge, cut = t.attention_route()
+        assert cluster == 1 and (merge, cut > 0) == ((False, False) if len(seqs) == 1 else (True, True))
         tl = t.timeline()
-        assert all(tl[c] > 0 for c in ("embed", "norm", "gemm", "rope", "attn", "lmhead", "verify")), (seq, tl)
+        assert all(tl[c] > 0 for c in ("embed", "norm", "gemm", "rope", "attn", "lmhead", "verify")), (seqs, tl)
         assert tl["busy"] == pytest.approx(sum(v for c, v in tl.items() if c not in ("busy", "span")), rel=1e-4)
+    assert t.graph_stats() == (2, 5, 2) and all(len(x) == 1 for x in launches.values()) and launches[1] != launches[n_seqs]
     _close(t)
 
 
