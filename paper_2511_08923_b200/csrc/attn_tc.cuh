@@ -147,10 +147,11 @@ static_assert(sizeof(Ctl) <= 512, "control block must fit its slot");
 // grids take the same figures, although a page costs them less: they were not fitted, and cuts come out somewhat finer than best.)
 constexpr float CLUSTER_MERGE = 2.f;                   // what sharing an item within a cluster adds
 // A stand-alone call is launched in clusters for the width of its page table, which is all the host knows; a tile whose own pages (known on the device) are
-// few is its cluster's first CTA's alone.  Shared where that takes at least CLUSTER_SAVES pages off the longest CTA (five SINGLE_PAGE: just above what
-// sharing costs).  Alone / shared, tables of 8 to 16 pages: 32/8 heads of 128, k = 4, clusters of eight, 2 pages per tile 6.9 / 8.1 us, 5 pages 7.9 / 8.3, 6 pages
-// 8.9 / 8.5; 12/2 heads, k = 16, clusters of four, 2 pages 7.9 / 9.8, 6 pages 10.4 / 10.3, 10 pages 12.3 / 10.8.  (A step's sizes are known on the host.)
-constexpr int CLUSTER_SAVES = 5;
+// few is its cluster's first CTA's alone.  Shared where that takes at least CLUSTER_SAVES pages off the longest CTA (four SINGLE_PAGE: what sharing costs).
+// Alone / shared, tables of 8 to 16 pages: 32/8 heads of 128, k = 4, clusters of eight, 2 pages per tile 7.2 / 8.1 us, 5 pages 7.9 / 8.4, 6 pages 8.9 / 8.4;
+// 12/2 heads, k = 16, clusters of four, 2 pages 8.0 / 9.8, 5 pages 9.9 / 10.2, 6 pages 10.4 / 10.3; 4/2 heads of 64, k = 4, 6 pages 7.7 / 6.9.  (A step's sizes
+// are known on the host.)
+constexpr int CLUSTER_SAVES = 4;
 __host__ __device__ constexpr bool cluster_shares(int n_pages, int log_size) { return n_pages - ((n_pages + (1 << log_size) - 1) >> log_size) >= CLUSTER_SAVES; }
 constexpr float OVERHEAD = 5.f, PAIR_PAGE = 1.05f, SINGLE_PAGE = 0.56f, PAIR_STORE = 2.5f, SINGLE_STORE = 1.5f, MERGE = 3.f;
 constexpr int PLAN_UNITS = 256;                        // up to this many units are planned; beyond, every unit is one item
@@ -162,8 +163,12 @@ struct PlanCost { int items, live, most; float sum, longest; };
 __host__ __device__ inline float plan_limit(float longest, int i) { return fmaxf(longest / (1.f + 0.5f * i), 0.1f) * 1.0001f; }
 __host__ __device__ inline int plan_pieces(float us, float limit, bool dbl) {
   const float n = us / limit, pages = us * (dbl ? 1.0001f / PAIR_PAGE : 1.0001f / SINGLE_PAGE);
-  const int up = (int)n + ((float)(int)n < n ? 1 : 0);
-  return up < (int)pages ? up : (int)pages;
+#ifdef __CUDA_ARCH__
+  return (int)fminf(ceilf(n), pages);
+#else
+  const int up = (int)n + ((float)(int)n < n ? 1 : 0);           // (the same without a library call)
+  return std::min(up, (int)pages);
+#endif
 }
 __host__ __device__ inline void plan_add(PlanCost &c, float us, float limit, bool dbl, int times = 1) {
   const int k = plan_pieces(us, limit, dbl);
@@ -359,6 +364,40 @@ __device__ __forceinline__ Item direct_item(const Args &a, int e) {
   return it;
 }
 
+// The end of a tile that its cluster does not share: both streams' halves merged and written.  A function of its own, called, so that its code does not
+// lie in the way of shared tiles (in place it cost them 0.1 - 0.2 us, as branches in their loop 0.3).
+template <int HD>
+__device__ __noinline__ void finish_alone(uint32_t o_addr, int t, int my_row, float m_ref, float l_run, int nj, bf16 *o, const float4 *xo, const float2 *xml) {
+  const float2 other = xml[(1 - t) * 128 + my_row];
+  const float M = fmaxf(m_ref, other.x);
+  const float wm = m_ref == -INFINITY ? 0.f : exp2f(m_ref - M), wo = other.x == -INFINITY ? 0.f : exp2f(other.x - M);
+  const float inv = 1.f / (wm * l_run + wo * other.y);
+#pragma unroll 1
+  for (int c = 0; c < HD / 2; c += 32) {
+    uint32_t w[32];
+    float v[32];
+    if (nj > 0) { sm100::tmem_ld32(o_addr + t * (HD / 2) + c, w); sm100::tmem_wait_ld(); }
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = nj > 0 ? __uint_as_float(w[i]) : 0.f;
+#pragma unroll
+    for (int i = 0; i < 32; i += 4) {
+      const float4 x = xo[(t * (HD / 8) + (c + i) / 4) * 128 + my_row];
+      v[i] = wm * v[i] + wo * x.x; v[i + 1] = wm * v[i + 1] + wo * x.y; v[i + 2] = wm * v[i + 2] + wo * x.z; v[i + 3] = wm * v[i + 3] + wo * x.w;
+    }
+    if (o) {
+#pragma unroll
+      for (int i = 0; i < 32; i += 8) {
+        uint4 u;
+        __nv_bfloat162 h0 = __floats2bfloat162_rn(v[i] * inv, v[i + 1] * inv), h1 = __floats2bfloat162_rn(v[i + 2] * inv, v[i + 3] * inv),
+                       h2 = __floats2bfloat162_rn(v[i + 4] * inv, v[i + 5] * inv), h3 = __floats2bfloat162_rn(v[i + 6] * inv, v[i + 7] * inv);
+        u.x = *reinterpret_cast<uint32_t *>(&h0); u.y = *reinterpret_cast<uint32_t *>(&h1);
+        u.z = *reinterpret_cast<uint32_t *>(&h2); u.w = *reinterpret_cast<uint32_t *>(&h3);
+        *reinterpret_cast<uint4 *>(o + t * (HD / 2) + c + i) = u;
+      }
+    }
+  }
+}
+
 // STREAMS = 1: one tile and one stream per CTA and two CTAs per SM, which fill each other's latencies as two streams do.  It serves calls that are
 // one wave that way and two otherwise (see attention_direct for both sides' figures).  DIRECT: no plan, see direct_item.
 // AHEAD (decode steps of few rows, whose CTAs become resident well before the RoPE kernel ends): what does not depend on that kernel is done ahead of
@@ -439,7 +478,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
   const int t = (warp - 4) >> 2;                         // softmax warps: stream
   const int my_row = (warp & 3) * 32 + lane;             // and this thread's MMA row = TMEM lane
   int my_slot = -1;                                      // and its slot, -1: none
-  const int c_cols = HD / 2 >> c_log, c_shift = 31 - __clz(c_cols);     // columns of a stream's half that a CTA of the cluster finishes (at least 8)
+  const int c_cols = (HD / 2) >> c_log, c_shift = 31 - __clz(c_cols);     // columns of a stream's half that a CTA of the cluster finishes (at least 8)
   if (warp == 0 || warp == 3) {
     // ===================== K producer / Q and V producer =====================
     // Lane i holds the i-th entry of a group of 32 entries of the page table, so that a page's load does not wait for
@@ -734,28 +773,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         }
       }
       sm100::named_bar_sync(13, 256);
-      if (ok) {
+      if (ok && (!CLUSTER || sharing)) {
         const float2 other = xml[(1 - t) * 128 + my_row];
         const float M = fmaxf(m_ref, other.x);
         const float wm = m_ref == -INFINITY ? 0.f : exp2f(m_ref - M), wo = other.x == -INFINITY ? 0.f : exp2f(other.x - M);
-        const float l = wm * l_run + wo * other.y, inv = (CLUSTER && sharing) || item.split ? 1.f : 1.f / l;
-        if (CLUSTER && DIRECT && __builtin_expect(!sharing, 0)) {       // (a short loop of its own, out of the way: as branches in the one below it cost shared tiles 0.3 us)
-#pragma unroll 1
-          for (int c = 0; c < HD / 2; c += 32) {
-            float v[32];
-            if (nj > 0) load32(t * (HD / 2) + c, v);
-            else {
-#pragma unroll
-              for (int i = 0; i < 32; ++i) v[i] = 0.f;
-            }
-#pragma unroll
-            for (int i = 0; i < 32; i += 4) {
-              const float4 x = xo[(t * (HD / 8) + (c + i) / 4) * 128 + my_row];
-              v[i] = wm * v[i] + wo * x.x; v[i + 1] = wm * v[i + 1] + wo * x.y; v[i + 2] = wm * v[i + 2] + wo * x.z; v[i + 3] = wm * v[i + 3] + wo * x.w;
-            }
-            write32(v, t * (HD / 2) + c, inv);
-          }
-        } else {
+        const float l = wm * l_run + wo * other.y, inv = CLUSTER || item.split ? 1.f : 1.f / l;
 #pragma unroll
         for (int c = 0; c < HD / 2; c += 32) {
           float v[32];
@@ -788,7 +810,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ 
         } else {
           if (t == 0 && my_slot >= 0 && item.split) a.part_ml[part * 128 + my_row] = make_float2(M, l);
         }
-        }
+      }
+      if constexpr (CLUSTER && DIRECT) {
+        if (ok && !sharing) finish_alone<HD>(o_addr, t, my_row, m_ref, l_run, nj, my_slot < 0 ? nullptr : o, xo, xml);
       }
     }
   }

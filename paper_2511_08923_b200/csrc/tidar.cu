@@ -698,10 +698,7 @@ DirectPlan attention_direct(const tidar_ctx *c, int n_seqs, int k, int n_pages) 
     DirectPlan pick{2, 1, 1};
     float best = n_pages * attn_tc::SINGLE_PAGE - 0.3f;
     for (int size = 2; size <= attn_tc::MAX_CLUSTER && size * 16 <= c->cfg.head_dim; size *= 2) {
-      // (Clusters on more than three quarters of the SMs leave the next call no room to start in, which short sequences under a wide table feel most: 144
-      // CTAs, 2 pages per tile 8.8 us instead of 8.2, where the full table's 13 pages would save only 0.2.  104 CTAs: 7.9 either way.)
-      const float crowd = 4 * tiles * size > 3 * c->n_sms ? 1.1f : 0.f;
-      const float t = (n_pages + size - 1) / size * attn_tc::SINGLE_PAGE + attn_tc::CLUSTER_MERGE + crowd;
+      const float t = (n_pages + size - 1) / size * attn_tc::SINGLE_PAGE + attn_tc::CLUSTER_MERGE;
       if (tiles <= c->max_clusters[size] && t < best) { best = t; pick.cluster = size; }
     }
     return pick;

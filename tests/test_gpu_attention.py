@@ -157,7 +157,7 @@ def test_attention_without_a_plan(hd, Hq, Hkv, k, ns, launches):
     (128, 8, 2, 1, [600], 8), (128, 8, 2, 4, [900, 0, 70, 320], 8),       # some tiles are not shared; six pages: CTAs of a sharing cluster without any
     (128, 12, 2, 16, [640], 4), (64, 4, 2, 8, [700, 1, 350, 64], 4),      # two unused rows per tile; head_dim 64
     (128, 32, 8, 16, [1000], 2), (64, 8, 8, 16, [900], 4),                # one head per KV head
-    (128, 32, 8, 16, [700], 1), (128, 8, 2, 4, [200], 1),                 # clusters would crowd the chip for little; too few pages
+    (128, 32, 8, 16, [400], 1), (128, 8, 2, 4, [200], 1),                 # too few pages
 ])
 def test_attention_shared_by_clusters(hd, Hq, Hkv, k, ns, size):
     t = _ctx(hd, Hq, Hkv, k, len(ns), 0)
@@ -169,7 +169,7 @@ def test_attention_shared_by_clusters(hd, Hq, Hkv, k, ns, size):
 
 
 @pytest.mark.parametrize("hd,Hq,Hkv,k,lens", [
-    (128, 32, 8, 4, [200]), (128, 32, 8, 16, [100]), (128, 12, 2, 16, [200]), (64, 4, 2, 8, [0, 50, 100, 200]),     # clusters of eight, two, four, eight
+    (128, 32, 8, 4, [100]), (128, 32, 8, 16, [100]), (128, 12, 2, 16, [200]), (64, 4, 2, 8, [0, 50, 100, 200]),     # clusters of eight, two, four, eight
 ])
 def test_a_page_table_wider_than_the_lengths_changes_nothing(hd, Hq, Hkv, k, lens):
     """Short sequences under a table wide enough for a call to be launched in clusters: bit for bit what the narrow table gives, for a tile of few pages
