@@ -413,7 +413,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // warps have nothing to do while the first item's MMAs run, so they first walk through the
     // epilogue once with every store and barrier operation switched off (dry), which
     // brings the code in; g.warm_epilogue is a run-time value so that both walks share one copy.
-    // Slabs and additions to the residual stream of the pair instances are walked through as well, where every worker has one item (see plan_gemm): 272 rows x 128 features leave a CTA in 3.6 - 3.9 us
+    // Slabs and additions to the residual stream of the pair instances are walked through as well, where every worker has one item that is long enough (see plan_gemm): 272 rows x 128 features leave a CTA in 3.6 - 3.9 us
     // then (4.6 - 6.4 before; 3.4 in a kernel that does nothing else, 28 B per cycle: the SM's port, whatever the instruction).  That walk
     // starts a little later, for the role warps' first rounds fetch code too (started at once, the first stage landed 0.3 us later).  Turning them
     // into a short loop over tensor memory instead was slower (8.3 us): a store holds its register until the port takes it.

@@ -391,8 +391,11 @@ gemm_tc::Args plan_gemm(const tidar_ctx *c, int mode, int R, int N, int K, int f
   // Partial sums and additions to the residual stream are walked through ahead (see the kernel) where every worker has one item: its store is then the
   // end of the launch.  With more, the first item's store runs beside the second's main loop and fetches the code for the last, and a walk
   // only costs.  (Down projection of the 1.5B class, launches timed one by one: 1400 rows, 72 items on 74 workers, 37.3 us without and 35.7 with;
-  // 1776 rows, 126 items, 45.7 and 47.6.)
-  a.warm_epilogue = mode != gemm_tc::MODE_SLAB || a.total_items() <= workers;
+  // 1776 rows, 126 items, 45.7 and 47.6.)  And where the main loop, 2.15 cycles per row + 50 and K block at 1.75 GHz, is longer than the nap and the walk
+  // leave behind: 16 K blocks of 272 rows and 24 of 160 gain, 12 of 208 (3.4 us) lose 0.3 us, 8 of 208 0.9, and a first pass of the tiny model, 4 and 11 K
+  // blocks, 168 -> 176 us.
+  const float loop_us = (float)((a.kb_total + a.S - 1) / a.S) * (2.15f * a.rb_rows + 50.f) / 1750.f;
+  a.warm_epilogue = mode != gemm_tc::MODE_SLAB || (a.total_items() <= workers && loop_us >= 4.f);
   return a;
 }
 

@@ -27,7 +27,7 @@ def _projections(model):
 
 
 @pytest.mark.parametrize("model", list(SHAPES))
-def test_epilogues_are_walked_through_only_ahead_of_a_workers_single_item(model):
+def test_epilogues_are_walked_through_only_ahead_of_a_workers_single_long_item(model):
     lib, out, seen = binding.load(), np.zeros(5, dtype=np.int32), set()
     for R in (1, 20, 96, 97, 272, 288, 289, 600, 1152, 1400, 1776, 2047, 4112):
         for swiglu, N, K in _projections(model):
@@ -36,9 +36,12 @@ def test_epilogues_are_walked_through_only_ahead_of_a_workers_single_item(model)
             small = R <= 96 or (not swiglu and R <= 288 and N * K <= 15_000_000)
             assert n_rb * rb_rows >= R and 1 <= S <= 8
             if not swiglu:
-                assert bool(walked) == (items <= (N_SMS if small else N_SMS // 2)), (R, N, K, out)
+                if small:
+                    continue                             # (their epilogue is never walked through)
+                loop = -(-(K // 64) // S) * (2.15 * rb_rows + 50) / 1750          # us
+                assert abs(loop - 4) < 1e-3 or bool(walked) == (items <= N_SMS // 2 and loop > 4), (R, N, K, out)
                 seen.add(walked)
-    assert seen == {0, 1} or model == "tiny"
+    assert seen == ({0} if model == "tiny" else {0, 1})
     assert lib.tidar_debug_plan_projection(None, N_SMS, 0, 1, 64, 64, binding._ip(out)) == -1
     assert lib.tidar_debug_plan_projection(C.byref(_cfg(model)), 0, 0, 1, 64, 64, binding._ip(out)) == -1
 
